@@ -204,10 +204,12 @@ int zipml_quantize_draw(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
     uint32_t* keys = cv.take<uint32_t>(2 * (size_t)n);
     float* inv = cv.take<float>((size_t)n);
     float* step_tmp = cv.take<float>((size_t)n);
-    rc = launch_column_range(ctx, A, m, n, lda, s, grid == ZIPML_GRID_SYMMETRIC, keys, feat_lo, nullptr, inv,
-                             feat_step ? feat_step : step_tmp);
-    if (rc != ZIPML_OK) return rc;
-    return launch_quantize(ctx, A, m, n, lda, bits, level_mode, feat_lo, inv, levels, seed, draw, plane1, plane2, row_bytes);
+    float* step = feat_step ? feat_step : step_tmp;
+    if (level_mode == ZIPML_LEVELS_UNIFORM) {
+        rc = launch_column_range(ctx, A, m, n, lda, s, grid == ZIPML_GRID_SYMMETRIC, keys, feat_lo, nullptr, inv, step);
+        if (rc != ZIPML_OK) return rc;
+    }
+    return launch_quantize(ctx, A, m, n, lda, bits, level_mode, feat_lo, inv, levels, seed, draw, plane1, plane2, row_bytes, keys, feat_lo, step);
 }
 
 int zipml_optimal_levels(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int32_t bits,

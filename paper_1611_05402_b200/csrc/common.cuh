@@ -50,28 +50,12 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
     return out;
 }
 
-// Random block of the sample feature pair (2p, 2p+1) of row `row`: words {2p copy 1, 2p copy 2,
-// 2p+1 copy 1, 2p+1 copy 2}; the top 24 bits of a word are the uniform integer.
-// `draw` numbers further independent pairs of quantizations of the same samples (0: the two samples of the SGD path).
-__device__ __forceinline__ Philox4 sample_block(uint64_t seed, uint64_t row, uint32_t pair, uint32_t draw) {
-    return philox4x32_10((uint32_t)row, (uint32_t)(row >> 32), pair, draw, (uint32_t)seed, (uint32_t)(seed >> 32));
-}
-
 // Uniform 24-bit integer for coordinate `coord` of the model (stream 3) / gradient (stream 4)
 // quantizer at (epoch, step).
 __device__ __forceinline__ uint32_t vector_u24(uint64_t seed, uint32_t epoch, uint32_t step, uint32_t coord,
                                                uint32_t stream) {
     const Philox4 b = philox4x32_10(coord >> 2, step, epoch, stream, (uint32_t)seed, (uint32_t)(seed >> 32));
     return b.v[coord & 3u] >> 8;
-}
-
-// up <=> u24 * 2^-24 < p, both sides fp32 (the product is exact).  Since u24 is an integer below 2^24 and
-// p * 2^24 is exact in fp32, that is u24 < ceil(p * 2^24): the threshold is computed once per element (one
-// conversion; int <-> float conversions issue at a sixteenth of the FMA rate) and compared as integers for
-// both copies.  p <= 0 or NaN gives 0 (never up), p >= 1 gives at least 2^24 (always up).
-__device__ __forceinline__ uint32_t up_threshold(float p) { return __float2uint_ru(__fmul_rn(p, 16777216.0f)); }
-__device__ __forceinline__ uint32_t round_up_if(uint32_t cell, uint32_t threshold, uint32_t word) {
-    return cell + ((word >> 8) < threshold ? 1u : 0u);
 }
 
 // Cell and up-probability on a uniform grid of s intervals (s < 2^22): t = (v - lo) * inv with every

@@ -67,9 +67,11 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
                         uint32_t* key_scratch /* 2n */, float* lo_out, float* hi_out, float* inv_out,
                         float* step_out);
 
+// Uniform levels: on the grid (lo, inv) that launch_column_range has found.  Level tables: lo, inv unused; the range is
+// found on the way (2n keys of scratch) and lo_out, step_out written as launch_column_range would.
 int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bits, int level_mode,
                     const float* lo, const float* inv, const float* levels, uint64_t seed, uint32_t draw, uint8_t* plane1,
-                    uint8_t* plane2, int64_t row_bytes);
+                    uint8_t* plane2, int64_t row_bytes, uint32_t* key_scratch, float* lo_out, float* step_out);
 int launch_code_weights(zipml_ctx* ctx, const zipml_dataset* d, const float* x, float* wtab, double* base);
 int launch_poly_rows(zipml_ctx* ctx, const zipml_dataset* d, const uint8_t* const* planes, int degree, const double* coef,
                      const float* wtab, const double* base, const float* scale, double* rows_out);

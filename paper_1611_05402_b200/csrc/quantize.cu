@@ -1,6 +1,8 @@
 // Column range scan and the quantize + pack kernel (paper Section 2.1; Supplement "Randomized
 // Quantization" and "Column Scaling"): two independent unbiased stochastic roundings of every
 // sample element onto its feature's level grid, written as two bit-packed planes.
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -178,205 +180,414 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 }
 
 // ---------------------------------------------------------------------------------------------
-// Quantize + pack.  A thread owns one 32-bit word column of the planes (FPW = 32/CB consecutive
-// features) for kQuantRows consecutive rows: the features' lo and inv are loaded once, the rows'
-// Philox chains are independent and overlap.  Per row it reads the FPW samples as float4s when the
-// row is 16-byte aligned, decides cell and up-probability in pinned fp32 arithmetic, draws one
-// Philox block per feature pair (four words = two features x two copies) and writes the two
-// words.  A pair whose up-probabilities are all 0 or 1 (values on a level: the zeros of sparse
-// rows, the column extremes) needs no random numbers -- the comparison u * 2^-24 < p is decided
-// without them -- and skips its Philox block; the codes are the same.  Words past the last
-// feature are written as zero so that the planes are fully defined.
-// Level tables: the block's tables are staged in shared memory as [level][feature slot of the
-// word][word column], so that the lanes of a warp (consecutive word columns) read consecutive
-// addresses; read from global memory, where the tables of neighbouring lanes lie FPW * L floats
-// apart, every look-up took 32 cache lines per warp and the kernel ran at a tenth of this rate.
+// Quantize + pack.  A thread owns four consecutive features (8, 16 or 32 bits of a plane's row) and kQuantRows
+// consecutive rows per pass: the features' lo and inv are loaded once, the rows' loads and Philox chains are
+// independent and overlap, and the next pass's samples are on their way while this pass draws.
+//   Cell and threshold.  With t = (v - lo) * inv rounded as the grid prescribes, tc = clamp(t, 0, s) and
+//     r = 2^23 + tc rounded down, the cell is the low byte of r, and 2^24 * p = 2^24 * (tc - floor tc) comes out of
+//     two exact FMAs; up <=> (word >> 8) < ceil(2^24 p) <=> word < ceil(2^24 p) << 8, so the draws are compared as
+//     they are (u24 * 2^-24 < p is exact in fp32, u24 an integer; p <= 0 or NaN: never up).  t >= s lands in code s
+//     with p = 0: no special case for the upper end.
+//   Draws.  One Philox block serves a feature pair: counter (row, row's upper half, pair, draw), words {first feature copy
+//     1, copy 2, second feature copy 1, copy 2}, the top 24 bits of a word the uniform integer.  The round keys depend on
+//     the seed alone and arrive as kernel parameters (an operand of the xor).  The 32 x 32 -> 64-bit products are what
+//     the rounds cost (half of the FMA pipe takes them): of the first two rounds' four, two depend only on the pair
+//     (kept for the thread's life) and two only on the row (shared by the thread's pairs): 17 a block, not 20.
+//   Sparse rows.  A pair whose two values are their features' lowest level has code 0 in both planes for certain.
+//     Where at most a quarter of a warp's pairs are anything else (5 % non-zeros: a tenth), the lanes put those in a
+//     queue in shared memory and share them out evenly -- cell, threshold, draw and all, one round per 512 elements
+//     instead of 16 per lane -- each answer or-ed into its owner's words.
+// Level tables: the block's tables are staged in shared memory as [level][feature of the thread][thread column], so
+// that a warp's look-ups are free of bank conflicts whatever its codes are; the cell is found by bisection and p by a
+// multiplication with the staged reciprocal of the cell's width, corrected (quotient below).  Such a call
+// needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
+// non-finite values, are gathered on the way.
+// What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 63 %; 24 warps per SM: fewer
+// registers per thread spill, more leave too few warps); sparse rows, issue slots and DRAM together.
+// Measured, whole call with the range pass, before -> now: 100,003 x 1,001 at 8 bits 395 -> 278 us, 65,536 x 32,768 of
+// 5 % non-zeros at 4 bits 6,127 -> 3,639 us; 500,000 x 512 on 3-bit tables 1,520 -> 890 us (no range pass any more).
 // ---------------------------------------------------------------------------------------------
-constexpr int kQuantRows = 4;          // rows per thread and pass
-constexpr int kQuantTableCols = 64;    // word columns per block with level tables (shared memory: L * FPW * 64 floats)
+constexpr int kQuantRows = 4;                  // rows per thread and pass
+constexpr int kQuantTableCols = 64;            // thread columns per block with level tables
+constexpr int kQuantQueue = 64;                // pairs that a warp shares out (of the 256 of a pass); more: each lane does its own
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 
-template <int CB, bool TABLE>
-__global__ void __launch_bounds__(256) quantize_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda,
-                                                       int bits, const float* __restrict__ lo,
-                                                       const float* __restrict__ inv, const float* __restrict__ levels,
-                                                       uint64_t seed, uint32_t draw, uint32_t* __restrict__ plane1,
-                                                       uint32_t* __restrict__ plane2, int64_t row_words, bool vec_ok,
-                                                       int passes) {
-    constexpr int FPW = 32 / CB;
-    extern __shared__ float lev_s[];                               // TABLE: [L][FPW][blockDim.x]
-    // blockDim = (word columns, row groups); blockIdx.x runs over the rows, blockIdx.y over the columns
-    const int64_t q = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    const int L = 1 << bits, s = L - 1;
+struct PhiloxKeys {                            // the ten round keys of one seed
+    uint32_t k0[10], k1[10];
+};
+
+static PhiloxKeys philox_keys(uint64_t seed) {
+    PhiloxKeys k;
+    uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
+    for (int r = 0; r < 10; ++r) { k.k0[r] = a; k.k1[r] = b; a += 0x9E3779B9u; b += 0xBB67AE85u; }
+    return k;
+}
+
+// Rounds FIRST .. 9 of philox4x32_10() with its key schedule given.
+template <int FIRST>
+__device__ __forceinline__ Philox4 philox_rounds(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const PhiloxKeys& key) {
+#pragma unroll
+    for (int r = FIRST; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)kPhiloxM0 * c0, p1 = (uint64_t)kPhiloxM1 * c2;
+        c0 = (uint32_t)(p1 >> 32) ^ c1 ^ key.k0[r];
+        c1 = (uint32_t)p1;
+        c2 = (uint32_t)(p0 >> 32) ^ c3 ^ key.k1[r];
+        c3 = (uint32_t)p0;
+    }
+    Philox4 out;
+    out.v[0] = c0; out.v[1] = c1; out.v[2] = c2; out.v[3] = c3;
+    return out;
+}
+
+// Integer steps of the kernel below, worded so that they run on the ALU pipe: the Philox products fill the half of the
+// FMA pipe that integer multiplies share, and left to itself the compiler puts shifts and additions there too.
+template <int S>
+__device__ __forceinline__ uint32_t shift_left(uint32_t v) {
+    uint32_t d;
+    if constexpr (S == 8) asm("prmt.b32 %0, %1, 0, 0x2104;" : "=r"(d) : "r"(v));
+    else asm("shf.l.wrap.b32 %0, 0, %1, %2;" : "=r"(d) : "r"(v), "n"(S));
+    return d;
+}
+template <uint32_t BIT>
+__device__ __forceinline__ void set_if_below(uint32_t& word, uint32_t a, uint32_t b) {
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}" : "+r"(word) : "r"(a), "r"(b), "n"(BIT));
+}
+
+// Four codes (in the low bits of each word, anything above) side by side, CB bits each; what lies above is undefined.
+template <int CB>
+__device__ __forceinline__ uint32_t pack_codes(const uint32_t (&c)[4]) {
+    if constexpr (CB == 8) return __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+    else {
+        constexpr uint32_t kMask = (1u << CB) - 1u;
+        return (c[0] & kMask) | shift_left<CB>(c[1] & kMask) | shift_left<2 * CB>(c[2] & kMask) | shift_left<3 * CB>(c[3]);
+    }
+}
+
+__device__ __noinline__ float divide_slowly(float num, float width) { return __fdiv_rn(num, width); }
+
+// num / width rounded to nearest, from rw = 1 / width rounded to nearest: two residual corrections (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990: a faithful quotient corrected once with the
+// correctly rounded reciprocal is the correctly rounded quotient, where nothing underflows).  rw = 0 stands for a
+// width of 0 (quotient 0), rw < 0 for widths outside [2^-40, 2^40]: the quotient comes out negative.  The caller
+// divides instead where the quotient of a positive num is below 2^-60: the residuals of the others are multiples of
+// 2^(-60 - 23 - 40 - 23) and cannot underflow.
+// Compared with CUDA's division on 2 x 10^10 pairs (widths 2^-40 .. 2^40, quotients 2^-60 .. 2): equal.
+__device__ __forceinline__ float quotient(float num, float width, float rw) {
+    float q = __fmul_rn(num, rw);
+    q = __fmaf_rn(__fmaf_rn(-q, width, num), rw, q);
+    return __fmaf_rn(__fmaf_rn(-q, width, num), rw, q);
+}
+
+template <int CB> struct QuantWord;
+template <> struct QuantWord<8> { using type = uint32_t; };
+template <> struct QuantWord<4> { using type = uint16_t; };
+template <> struct QuantWord<2> { using type = uint8_t; };
+
+// TB: 0 for a uniform grid of `bits` bits, else the bits of the level table.
+template <int CB, int TB>
+__global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda, int bits,
+                                                          const float* __restrict__ lo, const float* __restrict__ inv,
+                                                          const float* __restrict__ levels, uint32_t* lo_key, uint32_t* hi_key,
+                                                          DeviceStatus* status, const PhiloxKeys key, uint32_t draw,
+                                                          uint8_t* __restrict__ plane1, uint8_t* __restrict__ plane2, int64_t row_bytes,
+                                                          bool vec_ok, int passes, unsigned col_blocks, unsigned row_blocks) {
+    using Word = typename QuantWord<CB>::type;
+    constexpr bool TABLE = TB > 0;
+    constexpr int L = 1 << TB;                                     // TABLE: levels
+    __shared__ float4 val_s[8][kQuantRows][32];                    // samples of a warp's pass: [row][lane]
+    __shared__ __align__(16) uint32_t word_s[8][32][2 * kQuantRows];  // and its words: [lane][row][plane]
+    __shared__ uint8_t queue_s[8][kQuantQueue];                    // pairs to do: lane * 8 + row * 2 + pair
+    extern __shared__ float4 cell_s[];                             // TABLE: [L][4][tx] level, width of its cell, 1 / width, cell
+    const int tx = blockDim.x, tid = threadIdx.y * tx + threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* lev_s = reinterpret_cast<float*>(cell_s + L * 4 * tx);  // TABLE: [L][4][tx] levels
+    const unsigned row_block = blockIdx.x / col_blocks, col_block = blockIdx.x - row_block * col_blocks;
+    const int64_t g = (int64_t)col_block * tx + threadIdx.x;       // this thread's group of four features
+    const int64_t groups = row_bytes * 8 / (4 * CB);
+    const int64_t j0 = g * 4;
+    const int nf = (int)max((int64_t)0, min((int64_t)4, n - j0));  // real features of the group (0: padding)
     if constexpr (TABLE) {
-        const int tx = blockDim.x, nthreads = blockDim.x * blockDim.y, tid = threadIdx.y * blockDim.x + threadIdx.x;
-        const int64_t jb = (int64_t)blockIdx.y * tx * FPW;         // first feature of the block
-        // consecutive threads read consecutive floats of the n x L table
-        for (int idx = tid; idx < tx * FPW * L; idx += nthreads) {
-            const int f = idx / L, k = idx - f * L;                // feature within the block, level
-            const float val = (jb + f < n) ? __ldg(levels + (jb + f) * L + k) : 0.0f;
-            lev_s[(k * FPW + (f % FPW)) * tx + f / FPW] = val;
+        const int64_t jb = (int64_t)col_block * tx * 4;            // first feature of the block
+        for (int idx = tid; idx < tx * 4 * L; idx += 256) {        // consecutive threads read consecutive floats of the table
+            const int f = idx / L, k = idx - f * L;
+            const bool have = jb + f < n;
+            const float val = have ? __ldg(levels + (jb + f) * L + k) : 0.0f;
+            const float next = have && k < L - 1 ? __ldg(levels + (jb + f) * L + k + 1) : val;
+            const float width = __fsub_rn(next, val);
+            const float rw = !(width > 0.0f) ? 0.0f : (width >= 9.1e-13f && width <= 1.09e12f) ? __frcp_rn(width) : -1.0f;
+            const int at = (k * 4 + (f & 3)) * tx + (f >> 2);
+            lev_s[at] = k < L - 1 ? val : INFINITY;
+            cell_s[at] = make_float4(val, width, rw, __int_as_float(k));
         }
         __syncthreads();
     }
-    if (q >= row_words) return;
-    const int64_t j0 = q * FPW;
-    const int nf = (int)min((int64_t)FPW, n - j0);                 // real features of this word (<= 0: padding only)
-    float flo[TABLE ? 1 : FPW], finv[TABLE ? 1 : FPW];
-    if constexpr (!TABLE) {
+    // the value that has code 0 for certain: the lowest level (level tables: unless it is there twice)
+    float flo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, finv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float seen_lo[4], seen_hi[4], probe = 0.0f;                    // TABLE: the extremes of this thread's rows; NaN once a value is not finite
 #pragma unroll
-        for (int i = 0; i < FPW; ++i) {
-            flo[i] = i < nf ? __ldg(lo + j0 + i) : 0.0f;
-            finv[i] = i < nf ? __ldg(inv + j0 + i) : 0.0f;
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (!TABLE) {
+            if (i < nf) { flo[i] = __ldg(lo + j0 + i); finv[i] = __ldg(inv + j0 + i); }
+        } else {
+            seen_lo[i] = INFINITY; seen_hi[i] = -INFINITY;
+            if (i < nf) {
+                const float4 c = cell_s[i * tx + threadIdx.x];
+                flo[i] = c.y > 0.0f ? c.x : __int_as_float(0x7fffffff);
+            }
         }
     }
-    const bool vec = vec_ok && nf == FPW;
-    const int64_t row_first = ((int64_t)blockIdx.x * blockDim.y + threadIdx.y) * kQuantRows * passes;
-#pragma unroll 2
-    for (int rr = 0; rr < kQuantRows * passes; ++rr) {
-        const int64_t row = row_first + rr;
-        if (row >= m) break;
-        uint32_t w1 = 0u, w2 = 0u;
-        if (nf > 0) {
-            float v[FPW];
-            const float* src = A + row * lda + j0;
-            if (vec) {
+    const float top = (float)((1 << bits) - 1);
+    // the blocks run from the last rows to the first: the range pass has left the end of A in L2
+    const int64_t row_first = ((int64_t)(row_blocks - 1 - row_block) * blockDim.y + threadIdx.y) * kQuantRows * passes;
+    // (rows above 2^32: a block holds a power of two of them, at its multiple, so all its rows have the same upper half)
+    const uint32_t row_hi = (uint32_t)((uint64_t)row_first >> 32), pair0 = (uint32_t)(j0 >> 1);
+    uint32_t row0 = (uint32_t)row_first;
+    int left = (int)max((int64_t)0, min((int64_t)kQuantRows * passes, m - row_first));   // rows from this pass on
+    const float* src = A + row_first * lda + j0;                   // the row that is requested next
+    uint8_t* out1 = plane1 + row_first * row_bytes + g * (int64_t)sizeof(Word);
+    uint8_t* out2 = plane2 + row_first * row_bytes + g * (int64_t)sizeof(Word);
+    // cell (in the low bits) and threshold of value x of feature i of thread column `col`, whose lo and inv are given
+    auto decide = [&](float x, int i, int col, float x_lo, float x_inv, uint32_t& cell, uint32_t& threshold) {
+        float y;
+        if constexpr (!TABLE) {
+            const float tc = fminf(fmaxf(__fmul_rn(__fsub_rn(x, x_lo), x_inv), 0.0f), top);
+            const float big = __fadd_rd(tc, 8388608.0f);
+            cell = __float_as_uint(big);
+            // 2^24 (tc - floor tc); both products are exact, and so is the difference
+            y = __fmaf_rn(tc, 16777216.0f, -__fmaf_rn(big, 16777216.0f, -140737488355328.0f));
+        } else {
+            const int ls = 4 * tx;
+            int at = i * tx + col;                                 // level k at lev_s[k * ls + at]; the last one is staged as infinity
 #pragma unroll
-                for (int i = 0; i < FPW / 4; ++i) {
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(src) + i);
-                    v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+            for (int half = L >> 1; half > 0; half >>= 1)          // the largest k <= L - 2 whose level is <= x
+                if (lev_s[at + half * ls] <= x) at += half * ls;
+            const float4 c = cell_s[at];
+            const float num = __fsub_rn(x, c.x);
+            float p = quotient(num, c.y, c.z);
+            if (p < 8.7e-19f && num > 0.0f && c.y > 0.0f) p = divide_slowly(num, c.y);
+            const bool sure = num >= c.y && c.z != 0.0f;           // the upper end (a quotient of 1): always up
+            cell = (uint32_t)__float_as_int(c.w) + (sure ? 1u : 0u);
+            y = sure ? 0.0f : __fmul_rn(p, 16777216.0f);
+        }
+        threshold = shift_left<8>(__float2uint_ru(y));
+    };
+    // the part of the Philox rounds 0 and 1 that depends on the pair alone
+    uint32_t pair_lo[2];
+    uint64_t pair_p[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const uint64_t a = (uint64_t)kPhiloxM1 * (pair0 + p);
+        pair_lo[p] = (uint32_t)a ^ key.k0[1];
+        pair_p[p] = (uint64_t)kPhiloxM0 * ((uint32_t)(a >> 32) ^ row_hi ^ key.k0[0]);
+    }
+    // The rows of a warp, with everything that depends on the matrix's edges compiled out where it lies inside.
+    auto run = [&](auto inside) {
+        constexpr bool kInside = decltype(inside)::value;
+        float v[kQuantRows][4];
+        auto request = [&](int have) {                             // the next kQuantRows rows, of which `have` exist
+            if (kInside && vec_ok) {
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r, src += lda) {
+                    const float4 t = __ldg(reinterpret_cast<const float4*>(src));
+                    v[r][0] = t.x; v[r][1] = t.y; v[r][2] = t.z; v[r][3] = t.w;
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < FPW; ++i) v[i] = (i < nf) ? __ldg(src + i) : 0.0f;
+                for (int r = 0; r < kQuantRows; ++r, src += lda)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[r][i] = kInside || (r < have && i < nf) ? __ldg(src + i) : flo[i];
             }
-            if constexpr (FPW <= 8) {
-                // pass 1: cells and thresholds of all features; a threshold strictly between 0 and 2^24 needs a draw
-                uint32_t thr[FPW];
-                uint32_t need = 0u;                                     // pairs with at least one such feature
-    #pragma unroll
-                for (int i = 0; i < FPW; ++i) {
-                    thr[i] = 0u;
-                    if (i >= nf) continue;
-                    uint32_t cell;
-                    float p;
-                    if constexpr (!TABLE) {
-                        uniform_cell(v[i], flo[i], finv[i], s, cell, p);
-                    } else {
-                        const float* lev = lev_s + i * blockDim.x + threadIdx.x;       // level k at lev[k * FPW * blockDim.x]
-                        const int ls = FPW * blockDim.x;
-                        int l = 0;
-                        for (int k = 1; k <= s - 1; ++k) l = (lev[k * ls] <= v[i]) ? k : l;
-                        const float base = lev[l * ls];
-                        const float width = __fsub_rn(lev[(l + 1) * ls], base);
-                        cell = (uint32_t)l;
-                        p = width > 0.0f ? __fdiv_rn(__fsub_rn(v[i], base), width) : 0.0f;
-                    }
-                    const uint32_t t = up_threshold(p);
-                    const bool open = t > 0u && t < 16777216u;
-                    // decided without a draw: threshold 0 never up, 2^24 and more always up
-                    const uint32_t c = cell + (t >= 16777216u ? 1u : 0u);
-                    w1 |= c << (i * CB);
-                    w2 |= c << (i * CB);
-                    thr[i] = open ? t : 0u;                             // 0: this feature adds nothing in pass 2
-                    need |= open ? 1u << (i >> 1) : 0u;
+        };
+        auto store = [&](const uint32_t (&w1)[kQuantRows], const uint32_t (&w2)[kQuantRows]) {
+#pragma unroll
+            for (int r = 0; r < kQuantRows; ++r, out1 += row_bytes, out2 += row_bytes)
+                if (kInside || (r < left && g < groups)) {
+                    *reinterpret_cast<Word*>(out1) = (Word)w1[r];
+                    *reinterpret_cast<Word*>(out2) = (Word)w2[r];
                 }
-                // pass 2: one Philox block per pair that needs one.  Where every lane needs every pair (dense continuous
-                // data) the pairs run as independent unrolled chains; otherwise every lane walks its own short list, so
-                // a warp runs as many rounds as its busiest lane has pairs (sparse rows: about two of four).
-                auto apply = [&](int pr, const Philox4& rnd) {
-    #pragma unroll
-                    for (int i = 0; i < FPW / 2; ++i)
-                        if (i == pr) {
-                            w1 += ((rnd.v[0] >> 8) < thr[2 * i] ? 1u : 0u) << (2 * i * CB);
-                            w2 += ((rnd.v[1] >> 8) < thr[2 * i] ? 1u : 0u) << (2 * i * CB);
-                            w1 += ((rnd.v[2] >> 8) < thr[2 * i + 1] ? 1u : 0u) << ((2 * i + 1) * CB);
-                            w2 += ((rnd.v[3] >> 8) < thr[2 * i + 1] ? 1u : 0u) << ((2 * i + 1) * CB);
+        };
+        request(left);
+#pragma unroll 1
+        for (int pass = 0; pass < passes; ++pass, left -= kQuantRows, row0 += kQuantRows) {
+            if (!kInside && !__any_sync(0xffffffffu, left > 0)) break;
+            if constexpr (TABLE) {
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (kInside || (r < left && i < nf)) {
+                            seen_lo[i] = fminf(seen_lo[i], v[r][i]);
+                            seen_hi[i] = fmaxf(seen_hi[i], v[r][i]);
+                            probe = fmaf(v[r][i], 0.0f, probe);
                         }
-                };
-                constexpr uint32_t kAllPairs = (1u << (FPW / 2)) - 1u;
-                if (__all_sync(__activemask(), need == kAllPairs)) {
-    #pragma unroll
-                    for (int pr = 0; pr < FPW / 2; ++pr) apply(pr, sample_block(seed, (uint64_t)row, (uint32_t)((j0 >> 1) + pr), draw));
-                } else {
-                    while (need) {
-                        const int pr = __ffs(need) - 1;
-                        need &= need - 1u;
-                        apply(pr, sample_block(seed, (uint64_t)row, (uint32_t)((j0 >> 1) + pr), draw));
+            }
+            // a guess from the first row (dense or sparse data look alike in every row), the count where it says sparse
+            int total = 4 * kQuantQueue, count = 0;
+            uint32_t need = 0u;                                    // bit 2 r + p: pair p of row r is not certain
+            if (__popc(__ballot_sync(0xffffffffu, v[0][0] != flo[0] || v[0][1] != flo[1] || v[0][2] != flo[2] || v[0][3] != flo[3])) <= 20) {
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r)
+                    need |= (v[r][0] != flo[0] || v[r][1] != flo[1] ? 1u << (2 * r) : 0u) | (v[r][2] != flo[2] || v[r][3] != flo[3] ? 2u << (2 * r) : 0u);
+                count = __popc(need);
+                total = __reduce_add_sync(0xffffffffu, count);
+            }
+            if (total > kQuantQueue) {
+                uint32_t w[kQuantRows], thr[kQuantRows][4], any = 0u;
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) {
+                    uint32_t cell[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        decide(v[r][i], i, threadIdx.x, flo[i], finv[i], cell[i], thr[r][i]);
+                        if (TABLE && !kInside && i >= nf) cell[i] = thr[r][i] = 0u;
+                        any |= thr[r][i];
+                    }
+                    w[r] = pack_codes<CB>(cell);
+                }
+                if (pass + 1 < passes) request(left - kQuantRows);
+                // what the draws add: one bit per code
+                uint32_t u1[kQuantRows], u2[kQuantRows];
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) u1[r] = u2[r] = 0u;
+                if (__any_sync(0xffffffffu, any != 0u)) {          // (integers on a grid of integers: no draw at all)
+#pragma unroll
+                    for (int r = 0; r < kQuantRows; ++r) {
+                        const uint64_t a = (uint64_t)kPhiloxM0 * (row0 + r);
+                        const uint64_t b = (uint64_t)kPhiloxM1 * ((uint32_t)(a >> 32) ^ draw ^ key.k1[0]);
+                        Philox4 rnd[2];
+#pragma unroll
+                        for (int p = 0; p < 2; ++p)
+                            rnd[p] = philox_rounds<2>((uint32_t)(b >> 32) ^ pair_lo[p], (uint32_t)b,
+                                                      (uint32_t)(pair_p[p] >> 32) ^ (uint32_t)a ^ key.k1[1], (uint32_t)pair_p[p], key);
+                        set_if_below<1u>(u1[r], rnd[0].v[0], thr[r][0]);
+                        set_if_below<1u>(u2[r], rnd[0].v[1], thr[r][0]);
+                        set_if_below<1u << CB>(u1[r], rnd[0].v[2], thr[r][1]);
+                        set_if_below<1u << CB>(u2[r], rnd[0].v[3], thr[r][1]);
+                        set_if_below<1u << 2 * CB>(u1[r], rnd[1].v[0], thr[r][2]);
+                        set_if_below<1u << 2 * CB>(u2[r], rnd[1].v[1], thr[r][2]);
+                        set_if_below<1u << 3 * CB>(u1[r], rnd[1].v[2], thr[r][3]);
+                        set_if_below<1u << 3 * CB>(u2[r], rnd[1].v[3], thr[r][3]);
                     }
                 }
-        
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) { u1[r] += w[r]; u2[r] += w[r]; }
+                store(u1, u2);
             } else {
-                // sixteen features per word: the thresholds of a whole word would not fit the registers; pair by pair
+                uint4* mine = reinterpret_cast<uint4*>(word_s[warp][lane]);
+                mine[0] = mine[1] = make_uint4(0u, 0u, 0u, 0u);
+                int at = count;                                    // exclusive prefix sum over the warp
 #pragma unroll
-                for (int pr = 0; pr < FPW / 2; ++pr) {
-                    if (2 * pr >= nf) break;
-                    uint32_t cell[2] = {0u, 0u}, t[2] = {0u, 0u};
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int i = 2 * pr + h;
-                        if (i >= nf) break;
-                        float p;
-                        if constexpr (!TABLE) {
-                            uniform_cell(v[i], flo[i], finv[i], s, cell[h], p);
-                        } else {
-                            const float* lev = lev_s + i * blockDim.x + threadIdx.x;
-                            const int ls = FPW * blockDim.x;
-                            int l = 0;
-                            for (int k = 1; k <= s - 1; ++k) l = (lev[k * ls] <= v[i]) ? k : l;
-                            const float base = lev[l * ls];
-                            const float width = __fsub_rn(lev[(l + 1) * ls], base);
-                            cell[h] = (uint32_t)l;
-                            p = width > 0.0f ? __fdiv_rn(__fsub_rn(v[i], base), width) : 0.0f;
-                        }
-                        t[h] = up_threshold(p);
-                    }
-                    const bool random = (t[0] > 0u && t[0] < 16777216u) || (t[1] > 0u && t[1] < 16777216u);
-                    Philox4 rnd;
-                    if (random) rnd = sample_block(seed, (uint64_t)row, (uint32_t)((j0 >> 1) + pr), draw);
-                    else rnd.v[0] = rnd.v[1] = rnd.v[2] = rnd.v[3] = 0u;    // decided without them: 0 never up, 2^24 always up
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int i = 2 * pr + h;
-                        if (i >= nf) break;
-                        w1 |= round_up_if(cell[h], t[h], rnd.v[2 * h]) << (i * CB);
-                        w2 |= round_up_if(cell[h], t[h], rnd.v[2 * h + 1]) << (i * CB);
-                    }
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int up = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += up;
                 }
+                at -= count;
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) val_s[warp][r][lane] = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+#pragma unroll
+                for (int k = 0; k < 2 * kQuantRows; ++k)
+                    if (need >> k & 1u) queue_s[warp][at++] = (uint8_t)(lane * 2 * kQuantRows + k);
+                if (pass + 1 < passes) request(left - kQuantRows);
+                __syncwarp();
+#pragma unroll 1
+                for (int e0 = 0; e0 < total; e0 += 32) {
+                    const int q = queue_s[warp][min(e0 + lane, total - 1)];    // (lanes past the end repeat the last: or-ing twice is harmless)
+                    const int owner = q >> 3, r = (q >> 1) & 3, p = q & 1;
+                    const uint32_t row = __shfl_sync(0xffffffffu, row0, owner) + r, pair = __shfl_sync(0xffffffffu, pair0, owner) + p;
+                    const float2 x = reinterpret_cast<const float2*>(&val_s[warp][r][owner])[p];
+                    const int col = (warp * 32 + owner) & (tx - 1);            // tx is a power of two
+                    const int64_t j = 2 * (int64_t)pair;
+                    const int second = kInside || j + 1 < n ? 1 : 0;           // (a queued pair has at least its first feature)
+                    float2 xlo = make_float2(0.0f, 0.0f), xinv = xlo;
+                    if constexpr (!TABLE) {
+                        xlo = make_float2(__ldg(lo + j), __ldg(lo + j + second));
+                        xinv = make_float2(__ldg(inv + j), __ldg(inv + j + second));
+                    }
+                    uint32_t c0, c1, t0, t1;
+                    decide(x.x, 2 * p, col, xlo.x, xinv.x, c0, t0);
+                    decide(x.y, 2 * p + 1, col, xlo.y, xinv.y, c1, t1);
+                    constexpr uint32_t kMask = (1u << CB) - 1u;
+                    uint32_t w1 = c0 & kMask, w2 = w1;
+                    const Philox4 rnd = philox_rounds<0>(row, row_hi, pair, draw, key);
+                    if (rnd.v[0] < t0) w1 += 1u;
+                    if (rnd.v[1] < t0) w2 += 1u;
+                    if (second) {
+                        w1 += (c1 & kMask) << CB;
+                        w2 += (c1 & kMask) << CB;
+                        if (rnd.v[2] < t1) w1 += 1u << CB;
+                        if (rnd.v[3] < t1) w2 += 1u << CB;
+                    }
+                    // (a row's two pairs share its words: hence the atomics)
+                    atomicOr(&word_s[warp][owner][2 * r], w1 << (2 * p * CB));
+                    atomicOr(&word_s[warp][owner][2 * r + 1], w2 << (2 * p * CB));
+                }
+                __syncwarp();
+                const uint4 lower = mine[0], upper = mine[1];
+                const uint32_t w1[kQuantRows] = {lower.x, lower.z, upper.x, upper.z}, w2[kQuantRows] = {lower.y, lower.w, upper.y, upper.w};
+                store(w1, w2);
             }
         }
-        plane1[row * row_words + q] = w1;
-        plane2[row * row_words + q] = w2;
+    };
+    if (__all_sync(0xffffffffu, nf == 4 && left == kQuantRows * passes)) run(std::true_type{});
+    else run(std::false_type{});
+    if constexpr (TABLE) {
+        if (!(probe == 0.0f)) set_status(status, ZIPML_ERR_NONFINITE, 1);
+        // (a value that is beaten already needs no atomic: after the first blocks hardly any does)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < nf && seen_lo[i] <= seen_hi[i]) {
+                const uint32_t a = float_order_key(seen_lo[i]), b = float_order_key(seen_hi[i]);
+                if (a < *reinterpret_cast<volatile uint32_t*>(lo_key + j0 + i)) atomicMin(lo_key + j0 + i, a);
+                if (b > *reinterpret_cast<volatile uint32_t*>(hi_key + j0 + i)) atomicMax(hi_key + j0 + i, b);
+            }
     }
 }
 
 int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bits, int level_mode,
                     const float* lo, const float* inv, const float* levels, uint64_t seed, uint32_t draw, uint8_t* plane1,
-                    uint8_t* plane2, int64_t row_bytes) {
+                    uint8_t* plane2, int64_t row_bytes, uint32_t* key_scratch, float* lo_out, float* step_out) {
     const int cb = container_bits(bits);
-    const int64_t row_words = row_bytes / 4;
     const bool table = level_mode == ZIPML_LEVELS_TABLE;
-    // 256 threads: as many word columns as the row has (a power of two from 8 to 256; 64 with level tables),
-    // the rest row groups; with level tables a thread makes four passes, so that staging the tables pays
-    int tx = 8;
-    while (tx < (table ? kQuantTableCols : 256) && tx < row_words) tx *= 2;
+    const int64_t groups = row_bytes * 8 / (4 * cb);
+    // 256 threads: as many feature groups as the row has (a power of two from 4 to 256; 64 with level tables), the
+    // rest row groups.  More passes per thread share the loads of lo and inv (the staging of the tables), as
+    // long as the grid still covers the SMs several times over.
+    int tx = 4;
+    while (tx < (table ? kQuantTableCols : 256) && tx < groups) tx *= 2;
     const int ty = 256 / tx;
-    const int passes = table ? 4 : 1;
-    const size_t smem = table ? sizeof(float) * ((size_t)1 << bits) * (32 / cb) * tx : 0;
-    const int64_t rows_per_block = (int64_t)ty * kQuantRows * passes;
-    const int64_t row_blocks = (m + rows_per_block - 1) / rows_per_block;
-    const int64_t col_blocks = (row_words + tx - 1) / tx;
-    if (row_blocks > 0x7fffffffLL || col_blocks > 65535) return ZIPML_ERR_WORKSPACE;
-    const dim3 grid((unsigned)row_blocks, (unsigned)col_blocks), block((unsigned)tx, (unsigned)ty);
+    const int64_t col_blocks = (groups + tx - 1) / tx;
+    int passes = 1;
+    while (passes < (table ? 16 : 8) && (m / (ty * kQuantRows * passes * 2)) * col_blocks >= (int64_t)ctx->sm_count * 16) passes *= 2;
+    const size_t smem = table ? (sizeof(float4) + sizeof(float)) * ((size_t)4 << bits) * tx : 0;
+    auto blocks_of_rows = [&]() { return (m + (int64_t)ty * kQuantRows * passes - 1) / ((int64_t)ty * kQuantRows * passes); };
+    while (blocks_of_rows() > 0x7fffffffLL / col_blocks && passes < (1 << 20)) passes *= 2;      // the grid is one-dimensional, columns first
+    const int64_t row_blocks = blocks_of_rows();
+    if (row_blocks > 0x7fffffffLL / col_blocks) return ZIPML_ERR_WORKSPACE;
+    const dim3 grid((unsigned)(row_blocks * col_blocks)), block((unsigned)tx, (unsigned)ty);
     const bool vec_ok = (lda % 4 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
-    uint32_t* p1 = reinterpret_cast<uint32_t*>(plane1);
-    uint32_t* p2 = reinterpret_cast<uint32_t*>(plane2);
-#define ZIPML_LAUNCH_Q(CB_, T_) \
-    quantize_kernel<CB_, T_><<<grid, block, smem, ctx->stream>>>(A, m, n, lda, bits, lo, inv, levels, seed, draw, p1, p2, row_words, vec_ok, passes)
-    if (cb == 2) { if (table) ZIPML_LAUNCH_Q(2, true); else ZIPML_LAUNCH_Q(2, false); }
-    else if (cb == 4) { if (table) ZIPML_LAUNCH_Q(4, true); else ZIPML_LAUNCH_Q(4, false); }
-    else { ZIPML_LAUNCH_Q(8, false); }
-#undef ZIPML_LAUNCH_Q
+    const PhiloxKeys key = philox_keys(seed);
+    uint32_t* lo_key = key_scratch;
+    uint32_t* hi_key = key_scratch + n;
+    const unsigned nb = (unsigned)((n + 255) / 256);
+    if (table) range_init_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n);
+    auto launch = [&](auto kernel) -> int {
+        // (the kernel's own 25 KB of shared memory count towards the 48 KB that need no opt-in)
+        if (smem > 20 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_status(e);
+        }
+        kernel<<<grid, block, smem, ctx->stream>>>(A, m, n, lda, bits, lo, inv, levels, lo_key, hi_key, ctx->d_status, key, draw, plane1, plane2,
+                                                   row_bytes, vec_ok, passes, (unsigned)col_blocks, (unsigned)row_blocks);
+        return ZIPML_OK;
+    };
+    int rc;
+    if (!table) rc = cb == 2 ? launch(quantize_kernel<2, 0>) : cb == 4 ? launch(quantize_kernel<4, 0>) : launch(quantize_kernel<8, 0>);
+    else rc = bits == 1 ? launch(quantize_kernel<2, 1>) : bits == 2 ? launch(quantize_kernel<2, 2>) : bits == 3 ? launch(quantize_kernel<4, 3>) : launch(quantize_kernel<4, 4>);
+    if (rc != ZIPML_OK) return rc;
     ctx->launches += 1;
+    if (table) {
+        range_finalize_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n, (1 << bits) - 1, false, lo_out, nullptr, nullptr, step_out);
+        ctx->launches += 2;
+    }
     return cuda_status(cudaGetLastError());
 }
 

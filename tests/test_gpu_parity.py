@@ -67,6 +67,45 @@ def test_quantize_bit_exact(ctx, key, m, n, bits):
     assert (gds.plane2.cpu().numpy() == ods.plane2).all()
 
 
+# (a thread takes four features and four rows per pass, several passes once the matrix fills the device)
+@pytest.mark.parametrize("m,n,bits,levels,nonzero", [
+    (1, 3, 4, False, 0.3), (5, 17, 8, False, 0.05), (259, 66, 2, False, 0.05), (130, 1023, 4, False, 0.05), (66, 258, 1, True, 0.1),
+    (131, 257, 2, True, 0.05), (37, 61, 3, True, 0.02), (66, 130, 4, True, 0.5), (18_955, 1022, 8, False, 0.08),
+    (19_001, 1029, 4, False, 0.05), (75_805, 255, 3, True, 0.05),
+])
+def test_quantize_sparse_rows_and_edges_bit_exact(ctx, m, n, bits, levels, nonzero):
+    """Rows that are mostly their features' lowest level (a warp shares out the few others), beside dense ones, at the
+    edges of groups, warps and passes; with level tables also cells of width zero and of extreme widths."""
+    rng = np.random.default_rng(m + n)
+    A = np.where(rng.random((m, n)) < nonzero, rng.random((m, n)), 0.0).astype(np.float32)
+    A[m // 2:, : n // 3] = rng.random((m - m // 2, n // 3), dtype=np.float32)       # dense
+    kw = okw = {}
+    if levels:
+        A[:, -1] *= np.float32(1e20)
+        A[:, 0] *= np.float32(1e-30)
+        lo, hi = A.min(axis=0), A.max(axis=0)
+        table = np.sort(rng.random((n, 1 << bits), dtype=np.float32), axis=1) * (hi - lo)[:, None] + lo[:, None]
+        table = np.clip(table, lo[:, None], hi[:, None]).astype(np.float32)
+        table[:, 0], table[:, -1] = lo, hi
+        if bits > 1:
+            table[1::2, 1] = table[1::2, 0]                                         # the same level twice
+        table = np.sort(table, axis=1)
+        okw = dict(mode=oracle.TABLE, levels=table)
+        kw = dict(level_mode=binding.LEVELS_TABLE, levels=to_dev(table, ctx))
+    ods = oracle.quantize(A, bits, seed=99, **okw)
+    gds = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=99, **kw)
+    ctx.zipml_sync()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+    assert (gds.feat_lo.cpu().numpy() == ods.feat_lo).all()
+    if levels:
+        bad = to_dev(A, ctx)
+        bad[m - 1, n - 1] = float("inf")
+        ctx.zipml_quantize(bad, bits, seed=99, **kw)
+        with pytest.raises(binding.ZipmlError) as e:
+            ctx.zipml_sync()
+        assert e.value.code == binding.ERR_NONFINITE
+
+
 def test_quantize_strided_and_unaligned_input(ctx):
     _, A, _, _ = workload("c2", 200, 101, seed=3)
     big = torch.zeros((200, 131), dtype=torch.float32, device=ctx.device)
