@@ -830,6 +830,19 @@ def test_config5_step_shape(ctx):
     assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x_ref))
 
 
+@pytest.mark.parametrize("m,n,bits,bins", [(900, 33, 4, 15), (1200, 3, 2, 257), (600, 2, 3, 1023), (3000, 2, 4, 321), (2100, 65, 3, 64)])
+def test_optimal_levels_at_the_edges_of_rounds(ctx, m, n, bits, bins):
+    """Bins beside the strides of the search's rounds (4, 16, 64, 256), fewest bins for the levels, values that leave most
+    bins empty (ties), rows beside a histogram chunk's multiple."""
+    rng = np.random.default_rng(bins)
+    A = (np.exp(1.5 * rng.standard_normal((m, n))) * np.sign(rng.standard_normal((m, n)))).astype(np.float32)
+    A[:, 0] = rng.integers(0, 5, m)
+    lev, obj = oracle.optimal_levels(A, bits, bins)
+    glev, gobj = ctx.zipml_optimal_levels(to_dev(A, ctx), bits, bins, want_objective=True)
+    ctx.zipml_sync()
+    assert (gobj.cpu().numpy().astype(np.uint64) == obj).all() and (glev.cpu().numpy() == lev).all()
+
+
 def test_config4_step_shape_with_level_table(ctx):
     """Config 4 as it runs: n = 512, 3-bit variance-optimal levels from a 1,024-bin histogram, B = 512."""
     m, n, batch, lr = 3 * 512 + 100, 512, 512, 1e-3
