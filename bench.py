@@ -40,7 +40,7 @@ NCU_TRAFFIC = {
     ("c5", 7): (4 * (538.45e6 + 4.86e6), "profiles/sgd_column_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
 }
 ENGINE_KERNELS = {1: "sgd_kernel (stepwise launches)", 2: "sgd_kernel (persistent)", 3: "sgd_ring_kernel", 4: "sgd_lean_kernel",
-                  5: "sgd_cluster_kernel", 6: "sgd_stream_kernel", 7: "sgd_column_kernel"}
+                  5: "sgd_cluster_kernel", 6: "sgd_stream_kernel", 7: "sgd_column_kernel", 8: "sgd_solo_kernel"}
 
 
 def measured_peaks():
@@ -147,7 +147,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default="c5", help="c1..c5, c4u (see paper_1611_05402_b200/synth.py)")
     ap.add_argument("--m", type=int, default=None, help="override the number of samples (smaller profiling cases)")
-    ap.add_argument("--engine", default="auto", choices=["auto", "stepwise", "persistent", "ring", "lean", "cluster", "stream", "column"])
+    ap.add_argument("--engine", default="auto", choices=["auto", "stepwise", "persistent", "ring", "lean", "cluster", "stream", "column", "solo"])
     ap.add_argument("--chunk-rows", type=int, default=0, help="column engine: rows per chunk (0 = automatic)")
     ap.add_argument("--feature-parts", type=int, default=0)
     ap.add_argument("--row-parts", type=int, default=0)
@@ -219,7 +219,7 @@ def main():
     dev = torch.device("cuda", local_rank)
     engine = {"auto": binding.ENGINE_AUTO, "stepwise": binding.ENGINE_STEPWISE, "persistent": binding.ENGINE_PERSISTENT,
               "ring": binding.ENGINE_RING, "lean": binding.ENGINE_LEAN, "cluster": binding.ENGINE_CLUSTER,
-              "stream": binding.ENGINE_STREAM, "column": binding.ENGINE_COLUMN}[args.engine]
+              "stream": binding.ENGINE_STREAM, "column": binding.ENGINE_COLUMN, "solo": binding.ENGINE_SOLO}[args.engine]
 
     sharded = args.sharded and world > 1
     w, A, b, _ = synth.make(args.workload, m=args.m, device=dev, seed=base.seed + (0 if sharded else rank))

@@ -64,7 +64,8 @@ enum {
 };
 /* How zipml_sgd_epoch runs its minibatch chain.  Results do not depend on the choice. */
 enum {
-    ZIPML_ENGINE_AUTO = 0,      /* cluster, else lean, for steps of at most 2 MiB of codes; else column,
+    ZIPML_ENGINE_AUTO = 0,      /* solo for the smallest steps; cluster, else lean, for steps of at most
+                                   2 MiB of codes; else column,
                                    else stream, where they apply (wide rows, uniform grid, fp32 model
                                    and gradient), else ring                                           */
     ZIPML_ENGINE_STEPWISE = 1,  /* a few kernel launches per minibatch                               */
@@ -86,7 +87,7 @@ enum {
                                     model or gradient, batches above 8192 rows.
                                     zipml_sgd_params.stream_prefetch overrides how many eighths of the
                                     next step's tile are requested into L2 ahead of time               */
-    ZIPML_ENGINE_COLUMN = 7      /* one cooperative launch for large tiles on uniform grids with an fp32
+    ZIPML_ENGINE_COLUMN = 7,     /* one cooperative launch for large tiles on uniform grids with an fp32
                                     model and gradient, rows of 128 bytes .. 128 bytes x the number of
                                     SMs: a CTA owns a 128-byte column block of the packed rows for the
                                     whole launch; chunks of rows visit shared memory once for the dots
@@ -96,6 +97,10 @@ enum {
                                     barrier.  The only engine that takes ZIPML_LAYOUT_COLUMN_BLOCKS
                                     (where its copies are contiguous; AUTO picks it for such data).
                                     ZIPML_ERR_WORKSPACE for what it does not cover (as for STREAM)     */
+    ZIPML_ENGINE_SOLO = 8        /* one thread block for the whole chain: steps so small that handing
+                                   values between SMs costs more than their arithmetic.
+                                   ZIPML_ERR_WORKSPACE for more than 2,048 features or tiles above 48 KiB
+                                   a plane                                                            */
 };
 
 typedef struct zipml_ctx zipml_ctx;

@@ -245,7 +245,7 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (!b || !x || params->batch <= 0) return ZIPML_ERR_INVALID_ARG;
     if (params->model_bits != 0 && (params->model_bits < 2 || params->model_bits > 8)) return ZIPML_ERR_UNSUPPORTED;
     if (params->grad_bits != 0 && (params->grad_bits < 2 || params->grad_bits > 8)) return ZIPML_ERR_UNSUPPORTED;
-    if (params->engine < ZIPML_ENGINE_AUTO || params->engine > ZIPML_ENGINE_COLUMN) return ZIPML_ERR_INVALID_ARG;
+    if (params->engine < ZIPML_ENGINE_AUTO || params->engine > ZIPML_ENGINE_SOLO) return ZIPML_ERR_INVALID_ARG;
     if (params->epoch < 0 || params->epoch > 0xffffffffLL) return ZIPML_ERR_INVALID_ARG;
     if (params->reg < ZIPML_REG_NONE || params->reg > ZIPML_REG_LSSVM) return ZIPML_ERR_INVALID_ARG;
     if (params->reg != ZIPML_REG_NONE && params->reg != ZIPML_REG_NONNEG && !(params->reg_param >= 0.0f)) return ZIPML_ERR_INVALID_ARG;
@@ -278,14 +278,18 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (params->engine == ZIPML_ENGINE_CLUSTER) return launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
     if (params->engine == ZIPML_ENGINE_STREAM) return launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_COLUMN) return launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
+    if (params->engine == ZIPML_ENGINE_SOLO) return launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_AUTO && !linf) {
-        // Small minibatch tiles are bound by the step-to-step chain, not by HBM: one cluster whose CTAs
+        // Small minibatch tiles are bound by the step-to-step chain, not by HBM: the smallest stay on one SM;
+        // then one cluster whose CTAs
         // exchange through shared memory, else row parts exchanging through L2.  Larger tiles go to the
         // column engine (codes read once per step), the stream engine, then the ring engine.  Each engine
         // answers ZIPML_ERR_WORKSPACE when the shape does not fit it.
         const int64_t B = params->batch < data->m ? params->batch : data->m;
         const int64_t step_bytes = 2 * B * data->row_bytes;
         if (step_bytes <= (2ll << 20)) {
+            rc = launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, true);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
             rc = launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
             rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);

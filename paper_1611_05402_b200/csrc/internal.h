@@ -95,6 +95,9 @@ int launch_sgd_ring(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
                     int64_t first_step, int64_t num_steps, float* grad_out, bool probe_only);
 int launch_sgd_lean(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                     int64_t first_step, int64_t num_steps, float* grad_out);
+// Solo engine (one thread block).  With only_if_profitable it declines (ZIPML_ERR_WORKSPACE) steps that several SMs take faster.
+int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
+                    int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out);
 // Stream engine (uniform grids, fp32 model and gradient).  With only_if_profitable it declines

@@ -258,6 +258,59 @@ def test_sgd_epoch_parity(ctx, case, engine):
         assert rel(xb.cpu().numpy(), x_ref) <= MODEL_TOL
 
 
+@pytest.mark.parametrize("m,n,bits,batch,table", [
+    (100, 1, 2, 7, False), (300, 5, 8, 64, False), (90, 16, 4, 1, False), (1200, 23, 8, 512, False), (260, 61, 4, 33, False),
+    (700, 250, 2, 64, False), (70, 2048, 8, 16, False), (60, 1999, 4, 16, False), (300, 1000, 1, 16, False), (500, 37, 3, 100, True),
+    (130, 250, 2, 16, True), (40, 2000, 4, 3, True), (2500, 30, 6, 1024, False),
+])
+def test_solo_engine(ctx, m, n, bits, batch, table):
+    """The one-block engine at the edges of its lane splits (rows, words and features left over), with a batch order, a
+    ragged last batch, a step range, a regulariser and quantized model and gradient."""
+    _, A, b, _ = workload("c4" if table else "c1", m, n, seed=n)
+    kw = dict(mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 256)[0]) if table else {}
+    ods = oracle.quantize(A, bits, seed=3, **kw)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    T = (m + batch - 1) // batch
+    lr = 0.3 / n
+    order = np.random.default_rng(0).permutation(T).astype(np.int32)
+    x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
+    for kw in (dict(batch_order=order), dict(reg=binding.REG_LSSVM, reg_param=0.1)):
+        x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, **kw)
+        x_before, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, num_steps=T - 1, **kw)
+        _, g_ref = oracle.sgd_epoch(ods, b, x_before, batch, lr, first_step=T - 1, num_steps=1, want_grad=True, **kw)
+        x = to_dev(x0, ctx)
+        ctx.zipml_sgd_epoch(gds, db, x, batch, lr, engine=binding.ENGINE_SOLO, **kw)
+        ctx.zipml_sync()
+        assert ctx.zipml_last_engine() == binding.ENGINE_SOLO and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+        xb, seen = to_dev(x_before, ctx), torch.zeros(n, device=ctx.device)
+        g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+        ctx.zipml_sgd_epoch(gds, db, xb, batch, lr, first_step=T - 1, num_steps=1, engine=binding.ENGINE_SOLO, grad_out=g, model_out=seen, **kw)
+        ctx.zipml_sync()
+        assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL and (g[0] == g[1]).all()
+        assert (seen.cpu().numpy() == x_before).all() and rel(xb.cpu().numpy(), x_ref) <= MODEL_TOL
+    # one step end to end quantized: Q3 of the same model is the oracle's, up to a draw within 1e-4 of its threshold;
+    # the gradient is the one of the model that was seen
+    x, seen = to_dev(x0, ctx), torch.zeros(n, device=ctx.device)
+    g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+    kw = dict(seed=5, epoch=1, first_step=0, num_steps=1)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, model_bits=8, grad_bits=6, engine=binding.ENGINE_SOLO, grad_out=g, model_out=seen, **kw)
+    ctx.zipml_sync()
+    want, _ = oracle.quantize_vector(x0, 8, 5, 1, 0, 3)
+    margin, _ = q3_margins(x0, 8, 5, 1, 0)
+    seen = seen.cpu().numpy()
+    assert not ((seen != want) & (margin >= 1e-4)).any()
+    _, g_ref = oracle.sgd_epoch(ods, b, seen, batch, lr, want_grad=True, **kw)
+    assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL
+    g4, _ = oracle.quantize_vector(g[0].cpu().numpy(), 6, 5, 1, 0, 4)
+    assert (g[1].cpu().numpy() != g4).sum() <= 2
+    y = x0 - np.float32(lr) * g[1].cpu().numpy()
+    assert np.allclose(x.cpu().numpy(), y, rtol=1e-6, atol=1e-7)
+    if batch <= 16:
+        ctx.zipml_sgd_epoch(gds, db, to_dev(x0, ctx), batch, lr)
+        ctx.zipml_sync()
+        assert ctx.zipml_last_engine() == binding.ENGINE_SOLO               # what AUTO takes
+
+
 @pytest.mark.parametrize("contraction", [1, 2], ids=["fp32", "int8"])
 @pytest.mark.parametrize("case", SGD_CASES[:5], ids=lambda c: f"{c[0]}-{c[1]}x{c[2]}-b{c[3]}-B{c[4]}")
 def test_cluster_engine_both_contractions(ctx, case, contraction):
