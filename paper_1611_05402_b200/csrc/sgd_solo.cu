@@ -448,17 +448,24 @@ static size_t solo_smem_bytes(int cb, bool table, int bits, int words, int rc, i
                                                (size_t)slots * (2 * (size_t)rc * pitch + (size_t)((rc + 3) & ~3)));
 }
 
-// How many of a warp's 32 lanes, (lane >> shift) rows apart or words apart, fall into the fullest bank.
-static int bank_degree(int pitch, int shift, bool lanes_on_rows) {
-    int load[32] = {0}, worst = 0;
-    for (int l = 0; l < 32; ++l) {
-        const int inner = l & ((1 << shift) - 1), outer = l >> shift;
-        const int word = lanes_on_rows ? inner * pitch + outer : outer * pitch + inner;
-        const int d = ++load[word & 31];
-        if (d > worst) worst = d;
+// The fullest bank's share of a warp's 32 loads: 32 / run rows of `run` consecutive words each, rows pitch = 4 u words
+// apart, by [u % 8][log2 run].  (A table because a plan is made on every call: counted out there it cost 10 us of host time.)
+struct BankTable {
+    int degree[8][6];
+    constexpr BankTable() : degree() {
+        for (int u = 0; u < 8; ++u)
+            for (int s = 0; s <= 5; ++s) {
+                int load[32] = {0}, worst = 0;
+                for (int l = 0; l < 32; ++l) {
+                    const int bank = ((l >> s) * 4 * u + (l & ((1 << s) - 1))) & 31;
+                    ++load[bank];
+                    if (load[bank] > worst) worst = load[bank];
+                }
+                degree[u][s] = worst;
+            }
     }
-    return worst;
-}
+};
+static constexpr BankTable kBanks;
 
 template <int CB, bool TABLE>
 static const void* solo_kernel(int keep) {
@@ -476,7 +483,7 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
     const int B = (int)B64, row_words = (int)(d->row_bytes / 4), nw = (int)((d->n + fpw - 1) / fpw);
     const double unit = (table ? 7.0 : 4.2) * fpw + 6;              // instructions per word of both planes
     best->threads = 0;
-    for (int pad = 0; pad <= 28; pad += 4) {
+    for (const int pad : {0, 4, 8, 16}) {
         const int pitch = row_words + pad;
         int slots = kSoloMaxSlots;
         while (slots >= 2 && solo_smem_bytes(cb, table, d->bits, nw, B, pitch, slots) > (size_t)ctx->smem_optin) --slots;
@@ -491,7 +498,7 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
                 if (threads / g >= 1) {
                     const int turns = (B + threads / g - 1) / (threads / g), per = (nw + g - 1) / g;
                     const double instr = turns * (per * unit + (nw > g ? per * fpw * 0.5 : 0) + 5.0 * s + 14) + (table ? 0 : per * fpw * 1.5);
-                    const double lds = (double)turns * per * warps * (2.0 * bank_degree(pitch, s, false) + (table ? 2.0 * fpw * 2 : fpw / 4));
+                    const double lds = (double)turns * per * warps * (2.0 * kBanks.degree[(pitch / 4) % 8][s] + (table ? 2.0 * fpw * 2 : fpw / 4));
                     const double c = (instr * issue > lds ? instr * issue : lds) + 28.0 * s + 80;
                     if (c < best_a) { best_a = c; sa = s; }
                 }
@@ -499,7 +506,7 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
                 if (nw * g <= threads && (fpw >> (s < logf ? s : logf)) <= 4) {
                     const int per = (B + g - 1) / g, kept = fpw >> (s < logf ? s : logf);
                     const double instr = per * (unit + 4) + 3.0 * (fpw - kept) + 4.0 * s + kept * 12 + 20;
-                    const double lds = (double)per * warps * (2.0 * bank_degree(pitch, s, true) + 2 + (table ? 2.0 * fpw * 2 : 0));
+                    const double lds = (double)per * warps * (2.0 * kBanks.degree[(pitch / 4) % 8][5 - s] + 2 + (table ? 2.0 * fpw * 2 : 0));
                     const double c = (instr * issue > lds ? instr * issue : lds) + 28.0 * s + 100;
                     if (c < best_b) { best_b = c; sb = s; }
                 }
@@ -519,19 +526,19 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
     return ZIPML_OK;
 }
 
-// Whether AUTO takes this engine: by the multiply-adds of a dot pass, batch x features, which one SM has to get through.
-// Measured, us per step here / cluster or lean engine, on both sides of the lines: 4 bits 256 x 64 3.3 / 4.1, 64 x 250
-// 3.3 / 3.9, 37 x 512 4.5 / 4.3, 128 x 250 5.3 / 3.9; 2 bits 37 x 512 3.8 / 4.8, 1,024 x 23 8.3 / 7.4; 8 bits 512 x 23
-// 4.0 / 4.5, 128 x 64 2.6 / 3.8, 64 x 250 4.4 / 3.9, 256 x 64 4.1 / 3.9; tables (3 bits) 256 x 23 3.8 / 4.3, 128 x 64
-// 4.0 / 3.9, 37 x 250 4.3 / 4.0.  A quantized model or gradient costs the others an exchange more each: 4 bits 256 x 64 4.8
-// / 6.9, 64 x 512 7.0 / 7.1.  Up to 16 rows the others' exchanges grow with the features as fast as this engine's work:
-// 16 x 1,000 at 8 bits 3.7 / 4.8, 16 x 1,999 5.9 / 6.5, on 3-bit tables 7.4 / 8.6.
+// Whether AUTO takes this engine: by what a step has one SM get through, batch x (features + 8).  Measured, us per step
+// here / cluster engine, on both sides of the lines: 4 bits 256 x 64 3.3 / 4.2, 64 x 250 3.2 / 4.0, 800 x 23 5.2 / 5.0, 1,024 x 17
+// 5.8 / 5.0, 37 x 512 4.5 / 4.3; 2 bits 64 x 250 3.2 / 4.2, 37 x 333 4.6 / 4.0, 16 x 2,048 5.9 / 5.2; 8 bits 300 x 30 3.0 / 4.2, 512
+// x 23 4.0 / 4.5, 64 x 250 4.4 / 3.9, 16 x 1,000 3.7 / 3.9, 16 x 2,000 5.8 / 5.2; tables (3 bits) 256 x 23 3.8 / 4.3, 128 x 64 4.0 / 3.9,
+// 37 x 250 4.3 / 4.0, 16 x 1,999 7.4 / 8.6.  A quantized model or gradient costs the others an exchange more each: 8 bits 256
+// x 64 5.9 / 6.4, 4 bits 500 x 61 7.5 / 7.7, 37 x 512 7.3 / 7.2.
 static bool solo_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
     const int64_t B = p->batch < d->m ? p->batch : d->m;
-    if (B <= 16) return true;
-    int64_t limit = d->level_mode == ZIPML_LEVELS_TABLE ? 7000 : container_bits(d->bits) == 8 ? 12288 : 18432;
-    if (p->model_bits > 0 || p->grad_bits > 0) limit = limit * 3 / 2;
-    return B * d->n <= limit;
+    const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
+    if (table && B <= 16) return true;
+    int64_t limit = table ? 7500 : container_bits(d->bits) == 4 || B <= 16 ? 18500 : 14000;
+    if (p->model_bits > 0 || p->grad_bits > 0) limit = limit * 5 / 4;
+    return (table || d->n <= 1024) && B * (d->n + 8) <= limit;
 }
 
 int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
