@@ -98,6 +98,9 @@ int launch_sgd_lean(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
 // Solo engine (one thread block).  With only_if_profitable it declines (ZIPML_ERR_WORKSPACE) steps that several SMs take faster.
 int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                     int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable);
+// The cluster engine's int8 form on uniform grids (launch_sgd_cluster calls it).
+int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                     int64_t num_steps, float* grad_out);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out);
 // Stream engine (uniform grids, fp32 model and gradient).  With only_if_profitable it declines

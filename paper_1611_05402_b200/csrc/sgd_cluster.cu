@@ -844,6 +844,10 @@ int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
     const int fpw = 32 / cb;
     const int64_t T = (d->m + p->batch - 1) / p->batch;
+    if (!table && p->cluster_contraction != 1) {
+        const int rc = launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
+        if (rc != ZIPML_ERR_WORKSPACE) return rc;
+    }
     ClusterPlan plan;
     int rc = make_cluster_plan(ctx, d, p, &plan);
     if (rc != ZIPML_OK) return rc;

@@ -1,0 +1,633 @@
+// Cluster engine of zipml_sgd_epoch on uniform grids, int8 tensor cores: one thread-block cluster of nb <= 16 CTAs, the
+// minibatch cut into row parts, the packed row into slices that the CTAs own (Supplement "Double Sampling", footnote
+// form; "End-to-end Quantization").
+//
+// A small step is a chain of hand-overs; its arithmetic is little.  So everything that crosses a warp is kept to what
+// has to cross:
+//   * the model travels as what the dots need of it: the owner of a slice turns its w = step * x~ into four balanced
+//     base-128 digits per entry (int_digits.cuh) with the slice's own scale and stores them, as B fragments, into every
+//     CTA's shared memory (st.async, 16 bytes a thread), with the scale and the slice's part of lo^T x~ behind them;
+//   * a warp waits for its slice alone, multiplies its 32-byte slabs of the codes (mma.sync m16n8k32 u8 x s8: exact
+//     integer sums) and leaves 16 rows x 2 planes of partial dots;                                            barrier
+//   * a warp per 16 rows adds them up, subtracts the labels and writes the residuals' digits: 16 rows of plane 1 with
+//     r2 and 16 rows of plane 2 with r1 are the 32 entries of one contraction;                                barrier
+//   * a warp takes 16-byte columns of one slice (transposing ldmatrix), multiplies, centres the sums (codes less half
+//     the top code: nothing cancels later) and bulk-copies its part of the gradient into the owner's shared memory;
+//   * the owner adds the nb parts in a fixed order, applies Q4, updates its fp32 slice, applies Q3;           barrier
+//     and publishes.
+// Two extra warps copy the code tiles a few steps ahead (cp.async; rows lie an odd number of 16-byte units apart).
+// Buffer reuse: a CTA sends its part of step t after its warps have read the digits of step t (first barrier), and an
+// owner publishes after all parts have arrived: digits, parts and their sources are free when they are written again.
+// Every wait is bounded; when one gives up the CTA records ZIPML_ERR_TIMEOUT, skips its later waits, still issues every
+// store and copy, and all CTAs meet at a cluster barrier before they exit.
+#include <string.h>
+
+#include "int_digits.cuh"
+#include "sgd_common.cuh"
+
+namespace zipml {
+
+constexpr int kSliceWarps = 16;
+constexpr int kSliceThreads = 32 * kSliceWarps;   // without the copying warps
+constexpr int kSliceCopyWarps = 2;
+constexpr int kSliceMaxSlots = 8;
+constexpr int kSliceMaxCtas = 16;
+
+struct SliceArgs {
+    const uint8_t* p1;
+    const uint8_t* p2;
+    const float* lo;
+    const float* step;
+    const float* b;
+    float* x;
+    float* grad_out;             // null or 2n
+    float* model_out;            // null or n: the model the last executed step's gradient saw
+    const int32_t* order;        // device copy of the batch order, or null
+    unsigned long long* trace;
+    DeviceStatus* status;
+    int64_t m, batch, first_step, num_steps, row_bytes;
+    uint64_t seed;
+    uint32_t epoch;
+    float lr;
+    int reg;                     // ZIPML_REG_* and its fp32 constant
+    float reg_cst;
+    int n, bits;
+    int model_bits, grad_bits;
+    int nb, rc, rb;              // CTAs, rows per CTA, blocks of 16 rows
+    int owners, sps;             // CTAs that own a slice, 32-byte slabs per slice
+    int slabs, cols;             // 32-byte slabs and 16-byte columns that hold features
+    int a_parts, spw;            // dots: parts of a slice, slabs per part (a warp takes a part and RBC row blocks at a time)
+    int b_warps, cpw;            // gradient: warps per slice, 16-byte columns per warp
+    int p_shift;                 // 2^p_shift lanes share the sum of one owned feature
+    int pitch, slots;
+    int trace_steps;
+};
+
+struct alignas(16) SliceShared {
+    double base[kSliceWarps];    // owner: per-warp parts of lo^T x~
+    double red[2][kSliceWarps];  // owner: per-warp parts of the squared norms of gradient and model
+    double nrm_g[kSliceMaxCtas]; // squared norms of the owners' gradients and models
+    double nrm_x[kSliceMaxCtas];
+    uint64_t full[kSliceMaxSlots], empty[kSliceMaxSlots];
+    uint64_t w_bar[kSliceMaxCtas];   // a slice's digits have arrived
+    uint64_t part_bar, gn_bar, xn_bar;
+    float wmax[kSliceWarps];     // owner: per-warp maxima of |w|
+    float rmax[kSliceWarps];     // maxima of |residual| of a row block
+    int rows[kSliceMaxSlots];
+    int gave_up;
+    int pad[3];
+};
+
+__device__ __forceinline__ uint32_t slice_peer(const void* local_smem, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local_smem)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void slice_store16(uint32_t dst, uint4 v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];"
+                 ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void slice_store8(uint32_t dst, double v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+                 ::"r"(dst), "l"(__double_as_longlong(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void slice_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void slice_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void slice_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kSliceThreads) : "memory"); }
+
+// Bounded wait on a local phase; after the first failure of this CTA every wait is skipped.
+__device__ __forceinline__ void slice_wait(SliceShared* sh, uint64_t* bar, uint32_t parity, DeviceStatus* status, int where) {
+    if (mbar_try_wait(bar, parity)) return;
+    for (long long spin = 0; spin < kCopySpinLimit; ++spin) {
+        if (mbar_try_wait(bar, parity)) return;
+        if (*reinterpret_cast<volatile int*>(&sh->gave_up)) return;
+    }
+    sh->gave_up = 1;
+    set_status(status, ZIPML_ERR_TIMEOUT, where);
+}
+
+// l2 norm of a vector spread over the owners (v: this thread's share of the squares): per-CTA sums, one store to
+// every owner, added in CTA order.
+__device__ __noinline__ float slice_norm(double v, double* red, double* table, uint64_t* bar, uint32_t parity, int owners, SliceShared* sh,
+                                         DeviceStatus* status, int where) {
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    slice_bar();
+    if ((int)threadIdx.x < owners) {
+        double t = 0.0;
+        for (int w = 0; w < kSliceWarps; ++w) t += red[w];
+        slice_store8(slice_peer(table + blockIdx.x, threadIdx.x), t, slice_peer(bar, threadIdx.x));
+    }
+    slice_wait(sh, bar, parity, status, where);
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, 8u * (uint32_t)owners);     // the next one's
+    double t = 0.0;
+    for (int c = 0; c < owners; ++c) t += table[c];
+    return (float)sqrt(t);
+}
+
+__device__ __forceinline__ void slice_mark(const SliceArgs& a, int64_t it, int id) {
+    if (a.trace && blockIdx.x == 0 && threadIdx.x == 0 && it >= a.first_step && it - a.first_step < a.trace_steps) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %clock64;" : "=l"(t));
+        a.trace[(it - a.first_step) * 8 + id] = t;
+    }
+}
+
+__device__ __forceinline__ void slice_copy16(void* dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void slice_copy4(void* dst_smem, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void slice_arrive_after_copies(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Shared memory after SliceShared; SF = 32 sps NG features of a slice:
+//   wd[owners][sps NG 32 + 4]  words: digits of w [slab][group][t][half][digit], then the scale and lo^T x~ (doubles)
+//   psum[owners a_parts][rb][32]  doubles: partial dots in the order of the residuals' contraction
+//   rdig[rb][32]  words: digits of the residuals [t][half][digit... ] as B fragments
+//   gpart[owners][4 + SF]  this CTA's part of the gradient, slice by slice, behind its sum of residuals
+//   gbuf[nb][4 + SF]       the parts of the own slice
+//   wv[SF]                 w of the own slice
+//   ring[slots]: codes [2][16 rb][pitch], 32 bytes of slack, labels [rc]
+template <int CB, int RBC>
+__global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_slice_kernel(const SliceArgs a) {
+    constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
+    constexpr float QMAXF = (float)IntPath<CB>::QMAX;
+    constexpr int CT = NG == 4 ? 2 : 4;                  // columns that a warp takes at once in the gradient
+    static_assert(NS == 4, "a thread stores four digits at once");
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bi = blockIdx.x;
+    const int n = a.n, sps = a.sps, owners = a.owners, rb = a.rb, SF = 32 * sps * NG;
+    const int wd_words = sps * NG * 32 + 4, part_words = SF + 4;
+    SliceShared* sh = reinterpret_cast<SliceShared*>(s_raw);
+    uint32_t* wd = reinterpret_cast<uint32_t*>(s_raw + sizeof(SliceShared));
+    double* psum = reinterpret_cast<double*>(wd + owners * wd_words);
+    uint32_t* rdig = reinterpret_cast<uint32_t*>(psum + (size_t)owners * a.a_parts * rb * 32);
+    float* gpart = reinterpret_cast<float*>(rdig + rb * 32);
+    float* gbuf = gpart + owners * part_words;
+    float* wv = gbuf + a.nb * part_words;
+    unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wv + SF) + 127) & ~(uintptr_t)127);
+    const int plane_bytes = 16 * rb * a.pitch;
+    const int slot_bytes = (2 * plane_bytes + 32 + 4 * a.rc + 15) & ~15;
+    const int64_t step_end = a.first_step + a.num_steps;
+    const bool owner = bi < owners;
+    const uint32_t part_bytes = 4u * a.nb * (4 + (owner ? min(2 * sps, a.cols - bi * 2 * sps) : 0) * 16 * NG);
+
+    if (tid == 0) {
+        for (int s = 0; s < a.slots; ++s) {
+            mbar_init(sh->full + s, 32 * kSliceCopyWarps + 1);   // the copying lanes, and their leader for rows[]
+            mbar_init(sh->empty + s, kSliceWarps);
+            sh->rows[s] = 0;
+        }
+        for (int o = 0; o < owners; ++o) { mbar_init(sh->w_bar + o, 1); }
+        mbar_init(&sh->part_bar, 1);
+        mbar_init(&sh->gn_bar, 1);
+        mbar_init(&sh->xn_bar, 1);
+        sh->gave_up = 0;
+        mbar_fence_init();
+        for (int o = 0; o < owners; ++o) mbar_arrive_expect_tx(sh->w_bar + o, 4u * wd_words);
+        mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
+        mbar_arrive_expect_tx(&sh->gn_bar, 8u * owners);
+        mbar_arrive_expect_tx(&sh->xn_bar, 8u * owners);
+    }
+    __syncthreads();
+    slice_cluster_sync();                                // every CTA's barriers exist before anyone writes into it
+
+    if (warp >= kSliceWarps) {
+        // -------------------------------------------------------------------- the copying warps
+        constexpr int kLanes = 32 * kSliceCopyWarps;
+        const int me = tid - kSliceThreads;
+        const int units = (int)(a.row_bytes >> 4);       // 16-byte pieces of a row
+        const int r_step = kLanes / units, p_step = kLanes - r_step * units, r_first = me / units, p_first = me - r_first * units;
+        int slot = 0;
+        uint32_t parity = 1;                             // of the slots' emptiness: all are empty at first
+#pragma unroll 1
+        for (int64_t it = a.first_step; it < step_end; ++it) {
+            const int64_t first = (a.order ? (int64_t)a.order[it] : it) * a.batch, r0 = first + (int64_t)bi * a.rc;
+            const int rows = (int)max((int64_t)0, min((int64_t)a.rc, min(a.m, first + a.batch) - r0));
+            unsigned char* dst = ring + (size_t)slot * slot_bytes;
+            slice_wait(sh, sh->empty + slot, parity, a.status, 84);
+            const uint8_t* s1 = a.p1 + r0 * a.row_bytes;
+            const uint8_t* s2 = a.p2 + r0 * a.row_bytes;
+            // the pieces of the rows lie one after the other in memory: piece `me`, me + kLanes, ...
+            for (int r = r_first, p = p_first, at = me * 16; r < rows; at += kLanes * 16) {
+                unsigned char* to = dst + r * a.pitch + p * 16;
+                slice_copy16(to, s1 + at);
+                slice_copy16(to + plane_bytes, s2 + at);
+                r += r_step; p += p_step;
+                if (p >= units) { p -= units; ++r; }
+            }
+            float* labels = reinterpret_cast<float*>(dst + 2 * plane_bytes + 32);
+            for (int r = me; r < rows; r += kLanes) slice_copy4(labels + r, a.b + r0 + r);
+            slice_arrive_after_copies(sh->full + slot);
+            if (me == 0) { sh->rows[slot] = rows; mbar_arrive(sh->full + slot); }
+            if (++slot == a.slots) { slot = 0; parity ^= 1u; }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        slice_cluster_sync();
+        return;
+    }
+
+    // ------------------------------------------------------------------------ the computing warps
+    const int gl = lane >> 2, tl = lane & 3, lm = lane >> 3, l8 = lane & 7;
+    // dots: units of a part of a slice and RBC row blocks, dealt to the warps
+    const int a_all = owners * a.a_parts, a_units = a_all * ((rb + RBC - 1) / RBC);
+    // gradient: slice and columns of this warp
+    const int b_slice = warp / a.b_warps, bj = warp % a.b_warps;
+    const int col_begin = bj * a.cpw, col_end = b_slice < owners ? min(min(2 * sps, a.cols - b_slice * 2 * sps), col_begin + a.cpw) : 0;
+    // owner: feature of this thread
+    const int P = 1 << a.p_shift, pp = tid & (P - 1), k_own = tid >> a.p_shift;
+    const int f_own = bi * SF + k_own;
+    const bool mine = owner && k_own < SF && f_own < n;
+    const float c0f = (float)(1 << (a.bits - 1));
+    const int c0 = 1 << (a.bits - 1);
+    const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
+    const float mid = fmaf(c0f, st, lof);
+    float x = mine ? a.x[f_own] : 0.0f;
+    auto draw = [&](int64_t it, uint32_t stream) { return vector_u24(a.seed, a.epoch, (uint32_t)it, (uint32_t)f_own, stream); };
+    auto quantize = [&](float v, float M, int bits, uint32_t u24) {                  // VecQuant::apply with its draw given
+        if (!(M > 0.0f)) return 0.0f;
+        const float sm = (float)((1 << (bits - 1)) - 1);
+        const float t = __fmul_rn(__fdiv_rn(fabsf(v), M), sm);
+        float fl = floorf(t);
+        fl = fl > sm - 1.0f ? sm - 1.0f : fl;
+        const float p = __fsub_rn(t, fl);
+        const float mag = fl + ((__fmul_rn((float)u24, 5.9604644775390625e-08f) < p) ? 1.0f : 0.0f);
+        const float q = __fmul_rn(M, __fdiv_rn(mag, sm));
+        return v < 0.0f ? -q : q;
+    };
+
+    int slot = 0;
+    uint32_t parity = 0, w_parity = 0, part_parity = 0, gn_parity = 0, xn_parity = 0;
+#pragma unroll 1
+    for (int64_t it = a.first_step - 1; it < step_end; ++it) {
+        const bool last = it == step_end - 1;
+        uint32_t u_x = 0u;
+        if (it >= a.first_step) {
+            slice_mark(a, it, 0);
+            const unsigned char* tile = ring + (size_t)slot * slot_bytes;
+            const uint32_t tile_addr = smem_u32(tile);
+            slice_wait(sh, sh->full + slot, parity, a.status, 6);
+            const int rows = sh->rows[slot];
+            // -------------------------------------------------------------- dots
+#pragma unroll 1
+            for (int unit = warp; unit < a_units; unit += kSliceWarps) {
+                const int ws = unit % a_all, rb0 = unit / a_all * RBC, a_slice = ws / a.a_parts;
+                const int slab0 = (ws - a_slice * a.a_parts) * a.spw, slab1 = min(min(sps, a.slabs - a_slice * sps), slab0 + a.spw);
+                const bool keeper = slab0 == 0 && rb0 == 0;         // re-arms the slice's barrier
+                slice_wait(sh, sh->w_bar + a_slice, w_parity, a.status, 4);
+                if (keeper && lane == 0 && !last) mbar_arrive_expect_tx(sh->w_bar + a_slice, 4u * wd_words);
+                slice_mark(a, it, 1);
+                const uint32_t* wsl = wd + a_slice * wd_words;
+                const double delta = *reinterpret_cast<const double*>(wsl + wd_words - 4);
+                const double base = slab0 == 0 ? *reinterpret_cast<const double*>(wsl + wd_words - 2) : 0.0;
+                {
+                    int c[2][RBC][4];
+#pragma unroll
+                    for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+                        for (int i = 0; i < RBC; ++i)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) c[pl][i][e] = 0;
+                    // lane's address of a fragment: row l8 (+ 8 for the odd matrices), bytes 0 or 16 of the slab
+                    uint32_t addr = tile_addr + (uint32_t)((rb0 * 16 + l8 + (lm & 1) * 8) * a.pitch) + (uint32_t)((a_slice * sps + slab0) * 32 + (lm >> 1) * 16);
+                    const uint32_t* wq = wsl + slab0 * NG * 32 + tl * 8 + (gl & 3);
+#pragma unroll 1
+                    for (int ks = slab0; ks < slab1; ++ks, addr += 32u, wq += NG * 32) {
+                        uint32_t bf[NG][2];
+#pragma unroll
+                        for (int g = 0; g < NG; ++g) {
+                            bf[g][0] = gl < NS ? wq[g * 32] : 0u;
+                            bf[g][1] = gl < NS ? wq[g * 32 + 4] : 0u;
+                        }
+#pragma unroll
+                        for (int i = 0; i < RBC; ++i) {
+                            if (RBC == 1 || rb0 + i < rb) {
+                                uint32_t a1[4], a2[4];
+                                ldsm_x4(a1, addr + (uint32_t)(i * 16 * a.pitch));
+                                ldsm_x4(a2, addr + (uint32_t)(i * 16 * a.pitch + plane_bytes));
+#pragma unroll
+                                for (int g = 0; g < NG; ++g) {
+                                    mma_u8s8(c[0][i], group_bytes<CB>(a1[0], g), group_bytes<CB>(a1[1], g), group_bytes<CB>(a1[2], g),
+                                             group_bytes<CB>(a1[3], g), bf[g][0], bf[g][1]);
+                                    mma_u8s8(c[1][i], group_bytes<CB>(a2[0], g), group_bytes<CB>(a2[1], g), group_bytes<CB>(a2[2], g),
+                                             group_bytes<CB>(a2[3], g), bf[g][0], bf[g][1]);
+                                }
+                            }
+                        }
+                    }
+                    // lane t = 0 has digits 0, 1 of rows g and g + 8, lane t = 1 digits 2, 3: the first takes row g, the
+                    // other row g + 8.  Plane 1's dot belongs to r1, which meets plane 2's codes: entries 16 .. 31.
+#pragma unroll
+                    for (int i = 0; i < RBC; ++i) {
+                        if (RBC == 1 || rb0 + i < rb) {
+#pragma unroll
+                            for (int pl = 0; pl < 2; ++pl) {
+                                const int upper = c[pl][i][0] + 128 * c[pl][i][1], lower = c[pl][i][2] + 128 * c[pl][i][3];
+                                const int got = __shfl_xor_sync(0xffffffffu, tl == 0 ? lower : upper, 1);
+                                const long long v = tl == 0 ? (long long)upper + 16384ll * got : (long long)got + 16384ll * lower;
+                                const int k = (pl == 0 ? 16 : 0) + 4 * (gl >> 1) + (gl & 1) + 2 * tl;
+                                if (tl < 2) psum[((size_t)ws * rb + rb0 + i) * 32 + k] = (double)v * delta + base;
+                            }
+                        }
+                    }
+                }
+            }
+            uint32_t u_g = 0u;
+            if (a.grad_bits > 0 && mine && pp == 0) u_g = draw(it, 4u);
+            if (a.model_bits > 0 && mine && pp == 0) u_x = draw(it + 1, 3u);
+            slice_bar();
+
+            // -------------------------------------------------------------- residuals and their digits
+            if (warp < rb) {
+                const float* labels = reinterpret_cast<const float*>(tile + 2 * plane_bytes + 32);
+                const int row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
+                double d[4] = {row < rows ? -(double)labels[row] : 0.0, 0.0, 0.0, 0.0};
+                const double* ps = psum + warp * 32 + lane;
+                for (int w = 0; w < a_all; w += 4)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (w + i < a_all) d[i] += ps[(w + i) * rb * 32];
+                const float r = row < rows ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
+                float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(r))));
+                if (rb > 1) {                            // one scale for all row blocks
+                    if (lane == 0) sh->rmax[warp] = top;
+                    asm volatile("bar.sync 2, %0;" ::"r"(32 * rb) : "memory");
+                    for (int w2 = 0; w2 < rb; ++w2) top = fmaxf(top, sh->rmax[w2]);
+                } else if (lane == 0) {
+                    sh->rmax[0] = top;
+                }
+                const float inv = top > 0.0f ? QMAXF / top : 0.0f;
+                int digit[NS];
+                balanced_digits<NS>(__float2int_rn(r * inv), digit);
+                unsigned char* out = reinterpret_cast<unsigned char*>(rdig + warp * 32) + ((lane >> 2) & 3) * 32 + (lane >> 4) * 16 + (lane & 3);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) out[4 * s] = (unsigned char)digit[s];
+            }
+            slice_bar();
+            slice_mark(a, it, 2);
+
+            // -------------------------------------------------------------- the rows' part of the gradient
+            if (col_begin < col_end) {
+                float top = sh->rmax[0];
+                for (int w2 = 1; w2 < rb; ++w2) top = fmaxf(top, sh->rmax[w2]);
+                const float delta_r = __fdiv_rn(top, QMAXF);
+                float* part = gpart + b_slice * part_words;
+                const uint32_t row_addr = tile_addr + (uint32_t)((lane >> 4) * plane_bytes + (lane & 15) * a.pitch + b_slice * sps * 32);
+                const uint32_t* rq = rdig + tl * 8 + (gl & 3);
+#pragma unroll 1
+                for (int col0 = col_begin; col0 < col_end; col0 += CT) {
+                    int acc[CT][NG][4], ones[4] = {0, 0, 0, 0};
+#pragma unroll
+                    for (int ti = 0; ti < CT; ++ti)
+#pragma unroll
+                        for (int g = 0; g < NG; ++g)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) acc[ti][g][e] = 0;
+#pragma unroll 1
+                    for (int kb = 0; kb < rb; ++kb) {
+                        const uint32_t b0 = gl < NS ? rq[kb * 32] : 0u, b1 = gl < NS ? rq[kb * 32 + 4] : 0u;
+                        mma_u8s8(ones, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, b0, b1);
+#pragma unroll
+                        for (int ti = 0; ti < CT; ++ti) {
+                            if (col0 + ti < col_end) {
+                                uint32_t r4[4];
+                                ldsm_x4_trans(r4, row_addr + (uint32_t)(kb * 16 * a.pitch + (col0 + ti) * 16));
+                                const uint32_t pel = __byte_perm(r4[0], r4[1], 0x6420), pol = __byte_perm(r4[0], r4[1], 0x7531);
+                                const uint32_t peh = __byte_perm(r4[2], r4[3], 0x6420), poh = __byte_perm(r4[2], r4[3], 0x7531);
+#pragma unroll
+                                for (int g = 0; g < NG; ++g)
+                                    mma_u8s8(acc[ti][g], group_bytes<CB>(pel, g), group_bytes<CB>(pol, g), group_bytes<CB>(peh, g),
+                                             group_bytes<CB>(poh, g), b0, b1);
+                            }
+                        }
+                    }
+                    // sums of (code - c0) * residual; rows g, g + 8 of the accumulators are bytes 2g, 2g + 1 of the column
+                    const float weight = tl == 0 ? delta_r : 16384.0f * delta_r;
+#pragma unroll
+                    for (int ti = 0; ti < CT; ++ti) {
+                        if (col0 + ti < col_end) {
+#pragma unroll
+                            for (int g = 0; g < NG; ++g) {
+                                const int upper = (acc[ti][g][0] - c0 * ones[0]) + 128 * (acc[ti][g][1] - c0 * ones[1]);
+                                const int lower = (acc[ti][g][2] - c0 * ones[0]) + 128 * (acc[ti][g][3] - c0 * ones[1]);
+                                const float up = (float)upper * weight, low = (float)lower * weight;
+                                const float got = __shfl_xor_sync(0xffffffffu, tl == 0 ? low : up, 1);
+                                if (tl < 2) part[4 + ((col0 + ti) * 16 + 2 * gl + tl) * NG + g] = (tl == 0 ? up : low) + got;
+                            }
+                        }
+                    }
+                    if (bj == 0 && col0 == 0) {          // the sum of the residuals
+                        const float s = (float)(ones[0] + 128 * ones[1]) * weight;
+                        const float all = s + __shfl_xor_sync(0xffffffffu, s, 1);
+                        if (lane == 0) part[0] = all;
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    const int w0 = bj == 0 ? 0 : 4 + col_begin * 16 * NG, w1 = 4 + col_end * 16 * NG;
+                    slice_copy(slice_peer(gbuf + bi * part_words + w0, b_slice), part + w0, 4u * (w1 - w0), slice_peer(&sh->part_bar, b_slice));
+                }
+            }
+            if (lane == 0) mbar_arrive(sh->empty + slot);
+            if (++slot == a.slots) { slot = 0; parity ^= 1u; }
+            w_parity ^= 1u;
+            slice_mark(a, it, 3);
+
+            // -------------------------------------------------------------- the owner sums the parts and updates
+            if (owner) {
+                slice_wait(sh, &sh->part_bar, part_parity, a.status, 2);
+                part_parity ^= 1u;
+                if (tid == 0 && !last) mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
+                const int64_t t_now = a.order ? (int64_t)a.order[it] : it;
+                const double scale = 1.0 / (2.0 * (double)min(a.batch, a.m - t_now * a.batch));
+                double t = 0.0;
+                if (mine)
+                    for (int w = pp; w < a.nb; w += P) t += (double)fmaf(st, gbuf[w * part_words + 4 + k_own], mid * gbuf[w * part_words]);
+                for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                float g = (float)(t * scale);
+                const bool writes = mine && pp == 0;
+                if (last && a.grad_out && writes) a.grad_out[f_own] = g;
+                slice_mark(a, it, 4);
+                if (a.grad_bits > 0) {
+                    const float M = slice_norm(writes ? (double)g * (double)g : 0.0, sh->red[0], sh->nrm_g, &sh->gn_bar, gn_parity, owners, sh, a.status, 3);
+                    gn_parity ^= 1u;
+                    g = quantize(g, M, a.grad_bits, u_g);
+                }
+                if (last && a.grad_out && writes) a.grad_out[n + f_own] = g;
+                x = regularise(fmaf(-a.lr, g, x), x, a.reg, a.reg_cst);
+            }
+        } else if (a.model_bits > 0 && mine && pp == 0) {
+            u_x = draw(it + 1, 3u);
+        }
+        if (last) break;
+
+        // ------------------------------------------------------------------ publish what the next step sees
+        if (owner) {
+            float xt = x;
+            if (a.model_bits > 0) {
+                const float M = slice_norm(mine && pp == 0 ? (double)x * (double)x : 0.0, sh->red[1], sh->nrm_x, &sh->xn_bar, xn_parity, owners, sh, a.status, 8);
+                xn_parity ^= 1u;
+                xt = quantize(x, M, a.model_bits, u_x);
+            }
+            const bool writes = mine && pp == 0;
+            if (a.model_out && it + 2 == step_end && writes) a.model_out[f_own] = xt;
+            const float w = writes ? st * xt : 0.0f;
+            if (pp == 0 && k_own < SF) wv[k_own] = w;
+            const float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w))));
+            double bpart = writes ? (double)lof * (double)xt : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (o >= P) bpart += __shfl_xor_sync(0xffffffffu, bpart, o);
+            if (lane == 0) { sh->wmax[warp] = top; sh->base[warp] = bpart; }
+            slice_bar();
+            float wmax = 0.0f;
+#pragma unroll
+            for (int i = 0; i < kSliceWarps; ++i) wmax = fmaxf(wmax, sh->wmax[i]);
+            const float inv = wmax > 0.0f ? QMAXF / wmax : 0.0f;
+            const int items = 8 * sps * NG;
+            for (int idx = tid; idx < items * a.nb; idx += kSliceThreads) {
+                const int dest = idx / items, item = idx - dest * items;
+                const int half = item & 1, t = (item >> 1) & 3, gs = item >> 3, g = gs % NG, q = (gs / NG) * 8 + half * 4 + t;
+                const float* src = wv + q * 4 * NG + g;
+                const float v4[4] = {src[0], src[NG], src[2 * NG], src[3 * NG]};
+                slice_store16(slice_peer(wd + bi * wd_words + 4 * item, dest), digit_words<NS>(v4, inv), slice_peer(sh->w_bar + bi, dest));
+            }
+            if (tid >= kSliceThreads - a.nb) {           // the scale and lo^T x~
+                const int dest = tid - (kSliceThreads - a.nb);
+                double base = 0.0;
+#pragma unroll
+                for (int i = 0; i < kSliceWarps; ++i) base += sh->base[i];
+                const unsigned long long s = (unsigned long long)__double_as_longlong((double)wmax / (double)QMAXF), l = (unsigned long long)__double_as_longlong(base);
+                slice_store16(slice_peer(wd + bi * wd_words + wd_words - 4, dest), make_uint4((uint32_t)s, (uint32_t)(s >> 32), (uint32_t)l, (uint32_t)(l >> 32)),
+                              slice_peer(sh->w_bar + bi, dest));
+            }
+        }
+        slice_mark(a, it, 5);
+    }
+    if (mine && pp == 0) a.x[f_own] = x;
+    __syncwarp();
+    slice_cluster_sync();                                // nobody leaves while a copy may still target it
+}
+
+// ---------------------------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------------------------
+struct SlicePlan {
+    int nb, rc, rb, owners, sps, slabs, cols, a_parts, spw, b_warps, cpw, p_shift, pitch, slots;
+    size_t smem;
+};
+
+static size_t slice_smem_bytes(const SlicePlan& r, int ng, int slots) {
+    const size_t sf = (size_t)32 * r.sps * ng;
+    size_t bytes = sizeof(SliceShared) + 4 * (size_t)r.owners * ((size_t)r.sps * ng * 32 + 4) + 8 * (size_t)r.owners * r.a_parts * r.rb * 32 +
+                   4 * (size_t)r.rb * 32 + 4 * (size_t)(r.owners + r.nb) * (sf + 4) + 4 * sf + 128;
+    return bytes + (size_t)slots * (((size_t)2 * 16 * r.rb * r.pitch + 32 + 4 * r.rc + 15) & ~(size_t)15);
+}
+
+static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, SlicePlan* plan) {
+    const int cb = container_bits(d->bits), ng = 8 / cb;
+    const int64_t B = p->batch < d->m ? p->batch : d->m;
+    const int64_t used = (d->n * cb + 7) / 8, slabs = (used + 31) / 32;
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || slabs > 1024 || d->row_bytes > (1 << 16)) return ZIPML_ERR_WORKSPACE;
+    int64_t nb = p->grid_row_parts > 0 ? p->grid_row_parts : (B + 15) / 16;     // automatic: 16 rows per CTA
+    if (nb > kSliceMaxCtas) nb = kSliceMaxCtas;
+    if (nb > B) nb = B;
+    for (; nb <= kSliceMaxCtas && nb <= B; ++nb) {       // (more parts than asked for where a tile or a slice does not fit)
+        SlicePlan r;
+        r.rc = (int)((B + nb - 1) / nb);
+        r.nb = (int)((B + r.rc - 1) / r.rc);
+        r.rb = (r.rc + 15) / 16;
+        r.sps = (int)((slabs + r.nb - 1) / r.nb);
+        r.owners = (int)((slabs + r.sps - 1) / r.sps);
+        r.slabs = (int)slabs; r.cols = (int)((used + 15) / 16);
+        if (r.rb > kSliceWarps || 32 * r.sps * ng > kSliceThreads) continue;
+        const int per = kSliceWarps / r.owners;
+        r.spw = (r.sps + per - 1) / per;
+        r.a_parts = (r.sps + r.spw - 1) / r.spw;
+        r.cpw = (2 * r.sps + per - 1) / per;
+        r.b_warps = per;
+        r.p_shift = 0;
+        while (r.p_shift < 4 && (32 * r.sps * ng) << (r.p_shift + 1) <= kSliceThreads && (1 << r.p_shift) < r.nb) ++r.p_shift;
+        const int units = (int)(d->row_bytes / 16);
+        r.pitch = 16 * (units | 1);
+        r.slots = kSliceMaxSlots;
+        while (r.slots >= 2 && slice_smem_bytes(r, ng, r.slots) > (size_t)ctx->smem_optin) --r.slots;
+        if (r.slots < 2) continue;
+        r.smem = slice_smem_bytes(r, ng, r.slots);
+        *plan = r;
+        return ZIPML_OK;
+    }
+    return ZIPML_ERR_WORKSPACE;
+}
+
+int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                     int64_t num_steps, float* grad_out) {
+    SlicePlan plan;
+    int rc = make_slice_plan(ctx, d, p, &plan);
+    if (rc != ZIPML_OK) return rc;
+    const int cb = container_bits(d->bits);
+    const bool one = plan.rb == 1;
+    const void* kernel = cb == 2 ? (one ? (const void*)sgd_slice_kernel<2, 1> : (const void*)sgd_slice_kernel<2, 4>)
+                       : cb == 4 ? (one ? (const void*)sgd_slice_kernel<4, 1> : (const void*)sgd_slice_kernel<4, 4>)
+                                 : (one ? (const void*)sgd_slice_kernel<8, 1> : (const void*)sgd_slice_kernel<8, 4>);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+    if (e == cudaSuccess && plan.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return cuda_status(e);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)plan.nb);
+    cfg.blockDim = dim3(kSliceThreads + 32 * kSliceCopyWarps);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)plan.nb;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
+    if (clusters < 1) return ZIPML_ERR_WORKSPACE;
+    const int64_t T = (d->m + p->batch - 1) / p->batch;
+    SliceArgs a;
+    memset(&a, 0, sizeof(a));
+    if (p->batch_order) {
+        rc = ws_reserve(ctx, carve_size(sizeof(int32_t) * (size_t)T));
+        if (rc != ZIPML_OK) return rc;
+        e = cudaMemcpyAsync(ctx->ws, p->batch_order, sizeof(int32_t) * (size_t)T, cudaMemcpyHostToDevice, ctx->stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        a.order = reinterpret_cast<const int32_t*>(ctx->ws);
+    }
+    a.p1 = d->plane1; a.p2 = d->plane2; a.lo = d->feat_lo; a.step = d->feat_step;
+    a.b = b; a.x = x; a.grad_out = grad_out; a.model_out = p->model_out;
+    a.trace = reinterpret_cast<unsigned long long*>(p->trace);
+    a.trace_steps = p->trace ? p->trace_steps : 0;
+    a.status = ctx->d_status;
+    a.m = d->m; a.batch = p->batch < d->m ? p->batch : d->m; a.row_bytes = d->row_bytes;
+    a.first_step = first_step; a.num_steps = num_steps;
+    a.seed = p->seed; a.epoch = (uint32_t)p->epoch; a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
+    a.n = (int)d->n; a.bits = d->bits; a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
+    a.nb = plan.nb; a.rc = plan.rc; a.rb = plan.rb; a.owners = plan.owners; a.sps = plan.sps; a.slabs = plan.slabs; a.cols = plan.cols;
+    a.a_parts = plan.a_parts; a.spw = plan.spw; a.b_warps = plan.b_warps; a.cpw = plan.cpw;
+    a.p_shift = plan.p_shift; a.pitch = plan.pitch; a.slots = plan.slots;
+    void* params[] = {&a};
+    e = cudaLaunchKernelExC(&cfg, kernel, params);
+    if (e != cudaSuccess) return cuda_status(e);
+    ctx->launches += 1;
+    ctx->last_engine = ZIPML_ENGINE_CLUSTER;
+    return ZIPML_OK;
+}
+
+}  // namespace zipml

@@ -305,10 +305,54 @@ def test_solo_engine(ctx, m, n, bits, batch, table):
     assert (g[1].cpu().numpy() != g4).sum() <= 2
     y = x0 - np.float32(lr) * g[1].cpu().numpy()
     assert np.allclose(x.cpu().numpy(), y, rtol=1e-6, atol=1e-7)
-    if batch <= 16:
+    if batch <= 16 and n <= 1000:
         ctx.zipml_sgd_epoch(gds, db, to_dev(x0, ctx), batch, lr)
         ctx.zipml_sync()
         assert ctx.zipml_last_engine() == binding.ENGINE_SOLO               # what AUTO takes
+
+
+@pytest.mark.parametrize("m,n,bits,batch,parts", [
+    (50, 3, 8, 5, 0), (700, 33, 8, 130, 3), (900, 65, 4, 257, 0), (400, 1000, 8, 100, 0), (1100, 130, 2, 512, 2), (300, 2048, 2, 37, 0),
+    (70, 4090, 8, 33, 0), (600, 520, 6, 250, 16), (2100, 40, 4, 2048, 0), (64, 6100, 2, 16, 16),
+])
+def test_slice_form_of_the_cluster_engine(ctx, m, n, bits, batch, parts):
+    """The int8 form at the edges of its cuts: slabs, columns and slices left over, one and several row blocks, CTAs
+    without a slice or without rows, with a batch order, a regulariser and quantized model and gradient."""
+    _, A, b, _ = workload("c1", m, n, seed=n)
+    ods = oracle.quantize(A, bits, seed=3)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    T = (m + batch - 1) // batch
+    lr = 0.3 / n
+    order = np.random.default_rng(0).permutation(T).astype(np.int32)
+    x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
+    how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=2, grid_row_parts=parts)
+    for kw in (dict(batch_order=order), dict(reg=binding.REG_L2, reg_param=0.1)):
+        x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, **kw)
+        x_before, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, num_steps=T - 1, **kw)
+        _, g_ref = oracle.sgd_epoch(ods, b, x_before, batch, lr, first_step=T - 1, num_steps=1, want_grad=True, **kw)
+        x = to_dev(x0, ctx)
+        ctx.zipml_sgd_epoch(gds, db, x, batch, lr, **how, **kw)
+        ctx.zipml_sync()
+        assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+        xb, seen = to_dev(x_before, ctx), torch.zeros(n, device=ctx.device)
+        g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+        ctx.zipml_sgd_epoch(gds, db, xb, batch, lr, first_step=T - 1, num_steps=1, grad_out=g, model_out=seen, **how, **kw)
+        ctx.zipml_sync()
+        assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL and (g[0] == g[1]).all()
+        assert (seen.cpu().numpy() == x_before).all() and rel(xb.cpu().numpy(), x_ref) <= MODEL_TOL
+    x, seen = to_dev(x0, ctx), torch.zeros(n, device=ctx.device)
+    g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+    kw = dict(seed=5, epoch=1, first_step=0, num_steps=1)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, model_bits=8, grad_bits=6, grad_out=g, model_out=seen, **how, **kw)
+    ctx.zipml_sync()
+    want, _ = oracle.quantize_vector(x0, 8, 5, 1, 0, 3)
+    margin, _ = q3_margins(x0, 8, 5, 1, 0)
+    seen = seen.cpu().numpy()
+    assert not ((seen != want) & (margin >= 1e-4)).any()
+    _, g_ref = oracle.sgd_epoch(ods, b, seen, batch, lr, want_grad=True, **kw)
+    assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL
+    g4, _ = oracle.quantize_vector(g[0].cpu().numpy(), 6, 5, 1, 0, 4)
+    assert (g[1].cpu().numpy() != g4).sum() <= 3
 
 
 @pytest.mark.parametrize("contraction", [1, 2], ids=["fp32", "int8"])
