@@ -2,10 +2,15 @@
 // the bounded grid barrier and the row-scaled vector quantizer.
 #pragma once
 
+#include <cuda.h>
+
 #include "common.cuh"
 #include "internal.h"
 
 namespace zipml {
+
+// Tensor maps of the two planes for boxes of box_words x cr rows (sgd_ring.cu); wide_elements: boxes above 256 words.
+int encode_plane_maps(zipml_ctx* ctx, const zipml_dataset* d, int box_words, int cr, bool wide_elements, CUtensorMap* out);
 
 constexpr int kSgdThreads = 256;
 constexpr int kSgdWarps = kSgdThreads / 32;

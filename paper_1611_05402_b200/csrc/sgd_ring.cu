@@ -1154,7 +1154,7 @@ static int64_t plane_wc_check(int wc) { return (int64_t)wc; }
 
 // Tensor maps over the two planes seen as m x row_words matrices of 32-bit words.  The encoder is a
 // driver entry point looked up through the runtime (no link against the driver library).
-static int encode_plane_maps(zipml_ctx* ctx, const zipml_dataset* d, int box_words, int cr, bool wide_elements, CUtensorMap* out) {
+int encode_plane_maps(zipml_ctx* ctx, const zipml_dataset* d, int box_words, int cr, bool wide_elements, CUtensorMap* out) {
     typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -4,22 +4,31 @@
 //
 // A small step is a chain of hand-overs; its arithmetic is little.  So everything that crosses a warp is kept to what
 // has to cross:
-//   * the model travels as what the dots need of it: the owner of a slice turns its w = step * x~ into four balanced
-//     base-128 digits per entry (int_digits.cuh) with the slice's own scale and stores them, as B fragments, into every
-//     CTA's shared memory (st.async, 16 bytes a thread), with the scale and the slice's part of lo^T x~ behind them;
+//   * the model travels as what the dots need of it: the owner of a slice turns its w = step * x~ into fixed point with the
+//     slice's own power of two and stores the bytes (four balanced base-256 digits per entry: W + 0x80808080, xor
+//     0x80808080), as B fragments, into every CTA's shared memory (st.async, 16 bytes a thread), with the scale and the
+//     slice's part of lo^T x~ behind them;
 //   * a warp waits for its slice alone, multiplies its 32-byte slabs of the codes (mma.sync m16n8k32 u8 x s8: exact
 //     integer sums) and leaves 16 rows x 2 planes of partial dots;                                            barrier
 //   * a warp per 16 rows adds them up, subtracts the labels and writes the residuals' digits: 16 rows of plane 1 with
 //     r2 and 16 rows of plane 2 with r1 are the 32 entries of one contraction;                                barrier
 //   * a warp takes 16-byte columns of one slice (transposing ldmatrix), multiplies, centres the sums (codes less half
-//     the top code: nothing cancels later) and bulk-copies its part of the gradient into the owner's shared memory;
+//     the top code: nothing cancels later) and bulk-copies its part of the gradient, a low and a high integer per feature,
+//     into the owner's shared memory;
 //   * the owner adds the nb parts in a fixed order, applies Q4, updates its fp32 slice, applies Q3;           barrier
 //     and publishes.
-// Two extra warps copy the code tiles a few steps ahead (cp.async; rows lie an odd number of 16-byte units apart).
+// Codes of less than 8 bits are masked where they lie in their byte: the shift is in the digits (dots) or comes off the
+// sums (gradient).
+// The code tiles come a few steps ahead, one tensor copy per plane whose box is as wide as the distance of the rows in
+// shared memory, an odd number of 16-byte units (rows above 2 KB: a bulk copy each).
 // Buffer reuse: a CTA sends its part of step t after its warps have read the digits of step t (first barrier), and an
 // owner publishes after all parts have arrived: digits, parts and their sources are free when they are written again.
+// The step's machine code has to stay small: what does not fit the instruction cache is fetched again every step (with
+// everything inlined and unrolled, 64 to 78 KB, the kernel took twice as long).  So loops are rolled, rare paths and
+// random draws are out of line, and nothing is divided inside the loop.
 // Every wait is bounded; when one gives up the CTA records ZIPML_ERR_TIMEOUT, skips its later waits, still issues every
 // store and copy, and all CTAs meet at a cluster barrier before they exit.
+#include <cuda.h>
 #include <string.h>
 
 #include "int_digits.cuh"
@@ -28,8 +37,7 @@
 namespace zipml {
 
 constexpr int kSliceWarps = 16;
-constexpr int kSliceThreads = 32 * kSliceWarps;   // without the copying warps
-constexpr int kSliceCopyWarps = 2;
+constexpr int kSliceThreads = 32 * kSliceWarps;   // without the copying warp
 constexpr int kSliceMaxSlots = 8;
 constexpr int kSliceMaxCtas = 16;
 
@@ -53,29 +61,30 @@ struct SliceArgs {
     float reg_cst;
     int n, bits;
     int model_bits, grad_bits;
+    int whole, rows_last;        // batches below `whole` are full, that one has rows_last rows
+    double full_scale, last_scale;   // 1 / (2 rows)
     int nb, rc, rb;              // CTAs, rows per CTA, blocks of 16 rows
     int owners, sps;             // CTAs that own a slice, 32-byte slabs per slice
     int slabs, cols;             // 32-byte slabs and 16-byte columns that hold features
-    int a_parts, spw;            // dots: parts of a slice, slabs per part (a warp takes a part and RBC row blocks at a time)
-    int b_warps, cpw;            // gradient: warps per slice, 16-byte columns per warp
+    int a_parts, a_inv, spw;     // dots: parts of a slice, slabs per part (a warp takes a part and RBC row blocks at a time)
+    int b_parts, b_inv, cpw;     // gradient: parts of a slice, 16-byte columns per part
     int p_shift;                 // 2^p_shift lanes share the sum of one owned feature
-    int pitch, slots;
+    int pitch, slots, use_tmap;
     int trace_steps;
 };
 
 struct alignas(16) SliceShared {
-    double base[kSliceWarps];    // owner: per-warp parts of lo^T x~
-    double red[2][kSliceWarps];  // owner: per-warp parts of the squared norms of gradient and model
+    double base[16];             // owner: per-warp parts of lo^T x~ (entries past the warps stay zero, here and below)
+    double red[2][16];           // owner: per-warp parts of the squared norms of gradient and model
     double nrm_g[kSliceMaxCtas]; // squared norms of the owners' gradients and models
     double nrm_x[kSliceMaxCtas];
     uint64_t full[kSliceMaxSlots], empty[kSliceMaxSlots];
     uint64_t w_bar[kSliceMaxCtas];   // a slice's digits have arrived
     uint64_t part_bar, gn_bar, xn_bar;
-    float wmax[kSliceWarps];     // owner: per-warp maxima of |w|
-    float rmax[kSliceWarps];     // maxima of |residual| of a row block
-    int rows[kSliceMaxSlots];
+    float delta_r;               // value of a unit of the residuals' fixed point
+    float wmax[32];              // owner: per-warp maxima of |w|
+    float rmax[16];              // maxima of |residual| of a row block
     int gave_up;
-    int pad[3];
 };
 
 __device__ __forceinline__ uint32_t slice_peer(const void* local_smem, uint32_t rank) {
@@ -100,9 +109,49 @@ __device__ __forceinline__ void slice_cluster_sync() {
 }
 __device__ __forceinline__ void slice_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kSliceThreads) : "memory"); }
 
+// Power of two 2^k by which values up to `top` become integers within the range of four balanced base-256 digits
+// (2^31 - 2^31/128), `spare` bits kept back.  top = 0: 0.
+__device__ __forceinline__ int slice_exponent(float top, int spare) {
+    const int e = (int)(__float_as_uint(top * 1.01f) >> 23) - 127;
+    return min(126, 30 - spare - e);
+}
+__device__ __forceinline__ float slice_pow2(int k) { return k >= -126 ? __uint_as_float((uint32_t)(k + 127) << 23) : 0.0f; }
+// Sixteen doubles in a fixed order, four chains.
+__device__ __forceinline__ double slice_sum16(const double* v) {
+    double s[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+    for (int i = 4; i < 16; i += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[j] += v[i + j];
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
+// Codes of group g of a fragment register, where they lie in their bytes ...
+template <int CB>
+__device__ __forceinline__ uint32_t slice_codes(uint32_t u, int g) {
+    if constexpr (CB == 8) return u;
+    else return u & ((CB == 4 ? 0x0F0F0F0Fu : 0x03030303u) << (CB * g));
+}
+// ... and, for the dots, at most 4 bits up (2-bit codes: the upper pair is shifted down first).
+template <int CB>
+__device__ __forceinline__ uint32_t slice_dot_codes(uint32_t u, int g) {
+    if constexpr (CB == 2) return slice_codes<2>(g & 2 ? u >> 4 : u, g & 1);
+    else return slice_codes<CB>(u, g);
+}
+template <int CB>
+struct SliceShift {                                       // bits that a group's digits are shifted up by, against the lowest group
+    static constexpr int kMost = CB == 8 ? 0 : CB == 4 ? 4 : 2;
+    __device__ static constexpr int of(int g) { return CB == 8 ? 0 : CB == 4 ? (g == 0 ? 4 : 0) : (g & 1 ? 0 : 2); }
+};
+// D = A B + C with C's two columns given.
+__device__ __forceinline__ void slice_mma_from(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c0, int c1) {
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
+        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c0), "r"(c1));
+}
+
+
 // Bounded wait on a local phase; after the first failure of this CTA every wait is skipped.
-__device__ __forceinline__ void slice_wait(SliceShared* sh, uint64_t* bar, uint32_t parity, DeviceStatus* status, int where) {
-    if (mbar_try_wait(bar, parity)) return;
+__device__ __noinline__ void slice_wait_long(SliceShared* sh, uint64_t* bar, uint32_t parity, DeviceStatus* status, int where) {
+#pragma unroll 1
     for (long long spin = 0; spin < kCopySpinLimit; ++spin) {
         if (mbar_try_wait(bar, parity)) return;
         if (*reinterpret_cast<volatile int*>(&sh->gave_up)) return;
@@ -110,87 +159,96 @@ __device__ __forceinline__ void slice_wait(SliceShared* sh, uint64_t* bar, uint3
     sh->gave_up = 1;
     set_status(status, ZIPML_ERR_TIMEOUT, where);
 }
+__device__ __forceinline__ void slice_wait(SliceShared* sh, uint64_t* bar, uint32_t parity, DeviceStatus* status, int where) {
+    if (!mbar_try_wait(bar, parity)) slice_wait_long(sh, bar, parity, status, where);
+}
 
-// l2 norm of a vector spread over the owners (v: this thread's share of the squares): per-CTA sums, one store to
+__device__ __noinline__ float slice_regularise(float y, float x_old, int reg, float cst) { return regularise(y, x_old, reg, cst); }
+__device__ __noinline__ uint32_t slice_draw(uint64_t seed, uint32_t epoch, uint32_t step, uint32_t coord, uint32_t stream) {
+    return vector_u24(seed, epoch, step, coord, stream);
+}
+// VecQuant::apply with its draw given.
+__device__ __noinline__ float slice_quantize(float v, float M, int bits, uint32_t u24) {
+    if (!(M > 0.0f)) return 0.0f;
+    const float sm = (float)((1 << (bits - 1)) - 1);
+    const float t = __fmul_rn(__fdiv_rn(fabsf(v), M), sm);
+    float fl = floorf(t);
+    fl = fl > sm - 1.0f ? sm - 1.0f : fl;
+    const float p = __fsub_rn(t, fl);
+    const float mag = fl + ((__fmul_rn((float)u24, 5.9604644775390625e-08f) < p) ? 1.0f : 0.0f);
+    const float q = __fmul_rn(M, __fdiv_rn(mag, sm));
+    return v < 0.0f ? -q : q;
+}
+
+// l2 norm of a vector spread over the owners (v: this thread's share of the squares, in every `every`-th lane): per-CTA sums, one store to
 // every owner, added in CTA order.
-__device__ __noinline__ float slice_norm(double v, double* red, double* table, uint64_t* bar, uint32_t parity, int owners, SliceShared* sh,
+__device__ __noinline__ float slice_norm(double v, int every, double* red, double* table, uint64_t* bar, uint32_t parity, int owners, SliceShared* sh,
                                          DeviceStatus* status, int where) {
-    v = warp_sum(v);
+#pragma unroll 1
+    for (int o = 16; o >= every; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     slice_bar();
     if ((int)threadIdx.x < owners) {
-        double t = 0.0;
-        for (int w = 0; w < kSliceWarps; ++w) t += red[w];
-        slice_store8(slice_peer(table + blockIdx.x, threadIdx.x), t, slice_peer(bar, threadIdx.x));
+        slice_store8(slice_peer(table + blockIdx.x, threadIdx.x), slice_sum16(red), slice_peer(bar, threadIdx.x));
     }
     slice_wait(sh, bar, parity, status, where);
     if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, 8u * (uint32_t)owners);     // the next one's
-    double t = 0.0;
-    for (int c = 0; c < owners; ++c) t += table[c];
-    return (float)sqrt(t);
+    return (float)sqrt(slice_sum16(table));          // (entries past the owners stay zero)
 }
 
-__device__ __forceinline__ void slice_mark(const SliceArgs& a, int64_t it, int id) {
-    if (a.trace && blockIdx.x == 0 && threadIdx.x == 0 && it >= a.first_step && it - a.first_step < a.trace_steps) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %clock64;" : "=l"(t));
-        a.trace[(it - a.first_step) * 8 + id] = t;
-    }
+__device__ __noinline__ void slice_mark(unsigned long long* trace, int step, int id) {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %clock64;" : "=l"(t));
+    trace[step * 8 + id] = t;
 }
 
-__device__ __forceinline__ void slice_copy16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void slice_copy4(void* dst_smem, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void slice_arrive_after_copies(uint64_t* bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void slice_tensor_copy(void* dst_smem, const CUtensorMap* tm, int y, uint64_t* bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(smem_u32(dst_smem)), "l"(tm), "r"(0), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
 
 // Shared memory after SliceShared; SF = 32 sps NG features of a slice:
 //   wd[owners][sps NG 32 + 4]  words: digits of w [slab][group][t][half][digit], then the scale and lo^T x~ (doubles)
 //   psum[owners a_parts][rb][32]  doubles: partial dots in the order of the residuals' contraction
 //   rdig[rb][32]  words: digits of the residuals [t][half][digit... ] as B fragments
-//   gpart[owners][4 + SF]  this CTA's part of the gradient, slice by slice, behind its sum of residuals
-//   gbuf[nb][4 + SF]       the parts of the own slice
+//   gpart[owners][4 + 2 SF]  this CTA's part of the gradient, slice by slice, behind its sum of residuals and their scale
+//   gbuf[nb][4 + 2 SF]       the parts of the own slice
 //   wv[SF]                 w of the own slice
-//   ring[slots]: codes [2][16 rb][pitch], 32 bytes of slack, labels [rc]
+//   ring[slots]: codes [2][16 rb][pitch], 128 bytes of slack
 template <int CB, int RBC>
-__global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_slice_kernel(const SliceArgs a) {
+__global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const SliceArgs a, const __grid_constant__ CUtensorMap tm1,
+                                                                     const __grid_constant__ CUtensorMap tm2) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
-    constexpr float QMAXF = (float)IntPath<CB>::QMAX;
-    constexpr int CT = NG == 4 ? 2 : 4;                  // columns that a warp takes at once in the gradient
+    constexpr int CT = NG == 1 ? 2 : 1;                  // columns that a warp takes at once in the gradient
     static_assert(NS == 4, "a thread stores four digits at once");
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bi = blockIdx.x;
     const int n = a.n, sps = a.sps, owners = a.owners, rb = a.rb, SF = 32 * sps * NG;
-    const int wd_words = sps * NG * 32 + 4, part_words = SF + 4;
+    const int wd_words = sps * NG * 32 + 4, part_words = 2 * SF + 4;
     SliceShared* sh = reinterpret_cast<SliceShared*>(s_raw);
     uint32_t* wd = reinterpret_cast<uint32_t*>(s_raw + sizeof(SliceShared));
     double* psum = reinterpret_cast<double*>(wd + owners * wd_words);
-    uint32_t* rdig = reinterpret_cast<uint32_t*>(psum + (size_t)owners * a.a_parts * rb * 32);
-    float* gpart = reinterpret_cast<float*>(rdig + rb * 32);
-    float* gbuf = gpart + owners * part_words;
-    float* wv = gbuf + a.nb * part_words;
+    uint32_t* rdig = reinterpret_cast<uint32_t*>(psum + owners * a.a_parts * rb * 32);
+    int* gpart = reinterpret_cast<int*>(rdig + rb * 32);
+    int* gbuf = gpart + owners * part_words;
+    float* wv = reinterpret_cast<float*>(gbuf + a.nb * part_words);
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(wv + SF) + 127) & ~(uintptr_t)127);
-    const int plane_bytes = 16 * rb * a.pitch;
-    const int slot_bytes = (2 * plane_bytes + 32 + 4 * a.rc + 15) & ~15;
-    const int64_t step_end = a.first_step + a.num_steps;
+    const int plane_bytes = (16 * rb * a.pitch + 127) & ~127, slot_bytes = 2 * plane_bytes + 128;
     const bool owner = bi < owners;
-    const uint32_t part_bytes = 4u * a.nb * (4 + (owner ? min(2 * sps, a.cols - bi * 2 * sps) : 0) * 16 * NG);
+    const uint32_t part_bytes = 4u * a.nb * (4 + (owner ? min(2 * sps, a.cols - bi * 2 * sps) : 0) * 32 * NG);
 
     if (tid == 0) {
         for (int s = 0; s < a.slots; ++s) {
-            mbar_init(sh->full + s, 32 * kSliceCopyWarps + 1);   // the copying lanes, and their leader for rows[]
+            mbar_init(sh->full + s, 1);
             mbar_init(sh->empty + s, kSliceWarps);
-            sh->rows[s] = 0;
         }
         for (int o = 0; o < owners; ++o) { mbar_init(sh->w_bar + o, 1); }
         mbar_init(&sh->part_bar, 1);
         mbar_init(&sh->gn_bar, 1);
         mbar_init(&sh->xn_bar, 1);
         sh->gave_up = 0;
+        for (int c = 0; c < 16; ++c) sh->nrm_g[c] = sh->nrm_x[c] = sh->base[c] = sh->red[0][c] = sh->red[1][c] = 0.0;
+        for (int c = 0; c < 32; ++c) sh->wmax[c] = 0.0f;
         mbar_fence_init();
         for (int o = 0; o < owners; ++o) mbar_arrive_expect_tx(sh->w_bar + o, 4u * wd_words);
         mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
@@ -200,50 +258,54 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
     __syncthreads();
     slice_cluster_sync();                                // every CTA's barriers exist before anyone writes into it
 
-    if (warp >= kSliceWarps) {
-        // -------------------------------------------------------------------- the copying warps
-        constexpr int kLanes = 32 * kSliceCopyWarps;
-        const int me = tid - kSliceThreads;
-        const int units = (int)(a.row_bytes >> 4);       // 16-byte pieces of a row
-        const int r_step = kLanes / units, p_step = kLanes - r_step * units, r_first = me / units, p_first = me - r_first * units;
+    // steps are counted from the call's first one; a batch is named by its index
+    const int steps = (int)a.num_steps, whole = a.whole;
+    auto batch_at = [&](int k) { return k < steps ? (a.order ? __ldg(a.order + a.first_step + k) : (int)a.first_step + k) : 0; };
+    const int rows_full = min(a.rc, (int)a.batch - bi * a.rc), rows_last = min(a.rc, a.rows_last - bi * a.rc);
+    auto rows_of = [&](int batch) { return max(0, batch < whole ? rows_full : rows_last); };
+    if (warp == kSliceWarps) {
+        // -------------------------------------------------------------------- the copying warp
         int slot = 0;
         uint32_t parity = 1;                             // of the slots' emptiness: all are empty at first
 #pragma unroll 1
-        for (int64_t it = a.first_step; it < step_end; ++it) {
-            const int64_t first = (a.order ? (int64_t)a.order[it] : it) * a.batch, r0 = first + (int64_t)bi * a.rc;
-            const int rows = (int)max((int64_t)0, min((int64_t)a.rc, min(a.m, first + a.batch) - r0));
-            unsigned char* dst = ring + (size_t)slot * slot_bytes;
+        for (int k = 0; k < steps; ++k) {
+            const int batch = batch_at(k);
+            const int64_t r0 = batch * a.batch + (int64_t)bi * a.rc;
+            unsigned char* dst = ring + slot * slot_bytes;
             slice_wait(sh, sh->empty + slot, parity, a.status, 84);
-            const uint8_t* s1 = a.p1 + r0 * a.row_bytes;
-            const uint8_t* s2 = a.p2 + r0 * a.row_bytes;
-            // the pieces of the rows lie one after the other in memory: piece `me`, me + kLanes, ...
-            for (int r = r_first, p = p_first, at = me * 16; r < rows; at += kLanes * 16) {
-                unsigned char* to = dst + r * a.pitch + p * 16;
-                slice_copy16(to, s1 + at);
-                slice_copy16(to + plane_bytes, s2 + at);
-                r += r_step; p += p_step;
-                if (p >= units) { p -= units; ++r; }
+            if (a.use_tmap) {                            // (boxes that reach past the last row are filled up and count in full)
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)(a.rc * a.pitch));
+                    slice_tensor_copy(dst, &tm1, (int)r0, sh->full + slot);
+                    slice_tensor_copy(dst + plane_bytes, &tm2, (int)r0, sh->full + slot);
+                }
+            } else {
+                const int rows = rows_of(batch);
+                if (lane == 0) mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)rows * (uint32_t)a.row_bytes);
+                for (int i = lane; i < 2 * rows; i += 32)
+                    bulk_copy_g2s(dst + (i & 1) * plane_bytes + (i >> 1) * a.pitch, (i & 1 ? a.p2 : a.p1) + (r0 + (i >> 1)) * a.row_bytes, (uint32_t)a.row_bytes,
+                                  sh->full + slot);
             }
-            float* labels = reinterpret_cast<float*>(dst + 2 * plane_bytes + 32);
-            for (int r = me; r < rows; r += kLanes) slice_copy4(labels + r, a.b + r0 + r);
-            slice_arrive_after_copies(sh->full + slot);
-            if (me == 0) { sh->rows[slot] = rows; mbar_arrive(sh->full + slot); }
             if (++slot == a.slots) { slot = 0; parity ^= 1u; }
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
         slice_cluster_sync();
         return;
     }
 
-    // ------------------------------------------------------------------------ the computing warps
+    int batch = batch_at(0), batch_next = batch_at(1);
+    // labels: a lane of the first rb warps forms one residual, of this row of the CTA
+    const int res_row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
+    auto label_of = [&](int batch) { return warp < rb && res_row < rows_of(batch) ? __ldg(a.b + batch * a.batch + (int64_t)bi * a.rc + res_row) : 0.0f; };
+    float label = label_of(batch);
+
+    // ------------------------------------------------------------------------ the steps
     const int gl = lane >> 2, tl = lane & 3, lm = lane >> 3, l8 = lane & 7;
     // dots: units of a part of a slice and RBC row blocks, dealt to the warps
-    const int a_all = owners * a.a_parts, a_units = a_all * ((rb + RBC - 1) / RBC);
-    // gradient: slice and columns of this warp
-    const int b_slice = warp / a.b_warps, bj = warp % a.b_warps;
-    const int col_begin = bj * a.cpw, col_end = b_slice < owners ? min(min(2 * sps, a.cols - b_slice * 2 * sps), col_begin + a.cpw) : 0;
-    // owner: feature of this thread
+    const int a_all = owners * a.a_parts;
+    const int ws_first = warp % a_all, rb_first = warp / a_all * RBC, ws_more = kSliceWarps % a_all, rb_more = kSliceWarps / a_all * RBC;
+    // owner: the pieces of its digits and their destinations, dealt to the threads; feature of this thread
+    const int items = 8 * sps * NG, item_first = tid % items, dest_first = tid / items, item_more = kSliceThreads % items, dest_more = kSliceThreads / items;
     const int P = 1 << a.p_shift, pp = tid & (P - 1), k_own = tid >> a.p_shift;
     const int f_own = bi * SF + k_own;
     const bool mine = owner && k_own < SF && f_own < n;
@@ -251,41 +313,30 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
     const int c0 = 1 << (a.bits - 1);
     const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
     const float mid = fmaf(c0f, st, lof);
+    const float st_low = st / (float)(1 << (CB * (k_own % NG)));    // (codes were multiplied where they lie in their byte)
     float x = mine ? a.x[f_own] : 0.0f;
-    auto draw = [&](int64_t it, uint32_t stream) { return vector_u24(a.seed, a.epoch, (uint32_t)it, (uint32_t)f_own, stream); };
-    auto quantize = [&](float v, float M, int bits, uint32_t u24) {                  // VecQuant::apply with its draw given
-        if (!(M > 0.0f)) return 0.0f;
-        const float sm = (float)((1 << (bits - 1)) - 1);
-        const float t = __fmul_rn(__fdiv_rn(fabsf(v), M), sm);
-        float fl = floorf(t);
-        fl = fl > sm - 1.0f ? sm - 1.0f : fl;
-        const float p = __fsub_rn(t, fl);
-        const float mag = fl + ((__fmul_rn((float)u24, 5.9604644775390625e-08f) < p) ? 1.0f : 0.0f);
-        const float q = __fmul_rn(M, __fdiv_rn(mag, sm));
-        return v < 0.0f ? -q : q;
-    };
+    auto draw = [&](int k, uint32_t stream) { return slice_draw(a.seed, a.epoch, (uint32_t)a.first_step + (uint32_t)k, (uint32_t)f_own, stream); };
 
+    const int marked = bi == 0 && tid == 0 && a.trace ? a.trace_steps : -1;
     int slot = 0;
     uint32_t parity = 0, w_parity = 0, part_parity = 0, gn_parity = 0, xn_parity = 0;
 #pragma unroll 1
-    for (int64_t it = a.first_step - 1; it < step_end; ++it) {
-        const bool last = it == step_end - 1;
-        uint32_t u_x = 0u;
-        if (it >= a.first_step) {
-            slice_mark(a, it, 0);
-            const unsigned char* tile = ring + (size_t)slot * slot_bytes;
-            const uint32_t tile_addr = smem_u32(tile);
+    for (int step = -1; step < steps; ++step) {
+        const bool last = step == steps - 1;
+        uint32_t u_x = 0u, u_g = 0u;
+        const uint32_t tile_addr = smem_u32(ring) + (uint32_t)(slot * slot_bytes);
+        if (step >= 0) {
+            if (step < marked) slice_mark(a.trace, step, 0);
             slice_wait(sh, sh->full + slot, parity, a.status, 6);
-            const int rows = sh->rows[slot];
             // -------------------------------------------------------------- dots
 #pragma unroll 1
-            for (int unit = warp; unit < a_units; unit += kSliceWarps) {
-                const int ws = unit % a_all, rb0 = unit / a_all * RBC, a_slice = ws / a.a_parts;
+            for (int ws = ws_first, rb0 = rb_first; rb0 < rb;) {
+                const int a_slice = (ws * a.a_inv) >> 16;           // ws / a_parts
                 const int slab0 = (ws - a_slice * a.a_parts) * a.spw, slab1 = min(min(sps, a.slabs - a_slice * sps), slab0 + a.spw);
                 const bool keeper = slab0 == 0 && rb0 == 0;         // re-arms the slice's barrier
                 slice_wait(sh, sh->w_bar + a_slice, w_parity, a.status, 4);
                 if (keeper && lane == 0 && !last) mbar_arrive_expect_tx(sh->w_bar + a_slice, 4u * wd_words);
-                slice_mark(a, it, 1);
+                if (step < marked) slice_mark(a.trace, step, 1);
                 const uint32_t* wsl = wd + a_slice * wd_words;
                 const double delta = *reinterpret_cast<const double*>(wsl + wd_words - 4);
                 const double base = slab0 == 0 ? *reinterpret_cast<const double*>(wsl + wd_words - 2) : 0.0;
@@ -316,10 +367,10 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
                                 ldsm_x4(a2, addr + (uint32_t)(i * 16 * a.pitch + plane_bytes));
 #pragma unroll
                                 for (int g = 0; g < NG; ++g) {
-                                    mma_u8s8(c[0][i], group_bytes<CB>(a1[0], g), group_bytes<CB>(a1[1], g), group_bytes<CB>(a1[2], g),
-                                             group_bytes<CB>(a1[3], g), bf[g][0], bf[g][1]);
-                                    mma_u8s8(c[1][i], group_bytes<CB>(a2[0], g), group_bytes<CB>(a2[1], g), group_bytes<CB>(a2[2], g),
-                                             group_bytes<CB>(a2[3], g), bf[g][0], bf[g][1]);
+                                    mma_u8s8(c[0][i], slice_dot_codes<CB>(a1[0], g), slice_dot_codes<CB>(a1[1], g), slice_dot_codes<CB>(a1[2], g),
+                                             slice_dot_codes<CB>(a1[3], g), bf[g][0], bf[g][1]);
+                                    mma_u8s8(c[1][i], slice_dot_codes<CB>(a2[0], g), slice_dot_codes<CB>(a2[1], g), slice_dot_codes<CB>(a2[2], g),
+                                             slice_dot_codes<CB>(a2[3], g), bf[g][0], bf[g][1]);
                                 }
                             }
                         }
@@ -331,71 +382,79 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
                         if (RBC == 1 || rb0 + i < rb) {
 #pragma unroll
                             for (int pl = 0; pl < 2; ++pl) {
-                                const int upper = c[pl][i][0] + 128 * c[pl][i][1], lower = c[pl][i][2] + 128 * c[pl][i][3];
-                                const int got = __shfl_xor_sync(0xffffffffu, tl == 0 ? lower : upper, 1);
-                                const long long v = tl == 0 ? (long long)upper + 16384ll * got : (long long)got + 16384ll * lower;
+                                const long long upper = c[pl][i][0] + 256ll * c[pl][i][1], lower = c[pl][i][2] + 256ll * c[pl][i][3];
+                                const long long got = __shfl_xor_sync(0xffffffffu, tl == 0 ? lower : upper, 1);
+                                const long long v = tl == 0 ? upper + 65536ll * got : got + 65536ll * lower;
                                 const int k = (pl == 0 ? 16 : 0) + 4 * (gl >> 1) + (gl & 1) + 2 * tl;
-                                if (tl < 2) psum[((size_t)ws * rb + rb0 + i) * 32 + k] = (double)v * delta + base;
+                                if (tl < 2) psum[(ws * rb + rb0 + i) * 32 + k] = (double)v * delta + base;
                             }
                         }
                     }
                 }
+                ws += ws_more; rb0 += rb_more;
+                if (ws >= a_all) { ws -= a_all; rb0 += RBC; }
             }
-            uint32_t u_g = 0u;
-            if (a.grad_bits > 0 && mine && pp == 0) u_g = draw(it, 4u);
-            if (a.model_bits > 0 && mine && pp == 0) u_x = draw(it + 1, 3u);
+            if (a.grad_bits > 0 && mine && pp == 0) u_g = draw(step, 4u);
+            if (a.model_bits > 0 && mine && pp == 0) u_x = draw(step + 1, 3u);
             slice_bar();
 
             // -------------------------------------------------------------- residuals and their digits
             if (warp < rb) {
-                const float* labels = reinterpret_cast<const float*>(tile + 2 * plane_bytes + 32);
-                const int row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
-                double d[4] = {row < rows ? -(double)labels[row] : 0.0, 0.0, 0.0, 0.0};
+                double d[4] = {-(double)label, 0.0, 0.0, 0.0};
                 const double* ps = psum + warp * 32 + lane;
+#pragma unroll 1
                 for (int w = 0; w < a_all; w += 4)
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         if (w + i < a_all) d[i] += ps[(w + i) * rb * 32];
-                const float r = row < rows ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
+                const float r = res_row < rows_of(batch) ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
                 float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(r))));
                 if (rb > 1) {                            // one scale for all row blocks
                     if (lane == 0) sh->rmax[warp] = top;
                     asm volatile("bar.sync 2, %0;" ::"r"(32 * rb) : "memory");
+#pragma unroll 1
                     for (int w2 = 0; w2 < rb; ++w2) top = fmaxf(top, sh->rmax[w2]);
-                } else if (lane == 0) {
-                    sh->rmax[0] = top;
                 }
-                const float inv = top > 0.0f ? QMAXF / top : 0.0f;
-                int digit[NS];
-                balanced_digits<NS>(__float2int_rn(r * inv), digit);
+                const int k_r = slice_exponent(top, 0);
+                if (tid == 0) sh->delta_r = top <= 3.402823466e+38f ? slice_pow2(-k_r) : __int_as_float(0x7fffffff);
+                const uint32_t digits = ((uint32_t)__float2int_rn(r * slice_pow2(k_r)) + 0x80808080u) ^ 0x80808080u;
                 unsigned char* out = reinterpret_cast<unsigned char*>(rdig + warp * 32) + ((lane >> 2) & 3) * 32 + (lane >> 4) * 16 + (lane & 3);
 #pragma unroll
-                for (int s = 0; s < NS; ++s) out[4 * s] = (unsigned char)digit[s];
+                for (int s = 0; s < NS; ++s) out[4 * s] = (unsigned char)(digits >> (8 * s));
             }
+            const bool batch_full = batch < whole;
+            batch = batch_next;
+            batch_next = batch_at(step + 2);
+            label = label_of(batch);
             slice_bar();
-            slice_mark(a, it, 2);
+            if (step < marked) slice_mark(a.trace, step, 2);
 
             // -------------------------------------------------------------- the rows' part of the gradient
-            if (col_begin < col_end) {
-                float top = sh->rmax[0];
-                for (int w2 = 1; w2 < rb; ++w2) top = fmaxf(top, sh->rmax[w2]);
-                const float delta_r = __fdiv_rn(top, QMAXF);
-                float* part = gpart + b_slice * part_words;
+#pragma unroll 1
+            for (int unit = warp; unit < owners * a.b_parts; unit += kSliceWarps) {
+                const int b_slice = (unit * a.b_inv) >> 16, bj = unit - b_slice * a.b_parts;     // unit / b_parts
+                const int col_begin = bj * a.cpw, col_end = min(min(2 * sps, a.cols - b_slice * 2 * sps), col_begin + a.cpw);
+                if (col_begin >= col_end) continue;
+                int* part = gpart + b_slice * part_words;
                 const uint32_t row_addr = tile_addr + (uint32_t)((lane >> 4) * plane_bytes + (lane & 15) * a.pitch + b_slice * sps * 32);
                 const uint32_t* rq = rdig + tl * 8 + (gl & 3);
+                int ones[4] = {0, 0, 0, 0};              // the digits' sums
+#pragma unroll 1
+                for (int kb = 0; kb < rb; ++kb)
+                    mma_u8s8(ones, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, gl < NS ? rq[kb * 32] : 0u, gl < NS ? rq[kb * 32 + 4] : 0u);
+                // (sixteen row blocks: 512 products of a centred code and a digit, times 257, could pass 2^31: half of them)
+                const int half = RBC > 1 && rb > 15 ? 1 : 0, upper_weight = 256 >> half;
+                if (bj == 0) {                           // the sum of the residuals
+                    const float delta_r = sh->delta_r, s = (float)(ones[0] + 256 * ones[1]) * delta_r;
+                    const float upper = __shfl_down_sync(0xffffffffu, s, 1);
+                    if (lane == 0) *reinterpret_cast<float2*>(part) = make_float2(fmaf(upper, 65536.0f, s), half ? 2.0f * delta_r : delta_r);
+                }
 #pragma unroll 1
                 for (int col0 = col_begin; col0 < col_end; col0 += CT) {
-                    int acc[CT][NG][4], ones[4] = {0, 0, 0, 0};
-#pragma unroll
-                    for (int ti = 0; ti < CT; ++ti)
-#pragma unroll
-                        for (int g = 0; g < NG; ++g)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[ti][g][e] = 0;
+                    int acc[CT][NG][4];
 #pragma unroll 1
                     for (int kb = 0; kb < rb; ++kb) {
                         const uint32_t b0 = gl < NS ? rq[kb * 32] : 0u, b1 = gl < NS ? rq[kb * 32 + 4] : 0u;
-                        mma_u8s8(ones, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, b0, b1);
 #pragma unroll
                         for (int ti = 0; ti < CT; ++ti) {
                             if (col0 + ti < col_end) {
@@ -404,70 +463,76 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
                                 const uint32_t pel = __byte_perm(r4[0], r4[1], 0x6420), pol = __byte_perm(r4[0], r4[1], 0x7531);
                                 const uint32_t peh = __byte_perm(r4[2], r4[3], 0x6420), poh = __byte_perm(r4[2], r4[3], 0x7531);
 #pragma unroll
-                                for (int g = 0; g < NG; ++g)
-                                    mma_u8s8(acc[ti][g], group_bytes<CB>(pel, g), group_bytes<CB>(pol, g), group_bytes<CB>(peh, g),
-                                             group_bytes<CB>(poh, g), b0, b1);
+                                for (int g = 0; g < NG; ++g) {
+                                    // sums of (code - c0) * residual, codes where they lie: c0 times the digits' sums come off first
+                                    const int from = -(c0 << (CB * g));
+                                    if (RBC == 1 || kb == 0)
+                                        slice_mma_from(acc[ti][g], slice_codes<CB>(pel, g), slice_codes<CB>(pol, g), slice_codes<CB>(peh, g),
+                                                       slice_codes<CB>(poh, g), b0, b1, from * ones[0], from * ones[1]);
+                                    else
+                                        mma_u8s8(acc[ti][g], slice_codes<CB>(pel, g), slice_codes<CB>(pol, g), slice_codes<CB>(peh, g),
+                                                 slice_codes<CB>(poh, g), b0, b1);
+                                }
                             }
                         }
                     }
-                    // sums of (code - c0) * residual; rows g, g + 8 of the accumulators are bytes 2g, 2g + 1 of the column
-                    const float weight = tl == 0 ? delta_r : 16384.0f * delta_r;
+                    // rows g, g + 8 of the accumulators are bytes 2g, 2g + 1 of the column
 #pragma unroll
                     for (int ti = 0; ti < CT; ++ti) {
                         if (col0 + ti < col_end) {
 #pragma unroll
                             for (int g = 0; g < NG; ++g) {
-                                const int upper = (acc[ti][g][0] - c0 * ones[0]) + 128 * (acc[ti][g][1] - c0 * ones[1]);
-                                const int lower = (acc[ti][g][2] - c0 * ones[0]) + 128 * (acc[ti][g][3] - c0 * ones[1]);
-                                const float up = (float)upper * weight, low = (float)lower * weight;
-                                const float got = __shfl_xor_sync(0xffffffffu, tl == 0 ? low : up, 1);
-                                if (tl < 2) part[4 + ((col0 + ti) * 16 + 2 * gl + tl) * NG + g] = (tl == 0 ? up : low) + got;
+                                int* out = part + 4 + 2 * (((col0 + ti) * 16 + 2 * gl) * NG + g) + tl;
+                                if (tl < 2) {            // lane t = 0 has the lower digits, t = 1 the upper ones
+                                    out[0] = (acc[ti][g][0] >> half) + upper_weight * acc[ti][g][1];
+                                    out[2 * NG] = (acc[ti][g][2] >> half) + upper_weight * acc[ti][g][3];
+                                }
                             }
                         }
-                    }
-                    if (bj == 0 && col0 == 0) {          // the sum of the residuals
-                        const float s = (float)(ones[0] + 128 * ones[1]) * weight;
-                        const float all = s + __shfl_xor_sync(0xffffffffu, s, 1);
-                        if (lane == 0) part[0] = all;
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
-                    const int w0 = bj == 0 ? 0 : 4 + col_begin * 16 * NG, w1 = 4 + col_end * 16 * NG;
+                    const int w0 = bj == 0 ? 0 : 4 + col_begin * 32 * NG, w1 = 4 + col_end * 32 * NG;
                     slice_copy(slice_peer(gbuf + bi * part_words + w0, b_slice), part + w0, 4u * (w1 - w0), slice_peer(&sh->part_bar, b_slice));
                 }
             }
             if (lane == 0) mbar_arrive(sh->empty + slot);
             if (++slot == a.slots) { slot = 0; parity ^= 1u; }
             w_parity ^= 1u;
-            slice_mark(a, it, 3);
+            if (step < marked) slice_mark(a.trace, step, 3);
 
             // -------------------------------------------------------------- the owner sums the parts and updates
             if (owner) {
                 slice_wait(sh, &sh->part_bar, part_parity, a.status, 2);
                 part_parity ^= 1u;
                 if (tid == 0 && !last) mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
-                const int64_t t_now = a.order ? (int64_t)a.order[it] : it;
-                const double scale = 1.0 / (2.0 * (double)min(a.batch, a.m - t_now * a.batch));
                 double t = 0.0;
                 if (mine)
-                    for (int w = pp; w < a.nb; w += P) t += (double)fmaf(st, gbuf[w * part_words + 4 + k_own], mid * gbuf[w * part_words]);
+#pragma unroll 2
+                    for (int w = pp; w < a.nb; w += P) {
+                        const int2 v = *reinterpret_cast<const int2*>(gbuf + w * part_words + 4 + 2 * k_own);
+                        const float2 h = *reinterpret_cast<const float2*>(gbuf + w * part_words);
+                        t += (double)fmaf(st_low, fmaf((float)v.y, 65536.0f, (float)v.x) * h.y, mid * h.x);
+                    }
+#pragma unroll 1
                 for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                float g = (float)(t * scale);
+                float g = (float)(t * (batch_full ? a.full_scale : a.last_scale));
                 const bool writes = mine && pp == 0;
                 if (last && a.grad_out && writes) a.grad_out[f_own] = g;
-                slice_mark(a, it, 4);
+                if (step < marked) slice_mark(a.trace, step, 4);
                 if (a.grad_bits > 0) {
-                    const float M = slice_norm(writes ? (double)g * (double)g : 0.0, sh->red[0], sh->nrm_g, &sh->gn_bar, gn_parity, owners, sh, a.status, 3);
+                    const float M = slice_norm(writes ? (double)g * (double)g : 0.0, P, sh->red[0], sh->nrm_g, &sh->gn_bar, gn_parity, owners, sh, a.status, 3);
                     gn_parity ^= 1u;
-                    g = quantize(g, M, a.grad_bits, u_g);
+                    g = slice_quantize(g, M, a.grad_bits, u_g);
                 }
                 if (last && a.grad_out && writes) a.grad_out[n + f_own] = g;
-                x = regularise(fmaf(-a.lr, g, x), x, a.reg, a.reg_cst);
+                const float y = fmaf(-a.lr, g, x);
+                x = a.reg == ZIPML_REG_NONE ? y : slice_regularise(y, x, a.reg, a.reg_cst);
             }
         } else if (a.model_bits > 0 && mine && pp == 0) {
-            u_x = draw(it + 1, 3u);
+            u_x = draw(step + 1, 3u);
         }
         if (last) break;
 
@@ -475,44 +540,46 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
         if (owner) {
             float xt = x;
             if (a.model_bits > 0) {
-                const float M = slice_norm(mine && pp == 0 ? (double)x * (double)x : 0.0, sh->red[1], sh->nrm_x, &sh->xn_bar, xn_parity, owners, sh, a.status, 8);
+                const float M = slice_norm(mine && pp == 0 ? (double)x * (double)x : 0.0, P, sh->red[1], sh->nrm_x, &sh->xn_bar, xn_parity, owners, sh, a.status, 8);
                 xn_parity ^= 1u;
-                xt = quantize(x, M, a.model_bits, u_x);
+                xt = slice_quantize(x, M, a.model_bits, u_x);
             }
             const bool writes = mine && pp == 0;
-            if (a.model_out && it + 2 == step_end && writes) a.model_out[f_own] = xt;
+            if (a.model_out && step + 2 == steps && writes) a.model_out[f_own] = xt;
             const float w = writes ? st * xt : 0.0f;
             if (pp == 0 && k_own < SF) wv[k_own] = w;
             const float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w))));
             double bpart = writes ? (double)lof * (double)xt : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                if (o >= P) bpart += __shfl_xor_sync(0xffffffffu, bpart, o);
+#pragma unroll 1
+            for (int o = 16; o >= P; o >>= 1) bpart += __shfl_xor_sync(0xffffffffu, bpart, o);
             if (lane == 0) { sh->wmax[warp] = top; sh->base[warp] = bpart; }
             slice_bar();
-            float wmax = 0.0f;
-#pragma unroll
-            for (int i = 0; i < kSliceWarps; ++i) wmax = fmaxf(wmax, sh->wmax[i]);
-            const float inv = wmax > 0.0f ? QMAXF / wmax : 0.0f;
-            const int items = 8 * sps * NG;
-            for (int idx = tid; idx < items * a.nb; idx += kSliceThreads) {
-                const int dest = idx / items, item = idx - dest * items;
+            const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sh->wmax[lane])));
+            const int k_w = slice_exponent(wmax, SliceShift<CB>::kMost);
+            const float inv = slice_pow2(k_w);
+#pragma unroll 1
+            for (int item = item_first, dest = dest_first; dest < a.nb;) {
                 const int half = item & 1, t = (item >> 1) & 3, gs = item >> 3, g = gs % NG, q = (gs / NG) * 8 + half * 4 + t;
                 const float* src = wv + q * 4 * NG + g;
-                const float v4[4] = {src[0], src[NG], src[2 * NG], src[3 * NG]};
-                slice_store16(slice_peer(wd + bi * wd_words + 4 * item, dest), digit_words<NS>(v4, inv), slice_peer(sh->w_bar + bi, dest));
+                const float up = inv * (float)(1 << SliceShift<CB>::of(g));
+                uint32_t d[4];
+                transpose4x4((uint32_t)__float2int_rn(src[0] * up) + 0x80808080u, (uint32_t)__float2int_rn(src[NG] * up) + 0x80808080u,
+                             (uint32_t)__float2int_rn(src[2 * NG] * up) + 0x80808080u, (uint32_t)__float2int_rn(src[3 * NG] * up) + 0x80808080u, d);
+                slice_store16(slice_peer(wd + bi * wd_words + 4 * item, dest),
+                              make_uint4(d[0] ^ 0x80808080u, d[1] ^ 0x80808080u, d[2] ^ 0x80808080u, d[3] ^ 0x80808080u), slice_peer(sh->w_bar + bi, dest));
+                item += item_more; dest += dest_more;
+                if (item >= items) { item -= items; ++dest; }
             }
             if (tid >= kSliceThreads - a.nb) {           // the scale and lo^T x~
                 const int dest = tid - (kSliceThreads - a.nb);
-                double base = 0.0;
-#pragma unroll
-                for (int i = 0; i < kSliceWarps; ++i) base += sh->base[i];
-                const unsigned long long s = (unsigned long long)__double_as_longlong((double)wmax / (double)QMAXF), l = (unsigned long long)__double_as_longlong(base);
+                const unsigned long long s = wmax <= 3.402823466e+38f ? (unsigned long long)(1023 - k_w - SliceShift<CB>::kMost) << 52   // 2^-(k_w + kMost)
+                                                                      : 0x7fffffffffffffffull;
+                const unsigned long long l = (unsigned long long)__double_as_longlong(slice_sum16(sh->base));
                 slice_store16(slice_peer(wd + bi * wd_words + wd_words - 4, dest), make_uint4((uint32_t)s, (uint32_t)(s >> 32), (uint32_t)l, (uint32_t)(l >> 32)),
                               slice_peer(sh->w_bar + bi, dest));
             }
         }
-        slice_mark(a, it, 5);
+        if (step >= 0 && step < marked) slice_mark(a.trace, step, 5);
     }
     if (mine && pp == 0) a.x[f_own] = x;
     __syncwarp();
@@ -523,22 +590,22 @@ __global__ void __launch_bounds__(kSliceThreads + 32 * kSliceCopyWarps, 1) sgd_s
 // Host side
 // ---------------------------------------------------------------------------------------------
 struct SlicePlan {
-    int nb, rc, rb, owners, sps, slabs, cols, a_parts, spw, b_warps, cpw, p_shift, pitch, slots;
+    int nb, rc, rb, owners, sps, slabs, cols, a_parts, spw, b_parts, cpw, p_shift, pitch, slots;
     size_t smem;
 };
 
 static size_t slice_smem_bytes(const SlicePlan& r, int ng, int slots) {
     const size_t sf = (size_t)32 * r.sps * ng;
     size_t bytes = sizeof(SliceShared) + 4 * (size_t)r.owners * ((size_t)r.sps * ng * 32 + 4) + 8 * (size_t)r.owners * r.a_parts * r.rb * 32 +
-                   4 * (size_t)r.rb * 32 + 4 * (size_t)(r.owners + r.nb) * (sf + 4) + 4 * sf + 128;
-    return bytes + (size_t)slots * (((size_t)2 * 16 * r.rb * r.pitch + 32 + 4 * r.rc + 15) & ~(size_t)15);
+                   4 * (size_t)r.rb * 32 + 4 * (size_t)(r.owners + r.nb) * (2 * sf + 4) + 4 * sf + 128;
+    return bytes + (size_t)slots * (2 * (((size_t)16 * r.rb * r.pitch + 127) & ~(size_t)127) + 128);
 }
 
 static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, SlicePlan* plan) {
     const int cb = container_bits(d->bits), ng = 8 / cb;
     const int64_t B = p->batch < d->m ? p->batch : d->m;
     const int64_t used = (d->n * cb + 7) / 8, slabs = (used + 31) / 32;
-    if (d->level_mode != ZIPML_LEVELS_UNIFORM || slabs > 1024 || d->row_bytes > (1 << 16)) return ZIPML_ERR_WORKSPACE;
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || (d->m + B - 1) / B > 0x7ffffff0 || slabs > 1024 || d->row_bytes > (1 << 16)) return ZIPML_ERR_WORKSPACE;
     int64_t nb = p->grid_row_parts > 0 ? p->grid_row_parts : (B + 15) / 16;     // automatic: 16 rows per CTA
     if (nb > kSliceMaxCtas) nb = kSliceMaxCtas;
     if (nb > B) nb = B;
@@ -551,11 +618,11 @@ static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const z
         r.owners = (int)((slabs + r.sps - 1) / r.sps);
         r.slabs = (int)slabs; r.cols = (int)((used + 15) / 16);
         if (r.rb > kSliceWarps || 32 * r.sps * ng > kSliceThreads) continue;
-        const int per = kSliceWarps / r.owners;
+        const int per = r.owners < kSliceWarps ? kSliceWarps / r.owners : 1;
         r.spw = (r.sps + per - 1) / per;
         r.a_parts = (r.sps + r.spw - 1) / r.spw;
         r.cpw = (2 * r.sps + per - 1) / per;
-        r.b_warps = per;
+        r.b_parts = (2 * r.sps + r.cpw - 1) / r.cpw;
         r.p_shift = 0;
         while (r.p_shift < 4 && (32 * r.sps * ng) << (r.p_shift + 1) <= kSliceThreads && (1 << r.p_shift) < r.nb) ++r.p_shift;
         const int units = (int)(d->row_bytes / 16);
@@ -577,16 +644,16 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     if (rc != ZIPML_OK) return rc;
     const int cb = container_bits(d->bits);
     const bool one = plan.rb == 1;
-    const void* kernel = cb == 2 ? (one ? (const void*)sgd_slice_kernel<2, 1> : (const void*)sgd_slice_kernel<2, 4>)
-                       : cb == 4 ? (one ? (const void*)sgd_slice_kernel<4, 1> : (const void*)sgd_slice_kernel<4, 4>)
-                                 : (one ? (const void*)sgd_slice_kernel<8, 1> : (const void*)sgd_slice_kernel<8, 4>);
+    const void* kernel = cb == 2 ? (one ? (const void*)sgd_slice_kernel<2, 1> : (const void*)sgd_slice_kernel<2, 2>)
+                       : cb == 4 ? (one ? (const void*)sgd_slice_kernel<4, 1> : (const void*)sgd_slice_kernel<4, 2>)
+                                 : (one ? (const void*)sgd_slice_kernel<8, 1> : (const void*)sgd_slice_kernel<8, 2>);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
     if (e == cudaSuccess && plan.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return cuda_status(e);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)plan.nb);
-    cfg.blockDim = dim3(kSliceThreads + 32 * kSliceCopyWarps);
+    cfg.blockDim = dim3(kSliceThreads + 32);
     cfg.dynamicSmemBytes = plan.smem;
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
@@ -617,12 +684,17 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     a.status = ctx->d_status;
     a.m = d->m; a.batch = p->batch < d->m ? p->batch : d->m; a.row_bytes = d->row_bytes;
     a.first_step = first_step; a.num_steps = num_steps;
+    a.whole = (int)(d->m / a.batch); a.rows_last = (int)(d->m - a.whole * a.batch);
+    a.full_scale = 1.0 / (2.0 * (double)a.batch); a.last_scale = 1.0 / (2.0 * (double)(a.rows_last > 0 ? a.rows_last : 1));
     a.seed = p->seed; a.epoch = (uint32_t)p->epoch; a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
     a.n = (int)d->n; a.bits = d->bits; a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
     a.nb = plan.nb; a.rc = plan.rc; a.rb = plan.rb; a.owners = plan.owners; a.sps = plan.sps; a.slabs = plan.slabs; a.cols = plan.cols;
-    a.a_parts = plan.a_parts; a.spw = plan.spw; a.b_warps = plan.b_warps; a.cpw = plan.cpw;
+    a.a_parts = plan.a_parts; a.a_inv = 65536 / plan.a_parts + 1; a.spw = plan.spw; a.b_parts = plan.b_parts; a.b_inv = 65536 / plan.b_parts + 1; a.cpw = plan.cpw;
+    CUtensorMap tmaps[2];
+    memset(tmaps, 0, sizeof(tmaps));
+    a.use_tmap = d->m < (1ll << 31) - 4096 && encode_plane_maps(ctx, d, plan.pitch / 4, plan.rc, true, tmaps) == ZIPML_OK;
     a.p_shift = plan.p_shift; a.pitch = plan.pitch; a.slots = plan.slots;
-    void* params[] = {&a};
+    void* params[] = {&a, &tmaps[0], &tmaps[1]};
     e = cudaLaunchKernelExC(&cfg, kernel, params);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
