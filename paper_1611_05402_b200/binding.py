@@ -174,6 +174,32 @@ class SharedBase:
         return self.m * (self.row_bytes + 2 * self.up_row_bytes) + 4 * self.m
 
 
+class PreparedEpoch:
+    """zipml_sgd_epoch with its arguments marshalled once, for callers that take many short ranges of steps; calling it
+    runs from `first_step` on.  batch_order, if given, is the host array that the calls read (writable in place)."""
+
+    def __init__(self, ctx, data, b, x, params, keep, grad_out):
+        self.ctx, self.params, self.batch_order, self._tensors = ctx, params, keep, (data, b, x, grad_out)
+        self._call, self._data = lib().zipml_sgd_epoch, data.c_struct()
+        self._args = (ctx._h, C.byref(self._data), _ptr(b, torch.float32, ctx.device), _ptr(x, torch.float32, ctx.device), C.byref(params),
+                      _ptr(grad_out, torch.float32, ctx.device))
+
+    def __call__(self, first_step):
+        self.params.first_step = first_step
+        _check(self._call(*self._args), "zipml_sgd_epoch")
+
+
+class PreparedApply:
+    """zipml_sgd_apply_gradient on a fixed x, marshalled once; calling it applies a gradient at a step."""
+
+    def __init__(self, ctx, x, params):
+        self.ctx, self.params, self.x = ctx, params, x
+        self._call, self._x, self._p, self._n = lib().zipml_sgd_apply_gradient, _ptr(x, torch.float32, ctx.device), C.byref(params), x.numel()
+
+    def __call__(self, g, step):
+        _check(self._call(self.ctx._h, self._x, _ptr(g, torch.float32, self.ctx.device), self._n, self._p, step, None), "zipml_sgd_apply_gradient")
+
+
 class Context:
     """zipml_create / zipml_destroy bound to torch's current stream of `device`."""
 
@@ -369,6 +395,13 @@ class Context:
                                      _ptr(x, torch.float32, self.device), C.byref(p),
                                      _ptr(grad_out, torch.float32, self.device)), "zipml_sgd_epoch")
         del keep
+
+    def prepare_sgd_epoch(self, data, b, x, batch, lr, grad_out=None, **kw):
+        p, keep = self.sgd_params(batch, lr, **kw)
+        return PreparedEpoch(self, data, b, x, p, keep, grad_out)
+
+    def prepare_sgd_apply_gradient(self, x, lr, **kw):
+        return PreparedApply(self, x, self.sgd_params(1, lr, **kw)[0])
 
     def zipml_loss(self, mode, b, x, A=None, data=None, out=None):
         out = torch.empty(1, dtype=torch.float64, device=self.device) if out is None else out

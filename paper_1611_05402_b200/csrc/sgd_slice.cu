@@ -237,24 +237,30 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     const bool owner = bi < owners;
     const uint32_t part_bytes = 4u * a.nb * (4 + (owner ? min(2 * sps, a.cols - bi * 2 * sps) : 0) * 32 * NG);
 
-    if (tid == 0) {
-        for (int s = 0; s < a.slots; ++s) {
-            mbar_init(sh->full + s, 1);
-            mbar_init(sh->empty + s, kSliceWarps);
-        }
-        for (int o = 0; o < owners; ++o) { mbar_init(sh->w_bar + o, 1); }
+    if (tid < a.slots) {
+        mbar_init(sh->full + tid, 1);
+        mbar_init(sh->empty + tid, kSliceWarps);
+    } else if (tid >= 32 && tid < 32 + owners) {
+        mbar_init(sh->w_bar + tid - 32, 1);
+        mbar_arrive_expect_tx(sh->w_bar + tid - 32, 4u * wd_words);
+    } else if (tid == 64) {
         mbar_init(&sh->part_bar, 1);
-        mbar_init(&sh->gn_bar, 1);
-        mbar_init(&sh->xn_bar, 1);
-        sh->gave_up = 0;
-        for (int c = 0; c < 16; ++c) sh->nrm_g[c] = sh->nrm_x[c] = sh->base[c] = sh->red[0][c] = sh->red[1][c] = 0.0;
-        for (int c = 0; c < 32; ++c) sh->wmax[c] = 0.0f;
-        mbar_fence_init();
-        for (int o = 0; o < owners; ++o) mbar_arrive_expect_tx(sh->w_bar + o, 4u * wd_words);
         mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
+    } else if (tid == 65) {
+        mbar_init(&sh->gn_bar, 1);
         mbar_arrive_expect_tx(&sh->gn_bar, 8u * owners);
+    } else if (tid == 66) {
+        mbar_init(&sh->xn_bar, 1);
         mbar_arrive_expect_tx(&sh->xn_bar, 8u * owners);
+    } else if (tid == 67) {
+        sh->gave_up = 0;
+    } else if (tid >= 96 && tid < 128) {
+        sh->wmax[tid - 96] = 0.0f;
+    } else if (tid >= 128 && tid < 144) {
+        const int c = tid - 128;
+        sh->nrm_g[c] = sh->nrm_x[c] = sh->base[c] = sh->red[0][c] = sh->red[1][c] = 0.0;
     }
+    mbar_fence_init();
     __syncthreads();
     slice_cluster_sync();                                // every CTA's barriers exist before anyone writes into it
 

@@ -111,6 +111,7 @@ class ShardedEpoch:
         self.ctx, self.plan, self.data, self.b, self.x, self.lr = ctx, plan, data_local, b_local, x, lr
         self.model_bits, self.grad_bits, self.seed, self.epoch = model_bits, grad_bits, seed, epoch
         self.reg, self.reg_param, self.engine = reg, reg_param, engine
+        self._running = None                                       # the prepared calls, while run() is at work
         self.n = x.numel()
         self.g2 = torch.empty(2 * self.n, dtype=torch.float32, device=x.device)
         self.order = None if batch_order is None else [int(o) for o in batch_order]
@@ -118,29 +119,36 @@ class ShardedEpoch:
         # positions whose batch this rank does not hold are never executed; their entries only have to be valid
         self.order_local = None if self.order is None or not T_local else [min(o, T_local - 1) for o in self.order][:T_local]
 
+    # The step's two library calls, with everything marshalled that stays the same from step to step.
+    def _share_call(self):
+        return self.ctx.prepare_sgd_epoch(self.data, self.b, self.x, self.plan.local_batch, 0.0, model_bits=self.model_bits,   # lr = 0: x stays
+                                          num_steps=1, engine=self.engine, batch_order=self.order_local, grad_out=self.g2, seed=self.seed,
+                                          epoch=self.epoch)
+
+    def _apply_call(self):
+        return self.ctx.prepare_sgd_apply_gradient(self.x, self.lr, grad_bits=self.grad_bits, reg=self.reg, reg_param=self.reg_param,
+                                                   seed=self.seed, epoch=self.epoch)
+
     def share(self, pos, t, weight):
         """weight * the mean over the rank's rows of batch t of the symmetrised gradient, at the model (or its Q3
-        image for position pos) as it stands; zeros if the rank holds none of the batch."""
+        image for position pos) as it stands; zeros if the rank holds none of the batch.  (Good until the next call.)"""
         import torch
         if self.plan.count(t) == 0:
             return torch.zeros(self.n, dtype=torch.float32, device=self.x.device)
-        kw = dict(model_bits=self.model_bits, grad_bits=0, seed=self.seed, epoch=self.epoch, num_steps=1, engine=self.engine,
-                  first_step=pos, grad_out=self.g2)
+        call = self._running[0] if self._running else self._share_call()
         if self.order_local is not None:
             # the library keys Q3 by the position: the step runs at position pos of a local order that names t there
             if pos >= len(self.order_local):
                 raise ValueError("under a batch order a rank that holds fewer batches than the epoch has steps cannot "
                                  "take a position beyond its own count")
-            lo = list(self.order_local)
-            lo[pos] = t
-            kw["batch_order"] = lo
-        self.ctx.zipml_sgd_epoch(self.data, self.b, self.x, self.plan.local_batch, 0.0, **kw)   # lr = 0: x stays
-        return self.g2[:self.n] * weight
+            call.batch_order[pos] = t
+        call(pos)
+        g = self.g2[:self.n]
+        return g if weight == 1.0 else g * weight
 
     def apply(self, v, pos):
         """Q4 and the update on this rank's replica."""
-        self.ctx.zipml_sgd_apply_gradient(self.x, v.contiguous(), pos, self.lr, grad_bits=self.grad_bits, seed=self.seed,
-                                          epoch=self.epoch, reg=self.reg, reg_param=self.reg_param)
+        (self._running[1] if self._running else self._apply_call())(v.contiguous(), pos)
 
     def run(self, group=None, first_step=0, num_steps=None, all_reduce=None):
         """The epoch (or a range of its steps).  The ranks meet in one all-reduce of n floats per step
@@ -153,4 +161,8 @@ class ShardedEpoch:
             elif dist.is_available() and dist.is_initialized() and self.plan.world > 1:
                 dist.all_reduce(v, op=dist.ReduceOp.SUM, group=group)
 
-        run_steps(self.plan, self.share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
+        self._running = (self._share_call(), self._apply_call())
+        try:
+            run_steps(self.plan, self.share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
+        finally:
+            self._running = None
