@@ -75,7 +75,9 @@ enum {
     ZIPML_ENGINE_LEAN = 4,       /* one cooperative launch for small minibatch tiles: row parts only,
                                     two barriers and two packet exchanges per step                    */
     ZIPML_ENGINE_CLUSTER = 5,    /* one thread-block cluster (at most 16 row parts) for small tiles:
-                                    gradients and model travel between the CTAs' shared memories.
+                                    gradients and model travel between the CTAs' shared memories.  On
+                                    uniform grids with rows of up to some 3 KB several clusters, which
+                                    meet through L2, and minibatches of any size, in chunks.
                                     Uniform grids contract in fp32 or, on taller tiles, on the int8
                                     tensor cores; zipml_sgd_params.cluster_contraction overrides that
                                     choice                                                            */
@@ -156,7 +158,8 @@ typedef struct zipml_sgd_params {
     uint64_t seed;              /* keys the Q3/Q4 random draws                                       */
     const int32_t* batch_order; /* HOST pointer or NULL: T = ceil(m/B) batch indices; NULL = 0..T-1  */
     float lr;                   /* step length gamma, constant within the call                       */
-    int32_t grid_feature_parts; /* tuning, 0 = automatic: CTAs along the features                    */
+    int32_t grid_feature_parts; /* tuning, 0 = automatic: CTAs along the features (cluster engine on uniform
+                                   grids: an upper limit on its clusters)                            */
     int32_t grid_row_parts;     /* tuning, 0 = automatic: CTAs along the rows of a minibatch (stream
                                    engine: an upper limit on its CTAs, ignored where too few)        */
     int32_t trace_steps;        /* profiling: number of steps to trace (0 = none)                    */

@@ -28,6 +28,8 @@ static int grow(unsigned char** buf, size_t* have, size_t want, cudaStream_t str
 int ws_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->ws, &ctx->ws_bytes, bytes, ctx->stream); }
 int stage_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->stage, &ctx->stage_bytes, bytes, ctx->stream); }
 
+int exchange_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->exchange, &ctx->exchange_bytes, bytes, ctx->stream); }
+
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 struct DeviceGuard {
@@ -148,6 +150,7 @@ int zipml_destroy(zipml_ctx* ctx) {
     (void)cudaStreamSynchronize(ctx->stream);
     if (ctx->ws) (void)cudaFree(ctx->ws);
     if (ctx->stage) (void)cudaFree(ctx->stage);
+    if (ctx->exchange) (void)cudaFree(ctx->exchange);
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     (void)cudaGetLastError();
     delete ctx;
@@ -295,7 +298,14 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        // (also for small steps on rows too wide for the two above)
+        // Rows of up to some 3 KB: clusters that hold whole rows, however large the batch (8-bit codes, whose tensor work per
+        // byte is least, up to where the ring engine's 148 CTAs stream faster: 8,192 x 2,000 19.0 / 26.9 us per step,
+        // 16,384 x 2,000 36.9 / 35.2; at 4 bits 16,384 x 3,000 42.7 / 48.2).
+        if (step_bytes > (2ll << 20) && (container_bits(data->bits) < 8 || step_bytes <= (48ll << 20))) {
+            rc = launch_sgd_slice(ctx, data, b, x, params, first, count, grad_out);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
+        // (also for small steps on rows too wide for those above)
         rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, true);
         if (rc != ZIPML_ERR_WORKSPACE) return rc;
         rc = launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out, true);

@@ -24,6 +24,10 @@ struct zipml_ctx {
     // staging buffers of zipml_train_host (grown on demand)
     unsigned char* stage = nullptr;
     size_t stage_bytes = 0;
+    // words between the clusters of the cluster engine's int8 form, and the next tag (see sgd_slice.cu)
+    unsigned char* exchange = nullptr;
+    size_t exchange_bytes = 0;
+    uint32_t exchange_tag = 1;
     int64_t launches = 0;           // kernels launched so far (diagnostics)
     int last_engine = 0;            // engine of the latest zipml_sgd_epoch call (diagnostics)
     void* tmap_encode = nullptr;    // cuTensorMapEncodeTiled, resolved on first use
@@ -38,6 +42,7 @@ int check_dataset(const zipml_dataset* d);
 int cuda_status(cudaError_t e);                       // ZIPML_OK or ZIPML_ERR_CUDA (clears the sticky error)
 int ws_reserve(zipml_ctx* ctx, size_t bytes);         // grow ctx->ws to at least `bytes`
 int stage_reserve(zipml_ctx* ctx, size_t bytes);
+int exchange_reserve(zipml_ctx* ctx, size_t bytes);
 
 // The fp32 constant of zipml_sgd_params' regulariser for step length lr (see regularise() in common.cuh).
 inline float reg_constant(const zipml_sgd_params* p) {

@@ -21,6 +21,10 @@
 // sums (gradient).
 // The code tiles come a few steps ahead, one tensor copy per plane whose box is as wide as the distance of the rows in
 // shared memory, an odd number of 16-byte units (rows above 2 KB: a bulk copy each).
+// Larger minibatches take several clusters and several chunks of rows per CTA.  A CTA holds whole rows, so a chunk's dots,
+// residuals and gradient need nothing from the others: the codes are read once, and the gradient's parts add up in
+// shared memory until the last chunk.  The clusters hold replicas of the model: the owners of the same slice hand each
+// other their sums through L2 (self-validating 8-byte words, two buffers in turn) and add them in the same order.
 // Buffer reuse: a CTA sends its part of step t after its warps have read the digits of step t (first barrier), and an
 // owner publishes after all parts have arrived: digits, parts and their sources are free when they are written again.
 // The step's machine code has to stay small: what does not fit the instruction cache is fetched again every step (with
@@ -40,6 +44,7 @@ constexpr int kSliceWarps = 16;
 constexpr int kSliceThreads = 32 * kSliceWarps;   // without the copying warp
 constexpr int kSliceMaxSlots = 8;
 constexpr int kSliceMaxCtas = 16;
+constexpr int kSliceMaxClusters = 8;
 
 struct SliceArgs {
     const uint8_t* p1;
@@ -63,7 +68,10 @@ struct SliceArgs {
     int model_bits, grad_bits;
     int whole, rows_last;        // batches below `whole` are full, that one has rows_last rows
     double full_scale, last_scale;   // 1 / (2 rows)
-    int nb, rc, rb;              // CTAs, rows per CTA, blocks of 16 rows
+    int clusters, chunks;        // clusters; chunks of rows per CTA and step
+    int nb, rc, cr, rb;          // CTAs per cluster, rows per CTA, rows per chunk, blocks of 16 rows in a chunk
+    unsigned long long* exchange;    // [2][clusters][owners SF][2] words {fp32, tag} between the clusters
+    uint32_t tag;                // of the first step; greater than any that the buffer holds
     int owners, sps;             // CTAs that own a slice, 32-byte slabs per slice
     int slabs, cols;             // 32-byte slabs and 16-byte columns that hold features
     int a_parts, a_inv, spw;     // dots: parts of a slice, slabs per part (a warp takes a part and RBC row blocks at a time)
@@ -163,6 +171,24 @@ __device__ __forceinline__ void slice_wait(SliceShared* sh, uint64_t* bar, uint3
     if (!mbar_try_wait(bar, parity)) slice_wait_long(sh, bar, parity, status, where);
 }
 
+// A double, as the sum of two floats, handed over through L2: each 8-byte word carries the step's tag and is valid by itself.
+__device__ __forceinline__ void slice_post(unsigned long long* box, float hi, float low, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(box), "l"(t | __float_as_uint(hi)), "l"(t | __float_as_uint(low)) : "memory");
+}
+__device__ __noinline__ double slice_collect(SliceShared* sh, const unsigned long long* box, uint32_t tag, DeviceStatus* status) {
+    unsigned long long u, v;
+#pragma unroll 1
+    for (long long spin = 0; spin < kBarrierSpinLimit; ++spin) {
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(u), "=l"(v) : "l"(box) : "memory");
+        if ((uint32_t)(u >> 32) == tag && (uint32_t)(v >> 32) == tag) return (double)__uint_as_float((uint32_t)u) + (double)__uint_as_float((uint32_t)v);
+        if ((spin & 255) == 255 && *reinterpret_cast<volatile int*>(&sh->gave_up)) return 0.0;
+    }
+    sh->gave_up = 1;
+    set_status(status, ZIPML_ERR_TIMEOUT, 85);
+    return 0.0;
+}
+
 __device__ __noinline__ float slice_regularise(float y, float x_old, int reg, float cst) { return regularise(y, x_old, reg, cst); }
 __device__ __noinline__ uint32_t slice_draw(uint64_t seed, uint32_t epoch, uint32_t step, uint32_t coord, uint32_t stream) {
     return vector_u24(seed, epoch, step, coord, stream);
@@ -182,14 +208,14 @@ __device__ __noinline__ float slice_quantize(float v, float M, int bits, uint32_
 
 // l2 norm of a vector spread over the owners (v: this thread's share of the squares, in every `every`-th lane): per-CTA sums, one store to
 // every owner, added in CTA order.
-__device__ __noinline__ float slice_norm(double v, int every, double* red, double* table, uint64_t* bar, uint32_t parity, int owners, SliceShared* sh,
+__device__ __noinline__ float slice_norm(double v, int every, int rank, double* red, double* table, uint64_t* bar, uint32_t parity, int owners, SliceShared* sh,
                                          DeviceStatus* status, int where) {
 #pragma unroll 1
     for (int o = 16; o >= every; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     slice_bar();
     if ((int)threadIdx.x < owners) {
-        slice_store8(slice_peer(table + blockIdx.x, threadIdx.x), slice_sum16(red), slice_peer(bar, threadIdx.x));
+        slice_store8(slice_peer(table + rank, threadIdx.x), slice_sum16(red), slice_peer(bar, threadIdx.x));
     }
     slice_wait(sh, bar, parity, status, where);
     if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, 8u * (uint32_t)owners);     // the next one's
@@ -215,14 +241,14 @@ __device__ __forceinline__ void slice_tensor_copy(void* dst_smem, const CUtensor
 //   gbuf[nb][4 + 2 SF]       the parts of the own slice
 //   wv[SF]                 w of the own slice
 //   ring[slots]: codes [2][16 rb][pitch], 128 bytes of slack
-template <int CB, int RBC>
+template <int CB, int RBC, bool MANY>
 __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const SliceArgs a, const __grid_constant__ CUtensorMap tm1,
                                                                      const __grid_constant__ CUtensorMap tm2) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
     constexpr int CT = NG == 1 ? 2 : 1;                  // columns that a warp takes at once in the gradient
     static_assert(NS == 4, "a thread stores four digits at once");
     extern __shared__ __align__(16) unsigned char s_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bi = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cl = MANY ? blockIdx.x / a.nb : 0, bi = MANY ? blockIdx.x - cl * a.nb : blockIdx.x;
     const int n = a.n, sps = a.sps, owners = a.owners, rb = a.rb, SF = 32 * sps * NG;
     const int wd_words = sps * NG * 32 + 4, part_words = 2 * SF + 4;
     SliceShared* sh = reinterpret_cast<SliceShared*>(s_raw);
@@ -267,8 +293,9 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
     auto batch_at = [&](int k) { return k < steps ? (a.order ? __ldg(a.order + a.first_step + k) : (int)a.first_step + k) : 0; };
-    const int rows_full = min(a.rc, (int)a.batch - bi * a.rc), rows_last = min(a.rc, a.rows_last - bi * a.rc);
-    auto rows_of = [&](int batch) { return max(0, batch < whole ? rows_full : rows_last); };
+    const int row_base = (cl * a.nb + bi) * a.rc, chunks = MANY ? a.chunks : 1;
+    const int rows_full = min(a.rc, (int)a.batch - row_base), rows_last = min(a.rc, a.rows_last - row_base);
+    auto rows_of = [&](int batch, int chunk) { return max(0, min(a.cr, (batch < whole ? rows_full : rows_last) - chunk * a.cr)); };
     if (warp == kSliceWarps) {
         // -------------------------------------------------------------------- the copying warp
         int slot = 0;
@@ -276,23 +303,26 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll 1
         for (int k = 0; k < steps; ++k) {
             const int batch = batch_at(k);
-            const int64_t r0 = batch * a.batch + (int64_t)bi * a.rc;
-            unsigned char* dst = ring + slot * slot_bytes;
-            slice_wait(sh, sh->empty + slot, parity, a.status, 84);
-            if (a.use_tmap) {                            // (boxes that reach past the last row are filled up and count in full)
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)(a.rc * a.pitch));
-                    slice_tensor_copy(dst, &tm1, (int)r0, sh->full + slot);
-                    slice_tensor_copy(dst + plane_bytes, &tm2, (int)r0, sh->full + slot);
+#pragma unroll 1
+            for (int chunk = 0; chunk < chunks; ++chunk) {
+                const int64_t r0 = batch * a.batch + row_base + chunk * a.cr;
+                unsigned char* dst = ring + slot * slot_bytes;
+                slice_wait(sh, sh->empty + slot, parity, a.status, 84);
+                if (a.use_tmap) {                        // (boxes that reach past the last row are filled up and count in full)
+                    if (lane == 0) {
+                        mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)(a.cr * a.pitch));
+                        slice_tensor_copy(dst, &tm1, (int)r0, sh->full + slot);
+                        slice_tensor_copy(dst + plane_bytes, &tm2, (int)r0, sh->full + slot);
+                    }
+                } else {
+                    const int rows = rows_of(batch, chunk);
+                    if (lane == 0) mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)rows * (uint32_t)a.row_bytes);
+                    for (int i = lane; i < 2 * rows; i += 32)
+                        bulk_copy_g2s(dst + (i & 1) * plane_bytes + (i >> 1) * a.pitch, (i & 1 ? a.p2 : a.p1) + (r0 + (i >> 1)) * a.row_bytes,
+                                      (uint32_t)a.row_bytes, sh->full + slot);
                 }
-            } else {
-                const int rows = rows_of(batch);
-                if (lane == 0) mbar_arrive_expect_tx(sh->full + slot, 2u * (uint32_t)rows * (uint32_t)a.row_bytes);
-                for (int i = lane; i < 2 * rows; i += 32)
-                    bulk_copy_g2s(dst + (i & 1) * plane_bytes + (i >> 1) * a.pitch, (i & 1 ? a.p2 : a.p1) + (r0 + (i >> 1)) * a.row_bytes, (uint32_t)a.row_bytes,
-                                  sh->full + slot);
+                if (++slot == a.slots) { slot = 0; parity ^= 1u; }
             }
-            if (++slot == a.slots) { slot = 0; parity ^= 1u; }
         }
         __syncwarp();
         slice_cluster_sync();
@@ -302,8 +332,10 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     int batch = batch_at(0), batch_next = batch_at(1);
     // labels: a lane of the first rb warps forms one residual, of this row of the CTA
     const int res_row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
-    auto label_of = [&](int batch) { return warp < rb && res_row < rows_of(batch) ? __ldg(a.b + batch * a.batch + (int64_t)bi * a.rc + res_row) : 0.0f; };
-    float label = label_of(batch);
+    auto label_of = [&](int batch, int chunk) {
+        return warp < rb && res_row < rows_of(batch, chunk) ? __ldg(a.b + batch * a.batch + row_base + chunk * a.cr + res_row) : 0.0f;
+    };
+    float label = label_of(batch, 0);
 
     // ------------------------------------------------------------------------ the steps
     const int gl = lane >> 2, tl = lane & 3, lm = lane >> 3, l8 = lane & 7;
@@ -323,23 +355,27 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     float x = mine ? a.x[f_own] : 0.0f;
     auto draw = [&](int k, uint32_t stream) { return slice_draw(a.seed, a.epoch, (uint32_t)a.first_step + (uint32_t)k, (uint32_t)f_own, stream); };
 
-    const int marked = bi == 0 && tid == 0 && a.trace ? a.trace_steps : -1;
+    const int marked = blockIdx.x == 0 && tid == 0 && a.trace ? a.trace_steps : -1;
     int slot = 0;
     uint32_t parity = 0, w_parity = 0, part_parity = 0, gn_parity = 0, xn_parity = 0;
 #pragma unroll 1
     for (int step = -1; step < steps; ++step) {
         const bool last = step == steps - 1;
         uint32_t u_x = 0u, u_g = 0u;
-        const uint32_t tile_addr = smem_u32(ring) + (uint32_t)(slot * slot_bytes);
         if (step >= 0) {
             if (step < marked) slice_mark(a.trace, step, 0);
+            bool batch_full = true;
+#pragma unroll 1
+            for (int chunk = 0; chunk < chunks; ++chunk) {
+            const bool final_chunk = chunk == chunks - 1;
+            const uint32_t tile_addr = smem_u32(ring) + (uint32_t)(slot * slot_bytes);
             slice_wait(sh, sh->full + slot, parity, a.status, 6);
             // -------------------------------------------------------------- dots
 #pragma unroll 1
             for (int ws = ws_first, rb0 = rb_first; rb0 < rb;) {
                 const int a_slice = (ws * a.a_inv) >> 16;           // ws / a_parts
                 const int slab0 = (ws - a_slice * a.a_parts) * a.spw, slab1 = min(min(sps, a.slabs - a_slice * sps), slab0 + a.spw);
-                const bool keeper = slab0 == 0 && rb0 == 0;         // re-arms the slice's barrier
+                const bool keeper = slab0 == 0 && rb0 == 0 && chunk == 0;         // re-arms the slice's barrier
                 slice_wait(sh, sh->w_bar + a_slice, w_parity, a.status, 4);
                 if (keeper && lane == 0 && !last) mbar_arrive_expect_tx(sh->w_bar + a_slice, 4u * wd_words);
                 if (step < marked) slice_mark(a.trace, step, 1);
@@ -400,8 +436,8 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                 ws += ws_more; rb0 += rb_more;
                 if (ws >= a_all) { ws -= a_all; rb0 += RBC; }
             }
-            if (a.grad_bits > 0 && mine && pp == 0) u_g = draw(step, 4u);
-            if (a.model_bits > 0 && mine && pp == 0) u_x = draw(step + 1, 3u);
+            if (a.grad_bits > 0 && mine && pp == 0 && chunk == 0) u_g = draw(step, 4u);
+            if (a.model_bits > 0 && mine && pp == 0 && chunk == 0) u_x = draw(step + 1, 3u);
             slice_bar();
 
             // -------------------------------------------------------------- residuals and their digits
@@ -413,7 +449,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         if (w + i < a_all) d[i] += ps[(w + i) * rb * 32];
-                const float r = res_row < rows_of(batch) ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
+                const float r = res_row < rows_of(batch, chunk) ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
                 float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(r))));
                 if (rb > 1) {                            // one scale for all row blocks
                     if (lane == 0) sh->rmax[warp] = top;
@@ -428,10 +464,12 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll
                 for (int s = 0; s < NS; ++s) out[4 * s] = (unsigned char)(digits >> (8 * s));
             }
-            const bool batch_full = batch < whole;
-            batch = batch_next;
-            batch_next = batch_at(step + 2);
-            label = label_of(batch);
+            if (final_chunk) {
+                batch_full = batch < whole;
+                batch = batch_next;
+                batch_next = batch_at(step + 2);
+            }
+            label = label_of(batch, final_chunk ? 0 : chunk + 1);
             slice_bar();
             if (step < marked) slice_mark(a.trace, step, 2);
 
@@ -448,12 +486,15 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll 1
                 for (int kb = 0; kb < rb; ++kb)
                     mma_u8s8(ones, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, gl < NS ? rq[kb * 32] : 0u, gl < NS ? rq[kb * 32 + 4] : 0u);
-                // (sixteen row blocks: 512 products of a centred code and a digit, times 257, could pass 2^31: half of them)
-                const int half = RBC > 1 && rb > 15 ? 1 : 0, upper_weight = 256 >> half;
+                const float delta_r = sh->delta_r;
                 if (bj == 0) {                           // the sum of the residuals
-                    const float delta_r = sh->delta_r, s = (float)(ones[0] + 256 * ones[1]) * delta_r;
+                    const float s = (float)(ones[0] + 256 * ones[1]) * delta_r;
                     const float upper = __shfl_down_sync(0xffffffffu, s, 1);
-                    if (lane == 0) *reinterpret_cast<float2*>(part) = make_float2(fmaf(upper, 65536.0f, s), half ? 2.0f * delta_r : delta_r);
+                    if (lane == 0) {
+                        float2* head = reinterpret_cast<float2*>(part);
+                        const float all = fmaf(upper, 65536.0f, s);
+                        *head = MANY ? make_float2(chunk > 0 ? head->x + all : all, 1.0f) : make_float2(all, delta_r);
+                    }
                 }
 #pragma unroll 1
                 for (int col0 = col_begin; col0 < col_end; col0 += CT) {
@@ -489,14 +530,23 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll
                             for (int g = 0; g < NG; ++g) {
                                 int* out = part + 4 + 2 * (((col0 + ti) * 16 + 2 * gl) * NG + g) + tl;
-                                if (tl < 2) {            // lane t = 0 has the lower digits, t = 1 the upper ones
-                                    out[0] = (acc[ti][g][0] >> half) + upper_weight * acc[ti][g][1];
-                                    out[2 * NG] = (acc[ti][g][2] >> half) + upper_weight * acc[ti][g][3];
+                                // lane t = 0 has the lower digits, t = 1 the upper ones (fifteen row blocks at most: below 2^31)
+                                const int first = acc[ti][g][0] + 256 * acc[ti][g][1], second = acc[ti][g][2] + 256 * acc[ti][g][3];
+                                if (tl < 2) {
+                                    if constexpr (MANY) {          // chunks have scales of their own: they add up as floats
+                                        float* sum = reinterpret_cast<float*>(out);
+                                        sum[0] = fmaf((float)first, delta_r, chunk > 0 ? sum[0] : 0.0f);
+                                        sum[2 * NG] = fmaf((float)second, delta_r, chunk > 0 ? sum[2 * NG] : 0.0f);
+                                    } else {
+                                        out[0] = first;
+                                        out[2 * NG] = second;
+                                    }
                                 }
                             }
                         }
                     }
                 }
+                if (!final_chunk) continue;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
@@ -506,6 +556,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
             }
             if (lane == 0) mbar_arrive(sh->empty + slot);
             if (++slot == a.slots) { slot = 0; parity ^= 1u; }
+            }
             w_parity ^= 1u;
             if (step < marked) slice_mark(a.trace, step, 3);
 
@@ -520,20 +571,34 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                     for (int w = pp; w < a.nb; w += P) {
                         const int2 v = *reinterpret_cast<const int2*>(gbuf + w * part_words + 4 + 2 * k_own);
                         const float2 h = *reinterpret_cast<const float2*>(gbuf + w * part_words);
-                        t += (double)fmaf(st_low, fmaf((float)v.y, 65536.0f, (float)v.x) * h.y, mid * h.x);
+                        if constexpr (MANY) t += (double)fmaf(st_low, fmaf(__int_as_float(v.y), 65536.0f, __int_as_float(v.x)), mid * h.x);
+                        else t += (double)fmaf(st_low, fmaf((float)v.y, 65536.0f, (float)v.x) * h.y, mid * h.x);
                     }
 #pragma unroll 1
                 for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                if (MANY && a.clusters > 1) {
+                    const uint32_t tag = a.tag + (uint32_t)step;
+                    unsigned long long* box = a.exchange + ((size_t)(step & 1) * a.clusters * owners * SF + f_own) * 2;
+                    const size_t stride = (size_t)owners * SF * 2;
+                    const float hi = (float)t, low = (float)(t - (double)hi);
+                    if (mine && pp == 0) slice_post(box + cl * stride, hi, low, tag);
+                    t = 0.0;
+                    if (mine)
+#pragma unroll 1
+                        for (int c = pp; c < a.clusters; c += P) t += c == cl ? (double)hi + (double)low : slice_collect(sh, box + c * stride, tag, a.status);
+#pragma unroll 1
+                    for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                }
                 float g = (float)(t * (batch_full ? a.full_scale : a.last_scale));
                 const bool writes = mine && pp == 0;
-                if (last && a.grad_out && writes) a.grad_out[f_own] = g;
+                if (last && a.grad_out && writes && cl == 0) a.grad_out[f_own] = g;
                 if (step < marked) slice_mark(a.trace, step, 4);
                 if (a.grad_bits > 0) {
-                    const float M = slice_norm(writes ? (double)g * (double)g : 0.0, P, sh->red[0], sh->nrm_g, &sh->gn_bar, gn_parity, owners, sh, a.status, 3);
+                    const float M = slice_norm(writes ? (double)g * (double)g : 0.0, P, bi, sh->red[0], sh->nrm_g, &sh->gn_bar, gn_parity, owners, sh, a.status, 3);
                     gn_parity ^= 1u;
                     g = slice_quantize(g, M, a.grad_bits, u_g);
                 }
-                if (last && a.grad_out && writes) a.grad_out[n + f_own] = g;
+                if (last && a.grad_out && writes && cl == 0) a.grad_out[n + f_own] = g;
                 const float y = fmaf(-a.lr, g, x);
                 x = a.reg == ZIPML_REG_NONE ? y : slice_regularise(y, x, a.reg, a.reg_cst);
             }
@@ -546,12 +611,12 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
         if (owner) {
             float xt = x;
             if (a.model_bits > 0) {
-                const float M = slice_norm(mine && pp == 0 ? (double)x * (double)x : 0.0, P, sh->red[1], sh->nrm_x, &sh->xn_bar, xn_parity, owners, sh, a.status, 8);
+                const float M = slice_norm(mine && pp == 0 ? (double)x * (double)x : 0.0, P, bi, sh->red[1], sh->nrm_x, &sh->xn_bar, xn_parity, owners, sh, a.status, 8);
                 xn_parity ^= 1u;
                 xt = slice_quantize(x, M, a.model_bits, u_x);
             }
             const bool writes = mine && pp == 0;
-            if (a.model_out && step + 2 == steps && writes) a.model_out[f_own] = xt;
+            if (a.model_out && step + 2 == steps && writes && cl == 0) a.model_out[f_own] = xt;
             const float w = writes ? st * xt : 0.0f;
             if (pp == 0 && k_own < SF) wv[k_own] = w;
             const float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w))));
@@ -587,7 +652,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
         }
         if (step >= 0 && step < marked) slice_mark(a.trace, step, 5);
     }
-    if (mine && pp == 0) a.x[f_own] = x;
+    if (mine && pp == 0 && cl == 0) a.x[f_own] = x;
     __syncwarp();
     slice_cluster_sync();                                // nobody leaves while a copy may still target it
 }
@@ -596,7 +661,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 // Host side
 // ---------------------------------------------------------------------------------------------
 struct SlicePlan {
-    int nb, rc, rb, owners, sps, slabs, cols, a_parts, spw, b_parts, cpw, p_shift, pitch, slots;
+    int clusters, chunks, nb, rc, cr, rb, owners, sps, slabs, cols, a_parts, spw, b_parts, cpw, p_shift, pitch, slots;
     size_t smem;
 };
 
@@ -607,23 +672,37 @@ static size_t slice_smem_bytes(const SlicePlan& r, int ng, int slots) {
     return bytes + (size_t)slots * (2 * (((size_t)16 * r.rb * r.pitch + 127) & ~(size_t)127) + 128);
 }
 
-static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, SlicePlan* plan) {
+// How many clusters (most: as many as can be resident at once): one for 16 rows per CTA where a step has the work to pay
+// for their exchange (about 1.2 us), batch x (features + 128).  Measured, us per step with 1 / 2 / 4 / 8 clusters: 8 bits 512 x 1,000
+// 4.6 / 4.8 / 5.0 / 6.6, 1,024 x 1,000 8.5 / 6.1 / 5.1 / 5.6, 4,096 x 1,000 28.9 / 16.7 / 10.2 / 8.7, 2,400 x 287 7.1 / 6.6 / 6.2 / 5.3; 4 bits
+// 1,024 x 64 3.7 / 4.4 / 4.1 / 4.2, 4,096 x 64 7.5 / 5.4 / 5.0 / 5.0, 512 x 512 3.8 / 4.2 / 4.3 / 4.9, 384 x 4,035 10.8 / 8.2 / 8.7 / 10.5; 2 bits 1,024 x
+// 2,048 7.8 / 7.5 / 6.3 / 7.3.
+static int slice_clusters(int64_t B, int64_t n, int most) {
+    if (B * (n + 128) < 650000) return 1;
+    const int64_t want = (B + 16 * kSliceMaxCtas - 1) / (16 * kSliceMaxCtas);
+    return (int)(want > most ? most : want);
+}
+
+static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, int most_clusters, SlicePlan* plan) {
     const int cb = container_bits(d->bits), ng = 8 / cb;
     const int64_t B = p->batch < d->m ? p->batch : d->m;
     const int64_t used = (d->n * cb + 7) / 8, slabs = (used + 31) / 32;
-    if (d->level_mode != ZIPML_LEVELS_UNIFORM || (d->m + B - 1) / B > 0x7ffffff0 || slabs > 1024 || d->row_bytes > (1 << 16)) return ZIPML_ERR_WORKSPACE;
-    int64_t nb = p->grid_row_parts > 0 ? p->grid_row_parts : (B + 15) / 16;     // automatic: 16 rows per CTA
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || (d->m + B - 1) / B > 0x7ffffff0 || slabs > 1024 || d->row_bytes > (1 << 16) || B > (1 << 24)) return ZIPML_ERR_WORKSPACE;
+    int64_t clusters = p->grid_feature_parts > 0 ? p->grid_feature_parts : slice_clusters(B, d->n, most_clusters);
+    if (clusters > most_clusters) clusters = most_clusters;
+    const int64_t Bc = (B + clusters - 1) / clusters;
+    int64_t nb = p->grid_row_parts > 0 ? p->grid_row_parts : (Bc + 15) / 16;    // automatic: 16 rows per CTA
     if (nb > kSliceMaxCtas) nb = kSliceMaxCtas;
-    if (nb > B) nb = B;
-    for (; nb <= kSliceMaxCtas && nb <= B; ++nb) {       // (more parts than asked for where a tile or a slice does not fit)
+    if (nb > Bc) nb = Bc;
+    for (; nb <= kSliceMaxCtas && nb <= Bc; ++nb) {      // (more parts than asked for where a tile or a slice does not fit)
         SlicePlan r;
-        r.rc = (int)((B + nb - 1) / nb);
-        r.nb = (int)((B + r.rc - 1) / r.rc);
-        r.rb = (r.rc + 15) / 16;
+        r.clusters = (int)clusters;
+        r.rc = (int)((Bc + nb - 1) / nb);
+        r.nb = (int)((Bc + r.rc - 1) / r.rc);
         r.sps = (int)((slabs + r.nb - 1) / r.nb);
         r.owners = (int)((slabs + r.sps - 1) / r.sps);
         r.slabs = (int)slabs; r.cols = (int)((used + 15) / 16);
-        if (r.rb > kSliceWarps || 32 * r.sps * ng > kSliceThreads) continue;
+        if (32 * r.sps * ng > kSliceThreads) continue;
         const int per = r.owners < kSliceWarps ? kSliceWarps / r.owners : 1;
         r.spw = (r.sps + per - 1) / per;
         r.a_parts = (r.sps + r.spw - 1) / r.spw;
@@ -633,9 +712,17 @@ static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const z
         while (r.p_shift < 4 && (32 * r.sps * ng) << (r.p_shift + 1) <= kSliceThreads && (1 << r.p_shift) < r.nb) ++r.p_shift;
         const int units = (int)(d->row_bytes / 16);
         r.pitch = 16 * (units | 1);
+        // as few chunks as leave two slots, equally long
+        const int blocks = (r.rc + 15) / 16;
+        for (r.chunks = (blocks + 14) / 15; r.chunks <= blocks; ++r.chunks) {
+            r.rb = (blocks + r.chunks - 1) / r.chunks;
+            if (slice_smem_bytes(r, ng, 2) <= (size_t)ctx->smem_optin) break;
+        }
+        if (r.chunks > blocks) continue;
+        r.chunks = (blocks + r.rb - 1) / r.rb;
+        r.cr = r.chunks == 1 ? r.rc : 16 * r.rb;
         r.slots = kSliceMaxSlots;
-        while (r.slots >= 2 && slice_smem_bytes(r, ng, r.slots) > (size_t)ctx->smem_optin) --r.slots;
-        if (r.slots < 2) continue;
+        while (slice_smem_bytes(r, ng, r.slots) > (size_t)ctx->smem_optin) --r.slots;
         r.smem = slice_smem_bytes(r, ng, r.slots);
         *plan = r;
         return ZIPML_OK;
@@ -643,43 +730,58 @@ static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const z
     return ZIPML_ERR_WORKSPACE;
 }
 
+template <int CB>
+static const void* slice_kernel(int rb, bool many) {
+    if (many) return rb == 1 ? (const void*)sgd_slice_kernel<CB, 1, true> : (const void*)sgd_slice_kernel<CB, 2, true>;
+    return rb == 1 ? (const void*)sgd_slice_kernel<CB, 1, false> : (const void*)sgd_slice_kernel<CB, 2, false>;
+}
+
 int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                      int64_t num_steps, float* grad_out) {
-    SlicePlan plan;
-    int rc = make_slice_plan(ctx, d, p, &plan);
-    if (rc != ZIPML_OK) return rc;
     const int cb = container_bits(d->bits);
-    const bool one = plan.rb == 1;
-    const void* kernel = cb == 2 ? (one ? (const void*)sgd_slice_kernel<2, 1> : (const void*)sgd_slice_kernel<2, 2>)
-                       : cb == 4 ? (one ? (const void*)sgd_slice_kernel<4, 1> : (const void*)sgd_slice_kernel<4, 2>)
-                                 : (one ? (const void*)sgd_slice_kernel<8, 1> : (const void*)sgd_slice_kernel<8, 2>);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-    if (e == cudaSuccess && plan.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return cuda_status(e);
+    if (cb == 0) return ZIPML_ERR_UNSUPPORTED;
+    SlicePlan plan;
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)plan.nb);
-    cfg.blockDim = dim3(kSliceThreads + 32);
-    cfg.dynamicSmemBytes = plan.smem;
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)plan.nb;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
-    if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
-    if (clusters < 1) return ZIPML_ERR_WORKSPACE;
+    cudaLaunchAttribute attr[2];
+    const void* kernel = nullptr;
+    int rc;
+    // (clusters are taken back until all of them can be resident at once: they wait for one another)
+    for (int most = kSliceMaxClusters;;) {
+        rc = make_slice_plan(ctx, d, p, ctx->cooperative ? most : 1, &plan);
+        if (rc != ZIPML_OK) return rc;
+        const bool many = plan.clusters > 1 || plan.chunks > 1;
+        kernel = cb == 2 ? slice_kernel<2>(plan.rb, many) : cb == 4 ? slice_kernel<4>(plan.rb, many) : slice_kernel<8>(plan.rb, many);
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+        if (e == cudaSuccess && plan.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return cuda_status(e);
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(plan.nb * plan.clusters));
+        cfg.blockDim = dim3(kSliceThreads + 32);
+        cfg.dynamicSmemBytes = plan.smem;
+        cfg.stream = ctx->stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)plan.nb;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeCooperative;
+        attr[1].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
+        if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
+        if (fit < 1) return ZIPML_ERR_WORKSPACE;
+        if (fit >= plan.clusters) break;
+        most = fit;
+    }
+    if (plan.clusters > 1) cfg.numAttrs = 2;
     const int64_t T = (d->m + p->batch - 1) / p->batch;
     SliceArgs a;
     memset(&a, 0, sizeof(a));
     if (p->batch_order) {
         rc = ws_reserve(ctx, carve_size(sizeof(int32_t) * (size_t)T));
         if (rc != ZIPML_OK) return rc;
-        e = cudaMemcpyAsync(ctx->ws, p->batch_order, sizeof(int32_t) * (size_t)T, cudaMemcpyHostToDevice, ctx->stream);
+        const cudaError_t e = cudaMemcpyAsync(ctx->ws, p->batch_order, sizeof(int32_t) * (size_t)T, cudaMemcpyHostToDevice, ctx->stream);
         if (e != cudaSuccess) return cuda_status(e);
         a.order = reinterpret_cast<const int32_t*>(ctx->ws);
     }
@@ -694,14 +796,29 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     a.full_scale = 1.0 / (2.0 * (double)a.batch); a.last_scale = 1.0 / (2.0 * (double)(a.rows_last > 0 ? a.rows_last : 1));
     a.seed = p->seed; a.epoch = (uint32_t)p->epoch; a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
     a.n = (int)d->n; a.bits = d->bits; a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
-    a.nb = plan.nb; a.rc = plan.rc; a.rb = plan.rb; a.owners = plan.owners; a.sps = plan.sps; a.slabs = plan.slabs; a.cols = plan.cols;
+    a.clusters = plan.clusters; a.chunks = plan.chunks; a.nb = plan.nb; a.rc = plan.rc; a.cr = plan.cr; a.rb = plan.rb; a.owners = plan.owners; a.sps = plan.sps; a.slabs = plan.slabs; a.cols = plan.cols;
     a.a_parts = plan.a_parts; a.a_inv = 65536 / plan.a_parts + 1; a.spw = plan.spw; a.b_parts = plan.b_parts; a.b_inv = 65536 / plan.b_parts + 1; a.cpw = plan.cpw;
     CUtensorMap tmaps[2];
     memset(tmaps, 0, sizeof(tmaps));
-    a.use_tmap = d->m < (1ll << 31) - 4096 && encode_plane_maps(ctx, d, plan.pitch / 4, plan.rc, true, tmaps) == ZIPML_OK;
+    a.use_tmap = d->m < (1ll << 31) - 4096 && encode_plane_maps(ctx, d, plan.pitch / 4, plan.cr, true, tmaps) == ZIPML_OK;
     a.p_shift = plan.p_shift; a.pitch = plan.pitch; a.slots = plan.slots;
     void* params[] = {&a, &tmaps[0], &tmaps[1]};
-    e = cudaLaunchKernelExC(&cfg, kernel, params);
+    if (plan.clusters > 1) {
+        // tags go up from launch to launch, so the buffer is cleared only when it is new (or they would wrap)
+        const size_t bytes = (size_t)2 * plan.clusters * plan.owners * 32 * plan.sps * (8 / cb) * 16;
+        const bool stale = ctx->exchange_bytes < bytes || ctx->exchange_tag > 0xffffffffu - (uint32_t)num_steps - 1u;
+        rc = exchange_reserve(ctx, bytes);
+        if (rc != ZIPML_OK) return rc;
+        if (stale) {
+            const cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, ctx->exchange_bytes, ctx->stream);
+            if (e != cudaSuccess) return cuda_status(e);
+            ctx->exchange_tag = 1;
+        }
+        a.exchange = reinterpret_cast<unsigned long long*>(ctx->exchange);
+        a.tag = ctx->exchange_tag;
+        ctx->exchange_tag += (uint32_t)num_steps;
+    }
+    cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, params);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
     ctx->last_engine = ZIPML_ENGINE_CLUSTER;

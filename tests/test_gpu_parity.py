@@ -311,6 +311,44 @@ def test_solo_engine(ctx, m, n, bits, batch, table):
         assert ctx.zipml_last_engine() == binding.ENGINE_SOLO               # what AUTO takes
 
 
+@pytest.mark.parametrize("m,n,bits,batch,clusters,parts", [
+    (2600, 33, 8, 1200, 3, 0), (1500, 1000, 8, 700, 2, 0), (9000, 64, 4, 4096, 1, 0), (2000, 2048, 2, 900, 8, 0), (700, 130, 4, 300, 4, 5),
+    (900, 2000, 6, 450, 1, 4), (100, 500, 8, 40, 8, 1), (5000, 17, 2, 5000, 8, 16),
+])
+def test_several_clusters_and_chunks(ctx, m, n, bits, batch, clusters, parts):
+    """Clusters that meet through L2 and minibatches that go through shared memory in chunks: rows left over, CTAs and
+    clusters without rows, twice on one context (the exchange buffer is not cleared in between)."""
+    _, A, b, _ = workload("c1", m, n, seed=n)
+    ods = oracle.quantize(A, bits, seed=3)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    T = (m + batch - 1) // batch
+    lr = 0.3 / n
+    order = np.random.default_rng(0).permutation(T).astype(np.int32)
+    x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
+    how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=2, grid_feature_parts=clusters, grid_row_parts=parts)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, batch_order=order)
+    x_before, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, batch_order=order, num_steps=T - 1)
+    _, g_ref = oracle.sgd_epoch(ods, b, x_before, batch, lr, batch_order=order, first_step=T - 1, num_steps=1, want_grad=True)
+    for _ in range(2):
+        x = to_dev(x0, ctx)
+        ctx.zipml_sgd_epoch(gds, db, x, batch, lr, batch_order=order, **how)
+        ctx.zipml_sync()
+        assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+    xb = to_dev(x_before, ctx)
+    g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+    ctx.zipml_sgd_epoch(gds, db, xb, batch, lr, batch_order=order, first_step=T - 1, num_steps=1, grad_out=g, **how)
+    ctx.zipml_sync()
+    assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL and rel(xb.cpu().numpy(), x_ref) <= MODEL_TOL
+    x, seen = to_dev(x0, ctx), torch.zeros(n, device=ctx.device)
+    kw = dict(seed=5, epoch=1, first_step=0, num_steps=1)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, model_bits=8, grad_bits=6, grad_out=g, model_out=seen, **how, **kw)
+    ctx.zipml_sync()
+    _, g_ref = oracle.sgd_epoch(ods, b, seen.cpu().numpy(), batch, lr, want_grad=True, **kw)
+    assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL
+    g4, _ = oracle.quantize_vector(g[0].cpu().numpy(), 6, 5, 1, 0, 4)
+    assert (g[1].cpu().numpy() != g4).sum() <= 3
+
+
 @pytest.mark.parametrize("m,n,bits,batch,parts", [
     (50, 3, 8, 5, 0), (700, 33, 8, 130, 3), (900, 65, 4, 257, 0), (400, 1000, 8, 100, 0), (1100, 130, 2, 512, 2), (300, 2048, 2, 37, 0),
     (70, 4090, 8, 33, 0), (600, 520, 6, 250, 16), (2100, 40, 4, 2048, 0), (64, 6100, 2, 16, 16),
