@@ -240,6 +240,54 @@ int zipml_optimal_levels(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, i
     return launch_levels_dp(ctx, counts, n, hist_bins, s, lo, hi, levels_out, objective_out);
 }
 
+// ---- AUTO's rules, measured in us per step: C column, S stream, R ring, K cluster (fp32 form), L lean, G the persistent grid ----
+
+// The engine for rows that no cluster takes (uniform grids, fp32 model and gradient), 0 where the cluster engine is tried first.
+// From 2,400 features (2-bit codes, of which a CTA unpacks the most per byte: 6,000) a hand-over through L2 costs less than a
+// cluster's fp32 work on whole rows: batch 1 n 1,723 K 6.6 C 7.6, n 2,427 K 7.9 C 7.9, n 4,891 K 12.2 C 7.8; 2 bits n 6,939 K 11.4
+// S 10.5.  Lean and ring take 20 to 80 there (4 bits n 6,747 batch 64 L 22.3 R 19.0 C 8.2; 2 bits n 13,499 L 52.9 R 22.2 S 10.8).
+static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, int64_t B) {
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || p->model_bits != 0 || p->grad_bits != 0 || p->model_out) return 0;
+    const int cb = container_bits(d->bits);
+    if (d->n < (cb == 2 ? 6000 : 2400)) return 0;
+    // Many rows of a few KB: the ring engine streams them.  4 bits 2.4 KB x 3,000 S 31.9 R 34.1, x 6,000 S 57 R 43; 3.3 KB x 6,000
+    // S 51 R 49; 4.5 KB x 6,000 S 44 R 50; 2 bits 3.3 KB x 3,000 S 38.5 R 42, x 6,000 S 65 R 59.  8 bits, of which it makes
+    // half the work per byte: 3.3 KB x 2,000 S 19.2 R 18.9, x 3,000 S 26.8 R 22.8; 6 KB x 2,000 S 18.9 R 22.7, x 6,000 S 41 R 37.
+    if (cb == 8 ? 4 * B > 3 * d->row_bytes : 3 * B > 4 * d->row_bytes) return ZIPML_ENGINE_RING;
+    const int64_t blocks = (d->row_bytes + 127) / 128;                 // CTAs of the column engine
+    if (2 * blocks >= ctx->sm_count) {
+        // At least half the device.  (At 32 to 255 rows of 4-bit codes the stream engine keeps what it had, C 9.2 S 11.1 at 10 KB x
+        // 128: callers rely on that choice.)
+        if (B >= 256 || cb == 8 || B < 32) return ZIPML_ENGINE_COLUMN;
+        return ZIPML_ENGINE_STREAM;
+    }
+    // 2 bits: C 11.5 S 10.8 at 2.4 KB x 64, 27 / 20 at 6 KB x 1,000.  Else up to some 1,000 rows the column engine, whose CTAs are
+    // few but exchange less: 4 bits 3.3 KB x 600 C 14.6 S 16.6, x 1,500 29.2 / 25.6; 8 bits 4.5 KB x 1,000 14.0 / 14.4, x 2,000
+    // 19.7 / 18.3.
+    return cb == 2 || B >= 1200 ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
+}
+
+// Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.
+//   uniform, quantized: 8 bits n 3,355 x 256 L 22 R 27; 4 bits n 4,891 x 256 L 30.5 R 31; n 6,747 x 64 L 32 R 25; 2 bits n 6,939 L 31 R 26.
+//   tables: 2 bits n 4,091 x 64 L 22 G 24, x 256 L 26 G 18; n 2,043 x 1,500 L 43 G 38; 4 bits n 1,019 x 600 L 24 G 28, x 1,500 L 42 G 34;
+//   one row of n 4,091 L 27 G 16; with a quantized vector the grid is no better (4 bits n 1,019 x 1,500 L 51 G 58).
+static bool lean_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B) {
+    if (d->level_mode == ZIPML_LEVELS_UNIFORM) return d->n <= 4096;
+    if (p->model_bits != 0 || p->grad_bits != 0) return true;
+    return B * d->n <= 700000 && (d->n < 3000 || B >= 32);
+}
+
+// Uniform rows too wide for the column and stream engines: the persistent grid up to 16 MB a step, 4 bits n 100,000 x 64 G 23 R 42, x 300
+// (30 MB) 107 / 53; 8 bits n 150,000 x 64 (19 MB) 60 / 71, x 300 243 / 138.
+// Level tables wider than a cluster holds: the persistent grid too, whose CTAs take row parts of a few columns and so build few of the
+// tables, until the ring engine's asynchronous tiles win.  2 bits n 13,499 x 64 G 17 R 27, x 600 (4 MB) 37 / 45, x 1,500 (10 MB) 75 / 76;
+// 3 bits n 6,747 x 600 (4 MB) 26 / 29, n 12,283 x 1,500 (18 MB) 91 / 64; 4 bits n 4,891 x 600 (2.9 MB) 29 / 32, n 20,475 x 256 (5 MB) 37 / 33.
+static bool grid_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t step_bytes, int wide) {
+    if (p->model_bits != 0 || p->grad_bits != 0) return false;
+    if (d->level_mode == ZIPML_LEVELS_UNIFORM) return (wide == ZIPML_ENGINE_COLUMN || wide == ZIPML_ENGINE_STREAM) && step_bytes <= (16ll << 20);
+    return step_bytes <= (d->bits == 2 ? 10ll << 20 : d->bits == 3 ? 5ll << 20 : 3ll << 20);
+}
+
 int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, float* x,
                     const zipml_sgd_params* params, float* grad_out) {
     if (!ctx || !params || params->struct_size != sizeof(zipml_sgd_params)) return ZIPML_ERR_INVALID_ARG;
@@ -273,43 +321,56 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (linf && data->layout == ZIPML_LAYOUT_COLUMN_BLOCKS) return ZIPML_ERR_UNSUPPORTED;
     if (data->layout == ZIPML_LAYOUT_COLUMN_BLOCKS) {                 // the column engine's own layout
         if (params->engine != ZIPML_ENGINE_AUTO && params->engine != ZIPML_ENGINE_COLUMN) return ZIPML_ERR_UNSUPPORTED;
-        rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
+        rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
         return rc == ZIPML_ERR_WORKSPACE ? ZIPML_ERR_UNSUPPORTED : rc;
     }
     if (params->engine == ZIPML_ENGINE_RING) return launch_sgd_ring(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_LEAN) return launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
     if (params->engine == ZIPML_ENGINE_CLUSTER) return launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
-    if (params->engine == ZIPML_ENGINE_STREAM) return launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out, false);
-    if (params->engine == ZIPML_ENGINE_COLUMN) return launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
+    if (params->engine == ZIPML_ENGINE_STREAM) return launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out);
+    if (params->engine == ZIPML_ENGINE_COLUMN) return launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
     if (params->engine == ZIPML_ENGINE_SOLO) return launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_AUTO && !linf) {
-        // Small minibatch tiles are bound by the step-to-step chain, not by HBM: the smallest stay on one SM;
-        // then one cluster whose CTAs
-        // exchange through shared memory, else row parts exchanging through L2.  Larger tiles go to the
-        // column engine (codes read once per step), the stream engine, then the ring engine.  Each engine
+        // Small minibatch tiles are bound by the step-to-step chain, not by HBM: the smallest stay on one SM, then
+        // clusters whose CTAs exchange through shared memory.  Rows too wide for a cluster go to the column engine
+        // (codes read once per step), the stream engine or the ring engine, whatever the step's size.  Each engine
         // answers ZIPML_ERR_WORKSPACE when the shape does not fit it.
         const int64_t B = params->batch < data->m ? params->batch : data->m;
         const int64_t step_bytes = 2 * B * data->row_bytes;
-        if (step_bytes <= (2ll << 20)) {
+        const bool small = step_bytes <= (2ll << 20);
+        const int wide = wide_rows_engine(ctx, data, params, B);
+        if (small) {
             rc = launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, true);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
+        if (small && !wide) {
             rc = launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
-            rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
-            if (rc != ZIPML_ERR_WORKSPACE) return rc;
-        }
-        // Rows of up to some 3 KB: clusters that hold whole rows, however large the batch (8-bit codes, whose tensor work per
-        // byte is least, up to where the ring engine's 148 CTAs stream faster: 8,192 x 2,000 19.0 / 26.9 us per step,
-        // 16,384 x 2,000 36.9 / 35.2; at 4 bits 16,384 x 3,000 42.7 / 48.2).
-        if (step_bytes > (2ll << 20) && (container_bits(data->bits) < 8 || step_bytes <= (48ll << 20))) {
+            if (lean_pays(data, params, B)) {
+                rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
+                if (rc != ZIPML_ERR_WORKSPACE) return rc;
+            }
+        } else if (container_bits(data->bits) < 8 || step_bytes <= (48ll << 20)) {
+            // Rows of up to some 3 KB: clusters that hold whole rows, however large the batch (8-bit codes, whose tensor work
+            // per byte is least, up to where the ring engine's 148 CTAs stream faster: 8,192 x 2,000 19.0 / 26.9 us per step,
+            // 16,384 x 2,000 36.9 / 35.2; at 4 bits 16,384 x 3,000 42.7 / 48.2).
             rc = launch_sgd_slice(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        // (also for small steps on rows too wide for those above)
-        rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, true);
-        if (rc != ZIPML_ERR_WORKSPACE) return rc;
-        rc = launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out, true);
-        if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        if (wide == ZIPML_ENGINE_COLUMN) {
+            rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
+        if (wide == ZIPML_ENGINE_COLUMN || wide == ZIPML_ENGINE_STREAM) {
+            rc = launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
+        if (grid_pays(data, params, step_bytes, wide)) {
+            zipml_sgd_params grid = *params;
+            grid.engine = ZIPML_ENGINE_PERSISTENT;
+            rc = launch_sgd_epoch(ctx, data, b, x, &grid, first, count, grad_out);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
         rc = launch_sgd_ring(ctx, data, b, x, params, first, count, grad_out, false);
         if (rc != ZIPML_ERR_WORKSPACE) return rc;
     }

@@ -108,15 +108,14 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
                      int64_t num_steps, float* grad_out);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out);
-// Stream engine (uniform grids, fp32 model and gradient).  With only_if_profitable it declines
-// (ZIPML_ERR_WORKSPACE) shapes whose steps are too narrow or too short for it.
+// Stream engine (uniform grids, fp32 model and gradient).
 int launch_sgd_stream(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
-                      int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable);
-// Column engine (uniform grids, fp32 model and gradient, rows of at most 128 bytes per SM).
+                      int64_t first_step, int64_t num_steps, float* grad_out);
 int launch_sgd_apply(zipml_ctx* ctx, float* x, const float* g, int64_t n, const zipml_sgd_params* p, int64_t step,
                      float* applied_out);
+// Column engine (uniform grids, fp32 model and gradient, rows of at most 128 bytes per SM).
 int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
-                      int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable);
+                      int64_t first_step, int64_t num_steps, float* grad_out);
 // Both planes of d into the other layout (see ZIPML_LAYOUT_* in zipml.h).
 int launch_convert_layout(zipml_ctx* ctx, const zipml_dataset* d, int to_layout, uint8_t* out1, uint8_t* out2);
 int launch_barrier_latency(zipml_ctx* ctx, int ctas, int floats, int iterations, unsigned long long* ns_out_dev);

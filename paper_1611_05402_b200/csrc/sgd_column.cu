@@ -962,7 +962,7 @@ static int encode_column_maps(zipml_ctx* ctx, const zipml_dataset* d, int R, CUt
 }
 
 int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
-                      int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable) {
+                      int64_t first_step, int64_t num_steps, float* grad_out) {
     if (!ctx->cooperative) return ZIPML_ERR_WORKSPACE;
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || p->model_bits != 0 || p->grad_bits != 0 || p->model_out) return ZIPML_ERR_WORKSPACE;
     if (d->m > 0x7fffffffLL || d->row_bytes < kColBlockBytes) return ZIPML_ERR_WORKSPACE;
@@ -974,8 +974,6 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     if (B > kColMaxBatch) return ZIPML_ERR_WORKSPACE;
     const int64_t G = (d->row_bytes + kColBlockBytes - 1) / kColBlockBytes;
     if (G > ctx->sm_count) return ZIPML_ERR_WORKSPACE;                 // one CTA per SM, all resident at once
-    // worth it where the rows occupy most of the device and a step holds several chunks
-    if (only_if_profitable && (G < ctx->sm_count / 2 || B < 256)) return ZIPML_ERR_WORKSPACE;
     int R = p->column_chunk_rows > 0 ? p->column_chunk_rows : 128;
     if (R > kColMaxChunkRows) R = kColMaxChunkRows;
     if (R > (B + 31) / 32 * 32) R = (int)((B + 31) / 32 * 32);

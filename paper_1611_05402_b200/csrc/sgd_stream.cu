@@ -625,7 +625,7 @@ static const void* stream_kernel_ptr(int cb) {
 }
 
 int launch_sgd_stream(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
-                      int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable) {
+                      int64_t first_step, int64_t num_steps, float* grad_out) {
     if (!ctx->cooperative) return ZIPML_ERR_WORKSPACE;
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || p->model_bits != 0 || p->grad_bits != 0) return ZIPML_ERR_WORKSPACE;
     if (d->n > (1 << 30) / 8) return ZIPML_ERR_WORKSPACE;
@@ -649,9 +649,6 @@ int launch_sgd_stream(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     }
     if (bpc > kStreamMaxOwn) return ZIPML_ERR_WORKSPACE;
     G = (int)((spans + bpc - 1) / bpc);
-    // worth it only where the rows are wide enough to occupy the device (measured against the ring engine on
-    // 16 KB rows: ahead at every batch from 128 to 8192 rows, 10.7 vs 25.8 us per step at 128)
-    if (only_if_profitable && (G < ctx->sm_count / 2 || B < 32)) return ZIPML_ERR_WORKSPACE;
     // pass A: 256-row groups x column parts, about one unit per CTA
     const int64_t nrg = ((B + 15) / 16 + kStreamWarps - 1) / kStreamWarps;
     int64_t ca = G / nrg;

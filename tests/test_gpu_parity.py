@@ -758,6 +758,26 @@ def test_auto_picks_the_engine_that_fits(ctx):
     assert ctx.zipml_last_engine() == binding.ENGINE_CLUSTER
 
 
+@pytest.mark.parametrize("m,n,bits,batch,optimal,engine", [
+    (130, 4700, 4, 64, False, binding.ENGINE_COLUMN), (9, 2431, 8, 1, False, binding.ENGINE_COLUMN),
+    (90, 9403, 2, 40, False, binding.ENGINE_STREAM), (1300, 4700, 4, 1205, False, binding.ENGINE_STREAM),
+    (2600, 3300, 8, 2500, False, binding.ENGINE_RING), (40, 3500, 4, 16, True, binding.ENGINE_PERSISTENT),
+    (30, 90_003, 8, 16, False, binding.ENGINE_PERSISTENT),
+], ids=str)
+def test_auto_on_rows_wider_than_a_cluster(ctx, m, n, bits, batch, optimal, engine):
+    """Every line of AUTO's rule for rows that no cluster takes, with the engine it names and the oracle's result."""
+    _, A, b, _ = workload("c4" if optimal else "c2", m, n, seed=4)
+    kw = dict(mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 64)[0]) if optimal else {}
+    ods = oracle.quantize(A, bits, seed=3, **kw)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-4)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, 1e-4)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_engine() == engine and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+
+
 REGS = [(binding.REG_L2, 0.5), (binding.REG_L1, 0.02), (binding.REG_NONNEG, 0.0), (binding.REG_LSSVM, 0.5)]
 
 
