@@ -106,6 +106,9 @@ int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
 // The cluster engine's int8 form on uniform grids (launch_sgd_cluster calls it).
 int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                      int64_t num_steps, float* grad_out);
+// Its form on level tables.
+int launch_sgd_table(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                     int64_t num_steps, float* grad_out);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out);
 // Stream engine (uniform grids, fp32 model and gradient).

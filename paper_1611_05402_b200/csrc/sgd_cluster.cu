@@ -838,14 +838,23 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
     }
 }
 
+// Level tables: split by features, or by rows where the features make too few 16-byte units for the CTAs.  us per step by features / by
+// rows / lean: 3 bits n 64 (2 units) x 512 5.1 / 5.2 / 5.6, x 1,024 8.4 / 7.1 / 6.9, n 120 (4) x 1,024 6.5 / 7.2 / 7.2, x 2,048 11.5 / 11.3 / 10.0,
+// n 512 (16) x 512 3.6 / 6.5 / 8.3, x 2,048 8.7 / 15.3 / 14.5; 2 bits n 120 (2) x 256 4.0 / 4.8 / 5.1, x 512 6.2 / 6.3 / 5.9; n 1,019 (16) x 1,024
+// 7.5 / 14.3 / 13.4.
+static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
+    const int64_t B = p->batch < d->m ? p->batch : d->m, units = (d->n * container_bits(d->bits) + 127) / 128;
+    return B <= (container_bits(d->bits) == 2 ? 240 : 300) * units;
+}
+
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out) {
     const int cb = container_bits(d->bits);
     const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
     const int fpw = 32 / cb;
     const int64_t T = (d->m + p->batch - 1) / p->batch;
-    if (!table && p->cluster_contraction != 1) {
-        const int rc = launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
+    if (p->cluster_contraction != 1 && (!table || p->cluster_contraction == 2 || table_form_pays(d, p))) {
+        const int rc = table ? launch_sgd_table(ctx, d, b, x, p, first_step, num_steps, grad_out) : launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
         if (rc != ZIPML_ERR_WORKSPACE) return rc;
     }
     ClusterPlan plan;

@@ -393,6 +393,42 @@ def test_slice_form_of_the_cluster_engine(ctx, m, n, bits, batch, parts):
     assert (g[1].cpu().numpy() != g4).sum() <= 3
 
 
+# tables split by features: units of 16 bytes per CTA (parts: fewer CTAs, more units), one row and one past a pass of 128, 256 and 512
+# lanes, odd batches (rows travel in pairs), owners without rows, several boxes, a short last batch
+@pytest.mark.parametrize("m,n,bits,batch,parts", [
+    (3, 5, 1, 1, 0), (40, 33, 3, 17, 0), (700, 64, 2, 255, 0), (1100, 65, 3, 257, 2), (300, 31, 4, 129, 0), (1300, 513, 3, 513, 0),
+    (900, 700, 4, 300, 7), (160, 2047, 2, 33, 0), (70, 1500, 3, 64, 5), (2100, 300, 4, 1025, 0),
+], ids=str)
+def test_cluster_engine_on_tables_by_features(ctx, m, n, bits, batch, parts):
+    """Level tables split by features over the CTAs of a cluster, against the oracle: an epoch in a given order of the batches,
+    then one step with quantized model and gradient."""
+    _, A, b, _ = workload("c4", m, n, seed=bits)
+    levels = oracle.optimal_levels(A, bits, 64)[0] if bits > 1 else np.stack([A.min(0), A.max(0)], 1)
+    ods = oracle.quantize(A, bits, seed=5, mode=oracle.TABLE, levels=levels)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    T, lr = (m + batch - 1) // batch, 1e-3
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=2, grid_row_parts=parts)
+    order = np.random.default_rng(1).permutation(T).astype(np.int32)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, batch_order=order)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, batch_order=order, **how)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_engine() == binding.ENGINE_CLUSTER and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+    kw = dict(seed=5, epoch=1, first_step=T - 1, num_steps=1)
+    x, g, seen = to_dev(x0, ctx), torch.zeros((2, n), device=ctx.device), torch.zeros(n, device=ctx.device)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, model_bits=8, grad_bits=6, grad_out=g, model_out=seen, **how, **kw)
+    ctx.zipml_sync()
+    want, _ = oracle.quantize_vector(x0, 8, 5, 1, T - 1, 3)
+    margin, _ = q3_margins(x0, 8, 5, 1, T - 1)
+    assert not ((seen.cpu().numpy() != want) & (margin >= 1e-4)).any()
+    _, g_ref = oracle.sgd_epoch(ods, b, seen.cpu().numpy(), batch, lr, want_grad=True, **kw)
+    assert rel(g[0].cpu().numpy(), g_ref[0]) <= GRAD_TOL
+    g4, _ = oracle.quantize_vector(g[0].cpu().numpy(), 6, 5, 1, T - 1, 4)
+    assert (g[1].cpu().numpy() != g4).sum() <= 2
+    assert np.allclose(x.cpu().numpy(), x0 - np.float32(lr) * g[1].cpu().numpy(), rtol=1e-6, atol=1e-7)
+
+
 @pytest.mark.parametrize("contraction", [1, 2], ids=["fp32", "int8"])
 @pytest.mark.parametrize("case", SGD_CASES[:5], ids=lambda c: f"{c[0]}-{c[1]}x{c[2]}-b{c[3]}-B{c[4]}")
 def test_cluster_engine_both_contractions(ctx, case, contraction):
@@ -761,7 +797,7 @@ def test_auto_picks_the_engine_that_fits(ctx):
 @pytest.mark.parametrize("m,n,bits,batch,optimal,engine", [
     (130, 4700, 4, 64, False, binding.ENGINE_COLUMN), (9, 2431, 8, 1, False, binding.ENGINE_COLUMN),
     (90, 9403, 2, 40, False, binding.ENGINE_STREAM), (1300, 4700, 4, 1205, False, binding.ENGINE_STREAM),
-    (2600, 3300, 8, 2500, False, binding.ENGINE_RING), (40, 3500, 4, 16, True, binding.ENGINE_PERSISTENT),
+    (2600, 3300, 8, 2500, False, binding.ENGINE_RING), (30, 16_000, 4, 16, True, binding.ENGINE_PERSISTENT),
     (30, 90_003, 8, 16, False, binding.ENGINE_PERSISTENT),
 ], ids=str)
 def test_auto_on_rows_wider_than_a_cluster(ctx, m, n, bits, batch, optimal, engine):
