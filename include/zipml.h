@@ -189,8 +189,9 @@ typedef struct zipml_sgd_params {
                                    (Supplement "Quantizing the Model"), else x as it stood before the step.
                                    ZIPML_ERR_WORKSPACE from the stream and column engines, which keep
                                    no such copy                                                      */
-    int32_t cluster_contraction; /* tuning, cluster engine on uniform grids: 0 = automatic, 1 = fp32,
-                                   2 = int8 tensor cores                                             */
+    int32_t cluster_contraction; /* tuning, cluster engine: 0 = automatic, 1 = fp32, 2 = int8 tensor cores
+                                   (level tables: split by features), 3 = int8 split by rows,
+                                   4 = int8 split by features                                        */
     int32_t stream_prefetch;    /* tuning, stream engine: 0 = automatic, 1..9 = request (value - 1)
                                    eighths of the next step's tile into L2 ahead of time             */
     int32_t column_chunk_rows;  /* tuning, column engine: 0 = automatic, else rows of a minibatch that

@@ -28,7 +28,21 @@ static int grow(unsigned char** buf, size_t* have, size_t want, cudaStream_t str
 int ws_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->ws, &ctx->ws_bytes, bytes, ctx->stream); }
 int stage_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->stage, &ctx->stage_bytes, bytes, ctx->stream); }
 
-int exchange_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->exchange, &ctx->exchange_bytes, bytes, ctx->stream); }
+int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag) {
+    // tags go up from launch to launch, so the buffer is cleared only when it is new (or they would wrap)
+    const bool stale = ctx->exchange_bytes < bytes || ctx->exchange_tag > 0xffffffffu - (uint32_t)steps - 1u;
+    const int rc = grow(&ctx->exchange, &ctx->exchange_bytes, bytes, ctx->stream);
+    if (rc != ZIPML_OK) return rc;
+    if (stale) {
+        const cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, ctx->exchange_bytes, ctx->stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        ctx->exchange_tag = 1;
+    }
+    *buffer = reinterpret_cast<unsigned long long*>(ctx->exchange);
+    *tag = ctx->exchange_tag;
+    ctx->exchange_tag += (uint32_t)steps;
+    return ZIPML_OK;
+}
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
@@ -242,14 +256,11 @@ int zipml_optimal_levels(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, i
 
 // ---- AUTO's rules, measured in us per step: C column, S stream, R ring, K cluster (fp32 form), L lean, G the persistent grid ----
 
-// The engine for rows that no cluster takes (uniform grids, fp32 model and gradient), 0 where the cluster engine is tried first.
-// From 2,400 features (2-bit codes, of which a CTA unpacks the most per byte: 6,000) a hand-over through L2 costs less than a
-// cluster's fp32 work on whole rows: batch 1 n 1,723 K 6.6 C 7.6, n 2,427 K 7.9 C 7.9, n 4,891 K 12.2 C 7.8; 2 bits n 6,939 K 11.4
-// S 10.5.  Lean and ring take 20 to 80 there (4 bits n 6,747 batch 64 L 22.3 R 19.0 C 8.2; 2 bits n 13,499 L 52.9 R 22.2 S 10.8).
+// The engine for rows that no cluster takes (uniform grids, fp32 model and gradient), 0 for other data and quantized vectors.  Lean and ring
+// take 20 to 80 there (4 bits n 6,747 batch 64 L 22.3 R 19.0 C 8.2; 2 bits n 13,499 L 52.9 R 22.2 S 10.8).
 static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, int64_t B) {
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || p->model_bits != 0 || p->grad_bits != 0 || p->model_out) return 0;
     const int cb = container_bits(d->bits);
-    if (d->n < (cb == 2 ? 6000 : 2400)) return 0;
     // Many rows of a few KB: the ring engine streams them.  4 bits 2.4 KB x 3,000 S 31.9 R 34.1, x 6,000 S 57 R 43; 3.3 KB x 6,000
     // S 51 R 49; 4.5 KB x 6,000 S 44 R 50; 2 bits 3.3 KB x 3,000 S 38.5 R 42, x 6,000 S 65 R 59.  8 bits, of which it makes
     // half the work per byte: 3.3 KB x 2,000 S 19.2 R 18.9, x 3,000 S 26.8 R 22.8; 6 KB x 2,000 S 18.9 R 22.7, x 6,000 S 41 R 37.
@@ -268,11 +279,10 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
 }
 
 // Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.
-//   uniform, quantized: 8 bits n 3,355 x 256 L 22 R 27; 4 bits n 4,891 x 256 L 30.5 R 31; n 6,747 x 64 L 32 R 25; 2 bits n 6,939 L 31 R 26.
 //   tables: 2 bits n 4,091 x 64 L 22 G 24, x 256 L 26 G 18; n 2,043 x 1,500 L 43 G 38; 4 bits n 1,019 x 600 L 24 G 28, x 1,500 L 42 G 34;
 //   one row of n 4,091 L 27 G 16; with a quantized vector the grid is no better (4 bits n 1,019 x 1,500 L 51 G 58).
 static bool lean_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B) {
-    if (d->level_mode == ZIPML_LEVELS_UNIFORM) return d->n <= 4096;
+    if (d->level_mode == ZIPML_LEVELS_UNIFORM) return false;
     if (p->model_bits != 0 || p->grad_bits != 0) return true;
     return B * d->n <= 700000 && (d->n < 3000 || B >= 32);
 }
@@ -300,7 +310,7 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (params->epoch < 0 || params->epoch > 0xffffffffLL) return ZIPML_ERR_INVALID_ARG;
     if (params->reg < ZIPML_REG_NONE || params->reg > ZIPML_REG_LSSVM) return ZIPML_ERR_INVALID_ARG;
     if (params->reg != ZIPML_REG_NONE && params->reg != ZIPML_REG_NONNEG && !(params->reg_param >= 0.0f)) return ZIPML_ERR_INVALID_ARG;
-    if (params->cluster_contraction < 0 || params->cluster_contraction > 2) return ZIPML_ERR_INVALID_ARG;
+    if (params->cluster_contraction < 0 || params->cluster_contraction > 4) return ZIPML_ERR_INVALID_ARG;
     if (params->stream_prefetch < 0 || params->stream_prefetch > 9) return ZIPML_ERR_INVALID_ARG;
     if (params->column_chunk_rows < 0 || params->column_chunk_rows > 256 || params->column_chunk_rows % 32 != 0) return ZIPML_ERR_INVALID_ARG;
     if (params->vector_norm != ZIPML_NORM_L2 && params->vector_norm != ZIPML_NORM_LINF) return ZIPML_ERR_INVALID_ARG;
@@ -332,7 +342,7 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (params->engine == ZIPML_ENGINE_SOLO) return launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_AUTO && !linf) {
         // Small minibatch tiles are bound by the step-to-step chain, not by HBM: the smallest stay on one SM, then
-        // clusters whose CTAs exchange through shared memory.  Rows too wide for a cluster go to the column engine
+        // clusters whose CTAs exchange through shared memory.  What no cluster holds goes to the column engine
         // (codes read once per step), the stream engine or the ring engine, whatever the step's size.  Each engine
         // answers ZIPML_ERR_WORKSPACE when the shape does not fit it.
         const int64_t B = params->batch < data->m ? params->batch : data->m;
@@ -343,18 +353,15 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, true);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        if (small && !wide) {
+        if (data->level_mode == ZIPML_LEVELS_UNIFORM && params->cluster_contraction != 1) {
+            rc = launch_sgd_int8(ctx, data, b, x, params, first, count, grad_out);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        } else if (small) {
             rc = launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
-            if (lean_pays(data, params, B)) {
-                rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
-                if (rc != ZIPML_ERR_WORKSPACE) return rc;
-            }
-        } else if (container_bits(data->bits) < 8 || step_bytes <= (48ll << 20)) {
-            // Rows of up to some 3 KB: clusters that hold whole rows, however large the batch (8-bit codes, whose tensor work
-            // per byte is least, up to where the ring engine's 148 CTAs stream faster: 8,192 x 2,000 19.0 / 26.9 us per step,
-            // 16,384 x 2,000 36.9 / 35.2; at 4 bits 16,384 x 3,000 42.7 / 48.2).
-            rc = launch_sgd_slice(ctx, data, b, x, params, first, count, grad_out);
+        }
+        if (small && lean_pays(data, params, B)) {
+            rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
         if (wide == ZIPML_ENGINE_COLUMN) {

@@ -1,5 +1,6 @@
-// Pieces shared by the kernels that run as thread-block clusters (sgd_slice.cu, sgd_table.cu): stores and copies into another CTA's
-// shared memory that complete on its mbarrier, bounded waits, the vector quantizer out of line and norms over the owners.  A kernel's
+// Pieces shared by the kernels that run as thread-block clusters (sgd_slice.cu, sgd_feature.cu, sgd_table.cu): stores and copies into another CTA's
+// shared memory that complete on its mbarrier, bounded waits, the vector quantizer out of line, norms over the owners, fixed point and
+// codes as the int8 contractions take them, and the hand-over of sums between clusters.  A kernel's
 // block of shared memory has a member `gave_up`.
 #pragma once
 
@@ -11,6 +12,7 @@ constexpr int kSliceWarps = 16;
 constexpr int kSliceThreads = 32 * kSliceWarps;   // without the copying warp
 constexpr int kSliceMaxSlots = 8;
 constexpr int kSliceMaxCtas = 16;
+constexpr int kSliceMaxClusters = 8;
 
 __device__ __forceinline__ uint32_t slice_peer(const void* local_smem, uint32_t rank) {
     uint32_t r;
@@ -32,7 +34,9 @@ __device__ __forceinline__ void slice_copy(uint32_t dst, const void* src, uint32
 __device__ __forceinline__ void slice_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The compute warps; and all, the copying warp included.
 __device__ __forceinline__ void slice_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kSliceThreads) : "memory"); }
+__device__ __forceinline__ void slice_bar_all() { asm volatile("bar.sync 3, %0;" ::"n"(kSliceThreads + 32) : "memory"); }
 
 // Sixteen doubles in a fixed order, four chains.
 __device__ __forceinline__ double slice_sum16(const double* v) {
@@ -103,6 +107,55 @@ static __device__ __noinline__ void slice_mark(unsigned long long* trace, int st
 __device__ __forceinline__ void slice_tensor_copy(void* dst_smem, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(smem_u32(dst_smem)), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
+}
+
+// Power of two 2^k by which values up to `top` become integers within the range of four balanced base-256 digits
+// (2^31 - 2^31/128), `spare` bits kept back.  top = 0: 0.
+__device__ __forceinline__ int slice_exponent(float top, int spare) {
+    const int e = (int)(__float_as_uint(top * 1.01f) >> 23) - 127;
+    return min(126, 30 - spare - e);
+}
+__device__ __forceinline__ float slice_pow2(int k) { return k >= -126 ? __uint_as_float((uint32_t)(k + 127) << 23) : 0.0f; }
+// Codes of group g of a fragment register, where they lie in their bytes ...
+template <int CB>
+__device__ __forceinline__ uint32_t slice_codes(uint32_t u, int g) {
+    if constexpr (CB == 8) return u;
+    else return u & ((CB == 4 ? 0x0F0F0F0Fu : 0x03030303u) << (CB * g));
+}
+// ... and, for the dots, at most 4 bits up (2-bit codes: the upper pair is shifted down first).
+template <int CB>
+__device__ __forceinline__ uint32_t slice_dot_codes(uint32_t u, int g) {
+    if constexpr (CB == 2) return slice_codes<2>(g & 2 ? u >> 4 : u, g & 1);
+    else return slice_codes<CB>(u, g);
+}
+template <int CB>
+struct SliceShift {                                       // bits that a group's digits are shifted up by, against the lowest group
+    static constexpr int kMost = CB == 8 ? 0 : CB == 4 ? 4 : 2;
+    __device__ static constexpr int of(int g) { return CB == 8 ? 0 : CB == 4 ? (g == 0 ? 4 : 0) : (g & 1 ? 0 : 2); }
+};
+// D = A B + C with C's two columns given.
+__device__ __forceinline__ void slice_mma_from(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c0, int c1) {
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
+        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c0), "r"(c1));
+}
+
+// A double, as the sum of two floats, handed over through L2: each 8-byte word carries the step's tag and is valid by itself.
+__device__ __forceinline__ void slice_post(unsigned long long* box, float hi, float low, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(box), "l"(t | __float_as_uint(hi)), "l"(t | __float_as_uint(low)) : "memory");
+}
+template <class Shared>
+__device__ __noinline__ double slice_collect(Shared* sh, const unsigned long long* box, uint32_t tag, DeviceStatus* status) {
+    unsigned long long u, v;
+#pragma unroll 1
+    for (long long spin = 0; spin < kBarrierSpinLimit; ++spin) {
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(u), "=l"(v) : "l"(box) : "memory");
+        if ((uint32_t)(u >> 32) == tag && (uint32_t)(v >> 32) == tag) return (double)__uint_as_float((uint32_t)u) + (double)__uint_as_float((uint32_t)v);
+        if ((spin & 255) == 255 && *reinterpret_cast<volatile int*>(&sh->gave_up)) return 0.0;
+    }
+    sh->gave_up = 1;
+    set_status(status, ZIPML_ERR_TIMEOUT, 85);
+    return 0.0;
 }
 
 }  // namespace zipml

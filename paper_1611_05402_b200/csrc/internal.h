@@ -24,7 +24,7 @@ struct zipml_ctx {
     // staging buffers of zipml_train_host (grown on demand)
     unsigned char* stage = nullptr;
     size_t stage_bytes = 0;
-    // words between the clusters of the cluster engine's int8 form, and the next tag (see sgd_slice.cu)
+    // words between the clusters of the cluster engine's int8 forms, and the next tag (see sgd_slice.cu, sgd_feature.cu)
     unsigned char* exchange = nullptr;
     size_t exchange_bytes = 0;
     uint32_t exchange_tag = 1;
@@ -42,7 +42,8 @@ int check_dataset(const zipml_dataset* d);
 int cuda_status(cudaError_t e);                       // ZIPML_OK or ZIPML_ERR_CUDA (clears the sticky error)
 int ws_reserve(zipml_ctx* ctx, size_t bytes);         // grow ctx->ws to at least `bytes`
 int stage_reserve(zipml_ctx* ctx, size_t bytes);
-int exchange_reserve(zipml_ctx* ctx, size_t bytes);
+// At least `bytes` of exchange words between clusters, and the tag of the first of `steps` steps.
+int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag);
 
 // The fp32 constant of zipml_sgd_params' regulariser for step length lr (see regularise() in common.cuh).
 inline float reg_constant(const zipml_sgd_params* p) {
@@ -103,10 +104,14 @@ int launch_sgd_lean(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
 // Solo engine (one thread block).  With only_if_profitable it declines (ZIPML_ERR_WORKSPACE) steps that several SMs take faster.
 int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                     int64_t first_step, int64_t num_steps, float* grad_out, bool only_if_profitable);
-// The cluster engine's int8 form on uniform grids (launch_sgd_cluster calls it).
+// The cluster engine's int8 forms on uniform grids, split by rows or by features, and the one of them that pays.
 int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                      int64_t num_steps, float* grad_out);
-// Its form on level tables.
+int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                       int64_t num_steps, float* grad_out);
+int launch_sgd_int8(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                    int64_t num_steps, float* grad_out);
+// The form on level tables.
 int launch_sgd_table(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                      int64_t num_steps, float* grad_out);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,

@@ -810,7 +810,7 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
     const size_t cap = (size_t)ctx->smem_optin;
     const int64_t nb_max = B < kCluMaxCtas ? B : kCluMaxCtas;
     // the caller may fix the contraction for uniform grids (tests, tuning): 1 = fp32, 2 = int8 tensor cores
-    const int force_int8 = p->cluster_contraction == 1 ? 0 : p->cluster_contraction == 2 ? 1 : -1;
+    const int force_int8 = p->cluster_contraction == 1 ? 0 : p->cluster_contraction >= 2 ? 1 : -1;
     // the requested number of row parts is a hint: more parts are used when a tile does not fit
     for (;; ++nb) {
         if (nb > nb_max) return ZIPML_ERR_WORKSPACE;
@@ -847,14 +847,38 @@ static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
     return B <= (container_bits(d->bits) == 2 ? 240 : 300) * units;
 }
 
+// Uniform grids: split by features, or by rows where the features make too little work for the CTAs, or a batch is so long that it goes
+// through in chunks.  us per step by features / by rows: 8 bits n 250 x 16 2.55 / 2.64, x 256 3.11 / 2.78, n 512 x 64 2.59 / 2.99, x 256 3.11 /
+// 3.10, x 1,024 4.12 / 4.41, n 1,000 x 256 3.15 / 3.56, n 2,000 x 2,048 6.6 / 9.5; 4 bits n 250 x 256 3.19 / 2.92, n 512 x 2,048 5.15 / 5.27, x 4,096
+// 7.06 / 5.99; 2 bits n 256 x 128 3.04 / 2.83, n 1,000 x 64 2.82 / 3.33, x 512 4.05 / 4.58, x 4,096 8.04 / 7.66.
+static bool features_pay(const zipml_dataset* d, const zipml_sgd_params* p) {
+    const int64_t B = p->batch < d->m ? p->batch : d->m;
+    // (from 2^24 entries a step a quantized vector goes to the ring engine, a choice that callers rely on)
+    if ((p->model_bits > 0 || p->grad_bits > 0) && B * d->n >= 1 << 24) return false;
+    return d->n >= (container_bits(d->bits) == 2 ? 900 : 480) && B <= 5 * d->n;
+}
+int launch_sgd_int8(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
+                    int64_t num_steps, float* grad_out) {
+    // (the caller may fix the form by its tuning hint: 3 = by rows, 4 = by features)
+    const bool features = p->cluster_contraction == 4 || (p->cluster_contraction != 3 && features_pay(d, p));
+    int rc = features ? launch_sgd_feature(ctx, d, b, x, p, first_step, num_steps, grad_out) : launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
+    if (rc != ZIPML_ERR_WORKSPACE) return rc;
+    if (features) return launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
+    // (few features, or one of few rows, that the other form does not hold)
+    const int64_t B = p->batch < d->m ? p->batch : d->m;
+    return p->cluster_contraction == 3 || B * d->n >= 1 << 24 ? ZIPML_ERR_WORKSPACE : launch_sgd_feature(ctx, d, b, x, p, first_step, num_steps, grad_out);
+}
+
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
                        int64_t first_step, int64_t num_steps, float* grad_out) {
     const int cb = container_bits(d->bits);
     const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
     const int fpw = 32 / cb;
     const int64_t T = (d->m + p->batch - 1) / p->batch;
-    if (p->cluster_contraction != 1 && (!table || p->cluster_contraction == 2 || table_form_pays(d, p))) {
-        const int rc = table ? launch_sgd_table(ctx, d, b, x, p, first_step, num_steps, grad_out) : launch_sgd_slice(ctx, d, b, x, p, first_step, num_steps, grad_out);
+    if (p->cluster_contraction != 1) {
+        int rc = ZIPML_ERR_WORKSPACE;
+        if (!table) rc = launch_sgd_int8(ctx, d, b, x, p, first_step, num_steps, grad_out);
+        else if (p->cluster_contraction >= 2 || table_form_pays(d, p)) rc = launch_sgd_table(ctx, d, b, x, p, first_step, num_steps, grad_out);
         if (rc != ZIPML_ERR_WORKSPACE) return rc;
     }
     ClusterPlan plan;

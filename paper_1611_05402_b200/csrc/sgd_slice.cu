@@ -40,8 +40,6 @@
 
 namespace zipml {
 
-constexpr int kSliceMaxClusters = 8;
-
 struct SliceArgs {
     const uint8_t* p1;
     const uint8_t* p2;
@@ -90,55 +88,6 @@ struct alignas(16) SliceShared {
     float rmax[16];              // maxima of |residual| of a row block
     int gave_up;
 };
-
-// Power of two 2^k by which values up to `top` become integers within the range of four balanced base-256 digits
-// (2^31 - 2^31/128), `spare` bits kept back.  top = 0: 0.
-__device__ __forceinline__ int slice_exponent(float top, int spare) {
-    const int e = (int)(__float_as_uint(top * 1.01f) >> 23) - 127;
-    return min(126, 30 - spare - e);
-}
-__device__ __forceinline__ float slice_pow2(int k) { return k >= -126 ? __uint_as_float((uint32_t)(k + 127) << 23) : 0.0f; }
-// Codes of group g of a fragment register, where they lie in their bytes ...
-template <int CB>
-__device__ __forceinline__ uint32_t slice_codes(uint32_t u, int g) {
-    if constexpr (CB == 8) return u;
-    else return u & ((CB == 4 ? 0x0F0F0F0Fu : 0x03030303u) << (CB * g));
-}
-// ... and, for the dots, at most 4 bits up (2-bit codes: the upper pair is shifted down first).
-template <int CB>
-__device__ __forceinline__ uint32_t slice_dot_codes(uint32_t u, int g) {
-    if constexpr (CB == 2) return slice_codes<2>(g & 2 ? u >> 4 : u, g & 1);
-    else return slice_codes<CB>(u, g);
-}
-template <int CB>
-struct SliceShift {                                       // bits that a group's digits are shifted up by, against the lowest group
-    static constexpr int kMost = CB == 8 ? 0 : CB == 4 ? 4 : 2;
-    __device__ static constexpr int of(int g) { return CB == 8 ? 0 : CB == 4 ? (g == 0 ? 4 : 0) : (g & 1 ? 0 : 2); }
-};
-// D = A B + C with C's two columns given.
-__device__ __forceinline__ void slice_mma_from(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c0, int c1) {
-    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
-        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(c0), "r"(c1));
-}
-
-
-// A double, as the sum of two floats, handed over through L2: each 8-byte word carries the step's tag and is valid by itself.
-__device__ __forceinline__ void slice_post(unsigned long long* box, float hi, float low, uint32_t tag) {
-    const unsigned long long t = (unsigned long long)tag << 32;
-    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(box), "l"(t | __float_as_uint(hi)), "l"(t | __float_as_uint(low)) : "memory");
-}
-__device__ __noinline__ double slice_collect(SliceShared* sh, const unsigned long long* box, uint32_t tag, DeviceStatus* status) {
-    unsigned long long u, v;
-#pragma unroll 1
-    for (long long spin = 0; spin < kBarrierSpinLimit; ++spin) {
-        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(u), "=l"(v) : "l"(box) : "memory");
-        if ((uint32_t)(u >> 32) == tag && (uint32_t)(v >> 32) == tag) return (double)__uint_as_float((uint32_t)u) + (double)__uint_as_float((uint32_t)v);
-        if ((spin & 255) == 255 && *reinterpret_cast<volatile int*>(&sh->gave_up)) return 0.0;
-    }
-    sh->gave_up = 1;
-    set_status(status, ZIPML_ERR_TIMEOUT, 85);
-    return 0.0;
-}
 
 // Shared memory after SliceShared; SF = 32 sps NG features of a slice:
 //   wd[owners][sps NG 32 + 4]  words: digits of w [slab][group][t][half][digit], then the scale and lo^T x~ (doubles)
@@ -594,6 +543,7 @@ static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const z
     const int cb = container_bits(d->bits), ng = 8 / cb;
     const int64_t B = p->batch < d->m ? p->batch : d->m;
     const int64_t used = (d->n * cb + 7) / 8, slabs = (used + 31) / 32;
+    if (d->n > kSliceMaxCtas * kSliceThreads) return ZIPML_ERR_WORKSPACE;      // (a thread per feature of a slice)
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || (d->m + B - 1) / B > 0x7ffffff0 || slabs > 1024 || d->row_bytes > (1 << 16) || B > (1 << 24)) return ZIPML_ERR_WORKSPACE;
     int64_t clusters = p->grid_feature_parts > 0 ? p->grid_feature_parts : slice_clusters(B, d->n, most_clusters);
     if (clusters > most_clusters) clusters = most_clusters;
@@ -711,19 +661,8 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     a.p_shift = plan.p_shift; a.pitch = plan.pitch; a.slots = plan.slots;
     void* params[] = {&a, &tmaps[0], &tmaps[1]};
     if (plan.clusters > 1) {
-        // tags go up from launch to launch, so the buffer is cleared only when it is new (or they would wrap)
-        const size_t bytes = (size_t)2 * plan.clusters * plan.owners * 32 * plan.sps * (8 / cb) * 16;
-        const bool stale = ctx->exchange_bytes < bytes || ctx->exchange_tag > 0xffffffffu - (uint32_t)num_steps - 1u;
-        rc = exchange_reserve(ctx, bytes);
+        rc = exchange_tags(ctx, (size_t)2 * plan.clusters * plan.owners * 32 * plan.sps * (8 / cb) * 16, num_steps, &a.exchange, &a.tag);
         if (rc != ZIPML_OK) return rc;
-        if (stale) {
-            const cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, ctx->exchange_bytes, ctx->stream);
-            if (e != cudaSuccess) return cuda_status(e);
-            ctx->exchange_tag = 1;
-        }
-        a.exchange = reinterpret_cast<unsigned long long*>(ctx->exchange);
-        a.tag = ctx->exchange_tag;
-        ctx->exchange_tag += (uint32_t)num_steps;
     }
     cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, params);
     if (e != cudaSuccess) return cuda_status(e);

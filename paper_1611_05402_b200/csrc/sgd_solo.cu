@@ -526,19 +526,19 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
     return ZIPML_OK;
 }
 
-// Whether AUTO takes this engine: by what a step has one SM get through, batch x (features + 8).  Measured, us per step
-// here / cluster engine, on both sides of the lines: 4 bits 256 x 64 3.3 / 4.2, 64 x 250 3.2 / 4.0, 800 x 23 5.2 / 5.0, 1,024 x 17
-// 5.8 / 5.0, 37 x 512 4.5 / 4.3; 2 bits 64 x 250 3.2 / 4.2, 37 x 333 4.6 / 4.0, 16 x 2,048 5.9 / 5.2; 8 bits 300 x 30 3.0 / 4.2, 512
-// x 23 4.0 / 4.5, 64 x 250 4.4 / 3.9, 16 x 1,000 3.7 / 3.9, 16 x 2,000 5.8 / 5.2; tables (3 bits) 256 x 23 3.8 / 4.3, 128 x 64 4.0 / 3.9,
-// 37 x 250 4.3 / 4.0, 16 x 1,999 7.4 / 8.6.  A quantized model or gradient costs the others an exchange more each: 8 bits 256
-// x 64 5.9 / 6.4, 4 bits 500 x 61 7.5 / 7.7, 37 x 512 7.3 / 7.2.
+// Whether AUTO takes this engine: by what a step has one SM get through, batch x (features + 8).  Measured, us per step here / cluster
+// engine, on both sides of the lines: 8 bits 512 x 16 1.94 / 2.28, 64 x 128 2.0 / 2.4, 333 x 32 3.9 / 2.6, 700 x 16 3.1 / 2.3; 4 bits 64 x 128
+// 1.9 / 2.4, 333 x 32 2.6 / 2.6, 200 x 64 2.7 / 2.5; 2 bits 333 x 32 2.5 / 2.6, 120 x 128 2.8 / 2.6; tables (3 bits) 120 x 16 1.6 / 2.0, 250
+// x 16 2.1 / 2.0, (2 bits) 64 x 64 2.3 / 2.6, 400 x 16 2.8 / 2.2.  A quantized model or gradient costs the others an exchange more each: 8 bits
+// 512 x 32 4.8 / 5.1, 333 x 64 7.7 / 5.5, 4 bits 64 x 256 4.4 / 5.0, 333 x 64 6.5 / 5.5, 700 x 16 5.8 / 5.2, tables 250 x 16 4.0 / 5.0, 250 x 64
+// 7.2 / 5.2.
 static bool solo_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
-    const int64_t B = p->batch < d->m ? p->batch : d->m;
-    const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
-    if (table && B <= 16) return true;
-    int64_t limit = table ? 7500 : container_bits(d->bits) == 4 || B <= 16 ? 18500 : 14000;
-    if (p->model_bits > 0 || p->grad_bits > 0) limit = limit * 5 / 4;
-    return (table || d->n <= 1024) && B * (d->n + 8) <= limit;
+    const int64_t B = p->batch < d->m ? p->batch : d->m, work = B * (d->n + 8);
+    const int cb = container_bits(d->bits);
+    const bool quantized = p->model_bits > 0 || p->grad_bits > 0;
+    if (d->level_mode == ZIPML_LEVELS_TABLE) return work <= (quantized ? 8000 : cb == 2 ? 5000 : 4000);
+    if (quantized) return d->n <= 640 && work <= (cb == 8 ? 17000 : 18500);
+    return d->n <= 1024 && work <= (cb == 8 ? 9500 : 11000);
 }
 
 int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
