@@ -3,6 +3,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "cluster.cuh"
 #include "int_digits.cuh"
 #include "internal.h"
 
@@ -205,77 +206,89 @@ __global__ void __launch_bounds__(1024) loss_codes_table_kernel(const uint32_t* 
 // ---------------------------------------------------------------------------------------------
 // The same estimate for uniform grids on the int8 tensor cores: a pure streaming pass (no step-to-step
 // dependency), so it shows what the unpack-and-dot arithmetic of the SGD step reaches against HBM.
-// w = step * x becomes four balanced base-128 int8 digits per entry (one rounding, 2^-27 of the
+// w = step * x becomes four balanced base-256 int8 digits per entry (one rounding, 2^-27 of the
 // largest |w|); a warp takes 16 rows, its lanes load 16 bytes of codes per row and 64-byte span
 // straight from global memory (rows g and g+8 of lane group g; four lanes cover the span), and every
 // 8 bytes of a lane's 16 are one mma.sync m16n8k32 (u8 x s8) against the matching 8 bytes of each
 // digit's vector (digits in the byte order of the codes, so the operand's k order is simply the
-// lane's own byte order).  Digit sums are exact (32-bit sums moved into 64 bits before they can
-// wrap, whatever the row length); they are combined in double.
+// lane's own byte order).  Codes of less than 8 bits are masked where they lie in their byte, 2-bit
+// ones after one shift: the shifts are in the digits.  Digit sums are exact (32-bit sums moved into 64 bits
+// before they can wrap, whatever the row length); they are combined in double.
+// Few rows: kp warps of a block share 16 rows, a part of the spans each, and add their sums up.  The last block
+// adds the blocks' partial sums up in order.
 // ---------------------------------------------------------------------------------------------
-// Digit vectors of w: wdig[group][digit][byte of the row], row_bytes rounded up to 64 per vector.
+// Digit vectors of w: wdig[group][digit][byte of the row], row_bytes rounded up to 64 per vector.  Every block finds the largest |w|.
 template <int CB>
 __global__ void __launch_bounds__(1024) loss_digits_kernel(const float* __restrict__ lo, const float* __restrict__ step,
                                                            const float* __restrict__ x, int64_t n, int64_t vec_bytes,
-                                                           signed char* __restrict__ wdig, double* __restrict__ base_out) {
+                                                           signed char* __restrict__ wdig, double* __restrict__ base_out, unsigned* __restrict__ ticket) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS, FPW = 32 / CB;
     __shared__ double red[40];
     __shared__ float smax[32];
     double base = 0.0;
     float wm = 0.0f;
+#pragma unroll 4
     for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
         const float xv = x[j];
         wm = fmaxf(wm, fabsf(step[j] * xv));
-        base += (double)lo[j] * (double)xv;
+        if (blockIdx.x == 0) base += (double)lo[j] * (double)xv;
     }
     for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
     if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = wm;
     base = block_sum(base, red);                  // its barriers also publish smax
     float wmax = 0.0f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) wmax = fmaxf(wmax, smax[w]);
-    const float inv = wmax > 0.0f ? (float)IntPath<CB>::QMAX / wmax : 0.0f;
-    if (threadIdx.x == 0) { base_out[0] = base; base_out[1] = (double)wmax / (double)IntPath<CB>::QMAX; }
+    const float inv = wmax > 0.0f ? (float)IntPath<CB>::QMAX / wmax : 0.0f;          // (16 QMAX is within four balanced base-256 digits)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        base_out[0] = base;
+        base_out[1] = (double)wmax / ((double)IntPath<CB>::QMAX * (1 << SliceShift<CB>::kMost));
+        *ticket = 0u;
+    }
     // feature j sits in byte (j / FPW) * 4 + (j % FPW) / NG of the row, code group (j % FPW) % NG
-    for (int64_t idx = threadIdx.x; idx < vec_bytes * NG; idx += blockDim.x) {
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < vec_bytes * NG; idx += (int64_t)gridDim.x * blockDim.x) {
         const int64_t byte = idx / NG;
         const int g = (int)(idx - byte * NG);
         const int64_t j = (byte >> 2) * FPW + (byte & 3) * NG + g;
-        int d[NS];
-        balanced_digits<NS>(j < n ? __float2int_rn(step[j] * x[j] * inv) : 0, d);
+        const int whole = j < n ? __float2int_rn(step[j] * x[j] * inv) : 0;
+        const uint32_t d = ((uint32_t)(whole * (1 << SliceShift<CB>::of(g))) + 0x80808080u) ^ 0x80808080u;
 #pragma unroll
-        for (int s = 0; s < NS; ++s) wdig[((int64_t)g * NS + s) * vec_bytes + byte] = (signed char)d[s];
+        for (int s = 0; s < NS; ++s) wdig[((int64_t)g * NS + s) * vec_bytes + byte] = (signed char)(d >> (8 * s));
     }
 }
 
-constexpr int64_t kLossFlushSpans = 1024;
+constexpr int64_t kLossFlushSpans = 512;
 
 template <int CB>
 __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned char* __restrict__ p1, const unsigned char* __restrict__ p2,
-                                                              int64_t row_bytes, int64_t m, int64_t vec_bytes,
+                                                              int64_t row_bytes, int64_t m, int64_t vec_bytes, int kp_shift,
                                                               const signed char* __restrict__ wdig, const double* __restrict__ base_in,
-                                                              const float* __restrict__ b, double* __restrict__ partials) {
+                                                              const float* __restrict__ b, double* __restrict__ partials, unsigned* __restrict__ ticket,
+                                                              double scale, double* __restrict__ out) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
     __shared__ double red[40];
-    const int lane = threadIdx.x & 31, gl = lane >> 2, tl = lane & 3;
-    const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    __shared__ double parts[16][32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, gl = lane >> 2, tl = lane & 3, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int kp = 1 << kp_shift, part = warp & (kp - 1);
+    const int64_t first = (int64_t)blockIdx.x * (warps >> kp_shift) + (warp >> kp_shift), more = (int64_t)gridDim.x * (warps >> kp_shift);
     const double base = base_in[0], delta = base_in[1];
     const int64_t nblocks = (m + 15) / 16;
     const int64_t nspans = (row_bytes + 63) / 64;
+    const int64_t span0 = (nspans * part) >> kp_shift, span1 = (nspans * (part + 1)) >> kp_shift;
     double total = 0.0;
-    for (int64_t blk = warp_global; blk < nblocks; blk += nwarps) {
+    for (int64_t blk = first; blk < nblocks || kp > 1; blk += more) {      // (shared rows: one turn, for all warps)
         const int64_t ra = min(blk * 16 + gl, m - 1), rh = min(blk * 16 + gl + 8, m - 1);
         const unsigned char* a1 = p1 + ra * row_bytes + 16 * tl;
         const unsigned char* h1 = p1 + rh * row_bytes + 16 * tl;
         const unsigned char* a2 = p2 + ra * row_bytes + 16 * tl;
         const unsigned char* h2 = p2 + rh * row_bytes + 16 * tl;
-        // A span adds at most 2 * 32 * 255 * 64 to a 32-bit digit sum: they are moved into 64-bit sums every
-        // kLossFlushSpans spans (2^20 * 1024 < 2^31), so rows of any admitted length stay exact.
+        // A span adds at most 64 * 128 * 255 to a 32-bit digit sum: they are moved into 64-bit sums every
+        // kLossFlushSpans spans (2^21 * 512 < 2^31), so rows of any admitted length stay exact.
         long long s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0};
-        for (int64_t sp0 = 0; sp0 < nspans; sp0 += kLossFlushSpans) {
+        for (int64_t sp0 = span0; sp0 < span1; sp0 += kLossFlushSpans) {
         int c1[4] = {0, 0, 0, 0}, c2[4] = {0, 0, 0, 0};
-        const int64_t sp1 = min(nspans, sp0 + kLossFlushSpans);
-#pragma unroll 2
+        const int64_t sp1 = min(span1, sp0 + kLossFlushSpans);
+#pragma unroll 4
         for (int64_t sp = sp0; sp < sp1; ++sp) {
             const int64_t off = sp * 64;
             uint4 ua = make_uint4(0u, 0u, 0u, 0u), uh = ua, va = ua, vh = ua;
@@ -289,10 +302,10 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
             for (int g = 0; g < NG; ++g) {
                 uint4 bd = make_uint4(0u, 0u, 0u, 0u);            // digit gl of this lane's 16 bytes
                 if (gl < NS) bd = __ldg(reinterpret_cast<const uint4*>(wdig + ((int64_t)g * NS + gl) * vec_bytes + off + 16 * tl));
-                mma_u8s8(c1, group_bytes<CB>(ua.x, g), group_bytes<CB>(uh.x, g), group_bytes<CB>(ua.y, g), group_bytes<CB>(uh.y, g), bd.x, bd.y);
-                mma_u8s8(c1, group_bytes<CB>(ua.z, g), group_bytes<CB>(uh.z, g), group_bytes<CB>(ua.w, g), group_bytes<CB>(uh.w, g), bd.z, bd.w);
-                mma_u8s8(c2, group_bytes<CB>(va.x, g), group_bytes<CB>(vh.x, g), group_bytes<CB>(va.y, g), group_bytes<CB>(vh.y, g), bd.x, bd.y);
-                mma_u8s8(c2, group_bytes<CB>(va.z, g), group_bytes<CB>(vh.z, g), group_bytes<CB>(va.w, g), group_bytes<CB>(vh.w, g), bd.z, bd.w);
+                mma_u8s8(c1, slice_dot_codes<CB>(ua.x, g), slice_dot_codes<CB>(uh.x, g), slice_dot_codes<CB>(ua.y, g), slice_dot_codes<CB>(uh.y, g), bd.x, bd.y);
+                mma_u8s8(c1, slice_dot_codes<CB>(ua.z, g), slice_dot_codes<CB>(uh.z, g), slice_dot_codes<CB>(ua.w, g), slice_dot_codes<CB>(uh.w, g), bd.z, bd.w);
+                mma_u8s8(c2, slice_dot_codes<CB>(va.x, g), slice_dot_codes<CB>(vh.x, g), slice_dot_codes<CB>(va.y, g), slice_dot_codes<CB>(vh.y, g), bd.x, bd.y);
+                mma_u8s8(c2, slice_dot_codes<CB>(va.z, g), slice_dot_codes<CB>(vh.z, g), slice_dot_codes<CB>(va.w, g), slice_dot_codes<CB>(vh.w, g), bd.z, bd.w);
             }
         }
 #pragma unroll
@@ -302,12 +315,21 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
         double v[4];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const double q1 = (double)s1[2 * e] + 128.0 * (double)s1[2 * e + 1];
-            const double q2 = (double)s2[2 * e] + 128.0 * (double)s2[2 * e + 1];
-            v[2 * e] = q1 + 16384.0 * __shfl_down_sync(0xffffffffu, q1, 1);
-            v[2 * e + 1] = q2 + 16384.0 * __shfl_down_sync(0xffffffffu, q2, 1);
+            const double q1 = (double)(s1[2 * e] + 256 * s1[2 * e + 1]);
+            const double q2 = (double)(s2[2 * e] + 256 * s2[2 * e + 1]);
+            v[2 * e] = q1 + 65536.0 * __shfl_down_sync(0xffffffffu, q1, 1);
+            v[2 * e + 1] = q2 + 65536.0 * __shfl_down_sync(0xffffffffu, q2, 1);
         }
-        if (tl == 0) {
+        if (kp > 1) {
+            if (tl == 0)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) parts[warp][gl * 4 + e] = v[e];
+            __syncthreads();
+            for (int w = 1; w < kp; ++w)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] += part == 0 && tl == 0 ? parts[warp + w][gl * 4 + e] : 0.0;
+        }
+        if (tl == 0 && part == 0) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int64_t k = blk * 16 + gl + 8 * e;
@@ -317,9 +339,21 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
                 }
             }
         }
+        if (kp > 1) break;
     }
     total = block_sum(total, red);
-    if (threadIdx.x == 0) partials[blockIdx.x] = total;
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = total;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    total = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) total += *(volatile double*)(partials + i);
+    total = block_sum(total, red);
+    if (threadIdx.x == 0) *out = total * scale;
 }
 
 __global__ void loss_finish_kernel(const double* __restrict__ partials, int count, double scale, double* out) {
@@ -335,24 +369,36 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
     const int cb = container_bits(d->bits);
     const bool table = d->level_mode == ZIPML_LEVELS_TABLE;
     const int L = 1 << d->bits;
-    // scratch behind the partials: base and the fixed-point unit (2 doubles), then the w table or digit vectors
+    // scratch behind the partials: base and the fixed-point unit (2 doubles), then the w table or digit vectors and a counter
     double* base = partials + max_partials;
     float* wtab = reinterpret_cast<float*>(base + 2);
     if (!table) {
         // digit vectors take (8 / cb) * 4 * roundup64(row_bytes) bytes (the caller reserved them from the stride)
         const int64_t vec_bytes = (d->row_bytes + 63) / 64 * 64;
         signed char* wdig = reinterpret_cast<signed char*>(wtab);
-        int blocks = ctx->sm_count * 2;                            // 2 x 16 warps per SM, 16 rows per warp and turn
-        if (blocks > max_partials) blocks = max_partials;
-        const int64_t need = ((d->m + 15) / 16 + 15) / 16;
-        if (blocks > need) blocks = (int)need;
+        unsigned* ticket = reinterpret_cast<unsigned*>(wdig + (8 / cb) * 4 * vec_bytes);
+        // 16 warps per SM, 16 rows per warp and turn (four spans in flight take 128 registers a thread); with fewer rows smaller
+        // blocks, so that every SM has some, and where there are not rows for two warps of all schedulers several to 16 rows.
+        // Measured, us: 2 bits 1,000,000 x 2,048 253 with shifted codes and two spans -> 225 (4.7 TB/s, bound by the masks and
+        // products), 4 bits 1,000,000 x 1,000 270 -> 185 (5.5 TB/s), 8 bits 300,000 x 2,000 264 -> 257; few rows: 4 bits 3,997 x 6,576
+        // 99 -> 29, 245 x 2,710 42 -> 26, 2 bits 8,000 x 32,000 176 -> 63.
+        const int64_t turns = (d->m + 15) / 16, spans = vec_bytes / 64;
+        int warps = (int)(turns / ctx->sm_count), kp = 1, kp_shift = 0;
+        warps = warps > 16 ? 16 : warps < 1 ? 1 : warps;
+        while (kp < 16 && turns * kp < 8ll * ctx->sm_count && 2 * kp <= spans) { kp *= 2; ++kp_shift; }
+        if (kp > 1) warps = kp;
+        int64_t blocks = kp > 1 ? turns : (turns + warps - 1) / warps;
+        if (kp == 1 && blocks > ctx->sm_count) blocks = ctx->sm_count;
+        if (blocks > max_partials) return ZIPML_ERR_WORKSPACE;
+        const int64_t chunks = (vec_bytes * (8 / cb) + 1023) / 1024;
+        const int digit_blocks = (int)(chunks > 16 ? 16 : chunks);
+        const double scale = 1.0 / (2.0 * (double)d->m);
 #define ZIPML_LAUNCH_LI(CB_) \
-    loss_digits_kernel<CB_><<<1, 1024, 0, ctx->stream>>>(d->feat_lo, d->feat_step, x, d->n, vec_bytes, wdig, base); \
-    loss_codes_imma_kernel<CB_><<<blocks, 512, 0, ctx->stream>>>(d->plane1, d->plane2, d->row_bytes, d->m, vec_bytes, wdig, base, b, partials)
+    loss_digits_kernel<CB_><<<digit_blocks, 1024, 0, ctx->stream>>>(d->feat_lo, d->feat_step, x, d->n, vec_bytes, wdig, base, ticket); \
+    loss_codes_imma_kernel<CB_><<<(int)blocks, 32 * warps, 0, ctx->stream>>>(d->plane1, d->plane2, d->row_bytes, d->m, vec_bytes, kp_shift, wdig, base, b, partials, ticket, scale, loss_out)
         if (cb == 2) { ZIPML_LAUNCH_LI(2); } else if (cb == 4) { ZIPML_LAUNCH_LI(4); } else { ZIPML_LAUNCH_LI(8); }
 #undef ZIPML_LAUNCH_LI
-        loss_finish_kernel<<<1, 256, 0, ctx->stream>>>(partials, blocks, 1.0 / (2.0 * (double)d->m), loss_out);
-        ctx->launches += 3;
+        ctx->launches += 2;
         return cuda_status(cudaGetLastError());
     }
     if (table) {

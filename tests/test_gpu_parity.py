@@ -899,6 +899,18 @@ def test_loss_parity(ctx, key, m, n, bits):
     assert abs(got_c.item() - want_c) <= LOSS_TOL * max(abs(want_c), abs(want))
 
 
+@pytest.mark.parametrize("m,n,bits", [(1, 5, 8), (17, 700, 2), (50, 6577, 4), (2600, 130, 8), (2400, 65, 4), (20_000, 40, 2)], ids=str)
+def test_loss_codes_with_few_and_many_rows(ctx, m, n, bits):
+    """Several warps to 16 rows, a part of the spans each; blocks of fewer warps; several turns of a block."""
+    _, A, b, xs = workload("c2", m, n, seed=2)
+    x = (xs * 0.9).astype(np.float32)
+    ods = oracle.quantize(A, bits, seed=3)
+    want = oracle.loss_codes(ods, b, x)
+    got = ctx.zipml_loss(binding.LOSS_CODES, to_dev(b, ctx), to_dev(x, ctx), data=dev_dataset(ods, ctx))
+    ctx.zipml_sync()
+    assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
+
+
 def test_loss_codes_with_level_table_and_strided_dense(ctx):
     _, A, b, xs = workload("c4", 2000, 60, seed=1)
     lev, _ = oracle.optimal_levels(A, 3, 128)
