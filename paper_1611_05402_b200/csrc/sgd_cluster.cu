@@ -1,4 +1,5 @@
-// Cluster engine of zipml_sgd_epoch: one persistent launch of a single thread-block cluster, built
+// Cluster engine of zipml_sgd_epoch, split by rows and in fp32 (level tables with few features and long batches, and what its other
+// forms do not hold; sgd_feature.cu, sgd_slice.cu and sgd_table.cu have those): one persistent launch of a single thread-block cluster, built
 // for steps whose code tile is small (Supplement "Double Sampling", footnote form; "End-to-end
 // Quantization").
 //
@@ -35,7 +36,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include "int_digits.cuh"
 #include "sgd_common.cuh"
 
 namespace zipml {
@@ -43,7 +43,6 @@ namespace zipml {
 constexpr int kCluThreads = 512;
 constexpr int kCluWarps = kCluThreads / 32;
 constexpr int kCluMaxSlots = 8;
-constexpr int kCluCols = 4;                       // integer phase B: 16-byte tile columns per warp (half of it for 2-bit codes)
 constexpr int kCluMaxCtas = 16;                   // one bulk copy per warp and destination: at most kCluWarps CTAs
 static_assert(kCluMaxCtas <= kCluWarps, "a warp per destination CTA");
 
@@ -67,7 +66,6 @@ struct ClusterArgs {
     int reg;                     // ZIPML_REG_* and its fp32 constant
     float reg_cst;
     int n, bits, row_words, words;   // words = ceil(n / codes per word) <= row_words
-    int pitch;                       // words between consecutive rows of a tile in shared memory (>= row_words)
     int model_bits, grad_bits;
     int nb, rc, slots;
     int sub;                     // a CTA owns `sub` consecutive features (a multiple of 4)
@@ -79,8 +77,6 @@ struct ClusterShared {
     double red[kCluWarps];       // block sums
     double wbase[kCluWarps];     // per-warp parts of lo^T x~
     double ssum[kCluWarps];      // per-warp sums of the residuals
-    float fmax[kCluWarps];       // per-warp maxima (|w| of the word stage, then |residual|)
-    uint4 zero16;                // sixteen zero bytes: the unused columns of the digit operands point here
     double nrm_g[kCluMaxCtas];   // partial squared gradient norms, one per CTA
     double nrm_x[kCluMaxCtas];   // partial squared model norms
     unsigned long long full[kCluMaxSlots];
@@ -172,11 +168,10 @@ __device__ __forceinline__ void clu_mark(const ClusterArgs& a, int64_t it, int i
 //   gbuf[nb][sub]    the nb parts of the owned features (reduce-scatter destination)
 //   xpub[sub], xown[sub], gsub[sub]   staging of the published slice, master model, gradient of the step
 //   res[2*rc]        residuals (r1, r2) per row;   bsm[rc]  labels of the step's rows
-//   gred[256*FPW]    cross-group sums of phase B (parts narrower than the CTA)
+//   gred[512*FPW]    cross-group sums of phase B (parts narrower than the CTA)
 //   ring[slots][2][rc][row_words]  code tiles
-template <int CB, bool TABLE, bool IMMA>
+template <int CB, bool TABLE>
 __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const ClusterArgs a) {
-    static_assert(!(TABLE && IMMA), "level tables use the fp32 look-up path");
     constexpr int FPW = 32 / CB;
     constexpr int LOGF = (CB == 8) ? 2 : (CB == 4) ? 3 : 4;
     extern __shared__ __align__(16) unsigned char s_raw[];
@@ -192,16 +187,9 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
     float* los = tab + Fp;
     float* steps = los + Fp;
     float* lev = tab + (size_t)L * Fp;                   // table
-    constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
-    constexpr float QMAXF = (float)IntPath<CB>::QMAX;
-    const int pitch = a.pitch;
-    const int nks = (nw + 7) >> 3;                       // k-slabs of 8 words (32 bytes of codes)
-    const int ncol = (nw + 3) >> 2;                      // 16-byte columns of the tile
-    uint32_t* wdig = reinterpret_cast<uint32_t*>(steps + Fp);            // [k-slab][group][digit][8 words]
-    unsigned char* rdig = reinterpret_cast<unsigned char*>(wdig + (size_t)((rw + 7) >> 3) * NG * NS * 8);   // [32 rows][r1, r2][digit][32 B]
-    int* dacc = reinterpret_cast<int*>(rdig + (size_t)((a.rc + 31) / 32) * 256);                        // [row][plane][digit]
-    float* gred = TABLE ? lev + (size_t)L * Fp : steps + Fp;             // fp32 paths
-    float* xs = IMMA ? reinterpret_cast<float*>(dacc + ((a.rc + 15) & ~15) * 8) : gred + kCluThreads * FPW;
+    float* gred = TABLE ? lev + (size_t)L * Fp : steps + Fp;
+    const int lanes_q = min(kCluThreads, ((nw + 31) / 32) * 32), ngroups = kCluThreads / lanes_q;
+    float* xs = gred + (ngroups > 1 ? kCluThreads * FPW : 0);
     float* gpart = xs + Fs;
     float* gbuf = gpart + Fs;
     float* xpub = gbuf + Fs;
@@ -211,7 +199,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
     float* bsm = res + ((2 * a.rc + 3) & ~3);
     uint32_t* ring = reinterpret_cast<uint32_t*>(
         (reinterpret_cast<uintptr_t>(bsm + ((a.rc + 3) & ~3)) + 127) & ~(uintptr_t)127);
-    const size_t slot_words = (size_t)2 * a.rc * pitch;
+    const size_t slot_words = (size_t)2 * a.rc * rw;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bi = blockIdx.x;                           // the grid is one cluster: block index = rank
@@ -224,8 +212,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         bt = (int)min(a.batch, a.m - r0);
         rcnt = max(0, min(a.rc, bt - k0));
     };
-    // the tile of step `it` into `slot`, issued by one whole warp: one contiguous piece per plane, or, when the
-    // rows are padded apart in shared memory, one piece per row (the lanes share them)
+    // the tile of step `it` into `slot`, issued by one whole warp: one contiguous piece per plane
     auto issue_tile = [&](int64_t it, int slot) {
         int64_t r0; int bt, rcnt;
         step_rows(it, r0, bt, rcnt);
@@ -235,30 +222,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         __syncwarp();
         uint32_t* dst = ring + (size_t)slot * slot_words;
         const size_t src = (size_t)(r0 + k0) * rw;
-        if (pitch == rw) {
-            if (lane < 2 && rcnt > 0) bulk_copy_g2s(dst + (size_t)lane * a.rc * pitch, (lane ? a.p2 : a.p1) + src, bytes, full);
-        } else {
-            for (int i = lane; i < 2 * rcnt; i += 32) {
-                const int pl = i & 1, r = i >> 1;
-                bulk_copy_g2s(dst + (size_t)(pl * a.rc + r) * pitch, (pl ? a.p2 : a.p1) + src + (size_t)r * rw, (uint32_t)rw * 4u, full);
-            }
-        }
-    };
-
-    // the same for padded rows, called by every warp: lane 0 of warp w issues pieces w, w + 16, ...
-    auto issue_tile_rows = [&](int64_t it, int slot) {
-        int64_t r0; int bt, rcnt;
-        step_rows(it, r0, bt, rcnt);
-        uint64_t* full = reinterpret_cast<uint64_t*>(sh->full + slot);
-        if (lane != 0) return;
-        // (bytes that land before the count is armed are held against it: the phase cannot complete earlier)
-        if (warp == kCluWarps - 1) mbar_arrive_expect_tx(full, 2u * (uint32_t)rcnt * (uint32_t)rw * 4u);
-        uint32_t* dst = ring + (size_t)slot * slot_words;
-        const size_t src = (size_t)(r0 + k0) * rw;
-        for (int i = warp; i < 2 * rcnt; i += kCluWarps) {
-            const int pl = i & 1, r = i >> 1;
-            bulk_copy_g2s(dst + (size_t)(pl * a.rc + r) * pitch, (pl ? a.p2 : a.p1) + src + (size_t)r * rw, (uint32_t)rw * 4u, full);
-        }
+        if (lane < 2 && rcnt > 0) bulk_copy_g2s(dst + (size_t)lane * a.rc * rw, (lane ? a.p2 : a.p1) + src, bytes, full);
     };
 
     if (tid == 0) {
@@ -268,7 +232,6 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         mbar_init(reinterpret_cast<uint64_t*>(&sh->gn_bar), 1);
         mbar_init(reinterpret_cast<uint64_t*>(&sh->xn_bar), 1);
         sh->abort_flag = 0;
-        sh->zero16 = make_uint4(0u, 0u, 0u, 0u);
         mbar_fence_init();
     }
     for (int f = tid; f < Fp; f += kCluThreads) {
@@ -281,8 +244,6 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         }
     }
     for (int f = tid; f < Fs; f += kCluThreads) gpart[f] = 0.0f;       // features past n stay zero
-    if constexpr (IMMA)
-        for (int i = tid; i < ((a.rc + 15) & ~15) * 8; i += kCluThreads) dacc[i] = 0;
     for (int k = tid; k < sub; k += kCluThreads) xown[k] = (bi * sub + k < n) ? a.x[bi * sub + k] : 0.0f;
     __syncthreads();
     if (warp == 0)
@@ -293,11 +254,8 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
     const int P = 1 << a.p_shift;
     const int pp = tid & (P - 1);
     const int kpt = kCluThreads >> a.p_shift;                      // owned features handled per pass
-    const int lanes_q = min(kCluThreads, ((nw + 31) / 32) * 32);
-    const int ngroups = kCluThreads / lanes_q;
     const int group = tid / lanes_q, ql = tid - group * lanes_q;
     const uint32_t slice_bytes = (uint32_t)sub * 4u;
-    double delta_w = 0.0;                                          // one fixed-point unit of w, renewed with the model
 
     int slot = 0;                                                  // slot and mbarrier parity of the current step's tile
     uint32_t parity = 0;
@@ -318,290 +276,120 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
             clu_mark(a, it, 0);
             clu_wait(sh->full + slot, parity, sh, a.status, 6);
             const uint32_t* t1 = ring + (size_t)slot * slot_words;
-            const uint32_t* t2 = t1 + (size_t)a.rc * pitch;
+            const uint32_t* t2 = t1 + (size_t)a.rc * rw;
             clu_mark(a, it, 1);
 
-            if constexpr (IMMA) {
-                // ------------------------------------------------------ phase A: digit sums of the dots
-                // A k-slab is 8 words (32 bytes of codes) of a row; a warp takes every kCluWarps-th slab for
-                // each block of 16 rows and both planes: the code bytes come as A fragments straight from the
-                // tile (ldmatrix), each code group of the bytes meets its own digit vectors of w (B
-                // fragments), all in the same accumulators.  The warps' sums meet in dacc (integer sums: the
-                // order of the atomics does not matter).  Rows past the CTA's last one are read (clamped to
-                // the tile) and dropped; bytes past the row's last code meet zero digits.
-                const int gl = lane >> 2, tl = lane & 3, lm = lane >> 3, l8 = lane & 7;
-                const uint32_t wdig_addr = smem_u32(wdig), rdig_addr = smem_u32(rdig), zero_addr = smem_u32(&sh->zero16);
-                const uint32_t tile_addr = smem_u32(t1);
-                const uint32_t plane_bytes = (uint32_t)a.rc * (uint32_t)pitch * 4u;
-                const int nrb = (rcnt + 15) >> 4;
-#pragma unroll 1
-                for (int rb0 = 0; rb0 < nrb && warp < nks; rb0 += 4) {     // four blocks of 16 rows per pass
-                    int c[2][4][4];                                // [plane][row block][fragment]
-#pragma unroll
-                    for (int pl = 0; pl < 2; ++pl)
-#pragma unroll
-                        for (int rb = 0; rb < 4; ++rb)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) c[pl][rb][e] = 0;
-#pragma unroll 1
-                    for (int ks = warp; ks < nks; ks += kCluWarps) {
-                        uint32_t bf[NG][2];
-#pragma unroll
-                        for (int g = 0; g < NG; ++g)
-                            ldsm_x2(bf[g][0], bf[g][1],
-                                    l8 < NS ? wdig_addr + (uint32_t)(((ks * NG + g) * NS + l8) * 32 + (lm & 1) * 16) : zero_addr);
-#pragma unroll
-                        for (int rb = 0; rb < 4; ++rb) {
-                            if (rb0 + rb < nrb) {
-                                const uint32_t row = (uint32_t)min((rb0 + rb) * 16 + l8 + (lm & 1) * 8, a.rc - 1);
-                                const uint32_t addr = tile_addr + row * (uint32_t)pitch * 4u + (uint32_t)ks * 32u + (lm >> 1) * 16u;
-                                uint32_t a1[4], a2[4];
-                                ldsm_x4(a1, addr);
-                                ldsm_x4(a2, addr + plane_bytes);
-#pragma unroll
-                                for (int g = 0; g < NG; ++g) {
-                                    mma_u8s8(c[0][rb], group_bytes<CB>(a1[0], g), group_bytes<CB>(a1[1], g), group_bytes<CB>(a1[2], g),
-                                             group_bytes<CB>(a1[3], g), bf[g][0], bf[g][1]);
-                                    mma_u8s8(c[1][rb], group_bytes<CB>(a2[0], g), group_bytes<CB>(a2[1], g), group_bytes<CB>(a2[2], g),
-                                             group_bytes<CB>(a2[3], g), bf[g][0], bf[g][1]);
-                                }
-                            }
-                        }
-                    }
-                    if (tl < 2) {                                  // columns 2t, 2t+1 are digits; dacc is [row][plane][digit]
-#pragma unroll
-                        for (int rb = 0; rb < 4; ++rb) {
-                            if (rb0 + rb < nrb) {
-                                int* d = dacc + ((rb0 + rb) * 16 + gl) * 8 + 2 * tl;
-#pragma unroll
-                                for (int pl = 0; pl < 2; ++pl) {
-                                    atomicAdd(d + pl * 4, c[pl][rb][0]); atomicAdd(d + pl * 4 + 1, c[pl][rb][1]);
-                                    atomicAdd(d + 64 + pl * 4, c[pl][rb][2]); atomicAdd(d + 64 + pl * 4 + 1, c[pl][rb][3]);
-                                }
-                            }
-                        }
-                    }
-                }
-                __syncthreads();
-                // residuals, one thread per (row, plane); the sums are taken and cleared
-                double base = 0.0;                                 // lo^T x~
+            // ---------------------------------------------------------- phase A: dots and residuals
+            double base = 0.0;                                     // lo^T x~ (uniform grids)
+            if constexpr (!TABLE) {
 #pragma unroll
                 for (int w = 0; w < kCluWarps; ++w) base += sh->wbase[w];
-                double srow = 0.0;
-                float rmax = 0.0f;
+            }
+            double srow = 0.0;
 #pragma unroll 1
-                for (int idx = tid; idx < 32 * nrb; idx += kCluThreads) {
-                    const int4 dv = *reinterpret_cast<const int4*>(dacc + idx * 4);
-                    *reinterpret_cast<int4*>(dacc + idx * 4) = make_int4(0, 0, 0, 0);
-                    const int r = idx >> 1;
-                    if (r < rcnt) {
-                        const int dd[NS] = {dv.x, dv.y, dv.z, dv.w};
-                        const float rv = (float)((double)combine_digits<NS>(dd) * delta_w + base - (double)bsm[r]);
-                        res[idx] = rv;
-                        srow += (double)rv;
-                        rmax = fmaxf(rmax, fabsf(rv));
-                    }
-                }
-                srow = warp_sum(srow);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-                if (lane == 0) { sh->ssum[warp] = srow; sh->fmax[warp] = rmax; }
-                __syncthreads();
-                clu_mark(a, it, 2);
-                double S = 0.0;                                    // sum of r1 + r2 over the CTA's rows
-                float rho = 0.0f;
-#pragma unroll
-                for (int w = 0; w < kCluWarps; ++w) { S += sh->ssum[w]; rho = fmaxf(rho, sh->fmax[w]); }
-                const float inv_r = rho > 0.0f ? QMAXF / rho : 0.0f;
-                const float delta_rf = (float)((double)rho / (double)QMAXF), Sf = (float)S;
-                // digits of the residuals as B operands of phase B: per 32 rows and residual, per digit, 32 bytes
-                // in the row order the transposed code fragments come in (k = 16h + 4t + e <-> row 16h + 2t +
-                // (e & 1) + 8 (e >> 1)); rows past the CTA's last one count as zero
-                const int nslab = (rcnt + 31) >> 5;
-                for (int kk = tid; kk < 8 * nslab; kk += kCluThreads) {
-                    const int rbase = (kk >> 3) * 32 + ((kk >> 2) & 1) * 16 + 2 * (kk & 3);
-                    float v1[4], v2[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int k = rbase + (e & 1) + 8 * (e >> 1);
-                        v1[e] = k < rcnt ? res[2 * k] : 0.0f;
-                        v2[e] = k < rcnt ? res[2 * k + 1] : 0.0f;
-                    }
-                    const uint4 o1 = digit_words<NS>(v1, inv_r), o2 = digit_words<NS>(v2, inv_r);
-                    uint32_t* d1 = reinterpret_cast<uint32_t*>(rdig) + (size_t)((kk >> 3) * 2 * NS) * 8 + (kk & 7);
-                    d1[0] = o1.x; d1[8] = o1.y; d1[16] = o1.z; d1[24] = o1.w;
-                    d1[32] = o2.x; d1[40] = o2.y; d1[48] = o2.z; d1[56] = o2.w;
-                }
-                __syncthreads();
-
-                // ------------------------------------------------------ phase B: the rows' part of the gradient
-                // A task is a 16-byte column of the tile over 32 rows.  A transposing ldmatrix hands each lane the
-                // bytes {2g, 2g+1} of rows {2t, 2t+1} of the four 8-row groups; two permutes per half turn them
-                // into A fragments "byte 2g (or 2g+1) of the column, four rows", i.e. features x rows in the row
-                // order of the residual digits.  Each code group of the bytes meets the residual digits (plane 1
-                // those of r2, plane 2 those of r1) in its own accumulators.
-                constexpr int TI = (CB == 2) ? kCluCols / 2 : kCluCols;
-#pragma unroll 1
-                for (int col0 = 0; col0 < ncol; col0 += kCluWarps * TI) {      // the tile stays: wide rows take several passes
-                int acc[TI][NG][4];
-#pragma unroll
-                for (int ti = 0; ti < TI; ++ti)
-#pragma unroll
-                    for (int g = 0; g < NG; ++g)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[ti][g][e] = 0;
-#pragma unroll 1
-                for (int slab = 0; slab < nslab; ++slab) {
-#pragma unroll
-                    for (int pl = 0; pl < 2; ++pl) {
-                        uint32_t b0, b1;
-                        ldsm_x2(b0, b1, l8 < NS ? rdig_addr + (uint32_t)(((slab * 2 + (1 - pl)) * NS + l8) * 32 + (lm & 1) * 16) : zero_addr);
-                        const uint32_t row_addr = tile_addr + pl * plane_bytes + (uint32_t)min(slab * 32 + lane, a.rc - 1) * (uint32_t)pitch * 4u;
-#pragma unroll
-                        for (int ti = 0; ti < TI; ++ti) {
-                            const int col = col0 + warp + ti * kCluWarps;
-                            if (col < ncol) {
-                                uint32_t r4[4];
-                                ldsm_x4_trans(r4, row_addr + (uint32_t)col * 16u);
-                                const uint32_t pel = __byte_perm(r4[0], r4[1], 0x6420), pol = __byte_perm(r4[0], r4[1], 0x7531);
-                                const uint32_t peh = __byte_perm(r4[2], r4[3], 0x6420), poh = __byte_perm(r4[2], r4[3], 0x7531);
-#pragma unroll
-                                for (int g = 0; g < NG; ++g)
-                                    mma_u8s8(acc[ti][g], group_bytes<CB>(pel, g), group_bytes<CB>(pol, g), group_bytes<CB>(peh, g),
-                                             group_bytes<CB>(poh, g), b0, b1);
-                            }
-                        }
-                    }
-                }
-                // columns 2t, 2t+1 of lane t < 2 are digits 2t, 2t+1 (the pair in double, exact; the other pair
-                // comes from lane t+1); accumulator rows g, g+8 are bytes 2g, 2g+1 of the column
-#pragma unroll
-                for (int ti = 0; ti < TI; ++ti) {
-                    const int col = col0 + warp + ti * kCluWarps;
-                    if (col < ncol) {
-#pragma unroll
-                        for (int g = 0; g < NG; ++g) {
-#pragma unroll
-                            for (int odd = 0; odd < 2; ++odd) {
-                                // (the digit sums meet in 64-bit integers and are converted once: conversions to and
-                                // from double run at a sixteenth of the FMA rate and made up most of this epilogue)
-                                const long long pair = (long long)acc[ti][g][2 * odd] + 128ll * (long long)acc[ti][g][2 * odd + 1];
-                                const long long upper = __shfl_down_sync(0xffffffffu, pair, 1);
-                                const int byte_in_row = col * 16 + 2 * gl + odd;
-                                const int f = (byte_in_row >> 2) * FPW + (byte_in_row & 3) * NG + g;
-                                if (tl == 0 && f < n)
-                                    gpart[f] = fmaf(steps[f], (float)(pair + 16384ll * upper) * delta_rf, los[f] * Sf);
-                            }
-                        }
-                    }
-                }
-                }
-            } else {
-                // ---------------------------------------------------------- phase A: dots and residuals
-                double base = 0.0;                                     // lo^T x~ (uniform grids)
-                if constexpr (!TABLE) {
-#pragma unroll
-                    for (int w = 0; w < kCluWarps; ++w) base += sh->wbase[w];
-                }
-                double srow = 0.0;
-#pragma unroll 1
-                for (int r = warp; r < rcnt; r += kCluWarps) {
-                    const uint32_t* row1 = t1 + (size_t)r * pitch;
-                    const uint32_t* row2 = t2 + (size_t)r * pitch;
-                    float acc1 = 0.0f, acc2 = 0.0f;
+            for (int r = warp; r < rcnt; r += kCluWarps) {
+                const uint32_t* row1 = t1 + (size_t)r * rw;
+                const uint32_t* row2 = t2 + (size_t)r * rw;
+                float acc1 = 0.0f, acc2 = 0.0f;
 #pragma unroll 2
-                    for (int q = lane; q < nw; q += 32) {
-                        const uint32_t u1 = row1[q], u2 = row2[q];
+                for (int q = lane; q < nw; q += 32) {
+                    const uint32_t u1 = row1[q], u2 = row2[q];
+                    if constexpr (!TABLE) {
+                        float c1[FPW], c2[FPW];
+                        unpack_word<CB>(u1, c1);
+                        unpack_word<CB>(u2, c2);
+                        // the word's FPW entries of w lie together: 16-byte loads, a quarter of the load instructions
+                        const float4* wq = reinterpret_cast<const float4*>(wv) + (size_t)q * (FPW / 4);
+#pragma unroll
+                        for (int i4 = 0; i4 < FPW / 4; ++i4) {
+                            const float4 w4 = wq[i4];
+                            acc1 = fmaf(c1[4 * i4], w4.x, acc1); acc2 = fmaf(c2[4 * i4], w4.x, acc2);
+                            acc1 = fmaf(c1[4 * i4 + 1], w4.y, acc1); acc2 = fmaf(c2[4 * i4 + 1], w4.y, acc2);
+                            acc1 = fmaf(c1[4 * i4 + 2], w4.z, acc1); acc2 = fmaf(c2[4 * i4 + 2], w4.z, acc2);
+                            acc1 = fmaf(c1[4 * i4 + 3], w4.w, acc1); acc2 = fmaf(c2[4 * i4 + 3], w4.w, acc2);
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < FPW; ++i) {
+                            acc1 += tab[(code_at<CB>(u1, i) * FPW + i) * rw + q];
+                            acc2 += tab[(code_at<CB>(u2, i) * FPW + i) * rw + q];
+                        }
+                    }
+                }
+                // both sums with one butterfly: the upper half-warp ends up with plane 2, the lower with plane 1
+                const bool up = (lane & 16) != 0;
+                double d = (double)(up ? acc2 : acc1) + __shfl_xor_sync(0xffffffffu, (double)(up ? acc1 : acc2), 16);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                if ((lane & 15) == 0) {
+                    const float rv = (float)(d + base - (double)bsm[r]);
+                    res[2 * r + (up ? 1 : 0)] = rv;
+                    srow += (double)rv;
+                }
+            }
+            srow += __shfl_xor_sync(0xffffffffu, srow, 16);
+            if (lane == 0) sh->ssum[warp] = srow;
+            __syncthreads();
+            clu_mark(a, it, 2);
+
+            // ---------------------------------------------------------- phase B: the rows' part of the gradient
+            double S = 0.0;                                        // sum of r1 + r2 over the CTA's rows
+            if constexpr (!TABLE) {
+#pragma unroll
+                for (int w = 0; w < kCluWarps; ++w) S += sh->ssum[w];
+            }
+            const float Sf = (float)S;
+#pragma unroll 1
+            for (int q0 = 0; q0 < nw; q0 += lanes_q) {
+                const int q = q0 + ql;
+                const bool active = group < ngroups && q < nw;
+                float acc[FPW];
+#pragma unroll
+                for (int i = 0; i < FPW; ++i) acc[i] = 0.0f;
+                if (active) {
+#pragma unroll 2
+                    for (int r = group; r < rcnt; r += ngroups) {
+                        const uint32_t u1 = t1[(size_t)r * rw + q], u2 = t2[(size_t)r * rw + q];
+                        const float2 rv = *reinterpret_cast<const float2*>(res + 2 * r);
                         if constexpr (!TABLE) {
                             float c1[FPW], c2[FPW];
                             unpack_word<CB>(u1, c1);
                             unpack_word<CB>(u2, c2);
-                            // the word's FPW entries of w lie together: 16-byte loads, a quarter of the load instructions
-                            const float4* wq = reinterpret_cast<const float4*>(wv) + (size_t)q * (FPW / 4);
 #pragma unroll
-                            for (int i4 = 0; i4 < FPW / 4; ++i4) {
-                                const float4 w4 = wq[i4];
-                                acc1 = fmaf(c1[4 * i4], w4.x, acc1); acc2 = fmaf(c2[4 * i4], w4.x, acc2);
-                                acc1 = fmaf(c1[4 * i4 + 1], w4.y, acc1); acc2 = fmaf(c2[4 * i4 + 1], w4.y, acc2);
-                                acc1 = fmaf(c1[4 * i4 + 2], w4.z, acc1); acc2 = fmaf(c2[4 * i4 + 2], w4.z, acc2);
-                                acc1 = fmaf(c1[4 * i4 + 3], w4.w, acc1); acc2 = fmaf(c2[4 * i4 + 3], w4.w, acc2);
-                            }
+                            for (int i = 0; i < FPW; ++i) acc[i] = fmaf(c1[i], rv.y, fmaf(c2[i], rv.x, acc[i]));
                         } else {
 #pragma unroll
                             for (int i = 0; i < FPW; ++i) {
-                                acc1 += tab[(code_at<CB>(u1, i) * FPW + i) * rw + q];
-                                acc2 += tab[(code_at<CB>(u2, i) * FPW + i) * rw + q];
+                                const float l1 = lev[(code_at<CB>(u1, i) * FPW + i) * rw + q];
+                                const float l2 = lev[(code_at<CB>(u2, i) * FPW + i) * rw + q];
+                                acc[i] = fmaf(l1, rv.y, fmaf(l2, rv.x, acc[i]));
                             }
                         }
                     }
-                    // both sums with one butterfly: the upper half-warp ends up with plane 2, the lower with plane 1
-                    const bool up = (lane & 16) != 0;
-                    double d = (double)(up ? acc2 : acc1) + __shfl_xor_sync(0xffffffffu, (double)(up ? acc1 : acc2), 16);
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-                    if ((lane & 15) == 0) {
-                        const float rv = (float)(d + base - (double)bsm[r]);
-                        res[2 * r + (up ? 1 : 0)] = rv;
-                        srow += (double)rv;
-                    }
                 }
-                srow += __shfl_xor_sync(0xffffffffu, srow, 16);
-                if (lane == 0) sh->ssum[warp] = srow;
+                if (ngroups == 1) {                          // (wide rows: a thread has its columns' sums to itself)
+                    if (active)
+#pragma unroll
+                        for (int i = 0; i < FPW; ++i)
+                            if (q * FPW + i < n) gpart[q * FPW + i] = TABLE ? acc[i] : fmaf(steps[q * FPW + i], acc[i], los[q * FPW + i] * Sf);
+                    continue;
+                }
+                // the groups' sums meet in shared memory ([group][feature of the pass]); then one thread per
+                // feature adds them in order and writes the feature's entry of the CTA's part
+                if (q0 > 0) __syncthreads();
+                if (active) {
+#pragma unroll
+                    for (int i = 0; i < FPW; ++i) gred[(group * lanes_q + ql) * FPW + i] = acc[i];
+                }
                 __syncthreads();
-                clu_mark(a, it, 2);
-
-                // ---------------------------------------------------------- phase B: the rows' part of the gradient
-                double S = 0.0;                                        // sum of r1 + r2 over the CTA's rows
-                if constexpr (!TABLE) {
-#pragma unroll
-                    for (int w = 0; w < kCluWarps; ++w) S += sh->ssum[w];
-                }
-                const float Sf = (float)S;
 #pragma unroll 1
-                for (int q0 = 0; q0 < nw; q0 += lanes_q) {
-                    const int q = q0 + ql;
-                    const bool active = group < ngroups && q < nw;
-                    float acc[FPW];
-#pragma unroll
-                    for (int i = 0; i < FPW; ++i) acc[i] = 0.0f;
-                    if (active) {
-#pragma unroll 2
-                        for (int r = group; r < rcnt; r += ngroups) {
-                            const uint32_t u1 = t1[(size_t)r * pitch + q], u2 = t2[(size_t)r * pitch + q];
-                            const float2 rv = *reinterpret_cast<const float2*>(res + 2 * r);
-                            if constexpr (!TABLE) {
-                                float c1[FPW], c2[FPW];
-                                unpack_word<CB>(u1, c1);
-                                unpack_word<CB>(u2, c2);
-#pragma unroll
-                                for (int i = 0; i < FPW; ++i) acc[i] = fmaf(c1[i], rv.y, fmaf(c2[i], rv.x, acc[i]));
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < FPW; ++i) {
-                                    const float l1 = lev[(code_at<CB>(u1, i) * FPW + i) * rw + q];
-                                    const float l2 = lev[(code_at<CB>(u2, i) * FPW + i) * rw + q];
-                                    acc[i] = fmaf(l1, rv.y, fmaf(l2, rv.x, acc[i]));
-                                }
-                            }
-                        }
-                    }
-                    // the groups' sums meet in shared memory ([group][feature of the pass]); then one thread per
-                    // feature adds them in order and writes the feature's entry of the CTA's part
-                    if (q0 > 0) __syncthreads();
-                    if (active) {
-#pragma unroll
-                        for (int i = 0; i < FPW; ++i) gred[(group * lanes_q + ql) * FPW + i] = acc[i];
-                    }
-                    __syncthreads();
-#pragma unroll 1
-                    for (int fl = tid; fl < lanes_q * FPW; fl += kCluThreads) {
-                        const int f = q0 * FPW + fl;
-                        if (f < n) {
-                            float v = gred[fl];
-                            for (int g = 1; g < ngroups; ++g) v += gred[g * lanes_q * FPW + fl];
-                            if constexpr (!TABLE) v = fmaf(steps[f], v, los[f] * Sf);      // (fp32: conversions are slow)
-                            gpart[f] = v;
-                        }
+                for (int fl = tid; fl < lanes_q * FPW; fl += kCluThreads) {
+                    const int f = q0 * FPW + fl;
+                    if (f < n) {
+                        float v = gred[fl];
+                        for (int g = 1; g < ngroups; ++g) v += gred[g * lanes_q * FPW + fl];
+                        if constexpr (!TABLE) v = fmaf(steps[f], v, los[f] * Sf);      // (fp32: conversions are slow)
+                        gpart[f] = v;
                     }
                 }
             }
@@ -613,12 +401,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
                 bulk_copy_s2c(cluster_addr(gbuf + (size_t)bi * sub, warp), gpart + (size_t)warp * sub, slice_bytes,
                               cluster_addr(&sh->rs_bar, warp));
             // the tile is consumed: refill its slot while the parts travel
-            // (row-by-row tiles: the warps share the rows, since one warp issues its copies one after the other
-            // and a whole tile from one warp held the CTA's next barrier back by thousands of cycles)
-            if (it + a.slots < step_end) {
-                if (pitch == rw) { if (warp == kCluWarps - 1) issue_tile(it + a.slots, slot); }
-                else issue_tile_rows(it + a.slots, slot);
-            }
+            if (it + a.slots < step_end && warp == kCluWarps - 1) issue_tile(it + a.slots, slot);
             if (++slot == a.slots) { slot = 0; parity ^= 1u; }
             clu_mark(a, it, 3);
 
@@ -703,7 +486,6 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         clu_wait(&sh->ag_bar, ag_parity, sh, a.status, 4);
         ag_parity ^= 1u;
         double bpart = 0.0;
-        float wm = 0.0f;
 #pragma unroll 1
         for (int idx = tid; idx < Fp; idx += kCluThreads) {
             // level tables: consecutive threads take consecutive word columns of one feature slot, so that the L
@@ -712,12 +494,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
             const int q = TABLE ? idx % rw : idx >> LOGF, i = TABLE ? idx / rw : idx & (FPW - 1);
             const int f = TABLE ? q * FPW + i : idx;
             const float xt = (f < n) ? xs[f] : 0.0f;
-            if constexpr (IMMA) {
-                const float w = steps[f] * xt;
-                wv[f] = w;
-                wm = fmaxf(wm, fabsf(w));
-                bpart += (double)los[f] * (double)xt;
-            } else if constexpr (!TABLE) {
+            if constexpr (!TABLE) {
                 wv[f] = steps[f] * xt;
                 bpart += (double)los[f] * (double)xt;
             } else {
@@ -726,33 +503,10 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
         }
         if constexpr (!TABLE) {
             bpart = warp_sum(bpart);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-            if (lane == 0) { sh->wbase[warp] = bpart; sh->fmax[warp] = wm; }
+            if (lane == 0) sh->wbase[warp] = bpart;
         }
         if (tid < rcnt) bsm[tid] = breg;
         for (int r = tid + kCluThreads; r < rcnt; r += kCluThreads) bsm[r] = __ldg(a.b + r0 + k0 + r);
-        if constexpr (IMMA) {
-            // digits of w as B operands of phase A, scaled by the largest |w| of the whole vector: per k-slab
-            // (8 words), code group and digit a 32-byte k vector
-            __syncthreads();
-            float wmax = 0.0f;
-#pragma unroll
-            for (int w = 0; w < kCluWarps; ++w) wmax = fmaxf(wmax, sh->fmax[w]);
-            const float inv_w = wmax > 0.0f ? QMAXF / wmax : 0.0f;
-            delta_w = (double)wmax / (double)QMAXF;
-#pragma unroll 1
-            for (int item = tid; item < 8 * ((rw + 7) >> 3) * NG; item += kCluThreads) {
-                const int q = item / NG, g = item - q * NG;
-                uint4 o = make_uint4(0u, 0u, 0u, 0u);
-                if (q < rw) {
-                    const float v4[4] = {wv[q * FPW + g], wv[q * FPW + NG + g], wv[q * FPW + 2 * NG + g], wv[q * FPW + 3 * NG + g]};
-                    o = digit_words<NS>(v4, inv_w);
-                }
-                uint32_t* dst = wdig + (size_t)(((q >> 3) * NG + g) * NS) * 8 + (q & 7);
-                dst[0] = o.x; dst[8] = o.y; dst[16] = o.z; dst[24] = o.w;
-            }
-        }
         clu_mark(a, it, 6);
         __syncthreads();
         clu_mark(a, it, 7);
@@ -769,31 +523,25 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
 // Host side
 // ---------------------------------------------------------------------------------------------
 struct ClusterPlan {
-    int nb, rc, slots, sub, p_shift, pitch;
-    bool imma;                   // uniform grids: int8 tensor-core contraction instead of fp32 FMA
+    int nb, rc, slots, sub, p_shift;
     size_t smem;
 };
 
-// Rows of a tile lie `pitch` words apart in shared memory.  The integer path loads fragments of 8 rows x 16
-// bytes; they fall into 8 different bank groups when the pitch is an odd number of 16-byte units.
-static int cluster_pitch(bool imma, int row_words) { return (!imma || ((row_words / 4) & 1)) ? row_words : row_words + 4; }
-
-static size_t cluster_smem_bytes(int cb, bool table, bool imma, int row_words, int bits, int nb, int sub, int rc, int slots) {
+static size_t cluster_smem_bytes(int cb, bool table, int row_words, int words, int bits, int nb, int sub, int rc, int slots) {
     const size_t fpw = 32 / cb, Fp = (size_t)row_words * fpw, L = (size_t)1 << bits, Fs = (size_t)nb * sub;
     size_t bytes = (sizeof(ClusterShared) + 15) & ~(size_t)15;
-    if (imma) bytes += sizeof(float) * 3 * Fp + (size_t)((row_words + 7) / 8) * (8 / cb) * 4 * 32 + (size_t)((rc + 31) / 32) * 256 +
-                       sizeof(int) * (size_t)((rc + 15) & ~15) * 8;
-    else bytes += sizeof(float) * ((table ? 2 * L * Fp : 3 * Fp) + (size_t)kCluThreads * fpw);
+    const int lanes_q = (words + 31) / 32 * 32;                     // one group of threads: no meeting of groups
+    bytes += sizeof(float) * ((table ? 2 * L * Fp : 3 * Fp) + (2 * lanes_q <= kCluThreads ? (size_t)kCluThreads * fpw : 0));
     bytes += sizeof(float) * (3 * Fs + 3 * (size_t)sub + (size_t)((2 * rc + 3) & ~3) + (size_t)((rc + 3) & ~3));
     bytes += 128 + 64;                                              // slack to align the ring, and past its last row
-    bytes += sizeof(uint32_t) * (size_t)slots * 2 * rc * cluster_pitch(imma, row_words);
+    bytes += sizeof(uint32_t) * (size_t)slots * 2 * rc * row_words;
     return bytes;
 }
 
-static const void* cluster_kernel_ptr(int cb, bool table, bool imma) {
-    if (cb == 2) return table ? (const void*)sgd_cluster_kernel<2, true, false> : imma ? (const void*)sgd_cluster_kernel<2, false, true> : (const void*)sgd_cluster_kernel<2, false, false>;
-    if (cb == 4) return table ? (const void*)sgd_cluster_kernel<4, true, false> : imma ? (const void*)sgd_cluster_kernel<4, false, true> : (const void*)sgd_cluster_kernel<4, false, false>;
-    return imma ? (const void*)sgd_cluster_kernel<8, false, true> : (const void*)sgd_cluster_kernel<8, false, false>;
+static const void* cluster_kernel_ptr(int cb, bool table) {
+    if (cb == 2) return table ? (const void*)sgd_cluster_kernel<2, true> : (const void*)sgd_cluster_kernel<2, false>;
+    if (cb == 4) return table ? (const void*)sgd_cluster_kernel<4, true> : (const void*)sgd_cluster_kernel<4, false>;
+    return (const void*)sgd_cluster_kernel<8, false>;
 }
 
 static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zipml_sgd_params* p, ClusterPlan* plan) {
@@ -809,8 +557,7 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
     if (nb < 1) nb = 1;
     const size_t cap = (size_t)ctx->smem_optin;
     const int64_t nb_max = B < kCluMaxCtas ? B : kCluMaxCtas;
-    // the caller may fix the contraction for uniform grids (tests, tuning): 1 = fp32, 2 = int8 tensor cores
-    const int force_int8 = p->cluster_contraction == 1 ? 0 : p->cluster_contraction >= 2 ? 1 : -1;
+    const int words = (int)((d->n * cb + 31) / 32);
     // the requested number of row parts is a hint: more parts are used when a tile does not fit
     for (;; ++nb) {
         if (nb > nb_max) return ZIPML_ERR_WORKSPACE;
@@ -823,16 +570,11 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
         while (r.p_shift < 5 && ((int64_t)r.sub << (r.p_shift + 1)) <= kCluThreads && (1 << r.p_shift) < r.nb) ++r.p_shift;
         if ((uint64_t)2 * r.rc * row_words * 4 >= (1u << 20)) continue;                     // mbarrier tx-count range
         if ((uint64_t)r.nb * r.sub * 4 >= (1u << 20)) continue;
-        // the integer contraction pays its per-step digit conversions back on tiles of 24 KiB per plane and more
-        // (measured: 16 rows x 1 KB 6.6 vs 5.5 us per step in fp32; 64 rows x 512 B 17.3 vs 21.6 us)
-        r.imma = !table && (int64_t)r.rc * d->row_bytes >= 24 * 1024;
-        if (!table && force_int8 >= 0) r.imma = force_int8 != 0;
-        r.pitch = cluster_pitch(r.imma, (int)row_words);
         int slots = kCluMaxSlots;
-        while (slots >= 2 && cluster_smem_bytes(cb, table, r.imma, (int)row_words, d->bits, r.nb, r.sub, r.rc, slots) > cap) --slots;
+        while (slots >= 2 && cluster_smem_bytes(cb, table, (int)row_words, words, d->bits, r.nb, r.sub, r.rc, slots) > cap) --slots;
         if (slots < 2) continue;
         r.slots = slots;
-        r.smem = cluster_smem_bytes(cb, table, r.imma, (int)row_words, d->bits, r.nb, r.sub, r.rc, slots);
+        r.smem = cluster_smem_bytes(cb, table, (int)row_words, words, d->bits, r.nb, r.sub, r.rc, slots);
         *plan = r;
         return ZIPML_OK;
     }
@@ -884,7 +626,7 @@ int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     ClusterPlan plan;
     int rc = make_cluster_plan(ctx, d, p, &plan);
     if (rc != ZIPML_OK) return rc;
-    const void* kernel = cluster_kernel_ptr(cb, table, plan.imma);
+    const void* kernel = cluster_kernel_ptr(cb, table);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
     if (e != cudaSuccess) return cuda_status(e);
     if (plan.nb > 8) {
@@ -931,7 +673,7 @@ int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     a.words = (int)((d->n + fpw - 1) / fpw);
     a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
     a.nb = plan.nb; a.rc = plan.rc; a.slots = plan.slots;
-    a.sub = plan.sub; a.p_shift = plan.p_shift; a.pitch = plan.pitch;
+    a.sub = plan.sub; a.p_shift = plan.p_shift;
     if (p->batch_order) {
         int32_t* dev_order = reinterpret_cast<int32_t*>(ctx->ws + o_ord);
         e = cudaMemcpyAsync(dev_order, p->batch_order, sizeof(int32_t) * (size_t)T, cudaMemcpyHostToDevice, ctx->stream);

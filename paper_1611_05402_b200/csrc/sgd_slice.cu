@@ -1,4 +1,4 @@
-// Cluster engine of zipml_sgd_epoch on uniform grids, int8 tensor cores: one thread-block cluster of nb <= 16 CTAs, the
+// Cluster engine of zipml_sgd_epoch on uniform grids, int8 tensor cores, split by rows: one thread-block cluster of nb <= 16 CTAs, the
 // minibatch cut into row parts, the packed row into slices that the CTAs own (Supplement "Double Sampling", footnote
 // form; "End-to-end Quantization").
 //
