@@ -40,7 +40,7 @@ NCU_TRAFFIC = {
     ("c5", 7): (4 * (538.45e6 + 4.86e6), "profiles/sgd_column_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
 }
 ENGINE_KERNELS = {1: "sgd_kernel (stepwise launches)", 2: "sgd_kernel (persistent)", 3: "sgd_ring_kernel", 4: "sgd_lean_kernel",
-                  5: "sgd_cluster_kernel", 6: "sgd_stream_kernel", 7: "sgd_column_kernel", 8: "sgd_solo_kernel"}
+                  5: "sgd_feature_kernel, sgd_slice_kernel or sgd_table_kernel", 6: "sgd_stream_kernel", 7: "sgd_column_kernel", 8: "sgd_solo_kernel"}
 
 
 def measured_peaks():

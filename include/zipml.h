@@ -64,23 +64,22 @@ enum {
 };
 /* How zipml_sgd_epoch runs its minibatch chain.  Results do not depend on the choice. */
 enum {
-    ZIPML_ENGINE_AUTO = 0,      /* solo for the smallest steps; cluster, else lean, for steps of at most
-                                   2 MiB of codes; else column,
-                                   else stream, where they apply (wide rows, uniform grid, fp32 model
-                                   and gradient), else ring                                           */
+    ZIPML_ENGINE_AUTO = 0,      /* solo for the smallest steps; cluster where its forms hold the rows;
+                                   else column, else stream, by code width, row length and batch
+                                   (uniform grid, fp32 model and gradient), else ring; lean and
+                                   persistent on level tables no cluster holds                        */
     ZIPML_ENGINE_STEPWISE = 1,  /* a few kernel launches per minibatch                               */
     ZIPML_ENGINE_PERSISTENT = 2, /* one cooperative launch per call, grid barriers between the phases */
     ZIPML_ENGINE_RING = 3,       /* one cooperative launch; producer warp streams code chunks through a
                                     shared-memory ring, gradients meet by reduce-scatter / all-gather  */
     ZIPML_ENGINE_LEAN = 4,       /* one cooperative launch for small minibatch tiles: row parts only,
                                     two barriers and two packet exchanges per step                    */
-    ZIPML_ENGINE_CLUSTER = 5,    /* one thread-block cluster (at most 16 row parts) for small tiles:
-                                    gradients and model travel between the CTAs' shared memories.  On
-                                    uniform grids with rows of up to some 3 KB several clusters, which
-                                    meet through L2, and minibatches of any size, in chunks.
-                                    Uniform grids contract in fp32 or, on taller tiles, on the int8
-                                    tensor cores; zipml_sgd_params.cluster_contraction overrides that
-                                    choice                                                            */
+    ZIPML_ENGINE_CLUSTER = 5,    /* one thread-block cluster of at most 16 CTAs that exchange through their
+                                    shared memories, for small tiles.  On uniform grids split by features
+                                    (up to 8,192) or by rows (up to some 3 KB), on the int8 tensor cores,
+                                    several clusters, which meet through L2, and by rows minibatches of any
+                                    size, in chunks; level tables split by features or by rows.
+                                    zipml_sgd_params.cluster_contraction overrides the choice          */
     ZIPML_ENGINE_STREAM = 6,     /* one cooperative launch for large tiles on uniform grids with an fp32
                                     model and gradient: both passes of a step read the codes straight
                                     from global memory into int8 tensor-core fragments (the second pass
