@@ -332,13 +332,14 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
             step_parity ^= 1u;
             if (step < marked) slice_mark(a.trace, step, 3);
             // -------------------------------------------------------------- digits of the residuals, one scale for all rows
-            float top = 0.0f;
+            // (largest as bit patterns: a residual that is not a number wins, and the gradient is none either)
+            uint32_t top_bits = 0u;
 #pragma unroll 4
             for (int i = lane; i < 8 * a.rb; i += 32) {
-                const float4 v = reinterpret_cast<const float4*>(res)[i];
-                top = fmaxf(fmaxf(top, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+                const uint4 v = reinterpret_cast<const uint4*>(res)[i];
+                top_bits = max(max(top_bits, max(v.x & 0x7fffffffu, v.y & 0x7fffffffu)), max(v.z & 0x7fffffffu, v.w & 0x7fffffffu));
             }
-            top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+            const float top = __uint_as_float(__reduce_max_sync(0xffffffffu, top_bits));
             const int k_r = slice_exponent(top, 0);
             const float up_r = slice_pow2(k_r), delta_r = top <= 3.402823466e+38f ? slice_pow2(-k_r) : __int_as_float(0x7fffffff);
             int r_low = 0, r_high = 0;                   // sums of the integers' halves (some 2,000 entries a warp at most)

@@ -85,7 +85,7 @@ struct alignas(16) SliceShared {
     uint64_t part_bar, gn_bar, xn_bar;
     float delta_r;               // value of a unit of the residuals' fixed point
     float wmax[32];              // owner: per-warp maxima of |w|
-    float rmax[16];              // maxima of |residual| of a row block
+    uint32_t rmax[16];           // maxima of |residual| of a row block, as bit patterns
     int gave_up;
 };
 
@@ -306,13 +306,15 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                     for (int i = 0; i < 4; ++i)
                         if (w + i < a_all) d[i] += ps[(w + i) * rb * 32];
                 const float r = res_row < rows_of(batch, chunk) ? (float)((d[0] + d[1]) + (d[2] + d[3])) : 0.0f;
-                float top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(r))));
+                // (largest as bit patterns: a residual that is not a number wins, and the gradient is none either)
+                uint32_t top_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(r)));
                 if (rb > 1) {                            // one scale for all row blocks
-                    if (lane == 0) sh->rmax[warp] = top;
+                    if (lane == 0) sh->rmax[warp] = top_bits;
                     asm volatile("bar.sync 2, %0;" ::"r"(32 * rb) : "memory");
 #pragma unroll 1
-                    for (int w2 = 0; w2 < rb; ++w2) top = fmaxf(top, sh->rmax[w2]);
+                    for (int w2 = 0; w2 < rb; ++w2) top_bits = max(top_bits, sh->rmax[w2]);
                 }
+                const float top = __uint_as_float(top_bits);
                 const int k_r = slice_exponent(top, 0);
                 if (tid == 0) sh->delta_r = top <= 3.402823466e+38f ? slice_pow2(-k_r) : __int_as_float(0x7fffffff);
                 const uint32_t digits = ((uint32_t)__float2int_rn(r * slice_pow2(k_r)) + 0x80808080u) ^ 0x80808080u;

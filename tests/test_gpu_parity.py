@@ -434,6 +434,37 @@ def test_cluster_engine_on_tables_by_features(ctx, m, n, bits, batch, parts):
     assert np.allclose(x.cpu().numpy(), x0 - np.float32(lr) * g[1].cpu().numpy(), rtol=1e-6, atol=1e-7)
 
 
+FORMS = {                                                            # engine, contraction, bits, n, batch, clusters, table
+    "solo": (binding.ENGINE_SOLO, 0, 4, 64, 40, 0, False), "solo-table": (binding.ENGINE_SOLO, 0, 3, 64, 40, 0, True),
+    "features": (binding.ENGINE_CLUSTER, 4, 8, 500, 70, 0, False), "features-clusters": (binding.ENGINE_CLUSTER, 4, 4, 500, 300, 3, False),
+    "rows": (binding.ENGINE_CLUSTER, 3, 8, 500, 70, 0, False), "rows-blocks": (binding.ENGINE_CLUSTER, 3, 4, 64, 900, 1, False),
+    "rows-chunks": (binding.ENGINE_CLUSTER, 3, 8, 1000, 5000, 1, False), "rows-clusters": (binding.ENGINE_CLUSTER, 3, 2, 500, 900, 2, False),
+    "table-features": (binding.ENGINE_CLUSTER, 2, 3, 500, 70, 0, True), "fp32": (binding.ENGINE_CLUSTER, 1, 8, 500, 70, 0, False),
+    "table-rows": (binding.ENGINE_CLUSTER, 1, 2, 100, 300, 0, True),
+}
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("where", ["label", "label-nan-first", "model"])
+def test_values_that_are_not_numbers_reach_gradient_and_model(ctx, form, where):
+    """One label that is not a number, or an infinite model entry, leaves no finite gradient or model behind in any form: the
+    scales of the integer contractions must not drop it beside finite residuals."""
+    engine, contraction, bits, n, batch, clusters, table = FORMS[form]
+    _, A, b, _ = workload("c4" if table else "c1", batch, n, seed=2)
+    kw = dict(mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 64)[0]) if table else {}
+    gds = dev_dataset(oracle.quantize(A, bits, seed=3, **kw), ctx)
+    x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
+    if where == "model":
+        x0[n // 2] = np.inf
+    else:
+        b = b.copy()
+        b[0 if where == "label-nan-first" else batch - 3] = np.nan
+    x, g = to_dev(x0, ctx), torch.zeros((2, n), device=ctx.device)
+    ctx.zipml_sgd_epoch(gds, to_dev(b, ctx), x, batch, 1e-3, engine=engine, cluster_contraction=contraction, grid_feature_parts=clusters, grad_out=g)
+    ctx.zipml_sync()
+    assert not torch.isfinite(g).any() and not torch.isfinite(x).any()
+
+
 @pytest.mark.parametrize("contraction", [1, 2], ids=["fp32", "int8"])
 @pytest.mark.parametrize("case", SGD_CASES[:5], ids=lambda c: f"{c[0]}-{c[1]}x{c[2]}-b{c[3]}-B{c[4]}")
 def test_cluster_engine_both_contractions(ctx, case, contraction):
