@@ -729,18 +729,19 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             const ColStep st = col_step(a, a.first_step + t_rel);
             const ColStepParams& sp = sh->sp[t_rel & 1];
             const long long* dots = a.dots + (size_t)(t_rel % 3) * ngrp * 2 * a.bpad;
-            // the step's largest |label| completes the bound of its residuals
-            float bm = 0.0f;
+            // the step's largest |label| completes the bound of its residuals (as bit patterns: one that is not a number
+            // wins, and such a bound makes the gradients of this and the later steps none either)
+            uint32_t bm = 0u;
 #pragma unroll 1
-            for (int k = rt; k < st.bt; k += kColRThreads) bm = fmaxf(bm, fabsf(__ldg(a.b + st.row0 + k)));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-            if (lane == 0) sh->red_f[1][rw] = bm;
+            for (int k = rt; k < st.bt; k += kColRThreads) bm = max(bm, __float_as_uint(fabsf(__ldg(a.b + st.row0 + k))));
+            bm = __reduce_max_sync(0xffffffffu, bm);
+            if (lane == 0) sh->red_f[1][rw] = __uint_as_float(bm);
             named_barrier(kColNamedR, kColRThreads);
-            bm = 0.0f;
+            bm = 0u;
 #pragma unroll
-            for (int w = 0; w < kColRWarps; ++w) bm = fmaxf(bm, sh->red_f[1][w]);
-            const double rbound = (dbound + (double)bm) * 1.0001;
+            for (int w = 0; w < kColRWarps; ++w) bm = max(bm, __float_as_uint(sh->red_f[1][w]));
+            const double rbound = (dbound + (double)__uint_as_float(bm)) * 1.0001;
+            const bool bounded = rbound - rbound == 0.0;
             // The residuals' unit is a power of two as well (at most twice what the bound needs), so that a dot becomes
             // a residual by a shift and the label's own fixed-point value: integers only on the way to the digits.
             const int ed = rbound > 0.0 ? max(-900, min(900, col_exponent(rbound * (1.0 / (double)kColQmaxR)) + 1)) : 0;
@@ -899,13 +900,13 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             long long hi = 0, lo = 0;
 #pragma unroll
             for (int w = 0; w < kColRWarps; ++w) { rm = fmax(rm, sh->red_d[1][w]); hi += sh->red_l[0][w]; lo += sh->red_l[1][w]; }
-            dbound = (dbound * grow + fabs((double)a.lr) * rm * c2) * 1.0001;
+            dbound = bounded ? (dbound * grow + fabs((double)a.lr) * rm * c2) * 1.0001 : __longlong_as_double(0x7fffffffffffffffll);
             if (((q0 + c_last) & (kColRWarps - 1)) == rw) {      // the warp that holds the step's last chunk
                 if (lane == 0) {
                     ColStepParams& cur = sh->sp[t_rel & 1];
                     cur.inv_r = inv_delta;
                     cur.delta_r = delta_r;
-                    cur.rsum = (double)hi * 268435456.0 + (double)lo;
+                    cur.rsum = bounded ? (double)hi * 268435456.0 + (double)lo : __longlong_as_double(0x7fffffffffffffffll);
                     col_unit_of(dbound, sh->sp[(t_rel + 1) & 1].U, sh->sp[(t_rel + 1) & 1].invU);
                 }
                 __syncwarp();

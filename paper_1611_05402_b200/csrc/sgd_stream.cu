@@ -404,8 +404,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) sgd_stream_kernel(const Str
                 int R1 = 0, R2 = 0;
                 if (k < bt) {
                     const double2 d = rres[k];
-                    R1 = fixed_point((float)(d.x + base), inv_r);
-                    R2 = fixed_point((float)(d.y + base), inv_r);
+                    const float r1 = (float)(d.x + base), r2 = (float)(d.y + base);
+                    R1 = fixed_point(r1, inv_r);
+                    R2 = fixed_point(r2, inv_r);
+                    rsum += (double)((r1 - r1) + (r2 - r2));       // 0; a residual that is not a number reaches the gradient
                 }
                 rsum += (double)R1 + (double)R2;
                 int d1[NS], d2[NS];

@@ -440,7 +440,9 @@ FORMS = {                                                            # engine, c
     "rows": (binding.ENGINE_CLUSTER, 3, 8, 500, 70, 0, False), "rows-blocks": (binding.ENGINE_CLUSTER, 3, 4, 64, 900, 1, False),
     "rows-chunks": (binding.ENGINE_CLUSTER, 3, 8, 1000, 5000, 1, False), "rows-clusters": (binding.ENGINE_CLUSTER, 3, 2, 500, 900, 2, False),
     "table-features": (binding.ENGINE_CLUSTER, 2, 3, 500, 70, 0, True), "fp32": (binding.ENGINE_CLUSTER, 1, 8, 500, 70, 0, False),
-    "table-rows": (binding.ENGINE_CLUSTER, 1, 2, 100, 300, 0, True),
+    "table-rows": (binding.ENGINE_CLUSTER, 1, 2, 100, 300, 0, True), "column": (binding.ENGINE_COLUMN, 0, 4, 9001, 64, 0, False),
+    "stream": (binding.ENGINE_STREAM, 0, 2, 9403, 40, 0, False), "ring": (binding.ENGINE_RING, 0, 8, 3300, 250, 0, False),
+    "lean": (binding.ENGINE_LEAN, 0, 4, 9001, 64, 0, False), "grid": (binding.ENGINE_PERSISTENT, 0, 8, 1000, 64, 0, False),
 }
 
 
