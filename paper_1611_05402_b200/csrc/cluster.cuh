@@ -133,6 +133,10 @@ struct SliceShift {                                       // bits that a group's
     static constexpr int kMost = CB == 8 ? 0 : CB == 4 ? 4 : 2;
     __device__ static constexpr int of(int g) { return CB == 8 ? 0 : CB == 4 ? (g == 0 ? 4 : 0) : (g & 1 ? 0 : 2); }
 };
+// low + 65536 high: the integer's bits behind those of 1.5 x 2^52 (conversions to double run at a sixteenth of the FMA rate).
+__device__ __forceinline__ double slice_double(int low, int high) {
+    return __longlong_as_double(low + 65536ll * high + 0x4338000000000000ll) - 6755399441055744.0;
+}
 // D = A B + C with C's two columns given.
 __device__ __forceinline__ void slice_mma_from(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, int c0, int c1) {
     asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"

@@ -11,7 +11,8 @@
 //     plane 2 with r1 are the 32 entries of one contraction;                                                  barrier
 //   * gradient: a warp takes a column and a part of the row blocks (transposing ldmatrix) and leaves a low and a high integer per feature;
 //                                                                                                             barrier
-//   * sums over the parts, centred as integers (codes less half the top code: nothing cancels later); Q4, update, Q3, w;   barrier
+//   * sums over the parts, exact integers until they meet lo and step in double (codes less a constant centre in fp32 lost 10 to 37 times
+//     the precision on rows that are mostly zeros: 1.2e-6 of the gradient at 256 x 1,000, 4e-8 now); Q4, update, Q3, w;   barrier
 //     and the digits of w, four balanced base-256 digits per entry, with the power of two of the CTA's largest.            barrier
 // Bound by the chain of dependent instructions: some 660 a warp and step at 48 % of the issue slots (8 bits 256 x 1,000: dots 1.1 k cycles,
 // hand-overs 0.8 k and 0.2 k, digits of the residuals 0.7 k, gradient 0.7 k, update 0.6 k, digits of w 0.6 k); a quantized gradient and
@@ -53,7 +54,7 @@ struct FeatureArgs {
     int n, bits;
     int model_bits, grad_bits;
     int whole, rows_last;        // batches below `whole` are full, that one has rows_last rows
-    float full_scale, last_scale;    // 1 / (2 rows)
+    double full_scale, last_scale;   // 1 / (2 rows)
     int clusters, rows;          // clusters, rows per cluster
     unsigned long long* exchange;    // [2][clusters][nb F][2] words {fp32, tag} between the clusters
     uint32_t tag;                // of the first step; greater than any that the buffer holds
@@ -240,9 +241,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
     const int P = 1 << a.p_shift, pp = tid & (P - 1), k_own = tid >> a.p_shift, f_own = bi * F + k_own;
     const bool mine = k_own < F && f_own < n, writes = mine && pp == 0;
     const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
-    const int c0 = 1 << (a.bits - 1), shift = CB * (k_own % NG);
-    const float mid = fmaf((float)c0, st, lof);
-    const float st_low = st / (float)(1 << shift);     // (codes were multiplied where they lie in their byte)
+    const double lo_double = lof, st_low = (double)st / (double)(1 << (CB * (k_own % NG)));     // (codes were multiplied where they lie in their byte)
     float x = mine ? a.x[f_own] : 0.0f;
     auto draw = [&](int k, uint32_t stream) { return slice_draw(a.seed, a.epoch, (uint32_t)a.first_step + (uint32_t)k, (uint32_t)f_own, stream); };
 
@@ -415,22 +414,21 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
             for (int o = 1; o < P; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
             const int2 halves = sh->rsum[step & 1];
             if (tid == 0) sh->rsum[(step + 1) & 1] = make_int2(0, 0);
-            const long long all_r = halves.x + 65536ll * halves.y;
-            float g = fmaf(st_low, (float)(sum - all_r * (c0 << shift)), mid * (float)all_r) * delta_r;
+            double t = fma(st_low, (double)sum, lo_double * slice_double(halves.x, halves.y)) * (double)delta_r;
             if constexpr (MANY) {
                 const uint32_t tag = a.tag + (uint32_t)step;
                 unsigned long long* box = a.exchange + ((size_t)(step & 1) * a.clusters * a.nb * F + f_own) * 2;
                 const size_t stride = (size_t)a.nb * F * 2;
-                if (writes) slice_post(box + cl * stride, g, 0.0f, tag);
-                double t = 0.0;
+                const float hi = (float)t, low = (float)(t - (double)hi);
+                if (writes) slice_post(box + cl * stride, hi, low, tag);
+                t = 0.0;
                 if (mine)
 #pragma unroll 1
-                    for (int c = pp; c < a.clusters; c += P) t += c == cl ? (double)g : slice_collect(sh, box + c * stride, tag, a.status);
+                    for (int c = pp; c < a.clusters; c += P) t += c == cl ? (double)hi + (double)low : slice_collect(sh, box + c * stride, tag, a.status);
 #pragma unroll 1
                 for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                g = (float)t;
             }
-            g *= batch_full ? a.full_scale : a.last_scale;
+            float g = (float)(t * (batch_full ? a.full_scale : a.last_scale));
             if (last && a.grad_out && writes && cl == 0) a.grad_out[f_own] = g;
             if (step < marked) slice_mark(a.trace, step, 6);
             if (a.grad_bits > 0) {
@@ -590,7 +588,7 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     a.batch = B;
     a.first_step = first_step; a.num_steps = num_steps;
     a.whole = (int)(d->m / B); a.rows_last = (int)(d->m - a.whole * B);
-    a.full_scale = (float)(1.0 / (2.0 * (double)B)); a.last_scale = (float)(1.0 / (2.0 * (double)(a.rows_last > 0 ? a.rows_last : 1)));
+    a.full_scale = 1.0 / (2.0 * (double)B); a.last_scale = 1.0 / (2.0 * (double)(a.rows_last > 0 ? a.rows_last : 1));
     a.seed = p->seed; a.epoch = (uint32_t)p->epoch; a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
     a.n = (int)d->n; a.bits = d->bits; a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
     if (many) {

@@ -439,6 +439,7 @@ FORMS = {                                                            # engine, c
     "features": (binding.ENGINE_CLUSTER, 4, 8, 500, 70, 0, False), "features-clusters": (binding.ENGINE_CLUSTER, 4, 4, 500, 300, 3, False),
     "rows": (binding.ENGINE_CLUSTER, 3, 8, 500, 70, 0, False), "rows-blocks": (binding.ENGINE_CLUSTER, 3, 4, 64, 900, 1, False),
     "rows-chunks": (binding.ENGINE_CLUSTER, 3, 8, 1000, 5000, 1, False), "rows-clusters": (binding.ENGINE_CLUSTER, 3, 2, 500, 900, 2, False),
+    "rows-few-chunks": (binding.ENGINE_CLUSTER, 3, 8, 1999, 2000, 1, False),
     "table-features": (binding.ENGINE_CLUSTER, 2, 3, 500, 70, 0, True), "fp32": (binding.ENGINE_CLUSTER, 1, 8, 500, 70, 0, False),
     "table-rows": (binding.ENGINE_CLUSTER, 1, 2, 100, 300, 0, True), "column": (binding.ENGINE_COLUMN, 0, 4, 9001, 64, 0, False),
     "stream": (binding.ENGINE_STREAM, 0, 2, 9403, 40, 0, False), "ring": (binding.ENGINE_RING, 0, 8, 3300, 250, 0, False),
@@ -465,6 +466,56 @@ def test_values_that_are_not_numbers_reach_gradient_and_model(ctx, form, where):
     ctx.zipml_sgd_epoch(gds, to_dev(b, ctx), x, batch, 1e-3, engine=engine, cluster_contraction=contraction, grid_feature_parts=clusters, grad_out=g)
     ctx.zipml_sync()
     assert not torch.isfinite(g).any() and not torch.isfinite(x).any()
+
+
+def values64(ds, plane):
+    """Values of a plane in 64 bits, and its codes."""
+    codes = oracle.unpack_plane(plane, ds.n, ds.bits).astype(np.float64)
+    if ds.mode == oracle.UNIFORM:
+        return ds.feat_lo.astype(np.float64) + codes * ds.feat_step, codes
+    return np.take_along_axis(np.broadcast_to(ds.levels.astype(np.float64), (ds.m,) + ds.levels.shape), codes.astype(int)[:, :, None], 2)[:, :, 0], codes
+
+
+@pytest.mark.parametrize("form", ["features", "features-clusters"])
+@pytest.mark.parametrize("values", ["mostly-zeros", "both-signs", "apart-from-zero", "growing-residuals"])
+def test_a_gradient_has_the_precision_of_fp32_products(ctx, form, values):
+    """A step's gradient against 64 bits on rows that are mostly zeros, of both signs, far from zero, and with residuals that grow
+    from chunk to chunk.  Bound: a residual is
+    off by its own rounding to fp32 and by a rounding in each product of the dot (2^-24 of its size, products about the feature's value
+    nearest zero), a gradient entry by its rows' residuals and a rounding of its own.  Roundings of many rows and features do not add up in
+    size: a quarter of that, half of it where the sums of the products are fp32 as well."""
+    engine, contraction, bits, n, batch, clusters, table = FORMS[form]
+    rng = np.random.default_rng(5)
+    A = rng.uniform(-1, 1, (batch, n))
+    xs = rng.standard_normal(n) / np.sqrt(n)
+    if values == "mostly-zeros":
+        A, xs = np.where(rng.random((batch, n)) < 0.05, np.abs(A), 0.0), rng.random(n)
+    elif values == "apart-from-zero":
+        A = A + 5 * rng.standard_normal(n)
+    A = A.astype(np.float32)
+    b = (A @ xs + 0.05 * rng.standard_normal(batch)).astype(np.float32)
+    if values == "growing-residuals":
+        b += (rng.standard_normal(batch) * 2.0 ** (np.arange(batch) % 125 / 8)).astype(np.float32)
+    kw = dict(mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 64)[0]) if table else {}
+    ods = oracle.quantize(A, bits, seed=3, **kw)
+    x0 = (0.5 * xs).astype(np.float32)
+    x, g = to_dev(x0, ctx), torch.zeros((2, n), device=ctx.device)
+    ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-3, engine=engine, cluster_contraction=contraction,
+                        grid_feature_parts=clusters, grad_out=g)
+    ctx.zipml_sync()
+    want, bound, x64 = 0.0, 0.0, x0.astype(np.float64)
+    planes = [values64(ods, p) for p in (ods.plane1, ods.plane2)]
+    for (a, _), (q, codes) in (planes, planes[::-1]):
+        if table:
+            products = np.abs(q * x64)
+        else:
+            centre = np.clip(np.rint(-ods.feat_lo / np.where(ods.feat_step > 0, ods.feat_step, 1)), 0, (1 << bits) - 1)
+            products = np.abs((codes - centre) * ods.feat_step.astype(np.float64) * x64)
+        r = q @ x64 - b
+        want = want + a.T @ r / (2 * batch)
+        bound = bound + np.abs(a).T @ (np.abs(r) + products.sum(axis=1)) / (2 * batch) * 2.0 ** -24
+    bound = bound + np.abs(want) * 2.0 ** -24
+    assert np.linalg.norm(g[0].cpu().numpy() - want) <= (0.5 if engine == binding.ENGINE_SOLO else 0.25) * np.linalg.norm(bound)
 
 
 @pytest.mark.parametrize("contraction", [1, 2], ids=["fp32", "int8"])
