@@ -13,9 +13,11 @@
 //   * a warp per 16 rows adds them up, subtracts the labels and writes the residuals' digits: 16 rows of plane 1 with
 //     r2 and 16 rows of plane 2 with r1 are the 32 entries of one contraction;                                barrier
 //   * a warp takes 16-byte columns of one slice (transposing ldmatrix), multiplies, centres the sums (codes less half
-//     the top code: nothing cancels later) and bulk-copies its part of the gradient, a low and a high integer per feature,
-//     into the owner's shared memory;
-//   * the owner adds the nb parts in a fixed order, applies Q4, updates its fp32 slice, applies Q3;           barrier
+//     the top code) and bulk-copies its part of the gradient, a low and a high integer per feature, behind the sum of its
+//     residuals, into the owner's shared memory;
+//   * the owner adds the nb parts in a fixed order, in double from the integers on (the centred sums and the residuals' sum cancel on
+//     rows that are mostly zeros: joined in fp32 the gradient lost 10 to 25 times its precision there), applies Q4, updates its
+//     fp32 slice, applies Q3;                                                                                 barrier
 //     and publishes.
 // Codes of less than 8 bits are masked where they lie in their byte: the shift is in the digits (dots) or comes off the
 // sums (gradient).
@@ -23,7 +25,8 @@
 // shared memory, an odd number of 16-byte units (rows above 2 KB: a bulk copy each).
 // Larger minibatches take several clusters and several chunks of rows per CTA.  A CTA holds whole rows, so a chunk's dots,
 // residuals and gradient need nothing from the others: the codes are read once, and the gradient's parts add up in
-// shared memory until the last chunk.  The clusters hold replicas of the model: the owners of the same slice hand each
+// shared memory until the last chunk: as integers, whose unit the first chunk's residuals choose with two bits to spare (sums of fp32 lost
+// what the centre adds, sums of doubles cost 6 % at 8,192 x 1,999 at 8 bits), or as doubles over more rows than the integers hold.  The clusters hold replicas of the model: the owners of the same slice hand each
 // other their sums through L2 (self-validating 8-byte words, two buffers in turn) and add them in the same order.
 // Buffer reuse: a CTA sends its part of step t after its warps have read the digits of step t (first barrier), and an
 // owner publishes after all parts have arrived: digits, parts and their sources are free when they are written again.
@@ -83,7 +86,8 @@ struct alignas(16) SliceShared {
     uint64_t full[kSliceMaxSlots], empty[kSliceMaxSlots];
     uint64_t w_bar[kSliceMaxCtas];   // a slice's digits have arrived
     uint64_t part_bar, gn_bar, xn_bar;
-    float delta_r;               // value of a unit of the residuals' fixed point
+    float delta_r;               // value of a unit of the residuals' fixed point, not a number where a residual is none
+    int k_r;                     // else it is 2^-k_r
     float wmax[32];              // owner: per-warp maxima of |w|
     uint32_t rmax[16];           // maxima of |residual| of a row block, as bit patterns
     int gave_up;
@@ -93,13 +97,16 @@ struct alignas(16) SliceShared {
 //   wd[owners][sps NG 32 + 4]  words: digits of w [slab][group][t][half][digit], then the scale and lo^T x~ (doubles)
 //   psum[owners a_parts][rb][32]  doubles: partial dots in the order of the residuals' contraction
 //   rdig[rb][32]  words: digits of the residuals [t][half][digit... ] as B fragments
-//   gpart[owners][4 + 2 SF]  this CTA's part of the gradient, slice by slice, behind its sum of residuals and their scale
+//   gpart[owners][4 + 2 SF]  this CTA's part of the gradient, slice by slice, behind its sum of residuals and the sums' unit, two
+//                          doubles: integers, or (MODE 2) doubles without a unit
 //   gbuf[nb][4 + 2 SF]       the parts of the own slice
 //   wv[SF]                 w of the own slice
 //   ring[slots]: codes [2][16 rb][pitch], 128 bytes of slack
-template <int CB, int RBC, bool MANY>
+// MODE: 0 = one chunk in one cluster, else several: 1 = of at most fifteen row blocks together, 2 = of more.
+template <int CB, int RBC, int MODE>
 __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const SliceArgs a, const __grid_constant__ CUtensorMap tm1,
                                                                      const __grid_constant__ CUtensorMap tm2) {
+    constexpr bool MANY = MODE > 0;
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
     constexpr int CT = NG == 1 ? 2 : 1;                  // columns that a warp takes at once in the gradient
     static_assert(NS == 4, "a thread stores four digits at once");
@@ -203,17 +210,17 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     const int P = 1 << a.p_shift, pp = tid & (P - 1), k_own = tid >> a.p_shift;
     const int f_own = bi * SF + k_own;
     const bool mine = owner && k_own < SF && f_own < n;
-    const float c0f = (float)(1 << (a.bits - 1));
     const int c0 = 1 << (a.bits - 1);
     const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
-    const float mid = fmaf(c0f, st, lof);
-    const float st_low = st / (float)(1 << (CB * (k_own % NG)));    // (codes were multiplied where they lie in their byte)
+    const double mid = fma((double)c0, (double)st, (double)lof);
+    const double st_low = (double)st / (double)(1 << (CB * (k_own % NG)));    // (codes were multiplied where they lie in their byte)
     float x = mine ? a.x[f_own] : 0.0f;
     auto draw = [&](int k, uint32_t stream) { return slice_draw(a.seed, a.epoch, (uint32_t)a.first_step + (uint32_t)k, (uint32_t)f_own, stream); };
 
     const int marked = blockIdx.x == 0 && tid == 0 && a.trace ? a.trace_steps : -1;
     int slot = 0;
     uint32_t parity = 0, w_parity = 0, part_parity = 0, gn_parity = 0, xn_parity = 0;
+    int k_sum = 0;                                       // MODE 1: the unit of the sums over a step's chunks is 2^-k_sum
 #pragma unroll 1
     for (int step = -1; step < steps; ++step) {
         const bool last = step == steps - 1;
@@ -315,8 +322,9 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                     for (int w2 = 0; w2 < rb; ++w2) top_bits = max(top_bits, sh->rmax[w2]);
                 }
                 const float top = __uint_as_float(top_bits);
-                const int k_r = slice_exponent(top, 0);
-                if (tid == 0) sh->delta_r = top <= 3.402823466e+38f ? slice_pow2(-k_r) : __int_as_float(0x7fffffff);
+                int k_r = slice_exponent(top, 0);
+                if constexpr (MODE == 1) k_r = chunk > 0 && k_r >= k_sum ? k_sum : slice_exponent(top, 2);   // (two bits for the chunks to come)
+                if (tid == 0) { sh->delta_r = top <= 3.402823466e+38f ? slice_pow2(-k_r) : __int_as_float(0x7fffffff); sh->k_r = k_r; }
                 const uint32_t digits = ((uint32_t)__float2int_rn(r * slice_pow2(k_r)) + 0x80808080u) ^ 0x80808080u;
                 unsigned char* out = reinterpret_cast<unsigned char*>(rdig + warp * 32) + ((lane >> 2) & 3) * 32 + (lane >> 4) * 16 + (lane & 3);
 #pragma unroll
@@ -332,6 +340,9 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
             if (step < marked) slice_mark(a.trace, step, 2);
 
             // -------------------------------------------------------------- the rows' part of the gradient
+            const double unit_r = (double)sh->delta_r;
+            const int k_r = sh->k_r, coarser = MODE == 1 && chunk > 0 ? min(63, k_sum - k_r) : 0;    // bits that the sums so far come down
+            k_sum = k_r;
 #pragma unroll 1
             for (int unit = warp; unit < owners * a.b_parts; unit += kSliceWarps) {
                 const int b_slice = (unit * a.b_inv) >> 16, bj = unit - b_slice * a.b_parts;     // unit / b_parts
@@ -344,15 +355,21 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 #pragma unroll 1
                 for (int kb = 0; kb < rb; ++kb)
                     mma_u8s8(ones, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, gl < NS ? rq[kb * 32] : 0u, gl < NS ? rq[kb * 32 + 4] : 0u);
-                const float delta_r = sh->delta_r;
-                if (bj == 0) {                           // the sum of the residuals
-                    const float s = (float)(ones[0] + 256 * ones[1]) * delta_r;
-                    const float upper = __shfl_down_sync(0xffffffffu, s, 1);
+                if (bj == 0) {                           // the sum of the residuals, and the unit of the features' sums
+                    const int s = ones[0] + 256 * ones[1], upper = __shfl_down_sync(0xffffffffu, s, 1);
                     if (lane == 0) {
-                        float2* head = reinterpret_cast<float2*>(part);
-                        const float all = fmaf(upper, 65536.0f, s);
-                        *head = MANY ? make_float2(chunk > 0 ? head->x + all : all, 1.0f) : make_float2(all, delta_r);
+                        double2* head = reinterpret_cast<double2*>(part);
+                        *head = make_double2(fma(slice_double(s, upper), unit_r, MANY && chunk > 0 ? head->x : 0.0), __hiloint2double((1023 - k_r) << 20, 0));
                     }
+                }
+                if (MODE == 1 && coarser > 0) {          // (seldom: a chunk's largest residual is four times the earlier ones')
+#pragma unroll 1
+                    for (int w = 4 + col_begin * 32 * NG + 2 * lane; w < 4 + col_end * 32 * NG; w += 64) {
+                        int2* pair = reinterpret_cast<int2*>(part + w);
+                        const long long v = (pair->x + 65536ll * pair->y) >> coarser;
+                        *pair = make_int2((int)(v & 0xffff), (int)(v >> 16));
+                    }
+                    __syncwarp();
                 }
 #pragma unroll 1
                 for (int col0 = col_begin; col0 < col_end; col0 += CT) {
@@ -390,15 +407,13 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                                 int* out = part + 4 + 2 * (((col0 + ti) * 16 + 2 * gl) * NG + g) + tl;
                                 // lane t = 0 has the lower digits, t = 1 the upper ones (fifteen row blocks at most: below 2^31)
                                 const int first = acc[ti][g][0] + 256 * acc[ti][g][1], second = acc[ti][g][2] + 256 * acc[ti][g][3];
-                                if (tl < 2) {
-                                    if constexpr (MANY) {          // chunks have scales of their own: they add up as floats
-                                        float* sum = reinterpret_cast<float*>(out);
-                                        sum[0] = fmaf((float)first, delta_r, chunk > 0 ? sum[0] : 0.0f);
-                                        sum[2 * NG] = fmaf((float)second, delta_r, chunk > 0 ? sum[2 * NG] : 0.0f);
-                                    } else {
-                                        out[0] = first;
-                                        out[2 * NG] = second;
-                                    }
+                                if constexpr (MODE == 2) {         // (chunks with scales of their own, a feature to a lane)
+                                    const int got = __shfl_xor_sync(0xffffffffu, tl == 0 ? second : first, 1);
+                                    double* sum = reinterpret_cast<double*>(out - tl + 2 * NG * tl);
+                                    if (tl < 2) *sum = fma(slice_double(tl == 0 ? first : got, tl == 0 ? got : second), unit_r, chunk > 0 ? *sum : 0.0);
+                                } else if (tl < 2) {
+                                    out[0] = (MODE == 1 && chunk > 0 ? out[0] : 0) + first;
+                                    out[2 * NG] = (MODE == 1 && chunk > 0 ? out[2 * NG] : 0) + second;
                                 }
                             }
                         }
@@ -423,15 +438,21 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
                 slice_wait(sh, &sh->part_bar, part_parity, a.status, 2);
                 part_parity ^= 1u;
                 if (tid == 0 && !last) mbar_arrive_expect_tx(&sh->part_bar, part_bytes);
-                double t = 0.0;
+                double t = 0.0, all = 0.0;               // sums of the codes and of the residuals
                 if (mine)
 #pragma unroll 2
                     for (int w = pp; w < a.nb; w += P) {
-                        const int2 v = *reinterpret_cast<const int2*>(gbuf + w * part_words + 4 + 2 * k_own);
-                        const float2 h = *reinterpret_cast<const float2*>(gbuf + w * part_words);
-                        if constexpr (MANY) t += (double)fmaf(st_low, fmaf(__int_as_float(v.y), 65536.0f, __int_as_float(v.x)), mid * h.x);
-                        else t += (double)fmaf(st_low, fmaf((float)v.y, 65536.0f, (float)v.x) * h.y, mid * h.x);
+                        const int* part = gbuf + w * part_words;
+                        const double2 h = *reinterpret_cast<const double2*>(part);
+                        if constexpr (MODE == 2) {
+                            t += reinterpret_cast<const double*>(part)[2 + k_own];
+                        } else {
+                            const int2 v = *reinterpret_cast<const int2*>(part + 4 + 2 * k_own);
+                            t = fma(slice_double(v.x, v.y), h.y, t);
+                        }
+                        all += h.x;
                     }
+                t = fma(st_low, t, mid * all);
 #pragma unroll 1
                 for (int o = 1; o < P; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
                 if (MANY && a.clusters > 1) {
@@ -589,10 +610,14 @@ static int make_slice_plan(const zipml_ctx* ctx, const zipml_dataset* d, const z
     return ZIPML_ERR_WORKSPACE;
 }
 
+template <int CB, int RBC>
+static const void* slice_kernel(int mode) {
+    return mode == 0 ? (const void*)sgd_slice_kernel<CB, RBC, 0> : mode == 1 ? (const void*)sgd_slice_kernel<CB, RBC, 1> : (const void*)sgd_slice_kernel<CB, RBC, 2>;
+}
 template <int CB>
-static const void* slice_kernel(int rb, bool many) {
-    if (many) return rb == 1 ? (const void*)sgd_slice_kernel<CB, 1, true> : (const void*)sgd_slice_kernel<CB, 2, true>;
-    return rb == 1 ? (const void*)sgd_slice_kernel<CB, 1, false> : (const void*)sgd_slice_kernel<CB, 2, false>;
+static const void* slice_kernel(const SlicePlan& r) {
+    const int mode = r.clusters == 1 && r.chunks == 1 ? 0 : (r.rc + 15) / 16 <= 15 ? 1 : 2;
+    return r.rb == 1 ? slice_kernel<CB, 1>(mode) : slice_kernel<CB, 2>(mode);
 }
 
 int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
@@ -608,8 +633,7 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     for (int most = kSliceMaxClusters;;) {
         rc = make_slice_plan(ctx, d, p, ctx->cooperative ? most : 1, &plan);
         if (rc != ZIPML_OK) return rc;
-        const bool many = plan.clusters > 1 || plan.chunks > 1;
-        kernel = cb == 2 ? slice_kernel<2>(plan.rb, many) : cb == 4 ? slice_kernel<4>(plan.rb, many) : slice_kernel<8>(plan.rb, many);
+        kernel = cb == 2 ? slice_kernel<2>(plan) : cb == 4 ? slice_kernel<4>(plan) : slice_kernel<8>(plan);
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
         if (e == cudaSuccess && plan.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return cuda_status(e);
