@@ -14,13 +14,19 @@
 //   * the code tiles do not depend on the model: an extra warp runs a few steps ahead with cp.async copies into a ring
 //     of slots.  Rows lie `pitch` words apart, chosen with the lane splits (make_solo_plan) so that lanes on
 //     different rows meet different banks.
-// Codes are centred (value = mid + (code - c0) * step, c0 half the top code): the dot's two parts, mid^T x~ and the
-// codes', stay small instead of cancelling, and fp32 sums keep their precision.
+// Codes are centred per feature (value = mid + (code - centre) * step, the centre the code whose value is nearest zero): the
+// dot's two parts, mid^T x~ and the codes', stay small instead of cancelling, and fp32 sums of a lane keep their
+// precision -- on features of both signs as on rows that are mostly zeros, where one centre for all (half the top code) lost 10 to
+// 20 times of it.  The lanes' sums of a dot meet in double.  Where a feature lies apart from zero by more than its step ("far", found out
+// once per launch), mid^T x~ and the sum of the residuals are held in double too; elsewhere |mid| <= step and fp32 adds no
+// more than the codes' own rounding.
 // What bounds it: the latency of the chain load - unpack - FMA - butterfly - barrier, twice a step.
-// Measured, us per step, cluster engine -> here: 16 x 64 at 4 bits 3.65 -> 1.58, 256 x 16 at 8 bits 3.94 -> 2.24, 16 x
-// 1,000 at 8 bits 4.80 -> 3.68, 16 x 250 on 3-bit tables 3.80 -> 2.48; 64 x 64 at 4 bits with quantized model and
-// gradient 6.33 -> 3.58.
+// Measured, us per step of 200, cluster engine split by rows -> here: 16 x 64 at 4 bits 3.75 -> 1.08 (1.00 with one centre for all and every
+// sum in fp32), 64 x 64 at 8 bits 3.75 -> 1.45, 16 x 250 on 2-bit tables 4.27 -> 1.87; 64 x 64 at 4 bits with quantized model and
+// gradient 6.23 -> 3.00.
 #include <string.h>
+
+#include <type_traits>
 
 #include "sgd_common.cuh"
 
@@ -51,7 +57,7 @@ struct SoloArgs {
     int model_bits, grad_bits;
     int rc;                      // rows of a full batch
     int pitch;                   // words between rows of a tile in shared memory
-    int slots;                   // tiles in the ring (at least 2)
+    int slots;                   // tiles in the ring
     int a_shift;                 // 2^a_shift lanes share a row's dots
     int b_shift;                 // 2^b_shift lanes share a word column's gradient
     int copy_shift;              // 2^copy_shift lanes share the copy of a row
@@ -62,27 +68,38 @@ struct SoloShared {
     uint64_t full[kSoloMaxSlots], empty[kSoloMaxSlots];
     int rows[kSoloMaxSlots];     // rows of the slot's tile
     int gave_up;
+    int far;                     // a feature lies apart from zero by more than its step
 };
 constexpr size_t kSoloSharedBytes = (sizeof(SoloShared) + 15) & ~(size_t)15;
 
-// Codes of a word as floats minus c0 (bias = 2^23 + c0).
+// Codes of a word as floats minus their centres (bias = 2^23 + centre).
 template <int CB>
-__device__ __forceinline__ void unpack_centred(uint32_t w, float bias, float (&c)[32 / CB]) {
-    auto byte = [&](uint32_t bytes, int i) { return __uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7650 + i)) - bias; };
+__device__ __forceinline__ void unpack_centred(uint32_t w, const float (&bias)[32 / CB], float (&c)[32 / CB]) {
+    auto byte = [&](uint32_t bytes, int i, int f) { c[f] = __uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7650 + i)) - bias[f]; };
     if constexpr (CB == 8) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) c[i] = byte(w, i);
+        for (int i = 0; i < 4; ++i) byte(w, i, i);
     } else if constexpr (CB == 4) {
         const uint32_t even = w & 0x0F0F0F0Fu, odd = (w >> 4) & 0x0F0F0F0Fu;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { c[2 * i] = byte(even, i); c[2 * i + 1] = byte(odd, i); }
+        for (int i = 0; i < 4; ++i) { byte(even, i, 2 * i); byte(odd, i, 2 * i + 1); }
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const uint32_t t = (w >> (2 * k)) & 0x03030303u;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) c[4 * i + k] = byte(t, i);
+            for (int i = 0; i < 4; ++i) byte(t, i, 4 * i + k);
         }
+    }
+}
+
+// A word's entries of a quad array (see below).
+template <int FPW>
+__device__ __forceinline__ void solo_quads(float (&v)[FPW], const float4* quads, int nwq, int q) {
+#pragma unroll
+    for (int i = 0; i < FPW / 4; ++i) {
+        const float4 t = quads[i * nwq + q];
+        v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
     }
 }
 
@@ -124,7 +141,8 @@ __device__ __forceinline__ void solo_wait(SoloShared* sh, uint64_t* bar, uint32_
 // Shared memory; nwq = words rounded up to 8, a "quad array" holds 4 FPW nwq bytes as float4 [FPW / 4][nwq], feature
 // i of word q in component i & 3 of element [i >> 2][q] (lanes on neighbouring words read neighbouring 16 bytes):
 //   SoloShared
-//   quad arrays   ws (uniform: step * x~; table: x~) and for uniform grids mx (mid * x~)
+//   quad arrays   ws (uniform: step * x~; table: x~) and for uniform grids centre (2^23 + the feature's centre)
+//   uniform       mid^T x~: a quad array, or (far) doubles mx [FPW / KEEP][nwq], an owner's features' part each
 //   table         lev [L][FPW][nwq]
 //   float res[2 rc]        residuals (r1, r2) per row
 //   ring[slots]: codes [2][rc][pitch], labels [rc]
@@ -136,9 +154,10 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
     const int nw = a.words, nwq = (nw + 7) & ~7, n = a.n, L = 1 << a.bits, F = nwq * FPW;
     SoloShared* sh = reinterpret_cast<SoloShared*>(s_raw);
     float* ws = reinterpret_cast<float*>(s_raw + kSoloSharedBytes);
-    float* mx = ws + F;
-    float* lev = mx + (TABLE ? 0 : F);
-    float* res = lev + (TABLE ? L * F : 0);
+    float* centre = ws + F;
+    double* mx = reinterpret_cast<double*>(centre + (TABLE ? 0 : F));
+    float* lev = ws + F;
+    float* res = TABLE ? lev + L * F : reinterpret_cast<float*>(mx + F / (KEEP < 2 ? KEEP : 2));
     uint32_t* ring = reinterpret_cast<uint32_t*>(res + ((2 * a.rc + 3) & ~3));
     const int plane_words = a.rc * a.pitch, slot_words = 2 * plane_words + ((a.rc + 3) & ~3);
     if (tid < a.slots) {
@@ -146,7 +165,7 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         mbar_init(sh->empty + tid, 1);
         sh->rows[tid] = a.rc;
     }
-    if (tid == 0) sh->gave_up = 0;
+    if (tid == 0) sh->gave_up = sh->far = 0;
     // (a wait that has given up computes on whatever lies in its slot: no code may then point past the table)
     if (TABLE && L < (1 << CB))
         for (int i = tid; i < a.slots * slot_words; i += blockDim.x) ring[i] = 0u;
@@ -181,7 +200,6 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
     }
 
     // ---------------------------------------------------------------------- the computing warps
-    const float bias = 8388608.0f + (float)(1 << (a.bits - 1)), c0 = (float)(1 << (a.bits - 1));
     // the features that the butterfly over a word column leaves in this lane: KEEP consecutive ones, from `first` on
     const int GA = 1 << a.a_shift, GB = 1 << a.b_shift;
     const int la = tid & (GA - 1), lb = tid & (GB - 1), row_first = tid >> a.a_shift, row_stride = threads >> a.a_shift;
@@ -192,13 +210,14 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         if (s < a.b_shift && (lb >> s & 1)) first += FPW >> (s + 1);
     const int f0 = q * FPW + first, at0 = ((first >> 2) * nwq + q) * 4 + (first & 3);
     const bool owner = (tid >> a.b_shift) < nw && (lb >> LOGF) == 0;
-    float x[KEEP], st[KEEP], mid[KEEP];
+    float x[KEEP], st[KEEP];
+    double mid[KEEP];
     for (int f = tid; f < F; f += threads) ws[f] = 0.0f;           // (slots past the last feature stay zero)
     if constexpr (TABLE) {
         for (int f = tid; f < F; f += threads)
             for (int c = 0; c < L; ++c) lev[(c * FPW + (f & (FPW - 1))) * nwq + (f >> LOGF)] = f < n ? __ldg(a.levels + (size_t)f * L + c) : 0.0f;
     } else {
-        for (int f = tid; f < F; f += threads) mx[f] = 0.0f;
+        for (int f = tid; f < F; f += threads) { centre[f] = 8388608.0f; reinterpret_cast<float*>(mx)[f] = 0.0f; }
     }
     auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); };
     // l2 norm of the owners' values, summed in double in a fixed order
@@ -223,26 +242,43 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         }
     };
     // what the next step's dots see of the model
-    auto publish = [&](const float (&v)[KEEP], bool seen_last) {
+    auto publish = [&](auto far, const float (&v)[KEEP], bool seen_last) {
         if (!owner) return;
 #pragma unroll
         for (int k = 0; k < KEEP; ++k)
             if (f0 + k < n) {
                 if (seen_last && a.model_out) a.model_out[f0 + k] = v[k];
                 if constexpr (TABLE) ws[at0 + k] = v[k];
-                else { ws[at0 + k] = st[k] * v[k]; mx[at0 + k] = mid[k] * v[k]; }
+                else {
+                    ws[at0 + k] = st[k] * v[k];
+                    if constexpr (!decltype(far)::value) reinterpret_cast<float*>(mx)[at0 + k] = (float)mid[k] * v[k];
+                }
             }
+        if constexpr (!TABLE && decltype(far)::value) {
+            double base = 0.0;
+#pragma unroll
+            for (int k = 0; k < KEEP; ++k) base = fma(mid[k], (double)v[k], base);
+            mx[first / KEEP * nwq + q] = base;
+        }
     };
     bar();                                                         // the zeros are in place
+    bool far_lane = false;
 #pragma unroll
     for (int k = 0; k < KEEP; ++k) {
         const bool real = f0 + k < n;
         x[k] = real ? a.x[f0 + k] : 0.0f;
         if constexpr (!TABLE) {
             st[k] = real ? __ldg(a.step + f0 + k) : 0.0f;
-            mid[k] = real ? fmaf(c0, st[k], __ldg(a.lo + f0 + k)) : 0.0f;
+            const float lo = real ? __ldg(a.lo + f0 + k) : 0.0f;
+            // (any whole number would do: how the quotient is rounded does not matter)
+            const float c = fminf(fmaxf(rintf(__fdividef(-lo, st[k])), 0.0f), (float)((1 << a.bits) - 1));
+            mid[k] = fma((double)c, (double)st[k], (double)lo);
+            far_lane = far_lane || fabs(mid[k]) > (double)st[k];
+            if (owner) centre[at0 + k] = 8388608.0f + c;
         }
     }
+    auto run = [&](auto far) {
+    constexpr bool FAR = decltype(far)::value;
     if (a.model_bits > 0) {
         uint32_t u[KEEP];
         draws(a.first_step, 3u, u);
@@ -250,17 +286,25 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         float v[KEEP];
 #pragma unroll
         for (int k = 0; k < KEEP; ++k) v[k] = solo_quantize(x[k], M, a.model_bits, u[k]);
-        publish(v, a.num_steps == 1);
+        publish(far, v, a.num_steps == 1);
     } else {
-        publish(x, a.num_steps == 1);
+        publish(far, x, a.num_steps == 1);
     }
     bar();
 
     const float full_scale = 1.0f / (2.0f * (float)a.rc);
     const bool single = nw <= GA;                                  // a lane has one word of w: it keeps it for all its rows
     const float4* w4 = reinterpret_cast<const float4*>(ws) + (single ? min(la, nw - 1) : 0);
-    const float4* m4 = reinterpret_cast<const float4*>(mx);
+    [[maybe_unused]] const float4* c4 = reinterpret_cast<const float4*>(centre);
+    [[maybe_unused]] const float4* m4 = reinterpret_cast<const float4*>(mx);
     const int stride_shift = 31 - __clz(row_stride);               // (threads is a power of two)
+    // of the lane's word in the dots (where it has one), in the gradient; of 16 codes to a word anew in every step: too many registers
+    constexpr bool kKept = !TABLE && FPW <= 8;
+    [[maybe_unused]] float bias_a[FPW], bias_b[FPW];
+    if constexpr (kKept) {
+        solo_quads<FPW>(bias_a, c4, nwq, min(la, nw - 1));
+        solo_quads<FPW>(bias_b, c4, nwq, q);
+    }
     int slot = 0;
     uint32_t parity = 0;
 #pragma unroll 1
@@ -273,7 +317,7 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         const int rows = sh->rows[slot];
 
         // ---------------------------------------------------------------- dots and residuals
-        auto add_word = [&](int at, int col, const float (&w)[FPW], float& a1, float& a2) {
+        auto add_word = [&](int at, int col, const float (&w)[FPW], const float (&bias)[FPW], float& a1, float& a2) {
             const uint32_t u1 = t1[at], u2 = t2[at];
             if constexpr (!TABLE) {
                 float c1[FPW], c2[FPW];
@@ -289,44 +333,48 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
                 }
             }
         };
+        // mid^T x~ over the lane's words
+        float base = 0.0f;
+        [[maybe_unused]] double base_far = 0.0;
+        if constexpr (!TABLE) {
+            for (int c = la; c < nw; c += GA)
+                if constexpr (FAR) {
+#pragma unroll
+                    for (int i = 0; i < FPW / KEEP; ++i) base_far += mx[i * nwq + c];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < FPW / 4; ++i) { const float4 u = m4[i * nwq + c]; base += (u.x + u.y) + (u.z + u.w); }
+                }
+        }
         // the two dots of a row from the parts of its lanes: a residual each in its lanes 0 and 1
         auto finish_row = [&](int r, float label, float a1, float a2) {
             if (a.a_shift > 0) {
                 const bool odd = lane & 1;
-                float d = (odd ? a2 : a1) + __shfl_xor_sync(0xffffffffu, odd ? a1 : a2, 1);
+                double d = (double)(odd ? a2 : a1) + (double)__shfl_xor_sync(0xffffffffu, odd ? a1 : a2, 1);
+                if constexpr (FAR) d += base_far + __shfl_xor_sync(0xffffffffu, base_far, 1);
 #pragma unroll
                 for (int o = 2; o < 32; o <<= 1)
                     if (o < GA) d += __shfl_xor_sync(0xffffffffu, d, o);
-                if (la < 2 && r < rows) res[2 * r + la] = d - label;
+                if (la < 2 && r < rows) res[2 * r + la] = (float)(d - (double)label);
             } else if (r < rows) {
-                *reinterpret_cast<float2*>(res + 2 * r) = make_float2(a1 - label, a2 - label);
+                const double rest = base_far - (double)label;
+                *reinterpret_cast<float2*>(res + 2 * r) = make_float2((float)((double)a1 + rest), (float)((double)a2 + rest));
             }
         };
         const int row_turns = (rows + row_stride - 1) >> stride_shift;
         if (single) {
-            float w[FPW], base = 0.0f;
-#pragma unroll
-            for (int i = 0; i < FPW / 4; ++i) {
-                const float4 v = w4[i * nwq];
-                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
-                if constexpr (!TABLE) { const float4 u = m4[i * nwq + min(la, nw - 1)]; base += (u.x + u.y) + (u.z + u.w); }
-            }
+            float w[FPW];
+            solo_quads<FPW>(w, w4, nwq, 0);
+            if constexpr (!TABLE && !kKept) solo_quads<FPW>(bias_a, c4, nwq, min(la, nw - 1));
 #pragma unroll 2
             for (int turn = 0; turn < row_turns; ++turn) {
                 const int r = row_first + turn * row_stride, rr = min(r, rows - 1);     // (every lane takes part in the butterfly)
                 const float label = labels[rr];
                 float a1 = base, a2 = base;
-                if (la < nw) add_word(rr * a.pitch + la, la, w, a1, a2);
-                else a1 = a2 = 0.0f;
+                if (la < nw) add_word(rr * a.pitch + la, la, w, bias_a, a1, a2);
                 finish_row(r, label, a1, a2);
             }
         } else {
-            float base = 0.0f;
-            if constexpr (!TABLE) {
-                for (int c = la; c < nw; c += GA)
-#pragma unroll
-                    for (int i = 0; i < FPW / 4; ++i) { const float4 u = m4[i * nwq + c]; base += (u.x + u.y) + (u.z + u.w); }
-            }
 #pragma unroll 1
             for (int turn = 0; turn < row_turns; ++turn) {
                 const int r = row_first + turn * row_stride, rr = min(r, rows - 1);
@@ -334,13 +382,10 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
                 float a1 = base, a2 = base;
 #pragma unroll 2
                 for (int c = la; c < nw; c += GA) {
-                    float w[FPW];
-#pragma unroll
-                    for (int i = 0; i < FPW / 4; ++i) {
-                        const float4 v = w4[i * nwq + c];
-                        w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
-                    }
-                    add_word(rr * a.pitch + c, c, w, a1, a2);
+                    float w[FPW], bias[FPW];
+                    solo_quads<FPW>(w, w4, nwq, c);
+                    if constexpr (!TABLE) solo_quads<FPW>(bias, c4, nwq, c);
+                    add_word(rr * a.pitch + c, c, w, bias, a1, a2);
                 }
                 finish_row(r, label, a1, a2);
             }
@@ -348,10 +393,12 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         uint32_t u_g[KEEP], u_x[KEEP];
         if (a.grad_bits > 0) draws(it, 4u, u_g);
         if (a.model_bits > 0) draws(it + 1, 3u, u_x);
+        if constexpr (!TABLE && !kKept) solo_quads<FPW>(bias_b, c4, nwq, q);
         bar();
 
         // ---------------------------------------------------------------- gradient and update
-        float acc[FPW], sum = 0.0f;
+        float acc[FPW];
+        std::conditional_t<FAR, double, float> sum = 0;
 #pragma unroll
         for (int i = 0; i < FPW; ++i) acc[i] = 0.0f;
 #pragma unroll 2
@@ -360,8 +407,8 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
             const float2 rv = *reinterpret_cast<const float2*>(res + 2 * r);
             if constexpr (!TABLE) {
                 float c1[FPW], c2[FPW];
-                unpack_centred<CB>(u1, bias, c1);
-                unpack_centred<CB>(u2, bias, c2);
+                unpack_centred<CB>(u1, bias_b, c1);
+                unpack_centred<CB>(u2, bias_b, c2);
                 sum += rv.x + rv.y;
 #pragma unroll
                 for (int i = 0; i < FPW; ++i) acc[i] = fmaf(c1[i], rv.y, fmaf(c2[i], rv.x, acc[i]));
@@ -393,7 +440,7 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
         float g[KEEP];
 #pragma unroll
         for (int k = 0; k < KEEP; ++k) {
-            if constexpr (!TABLE) g[k] = fmaf(st[k], acc[k], mid[k] * sum) * scale;
+            if constexpr (!TABLE) g[k] = fmaf(st[k], acc[k], FAR ? (float)(mid[k] * sum) : (float)mid[k] * (float)sum) * scale;
             else g[k] = acc[k] * scale;
         }
         if (last && a.grad_out && owner)
@@ -419,14 +466,23 @@ __global__ void __launch_bounds__(kSoloMaxThreads + 32, 1) sgd_solo_kernel(const
             float v[KEEP];
 #pragma unroll
             for (int k = 0; k < KEEP; ++k) v[k] = solo_quantize(x[k], M, a.model_bits, u_x[k]);
-            publish(v, left == 2);
+            publish(far, v, left == 2);
         } else {
-            publish(x, left == 2);
+            publish(far, x, left == 2);
         }
         bar();
         if (tid == 0) mbar_arrive(sh->empty + slot);
         if (++slot == a.slots) { slot = 0; parity ^= 1u; }
     }
+    };
+    bool far = false;
+    if constexpr (!TABLE) {
+        if (far_lane) sh->far = 1;
+        bar();
+        far = *reinterpret_cast<volatile int*>(&sh->far) != 0;
+    }
+    if (far) run(std::integral_constant<bool, !TABLE>{});
+    else run(std::false_type{});
     if (owner)
 #pragma unroll
         for (int k = 0; k < KEEP; ++k)
@@ -444,7 +500,7 @@ struct SoloPlan {
 
 static size_t solo_smem_bytes(int cb, bool table, int bits, int words, int rc, int pitch, int slots) {
     const size_t F = (size_t)((words + 7) & ~7) * (32 / cb);
-    return kSoloSharedBytes + sizeof(float) * (F * (table ? 1 + ((size_t)1 << bits) : 2) + (size_t)((2 * rc + 3) & ~3) +
+    return kSoloSharedBytes + sizeof(float) * (F * (table ? 1 + ((size_t)1 << bits) : 4) + (size_t)((2 * rc + 3) & ~3) +
                                                (size_t)slots * (2 * (size_t)rc * pitch + (size_t)((rc + 3) & ~3)));
 }
 
@@ -485,9 +541,10 @@ static int make_solo_plan(const zipml_ctx* ctx, const zipml_dataset* d, const zi
     best->threads = 0;
     for (const int pad : {0, 4, 8, 16}) {
         const int pitch = row_words + pad;
+        // two tiles at least; one where the tallest tiles of the narrowest rows leave no more (they fit beside half the quad arrays)
         int slots = kSoloMaxSlots;
-        while (slots >= 2 && solo_smem_bytes(cb, table, d->bits, nw, B, pitch, slots) > (size_t)ctx->smem_optin) --slots;
-        if (slots < 2) break;
+        while (slots >= 1 && solo_smem_bytes(cb, table, d->bits, nw, B, pitch, slots) > (size_t)ctx->smem_optin) --slots;
+        if (slots < 2 && (pad > 0 || table || solo_smem_bytes(cb, table, d->bits, nw, B, pitch, 2) - 8 * (size_t)((nw + 7) & ~7) * fpw > (size_t)ctx->smem_optin)) break;
         for (int threads = 32; threads <= kSoloMaxThreads; threads *= 2) {
             const int warps = threads / 32;
             const double issue = warps <= 4 ? 2.0 : warps == 8 ? 2.4 : 4.0;    // cycles per instruction of a warp

@@ -476,7 +476,7 @@ def values64(ds, plane):
     return np.take_along_axis(np.broadcast_to(ds.levels.astype(np.float64), (ds.m,) + ds.levels.shape), codes.astype(int)[:, :, None], 2)[:, :, 0], codes
 
 
-@pytest.mark.parametrize("form", ["features", "features-clusters", "rows", "rows-blocks", "rows-chunks", "rows-clusters",
+@pytest.mark.parametrize("form", ["solo", "solo-table", "features", "features-clusters", "rows", "rows-blocks", "rows-chunks", "rows-clusters",
                                   "rows-few-chunks"])
 @pytest.mark.parametrize("values", ["mostly-zeros", "both-signs", "apart-from-zero", "growing-residuals"])
 def test_a_gradient_has_the_precision_of_fp32_products(ctx, form, values):
