@@ -21,6 +21,21 @@ struct IntPath {
     static constexpr int NG = 8 / CB;                              // groups of four codes in a 32-bit word
 };
 
+// The fixed point of values up to `top`: the largest power of two that keeps them within QMAX (a multiplication by it rounds
+// nothing; QMAX / top itself added a rounding of 2^-25 to every value, the same one for all rows of a step), and
+// its inverse; not a number where top is none.
+struct FixedPoint {
+    float scale;
+    double unit;
+};
+__device__ __forceinline__ FixedPoint fixed_point_of(float top, int qmax) {
+    int k = min(126, 26 - ((int)(__float_as_uint(top) >> 23) - 127));      // top 2^k below 2^27
+    float scale = __uint_as_float((uint32_t)(k + 127) << 23);
+    if (top * scale > (float)qmax) { --k; scale *= 0.5f; }
+    if (!(top > 0.0f)) return FixedPoint{0.0f, 0.0};
+    return FixedPoint{scale, top <= 3.402823466e+38f ? __hiloint2double((1023 - k) << 20, 0) : __longlong_as_double(0x7fffffffffffffffll)};
+}
+
 // The four codes of group g of a word, one per byte: byte b holds feature b * NG + g of the word.
 template <int CB>
 __device__ __forceinline__ uint32_t group_bytes(uint32_t u, int g) {

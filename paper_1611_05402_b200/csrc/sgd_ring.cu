@@ -222,7 +222,6 @@ __global__ void __launch_bounds__(kRingThreads, 1) sgd_ring_kernel(const SgdArgs
                                                                   const __grid_constant__ CUtensorMap tm2) {
     constexpr int FPW = 32 / CB;
     constexpr int NS = IntPath<CB>::NS, NG = IntPath<CB>::NG;
-    constexpr float QMAXF = (float)IntPath<CB>::QMAX;
     extern __shared__ __align__(16) unsigned char s_raw[];
     RingShared* sh = reinterpret_cast<RingShared*>(s_raw);
     const int L = 1 << a.bits;
@@ -395,18 +394,18 @@ __global__ void __launch_bounds__(kRingThreads, 1) sgd_ring_kernel(const SgdArgs
             base_w = 0.0;
 #pragma unroll
             for (int w = 0; w < kRingWarps; ++w) base_w += sh->wbase[w];
-            const float inv = wmax > 0.0f ? QMAXF / wmax : 0.0f;
+            const FixedPoint fp = fixed_point_of(wmax, IntPath<CB>::QMAX);
             if (have) {
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
                     // B operand of phase A: per k-slab (8 words), group and digit a 32-byte k vector
                     const float v4[4] = {wv[0 * NG + g], wv[1 * NG + g], wv[2 * NG + g], wv[3 * NG + g]};
-                    const uint4 o = digit_words<NS>(v4, inv);
+                    const uint4 o = digit_words<NS>(v4, fp.scale);
                     uint32_t* dst = wd32 + (size_t)(((q >> 3) * NG + g) * NS) * 8 + (q & 7);
                     dst[0] = o.x; dst[8] = o.y; dst[16] = o.z; dst[24] = o.w;
                 }
             }
-            return (double)wmax / (double)QMAXF;
+            return fp.unit;
         } else {
             if (have) {
 #pragma unroll
@@ -715,8 +714,8 @@ __global__ void __launch_bounds__(kRingThreads, 1) sgd_ring_kernel(const SgdArgs
             float rho = 0.0f;
 #pragma unroll
             for (int w = 0; w < kRingWarps; ++w) rho = fmaxf(rho, sh->fmax[16 + w]);
-            const float inv = rho > 0.0f ? QMAXF / rho : 0.0f;
-            delta_r = (double)rho / (double)QMAXF;
+            const FixedPoint fp = fixed_point_of(rho, IntPath<CB>::QMAX);
+            delta_r = fp.unit;
             // digits of the residuals as B operands of phase B: per 32 rows and residual, per digit, 32 bytes
             // in the row order the transposed code fragments come in (k = 16h + 4t + e <-> row 16h + 2t +
             // (e & 1) + 8 (e >> 1)); rows past the batch count as zero
@@ -730,7 +729,7 @@ __global__ void __launch_bounds__(kRingThreads, 1) sgd_ring_kernel(const SgdArgs
                     v1[e] = k < rcnt ? res[2 * k] : 0.0f;
                     v2[e] = k < rcnt ? res[2 * k + 1] : 0.0f;
                 }
-                const uint4 o1 = digit_words<NS>(v1, inv), o2 = digit_words<NS>(v2, inv);
+                const uint4 o1 = digit_words<NS>(v1, fp.scale), o2 = digit_words<NS>(v2, fp.scale);
                 uint32_t* d1 = rd32w + (size_t)((kk >> 3) * 2 * NS) * 8 + (kk & 7);
                 d1[0] = o1.x; d1[8] = o1.y; d1[16] = o1.z; d1[24] = o1.w;
                 d1[32] = o2.x; d1[40] = o2.y; d1[48] = o2.z; d1[56] = o2.w;

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) sgd_stream_kernel(const Str
 
     // own features into shared memory; digits of w for the first step, from the caller's model
     {
-        const float inv = bound > 0.0f ? (float)QMAX / bound : 0.0f;
+        const float inv = fixed_point_of(bound, QMAX).scale;
         for (int idx = tid; idx < own_n; idx += kStreamThreads) {
             const int bl = idx / NG, grp = idx - bl * NG;
             const int64_t byte = (int64_t)cb0 * CW + bl;
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) sgd_stream_kernel(const Str
             long long* z = a.dots + (size_t)((t_rel + 2) % 3) * 2 * a.bpad;
             for (int i = cta * kStreamThreads + tid; i < 2 * a.bpad; i += G * kStreamThreads) z[i] = 0;
         }
-        const double delta_w = (double)bound / (double)QMAX;
+        const double delta_w = fixed_point_of(bound, QMAX).unit;
         float rmax = 0.0f, pm = 0.0f;
         double pb = 0.0;
         if (t_rel > 0) {                   // the owners' parts of max |w| and lo^T x of the model this step saw
@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) sgd_stream_kernel(const Str
             block_reduce_mms(rmax, unused, none, shf, shd);
         }
         stream_mark(a, t_rel, 7);
-        const float inv_r = rmax > 0.0f ? (float)QMAX / rmax : 0.0f;
-        const double delta_r = (double)rmax / (double)QMAX;
+        const FixedPoint fixed_r = fixed_point_of(rmax, QMAX);
+        const float inv_r = fixed_r.scale;
+        const double delta_r = fixed_r.unit;
         double rsum = 0.0;                 // sum of all fixed-point residuals (exact in double)
         // a thread takes rows t, t+4, t+8, t+12 of a group of 16: their digits are one 32-bit word of pass B's operand
         for (int q4 = tid; q4 < a.bpad / 4; q4 += kStreamThreads) {
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) sgd_stream_kernel(const Str
         {
             const double scale = 1.0 / (2.0 * (double)bt);
             const double lo_term = delta_r * rsum;
-            const float inv = bound_next > 0.0f ? (float)QMAX / bound_next : 0.0f;
+            const float inv = fixed_point_of(bound_next, QMAX).scale;
             float pmax = 0.0f, unused = 0.0f;
             double pbase = 0.0;
             for (int idx = tid; idx < own_n; idx += kStreamThreads) {
