@@ -376,18 +376,19 @@ __global__ void __launch_bounds__(kRingThreads, 1) sgd_ring_kernel(const SgdArgs
     auto word_stage = [&](bool have, int q, const float (&xt)[FPW]) -> double {
         if constexpr (!TABLE) {
             float wv[FPW];
-            float lsum = 0.0f, m = 0.0f;
+            float m = 0.0f;
+            double lsum = 0.0;
 #pragma unroll
             for (int i = 0; i < FPW; ++i) {
                 const int f = q * FPW + i;
                 float sv = 0.0f, lv = 0.0f;
                 if (have && f < fcnt) { sv = __ldg(a.step + j0 + f); lv = __ldg(a.lo + j0 + f); }
                 wv[i] = sv * xt[i];
-                lsum = fmaf(lv, xt[i], lsum);
+                lsum = fma((double)lv, (double)xt[i], lsum);
                 m = fmaxf(m, fabsf(wv[i]));
             }
             {
-                const double wb = warp_sum((double)lsum);
+                const double wb = warp_sum(lsum);
                 if (lane == 0) sh->wbase[warp] = wb;
             }
             const float wmax = consumer_max(m, sh, 0);     // its barrier also publishes wbase
