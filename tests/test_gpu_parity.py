@@ -477,11 +477,11 @@ def values64(ds, plane):
 
 
 @pytest.mark.parametrize("form", ["solo", "solo-table", "features", "features-clusters", "rows", "rows-blocks", "rows-chunks", "rows-clusters",
-                                  "rows-few-chunks"])
-@pytest.mark.parametrize("values", ["mostly-zeros", "both-signs", "apart-from-zero", "growing-residuals"])
+                                  "rows-few-chunks", "column", "stream", "ring"])
+@pytest.mark.parametrize("values", ["mostly-zeros", "near-the-solution", "both-signs", "apart-from-zero", "growing-residuals"])
 def test_a_gradient_has_the_precision_of_fp32_products(ctx, form, values):
-    """A step's gradient against 64 bits on rows that are mostly zeros, of both signs, far from zero, and with residuals that grow
-    from chunk to chunk.  Bound: a residual is
+    """A step's gradient against 64 bits on rows that are mostly zeros (also with residuals that are small against the dots), of
+    both signs, far from zero, and with residuals that grow from chunk to chunk.  Bound: a residual is
     off by its own rounding to fp32 and by a rounding in each product of the dot (2^-24 of its size, products about the feature's value
     nearest zero), a gradient entry by its rows' residuals and a rounding of its own.  Roundings of many rows and features do not add up in
     size: a quarter of that, half of it where the sums of the products are fp32 as well."""
@@ -489,7 +489,7 @@ def test_a_gradient_has_the_precision_of_fp32_products(ctx, form, values):
     rng = np.random.default_rng(5)
     A = rng.uniform(-1, 1, (batch, n))
     xs = rng.standard_normal(n) / np.sqrt(n)
-    if values == "mostly-zeros":
+    if values in ("mostly-zeros", "near-the-solution"):
         A, xs = np.where(rng.random((batch, n)) < 0.05, np.abs(A), 0.0), rng.random(n)
     elif values == "apart-from-zero":
         A = A + 5 * rng.standard_normal(n)
@@ -499,7 +499,7 @@ def test_a_gradient_has_the_precision_of_fp32_products(ctx, form, values):
         b += (rng.standard_normal(batch) * 2.0 ** (np.arange(batch) % 125 / 8)).astype(np.float32)
     kw = dict(mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 64)[0]) if table else {}
     ods = oracle.quantize(A, bits, seed=3, **kw)
-    x0 = (0.5 * xs).astype(np.float32)
+    x0 = (xs if values == "near-the-solution" else 0.5 * xs).astype(np.float32)
     x, g = to_dev(x0, ctx), torch.zeros((2, n), device=ctx.device)
     ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-3, engine=engine, cluster_contraction=contraction,
                         grid_feature_parts=clusters, grad_out=g)
