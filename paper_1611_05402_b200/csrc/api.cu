@@ -29,18 +29,20 @@ int ws_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->ws, &ctx->ws_by
 int stage_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->stage, &ctx->stage_bytes, bytes, ctx->stream); }
 
 int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag) {
-    // tags go up from launch to launch, so the buffer is cleared only when it is new (or they would wrap)
-    const bool stale = ctx->exchange_bytes < bytes || ctx->exchange_tag > 0xffffffffu - (uint32_t)steps - 1u;
-    const int rc = grow(&ctx->exchange, &ctx->exchange_bytes, bytes, ctx->stream);
-    if (rc != ZIPML_OK) return rc;
-    if (stale) {
-        const cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, ctx->exchange_bytes, ctx->stream);
+    if (bytes > kExchangeBytes) return ZIPML_ERR_WORKSPACE;
+    // Tags go up from launch to launch, so the buffer is cleared only before they would wrap.  A launch that is recorded into a
+    // graph keeps its tags from replay to replay: there the clearing is recorded with it.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess) (void)cudaGetLastError();
+    const bool recorded = capture != cudaStreamCaptureStatusNone, wraps = ctx->exchange_tag > 0xffffffffu - (uint32_t)steps - 1u;
+    if (recorded || wraps) {
+        const cudaError_t e = cudaMemsetAsync(ctx->exchange, 0, kExchangeBytes, ctx->stream);
         if (e != cudaSuccess) return cuda_status(e);
-        ctx->exchange_tag = 1;
     }
     *buffer = reinterpret_cast<unsigned long long*>(ctx->exchange);
-    *tag = ctx->exchange_tag;
-    ctx->exchange_tag += (uint32_t)steps;
+    *tag = wraps ? 1u : ctx->exchange_tag;
+    // (a recorded clearing has not happened yet: the next launch that runs at once clears too)
+    ctx->exchange_tag = recorded && wraps ? 0xffffffffu : *tag + (uint32_t)steps;
     return ZIPML_OK;
 }
 
@@ -153,7 +155,14 @@ int zipml_create(zipml_ctx** ctx_out, int device, void* cuda_stream) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->cooperative, cudaDevAttrCooperativeLaunch, device);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->d_status), sizeof(DeviceStatus));
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_status, 0, sizeof(DeviceStatus), ctx->stream);
-    if (e != cudaSuccess) { if (ctx->d_status) (void)cudaFree(ctx->d_status); delete ctx; return cuda_status(e); }
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->exchange), kExchangeBytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->exchange, 0, kExchangeBytes, ctx->stream);
+    if (e != cudaSuccess) {
+        if (ctx->d_status) (void)cudaFree(ctx->d_status);
+        if (ctx->exchange) (void)cudaFree(ctx->exchange);
+        delete ctx;
+        return cuda_status(e);
+    }
     *ctx_out = ctx;
     return ZIPML_OK;
 }

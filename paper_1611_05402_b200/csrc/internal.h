@@ -25,8 +25,7 @@ struct zipml_ctx {
     unsigned char* stage = nullptr;
     size_t stage_bytes = 0;
     // words between the clusters of the cluster engine's int8 forms, and the next tag (see sgd_slice.cu, sgd_feature.cu)
-    unsigned char* exchange = nullptr;
-    size_t exchange_bytes = 0;
+    unsigned char* exchange = nullptr;   // kExchangeBytes, for the context's life (recorded launches hold its address)
     uint32_t exchange_tag = 1;
     int64_t launches = 0;           // kernels launched so far (diagnostics)
     int last_engine = 0;            // engine of the latest zipml_sgd_epoch call (diagnostics)
@@ -42,7 +41,9 @@ int check_dataset(const zipml_dataset* d);
 int cuda_status(cudaError_t e);                       // ZIPML_OK or ZIPML_ERR_CUDA (clears the sticky error)
 int ws_reserve(zipml_ctx* ctx, size_t bytes);         // grow ctx->ws to at least `bytes`
 int stage_reserve(zipml_ctx* ctx, size_t bytes);
-// At least `bytes` of exchange words between clusters, and the tag of the first of `steps` steps.
+// `bytes` of exchange words between clusters, and the tag of the first of `steps` steps.  At most two buffers in turn, 8 clusters, 16
+// bytes for each of 8,192 features and what the last slice or column has past them.
+constexpr size_t kExchangeBytes = 2 * 8 * (8192 + 1024) * 16;
 int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag);
 
 // The fp32 constant of zipml_sgd_params' regulariser for step length lr (see regularise() in common.cuh).

@@ -398,6 +398,42 @@ def test_slice_form_of_the_cluster_engine(ctx, m, n, bits, batch, parts, form):
     assert (g[1].cpu().numpy() != g4).sum() <= 3
 
 
+@pytest.mark.parametrize("form", [3, 4], ids=["rows", "features"])
+@pytest.mark.parametrize("steps", [1, 2, 5])
+def test_recorded_steps_on_several_clusters_replay(ctx, form, steps):
+    """An epoch on clusters that meet through L2, recorded into a graph (on a context that has not run any before): every replay is the
+    plain call, whatever the replay before it or a plain call in between has left in the exchange buffer."""
+    m, n, batch = 1000 * steps - 300, 600, 1000
+    _, A, b, _ = workload("c1", m, n, seed=1)
+    gds, db = dev_dataset(oracle.quantize(A, 4, seed=3), ctx), to_dev(b, ctx)
+    how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=form, grid_feature_parts=4)
+    starts = [to_dev((np.random.default_rng(k).standard_normal(n) * 0.1).astype(np.float32), ctx) for k in range(3)]
+    wants = []
+    for x0 in starts:
+        x = x0.clone()
+        ctx.zipml_sgd_epoch(gds, db, x, batch, 1e-3, **how)
+        wants.append(x)
+    ctx.zipml_sync()
+    stream = torch.cuda.Stream(ctx.device)
+    stream.wait_stream(torch.cuda.current_stream(ctx.device))
+    with torch.cuda.stream(stream), binding.Context(ctx.device, stream=stream) as other:
+        x = starts[0].clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            other.zipml_sgd_epoch(gds, db, x, batch, 1e-3, **how)
+        for k in (0, 1, 2, 1, 0):
+            x.copy_(starts[k])
+            graph.replay()
+            other.zipml_sync()
+            assert (x == wants[k]).all()
+            if k == 2:
+                y = starts[0].clone()
+                other.zipml_sgd_epoch(gds, db, y, batch, 1e-3, **how)
+                other.zipml_sync()
+                assert (y == wants[0]).all()
+        del graph
+
+
 # tables split by features: units of 16 bytes per CTA (parts: fewer CTAs, more units), one row and one past a pass of 128, 256 and 512
 # lanes, odd batches (rows travel in pairs), owners without rows, several boxes, a short last batch
 @pytest.mark.parametrize("m,n,bits,batch,parts", [
