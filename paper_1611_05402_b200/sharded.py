@@ -131,7 +131,10 @@ class ShardedEpoch:
 
     def share(self, pos, t, weight):
         """weight * the mean over the rank's rows of batch t of the symmetrised gradient, at the model (or its Q3
-        image for position pos) as it stands; zeros if the rank holds none of the batch.  (Good until the next call.)"""
+        image for position pos) as it stands; zeros if the rank holds none of the batch.  A tensor of its own."""
+        return self._share(pos, t, weight, own=True)
+
+    def _share(self, pos, t, weight, own):
         import torch
         if self.plan.count(t) == 0:
             return torch.zeros(self.n, dtype=torch.float32, device=self.x.device)
@@ -144,7 +147,7 @@ class ShardedEpoch:
             call.batch_order[pos] = t
         call(pos)
         g = self.g2[:self.n]
-        return g if weight == 1.0 else g * weight
+        return g * weight if own or weight != 1.0 else g
 
     def apply(self, v, pos):
         """Q4 and the update on this rank's replica."""
@@ -155,14 +158,19 @@ class ShardedEpoch:
         (torch.distributed on `group`; `all_reduce(v)` replaces it, e.g. for ranks emulated in one process)."""
         import torch.distributed as dist
 
+        meet = all_reduce is not None or (dist.is_available() and dist.is_initialized() and self.plan.world > 1)
+
         def reduce(v):
             if all_reduce is not None:
                 all_reduce(v)
-            elif dist.is_available() and dist.is_initialized() and self.plan.world > 1:
+            elif meet:
                 dist.all_reduce(v, op=dist.ReduceOp.SUM, group=group)
+
+        def share(pos, t, weight):                                 # (nobody writes into it where the ranks do not meet)
+            return self._share(pos, t, weight, own=meet)
 
         self._running = (self._share_call(), self._apply_call())
         try:
-            run_steps(self.plan, self.share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
+            run_steps(self.plan, share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
         finally:
             self._running = None

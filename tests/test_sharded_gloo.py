@@ -112,6 +112,41 @@ def test_two_ranks_reproduce_the_single_rank_oracle_epoch(tmp_path):
         assert np.abs(want).max() > 1e-2                                  # the epoch did move x
 
 
+class _FakeContext:
+    """The library's two calls of a step, on CPU tensors: the gradient of position p is x + p + 1, the update x - lr v."""
+
+    def prepare_sgd_epoch(self, data, b, x, batch, lr, grad_out=None, **kw):
+        def call(pos):
+            grad_out[:x.numel()] = x + pos + 1
+        call.batch_order = kw["batch_order"]
+        return call
+
+    def prepare_sgd_apply_gradient(self, x, lr, **kw):
+        return lambda v, pos: x.sub_(lr * v)
+
+
+def _fake_rank(n=5, steps=3):
+    from paper_1611_05402_b200.sharded import ShardedEpoch
+    return ShardedEpoch(_FakeContext(), ShardPlan(4 * steps, 4, 0, 1), None, torch.zeros(4 * steps), torch.zeros(n), 0.5)
+
+
+def test_a_share_is_the_callers_own():
+    rank = _fake_rank()
+    shares = [rank.share(pos, pos, 1.0) for pos in range(3)]
+    assert [s[0].item() for s in shares] == [1.0, 2.0, 3.0]
+    shares[2].zero_()
+    assert rank.g2[0].item() == 3.0
+
+    def doubled(v):                            # ranks meet in place: the gradient that the last step left stays the rank's own
+        v.mul_(2)
+
+    rank.run(all_reduce=doubled)
+    x = 0.0
+    for pos in range(3):
+        g, x = x + pos + 1, x - 0.5 * 2 * (x + pos + 1)
+    assert torch.allclose(rank.x, torch.full((5,), x)) and torch.allclose(rank.g2[:5], torch.full((5,), g))
+
+
 def test_partition_covers_every_row_once():
     for m, batch, world in [(203, 16, 2), (197, 16, 2), (64, 16, 4), (1000, 24, 8), (5, 8, 2)]:
         seen = np.zeros(m, int)
