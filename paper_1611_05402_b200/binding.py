@@ -176,27 +176,36 @@ class SharedBase:
 
 class PreparedEpoch:
     """zipml_sgd_epoch with its arguments marshalled once, for callers that take many short ranges of steps; calling it
-    runs from `first_step` on.  batch_order, if given, is the host array that the calls read (writable in place)."""
+    runs from `first_step` on.  batch_order, if given, is the host array that the calls read (writable in place).  Marshalled
+    anew once one of the tensors lies elsewhere."""
 
     def __init__(self, ctx, data, b, x, params, keep, grad_out):
         self.ctx, self.params, self.batch_order, self._tensors = ctx, params, keep, (data, b, x, grad_out)
-        self._call, self._data = lib().zipml_sgd_epoch, data.c_struct()
-        self._args = (ctx._h, C.byref(self._data), _ptr(b, torch.float32, ctx.device), _ptr(x, torch.float32, ctx.device), C.byref(params),
-                      _ptr(grad_out, torch.float32, ctx.device))
+        self._call, self._at = lib().zipml_sgd_epoch, None
 
     def __call__(self, first_step):
+        data, b, x, grad_out = self._tensors
+        at = (data.plane1.data_ptr(), data.plane2.data_ptr(), b.data_ptr(), x.data_ptr(), None if grad_out is None else grad_out.data_ptr())
+        if at != self._at:
+            device = self.ctx.device
+            self._data = data.c_struct()
+            self._args = (self.ctx._h, C.byref(self._data), _ptr(b, torch.float32, device), _ptr(x, torch.float32, device), C.byref(self.params),
+                          _ptr(grad_out, torch.float32, device))
+            self._at = at
         self.params.first_step = first_step
         _check(self._call(*self._args), "zipml_sgd_epoch")
 
 
 class PreparedApply:
-    """zipml_sgd_apply_gradient on a fixed x, marshalled once; calling it applies a gradient at a step."""
+    """zipml_sgd_apply_gradient on an x, marshalled once (anew where it lies elsewhere); calling it applies a gradient at a step."""
 
     def __init__(self, ctx, x, params):
         self.ctx, self.params, self.x = ctx, params, x
-        self._call, self._x, self._p, self._n = lib().zipml_sgd_apply_gradient, _ptr(x, torch.float32, ctx.device), C.byref(params), x.numel()
+        self._call, self._p, self._at = lib().zipml_sgd_apply_gradient, C.byref(params), None
 
     def __call__(self, g, step):
+        if self.x.data_ptr() != self._at:
+            self._x, self._n, self._at = _ptr(self.x, torch.float32, self.ctx.device), self.x.numel(), self.x.data_ptr()
         _check(self._call(self.ctx._h, self._x, _ptr(g, torch.float32, self.ctx.device), self._n, self._p, step, None), "zipml_sgd_apply_gradient")
 
 

@@ -111,7 +111,6 @@ class ShardedEpoch:
         self.ctx, self.plan, self.data, self.b, self.x, self.lr = ctx, plan, data_local, b_local, x, lr
         self.model_bits, self.grad_bits, self.seed, self.epoch = model_bits, grad_bits, seed, epoch
         self.reg, self.reg_param, self.engine = reg, reg_param, engine
-        self._running = None                                       # the prepared calls, while run() is at work
         self.n = x.numel()
         self.g2 = torch.empty(2 * self.n, dtype=torch.float32, device=x.device)
         self.order = None if batch_order is None else [int(o) for o in batch_order]
@@ -119,7 +118,20 @@ class ShardedEpoch:
         # positions whose batch this rank does not hold are never executed; their entries only have to be valid
         self.order_local = None if self.order is None or not T_local else [min(o, T_local - 1) for o in self.order][:T_local]
 
+    _calls = None                                                  # the two below, kept until an attribute changes
+    _alone = False                                                 # run() is at work and nobody else sees a share
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if name != "_calls":
+            object.__setattr__(self, "_calls", None)
+
     # The step's two library calls, with everything marshalled that stays the same from step to step.
+    def _prepared(self):
+        if self._calls is None:
+            self._calls = (self._share_call(), self._apply_call())
+        return self._calls
+
     def _share_call(self):
         return self.ctx.prepare_sgd_epoch(self.data, self.b, self.x, self.plan.local_batch, 0.0, model_bits=self.model_bits,   # lr = 0: x stays
                                           num_steps=1, engine=self.engine, batch_order=self.order_local, grad_out=self.g2, seed=self.seed,
@@ -132,13 +144,10 @@ class ShardedEpoch:
     def share(self, pos, t, weight):
         """weight * the mean over the rank's rows of batch t of the symmetrised gradient, at the model (or its Q3
         image for position pos) as it stands; zeros if the rank holds none of the batch.  A tensor of its own."""
-        return self._share(pos, t, weight, own=True)
-
-    def _share(self, pos, t, weight, own):
-        import torch
         if self.plan.count(t) == 0:
+            import torch
             return torch.zeros(self.n, dtype=torch.float32, device=self.x.device)
-        call = self._running[0] if self._running else self._share_call()
+        call = self._prepared()[0]
         if self.order_local is not None:
             # the library keys Q3 by the position: the step runs at position pos of a local order that names t there
             if pos >= len(self.order_local):
@@ -147,11 +156,11 @@ class ShardedEpoch:
             call.batch_order[pos] = t
         call(pos)
         g = self.g2[:self.n]
-        return g * weight if own or weight != 1.0 else g
+        return g if self._alone and weight == 1.0 else g * weight
 
     def apply(self, v, pos):
         """Q4 and the update on this rank's replica."""
-        (self._running[1] if self._running else self._apply_call())(v.contiguous(), pos)
+        self._prepared()[1](v.contiguous(), pos)
 
     def run(self, group=None, first_step=0, num_steps=None, all_reduce=None):
         """The epoch (or a range of its steps).  The ranks meet in one all-reduce of n floats per step
@@ -166,11 +175,8 @@ class ShardedEpoch:
             elif meet:
                 dist.all_reduce(v, op=dist.ReduceOp.SUM, group=group)
 
-        def share(pos, t, weight):                                 # (nobody writes into it where the ranks do not meet)
-            return self._share(pos, t, weight, own=meet)
-
-        self._running = (self._share_call(), self._apply_call())
+        self._alone = not meet
         try:
-            run_steps(self.plan, share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
+            run_steps(self.plan, self.share, reduce, self.apply, order=self.order, first_step=first_step, num_steps=num_steps)
         finally:
-            self._running = None
+            self._alone = False

@@ -147,6 +147,25 @@ def test_a_share_is_the_callers_own():
     assert torch.allclose(rank.x, torch.full((5,), x)) and torch.allclose(rank.g2[:5], torch.full((5,), g))
 
 
+def test_a_rank_follows_its_attributes_from_step_to_step():
+    """What the meeting of the ranks changes (a step length by schedule, another replica) holds from there on, as it does
+    between runs."""
+    rank = _fake_rank(steps=4)
+    first, second = rank.x, torch.full((5,), 10.0)
+
+    def schedule(v):
+        rank.lr *= 0.5
+        if v[0].item() > 2.0:                  # after the second step's gradient: the update already goes to the other replica
+            rank.x = second
+
+    rank.run(all_reduce=schedule, num_steps=2)
+    # step 0: gradient 1, lr 1/4; step 1: gradient -1/4 + 2, lr 1/8
+    assert torch.allclose(first, torch.full((5,), -0.25 - 0.125 * 1.75)) and (second == 10.0).all()
+    rank.run(all_reduce=schedule, first_step=2, num_steps=1)
+    g = -0.25 - 0.125 * 1.75 + 3
+    assert torch.allclose(second, torch.full((5,), 10.0 - 0.0625 * g))
+
+
 def test_partition_covers_every_row_once():
     for m, batch, world in [(203, 16, 2), (197, 16, 2), (64, 16, 4), (1000, 24, 8), (5, 8, 2)]:
         seen = np.zeros(m, int)
