@@ -39,8 +39,6 @@ NCU_TRAFFIC = {
     ("c5", 6): (4 * (591.80e6 + 6.29e6), "profiles/sgd_stream_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
     ("c5", 7): (4 * (538.45e6 + 4.86e6), "profiles/sgd_column_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
 }
-ENGINE_KERNELS = {1: "sgd_kernel (stepwise launches)", 2: "sgd_kernel (persistent)", 3: "sgd_ring_kernel", 4: "sgd_lean_kernel",
-                  5: "sgd_feature_kernel, sgd_slice_kernel or sgd_table_kernel", 6: "sgd_stream_kernel", 7: "sgd_column_kernel", 8: "sgd_solo_kernel"}
 
 
 def measured_peaks():
@@ -304,7 +302,7 @@ def main():
                 "traffic": NCU_TRAFFIC.get((args.workload, ctx.zipml_last_engine()), (None, None))[0] if args.m is None else None,
                 "traffic_source": NCU_TRAFFIC.get((args.workload, ctx.zipml_last_engine()), (None, None))[1] if args.m is None else None,
                 "peak_kind": f"of {peak_kind} copy rate", "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS,
-                "kernel": ENGINE_KERNELS.get(ctx.zipml_last_engine(), "?") + " (one launch per epoch)",
+                "kernel": ctx.zipml_last_kernel() + (" (several launches per step)" if ctx.zipml_last_engine() == binding.ENGINE_STEPWISE else " (one launch per epoch)"),
                 "algorithmic_bytes_per_launch": packed_bytes,
                 "launch_ms_avg": epoch_avg_ms, "launch_ms_min": epoch_ms[0],
                 "epoch_samples_per_s": w.m / (epoch_avg_ms * 1e-3),
@@ -391,7 +389,7 @@ def main():
             t_ep = sum(a_.elapsed_time(b_) for a_, b_ in evs) / len(evs)         # a mean, like the headline
             To = (wo.m + wo.batch - 1) // wo.batch
             lm = latency_model(ctx, ctx.zipml_last_engine(), wo.n, dso.packed_bytes / To, peak)
-            others[key] = {"workload": wo.name, "kernel": ENGINE_KERNELS.get(ctx.zipml_last_engine(), "?"), "epoch_ms": t_ep, "us_per_step": 1e3 * t_ep / To,
+            others[key] = {"workload": wo.name, "kernel": ctx.zipml_last_kernel(), "epoch_ms": t_ep, "us_per_step": 1e3 * t_ep / To,
                            "samples_per_s": wo.m / (t_ep * 1e-3), "packed_GB/s": dso.packed_bytes / (t_ep * 1e-3) / 1e9,
                            "frac_of_copy_rate": dso.packed_bytes / (t_ep * 1e-3) / 1e9 / peak,
                            "ceiling_frac": lm["ceiling_frac"] if lm else None, "chain_floor_us": lm["chain_floor_us"] if lm else None,

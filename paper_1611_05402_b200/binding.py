@@ -21,7 +21,7 @@ ENGINE_AUTO, ENGINE_STEPWISE, ENGINE_PERSISTENT, ENGINE_RING, ENGINE_LEAN, ENGIN
 
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", "libzipml.so")
 EXPORTS = ["zipml_up_row_bytes", "zipml_shared_base_encode", "zipml_shared_base_decode", "zipml_loss_shared_base",
-           "zipml_sgd_epoch_shared_base", "zipml_sgd_apply_gradient", "zipml_quantize_draw", "zipml_poly_rows", "zipml_weighted_plane_mean", "zipml_column_blocks_bytes", "zipml_convert_layout", "zipml_create", "zipml_destroy", "zipml_sync", "zipml_kernel_launches", "zipml_last_engine", "zipml_barrier_latency", "zipml_wait_probe", "zipml_strerror", "zipml_row_bytes", "zipml_quantize",
+           "zipml_sgd_epoch_shared_base", "zipml_sgd_apply_gradient", "zipml_quantize_draw", "zipml_poly_rows", "zipml_weighted_plane_mean", "zipml_column_blocks_bytes", "zipml_convert_layout", "zipml_create", "zipml_destroy", "zipml_sync", "zipml_kernel_launches", "zipml_last_engine", "zipml_last_kernel", "zipml_barrier_latency", "zipml_wait_probe", "zipml_strerror", "zipml_row_bytes", "zipml_quantize",
            "zipml_optimal_levels", "zipml_sgd_epoch", "zipml_loss", "zipml_train_host",
            "zipml_loss_codes_static"]
 
@@ -77,6 +77,8 @@ def lib():
         L.zipml_kernel_launches.restype = i64
         L.zipml_last_engine.argtypes = [vp]
         L.zipml_last_engine.restype = C.c_int32
+        L.zipml_last_kernel.argtypes = [vp]
+        L.zipml_last_kernel.restype = C.c_char_p
         L.zipml_barrier_latency.argtypes = [vp, i32, i32, i32, vp]
         L.zipml_wait_probe.argtypes = [vp, i64]
         L.zipml_strerror.argtypes = [C.c_int]
@@ -252,6 +254,9 @@ class Context:
 
     def zipml_last_engine(self):
         return int(lib().zipml_last_engine(self._h))
+
+    def zipml_last_kernel(self):
+        return lib().zipml_last_kernel(self._h).decode()
 
     def zipml_barrier_latency(self, ctas, floats_per_cta=0, iterations=1000):
         """Nanoseconds per step of the SGD step's communication skeleton on `ctas` CTAs."""

@@ -184,6 +184,8 @@ int64_t zipml_kernel_launches(const zipml_ctx* ctx) { return ctx ? ctx->launches
 
 int32_t zipml_last_engine(const zipml_ctx* ctx) { return ctx ? ctx->last_engine : 0; }
 
+const char* zipml_last_kernel(const zipml_ctx* ctx) { return ctx ? ctx->last_kernel : ""; }
+
 int zipml_sync(zipml_ctx* ctx) {
     if (!ctx) return ZIPML_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);

@@ -28,7 +28,9 @@ struct zipml_ctx {
     unsigned char* exchange = nullptr;   // kExchangeBytes, for the context's life (recorded launches hold its address)
     uint32_t exchange_tag = 1;
     int64_t launches = 0;           // kernels launched so far (diagnostics)
-    int last_engine = 0;            // engine of the latest zipml_sgd_epoch call (diagnostics)
+    int last_engine = 0;            // engine of the latest zipml_sgd_epoch call, and its kernel (diagnostics)
+    const char* last_kernel = "";
+    void ran(int engine, const char* kernel) { last_engine = engine; last_kernel = kernel; }
     void* tmap_encode = nullptr;    // cuTensorMapEncodeTiled, resolved on first use
 };
 

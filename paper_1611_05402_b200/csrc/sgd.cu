@@ -663,7 +663,7 @@ int launch_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
             if (e != cudaSuccess) return cuda_status(e);
             ctx->launches += 1;
         }
-        ctx->last_engine = ZIPML_ENGINE_PERSISTENT;
+        ctx->ran(ZIPML_ENGINE_PERSISTENT, "sgd_kernel");
         return ZIPML_OK;
     }
 
@@ -679,7 +679,7 @@ int launch_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
             ctx->launches += 1;
         }
     }
-    ctx->last_engine = ZIPML_ENGINE_STEPWISE;
+    ctx->ran(ZIPML_ENGINE_STEPWISE, "sgd_kernel");
     return ZIPML_OK;
 }
 

@@ -1047,7 +1047,7 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     e = cudaLaunchCooperativeKernel(kernel, dim3((unsigned)G), dim3(kColThreads), params, smem, ctx->stream);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
-    ctx->last_engine = ZIPML_ENGINE_COLUMN;
+    ctx->ran(ZIPML_ENGINE_COLUMN, "sgd_column_kernel");
     return ZIPML_OK;
 }
 

@@ -599,7 +599,7 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     e = cudaLaunchKernelExC(&cfg, kernel, params);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
-    ctx->last_engine = ZIPML_ENGINE_CLUSTER;
+    ctx->ran(ZIPML_ENGINE_CLUSTER, "sgd_feature_kernel");
     return ZIPML_OK;
 }
 

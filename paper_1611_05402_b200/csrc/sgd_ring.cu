@@ -1276,7 +1276,7 @@ int launch_sgd_ring(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
         if (e != cudaSuccess) return cuda_status(e);
         ctx->launches += 1;
     }
-    ctx->last_engine = ZIPML_ENGINE_RING;
+    ctx->ran(ZIPML_ENGINE_RING, "sgd_ring_kernel");
     return ZIPML_OK;
 }
 

@@ -693,7 +693,7 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, params);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
-    ctx->last_engine = ZIPML_ENGINE_CLUSTER;
+    ctx->ran(ZIPML_ENGINE_CLUSTER, "sgd_slice_kernel");
     return ZIPML_OK;
 }
 

@@ -638,7 +638,7 @@ int launch_sgd_solo(zipml_ctx* ctx, const zipml_dataset* d, const float* b, floa
     e = cudaLaunchKernel(kernel, dim3(1), dim3((unsigned)plan.threads + 32u), params, plan.smem, ctx->stream);
     if (e != cudaSuccess) return cuda_status(e);
     ctx->launches += 1;
-    ctx->last_engine = ZIPML_ENGINE_SOLO;
+    ctx->ran(ZIPML_ENGINE_SOLO, "sgd_solo_kernel");
     return ZIPML_OK;
 }
 

@@ -732,7 +732,7 @@ int launch_sgd_stream(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
         if (e != cudaSuccess) return cuda_status(e);
         ctx->launches += 1;
     }
-    ctx->last_engine = ZIPML_ENGINE_STREAM;
+    ctx->ran(ZIPML_ENGINE_STREAM, "sgd_stream_kernel");
     return ZIPML_OK;
 }
 
