@@ -540,39 +540,45 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     // 5.72 / 4.84.  (Eight of sixteen CTAs are seldom resident at once.)
     const int64_t cols_all = (d->n * cb + 127) / 128;
     int64_t clusters = p->grid_feature_parts > 0 ? p->grid_feature_parts : B < 448 ? 1 : B >= 1024 && (cols_all + (cols_all + 15) / 16 - 1) / ((cols_all + 15) / 16) <= 12 ? 8 : 4;
-    const int most = ctx->cooperative ? kSliceMaxClusters : 1;
-    if (clusters > most) clusters = most;
-    while (!feature_plan(ctx, d, p, clusters, &a, &smem))
-        if (++clusters > most) return ZIPML_ERR_WORKSPACE;
+    const void* kernel = nullptr;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    cudaError_t e;
+    // (clusters are taken back until all of them can be resident at once: they wait for one another)
+    for (int most = ctx->cooperative ? kSliceMaxClusters : 1;;) {
+        if (clusters > most) clusters = most;
+        while (!feature_plan(ctx, d, p, clusters, &a, &smem))
+            if (++clusters > most) return ZIPML_ERR_WORKSPACE;
+        const bool many = a.clusters > 1;
+        kernel = cb == 2 ? feature_kernel<2>(many) : cb == 4 ? feature_kernel<4>(many) : feature_kernel<8>(many);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess && a.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return cuda_status(e);
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(a.nb * a.clusters));
+        cfg.blockDim = dim3(kSliceThreads + 32);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = ctx->stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)a.nb;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeCooperative;
+        attr[1].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
+        if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
+        if (fit < 1) return ZIPML_ERR_WORKSPACE;
+        if (fit >= a.clusters) break;
+        most = fit;
+    }
+    if (a.clusters > 1) cfg.numAttrs = 2;
     CUtensorMap tmaps[2];
     memset(tmaps, 0, sizeof(tmaps));
     int rc = encode_plane_maps(ctx, d, a.pitch / 4, a.box_rows, true, tmaps);
     if (rc != ZIPML_OK) return ZIPML_ERR_WORKSPACE;              // (also where a box would be wider than 256 elements)
-    const bool many = a.clusters > 1;
-    const void* kernel = cb == 2 ? feature_kernel<2>(many) : cb == 4 ? feature_kernel<4>(many) : feature_kernel<8>(many);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && a.nb > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return cuda_status(e);
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)(a.nb * a.clusters));
-    cfg.blockDim = dim3(kSliceThreads + 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)a.nb;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int fit = 0;
-    e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
-    if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
-    if (fit < a.clusters) return ZIPML_ERR_WORKSPACE;            // (they wait for one another)
-    if (many) cfg.numAttrs = 2;
     if (p->batch_order) {
         rc = ws_reserve(ctx, carve_size(sizeof(int32_t) * (size_t)T));
         if (rc != ZIPML_OK) return rc;
@@ -591,7 +597,7 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     a.full_scale = 1.0 / (2.0 * (double)B); a.last_scale = 1.0 / (2.0 * (double)(a.rows_last > 0 ? a.rows_last : 1));
     a.seed = p->seed; a.epoch = (uint32_t)p->epoch; a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
     a.n = (int)d->n; a.bits = d->bits; a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
-    if (many) {
+    if (a.clusters > 1) {
         rc = exchange_tags(ctx, (size_t)2 * a.clusters * a.nb * 16 * a.cols * (8 / cb) * 16, num_steps, &a.exchange, &a.tag);
         if (rc != ZIPML_OK) return rc;
     }

@@ -327,6 +327,7 @@ def test_several_clusters_and_chunks(ctx, m, n, bits, batch, clusters, parts, fo
     order = np.random.default_rng(0).permutation(T).astype(np.int32)
     x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
     how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=form, grid_feature_parts=clusters, grid_row_parts=parts)
+    kernel = {3: "sgd_slice_kernel", 4: "sgd_feature_kernel"}[form]            # (fewer clusters where they are not all resident at once)
     x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, batch_order=order)
     x_before, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, batch_order=order, num_steps=T - 1)
     _, g_ref = oracle.sgd_epoch(ods, b, x_before, batch, lr, batch_order=order, first_step=T - 1, num_steps=1, want_grad=True)
@@ -334,7 +335,7 @@ def test_several_clusters_and_chunks(ctx, m, n, bits, batch, clusters, parts, fo
         x = to_dev(x0, ctx)
         ctx.zipml_sgd_epoch(gds, db, x, batch, lr, batch_order=order, **how)
         ctx.zipml_sync()
-        assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+        assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
     xb = to_dev(x_before, ctx)
     g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
     ctx.zipml_sgd_epoch(gds, db, xb, batch, lr, batch_order=order, first_step=T - 1, num_steps=1, grad_out=g, **how)
@@ -369,6 +370,9 @@ def test_slice_form_of_the_cluster_engine(ctx, m, n, bits, batch, parts, form):
     order = np.random.default_rng(0).permutation(T).astype(np.int32)
     x0 = (np.random.default_rng(1).standard_normal(n) * 0.1).astype(np.float32)
     how = dict(engine=binding.ENGINE_CLUSTER, cluster_contraction=form, grid_row_parts=parts)
+    # (by rows a slice of the features has to fit a CTA's threads: not with as few rows as here beside so many features)
+    declines = form == 3 and (m, n) in ((70, 4090), (9, 700))
+    kernel = "sgd_cluster_kernel" if declines else {3: "sgd_slice_kernel", 4: "sgd_feature_kernel"}[form]
     for kw in (dict(batch_order=order), dict(reg=binding.REG_L2, reg_param=0.1)):
         x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, **kw)
         x_before, _ = oracle.sgd_epoch(ods, b, x0, batch, lr, num_steps=T - 1, **kw)
@@ -376,7 +380,7 @@ def test_slice_form_of_the_cluster_engine(ctx, m, n, bits, batch, parts, form):
         x = to_dev(x0, ctx)
         ctx.zipml_sgd_epoch(gds, db, x, batch, lr, **how, **kw)
         ctx.zipml_sync()
-        assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+        assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
         xb, seen = to_dev(x_before, ctx), torch.zeros(n, device=ctx.device)
         g = torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
         ctx.zipml_sgd_epoch(gds, db, xb, batch, lr, first_step=T - 1, num_steps=1, grad_out=g, model_out=seen, **how, **kw)
@@ -455,7 +459,7 @@ def test_cluster_engine_on_tables_by_features(ctx, m, n, bits, batch, parts):
     x = to_dev(x0, ctx)
     ctx.zipml_sgd_epoch(gds, db, x, batch, lr, batch_order=order, **how)
     ctx.zipml_sync()
-    assert ctx.zipml_last_engine() == binding.ENGINE_CLUSTER and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+    assert ctx.zipml_last_kernel() == "sgd_table_kernel" and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
     kw = dict(seed=5, epoch=1, first_step=T - 1, num_steps=1)
     x, g, seen = to_dev(x0, ctx), torch.zeros((2, n), device=ctx.device), torch.zeros(n, device=ctx.device)
     ctx.zipml_sgd_epoch(gds, db, x, batch, lr, model_bits=8, grad_bits=6, grad_out=g, model_out=seen, **how, **kw)
