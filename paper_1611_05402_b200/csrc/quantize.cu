@@ -313,7 +313,8 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
             const float val = have ? __ldg(levels + (jb + f) * L + k) : 0.0f;
             const float next = have && k < L - 1 ? __ldg(levels + (jb + f) * L + k + 1) : val;
             const float width = __fsub_rn(next, val);
-            const float rw = !(width > 0.0f) ? 0.0f : (width >= 9.1e-13f && width <= 1.09e12f) ? __frcp_rn(width) : -1.0f;
+            // (a width that overflows takes no value up either: its quotients are 0 or none)
+            const float rw = !(width > 0.0f && width <= 3.402823466e+38f) ? 0.0f : (width >= 9.1e-13f && width <= 1.09e12f) ? __frcp_rn(width) : -1.0f;
             const int at = (k * 4 + (f & 3)) * tx + (f >> 2);
             lev_s[at] = k < L - 1 ? val : INFINITY;
             cell_s[at] = make_float4(val, width, rw, __int_as_float(k));

@@ -106,6 +106,22 @@ def test_quantize_sparse_rows_and_edges_bit_exact(ctx, m, n, bits, levels, nonze
         assert e.value.code == binding.ERR_NONFINITE
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3])
+def test_quantize_onto_levels_whose_distance_overflows(ctx, bits):
+    """Cells wider than the largest float, beside cells of ordinary width: bit for bit what the pinned arithmetic gives."""
+    m, n = 70, 9
+    rng = np.random.default_rng(bits)
+    A = (rng.uniform(-1, 1, (m, n)) * 3.0e38).astype(np.float32)
+    A[0], A[1] = -3.0e38, 3.0e38
+    levels = np.sort(rng.uniform(-3.0e38, 3.0e38, (n, 1 << bits)).astype(np.float32), axis=1)
+    levels[:, 1:-1] = np.where(np.arange(n)[:, None] < 4, 2.9e38, levels[:, 1:-1])
+    levels[:, 0], levels[:, -1] = -3.0e38, 3.0e38
+    ods = oracle.quantize(A, bits, seed=7, mode=oracle.TABLE, levels=levels)
+    gds = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=7, level_mode=binding.LEVELS_TABLE, levels=to_dev(levels, ctx))
+    ctx.zipml_sync()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+
+
 def test_quantize_strided_and_unaligned_input(ctx):
     _, A, _, _ = workload("c2", 200, 101, seed=3)
     big = torch.zeros((200, 131), dtype=torch.float32, device=ctx.device)
