@@ -67,6 +67,8 @@ struct ClusterArgs {
     float reg_cst;
     int n, bits, row_words, words;   // words = ceil(n / codes per word) <= row_words
     int model_bits, grad_bits;
+    int pitch;                       // words between the rows of a tile in shared memory: row_words (as an argument of its own: addressed through
+                                     // row_words the kernel on 2-bit tables took 0.4 us a step longer, 5.3 -> 5.7 at 300 rows x 64)
     int nb, rc, slots;
     int sub;                     // a CTA owns `sub` consecutive features (a multiple of 4)
     int p_shift;                 // 2^p_shift lanes share the sum of one owned feature
@@ -199,7 +201,8 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
     float* bsm = res + ((2 * a.rc + 3) & ~3);
     uint32_t* ring = reinterpret_cast<uint32_t*>(
         (reinterpret_cast<uintptr_t>(bsm + ((a.rc + 3) & ~3)) + 127) & ~(uintptr_t)127);
-    const size_t slot_words = (size_t)2 * a.rc * rw;
+    const int pitch = a.pitch;
+    const size_t slot_words = (size_t)2 * a.rc * pitch;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bi = blockIdx.x;                           // the grid is one cluster: block index = rank
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
             clu_mark(a, it, 0);
             clu_wait(sh->full + slot, parity, sh, a.status, 6);
             const uint32_t* t1 = ring + (size_t)slot * slot_words;
-            const uint32_t* t2 = t1 + (size_t)a.rc * rw;
+            const uint32_t* t2 = t1 + (size_t)a.rc * pitch;
             clu_mark(a, it, 1);
 
             // ---------------------------------------------------------- phase A: dots and residuals
@@ -288,8 +291,8 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
             double srow = 0.0;
 #pragma unroll 1
             for (int r = warp; r < rcnt; r += kCluWarps) {
-                const uint32_t* row1 = t1 + (size_t)r * rw;
-                const uint32_t* row2 = t2 + (size_t)r * rw;
+                const uint32_t* row1 = t1 + (size_t)r * pitch;
+                const uint32_t* row2 = t2 + (size_t)r * pitch;
                 float acc1 = 0.0f, acc2 = 0.0f;
 #pragma unroll 2
                 for (int q = lane; q < nw; q += 32) {
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) sgd_cluster_kernel(const Clust
                 if (active) {
 #pragma unroll 2
                     for (int r = group; r < rcnt; r += ngroups) {
-                        const uint32_t u1 = t1[(size_t)r * rw + q], u2 = t2[(size_t)r * rw + q];
+                        const uint32_t u1 = t1[(size_t)r * pitch + q], u2 = t2[(size_t)r * pitch + q];
                         const float2 rv = *reinterpret_cast<const float2*>(res + 2 * r);
                         if constexpr (!TABLE) {
                             float c1[FPW], c2[FPW];
@@ -673,7 +676,7 @@ int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
     a.words = (int)((d->n + fpw - 1) / fpw);
     a.model_bits = p->model_bits; a.grad_bits = p->grad_bits;
     a.nb = plan.nb; a.rc = plan.rc; a.slots = plan.slots;
-    a.sub = plan.sub; a.p_shift = plan.p_shift;
+    a.pitch = a.row_words; a.sub = plan.sub; a.p_shift = plan.p_shift;
     if (p->batch_order) {
         int32_t* dev_order = reinterpret_cast<int32_t*>(ctx->ws + o_ord);
         e = cudaMemcpyAsync(dev_order, p->batch_order, sizeof(int32_t) * (size_t)T, cudaMemcpyHostToDevice, ctx->stream);
