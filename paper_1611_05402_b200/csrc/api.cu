@@ -290,12 +290,19 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
 }
 
 // Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.
-//   tables: 2 bits n 4,091 x 64 L 22 G 24, x 256 L 26 G 18; n 2,043 x 1,500 L 43 G 38; 4 bits n 1,019 x 600 L 24 G 28, x 1,500 L 42 G 34;
-//   one row of n 4,091 L 27 G 16; with a quantized vector the grid is no better (4 bits n 1,019 x 1,500 L 51 G 58).
+//   tables: 3 bits n 600 x 1,207 L 13.7 G 21.2, x 2,414 L 21.5 G 23.8, x 3,276 L 27 G 25; n 512 x 2,867 L 18.5 G 20.1, x 3,891 L 22.9 G 21.5;
+//   n 300 x 3,276 L 19.1 G 20.7, x 4,587 L 24.3 G 22.9; n 700 x 1,489 L 15.8 G 16.6, x 2,084 L 20.0 G 19.0; n 1,000 x 1,024 L 15.4 G 16.6, x 1,433
+//   L 18.5 G 18.2; n 1,400 x 521 L 16.0 G 14.0.  4 bits n 600 x 2,414 L 23.0 G 26.2; n 850 x 1,213 L 17.6 G 17.9, x 1,698 L 21.7 G 19.7; n 1,000 x
+//   716 L 17.6 G 15.6.  2 bits n 600 x 3,276 L 25.2 G 27.9, x 4,587 L 32.6 G 30.2; n 1,000 x 2,048 L 20.1 G 22.3, x 2,867 L 25.2 G 24.3; n 1,400 x
+//   1,042 L 18.9 G 19.3, x 1,489 L 22.6 G 21.2; n 2,000 x 716 L 18.5 G 19.2, x 1,024 L 22.4 G 21.0; n 4,091 x 64 L 22 G 24, x 256 L 26 G 18.
+//   One row of n 4,091 L 27 G 16.  With a quantized vector the grid is seldom better (3 bits n 600 x 1,207 L 17.6 G 24.8).
 static bool lean_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B) {
     if (d->level_mode == ZIPML_LEVELS_UNIFORM) return false;
     if (p->model_bits != 0 || p->grad_bits != 0) return true;
-    return B * d->n <= 700000 && (d->n < 3000 || B >= 32);
+    if (d->n >= 3000) return B * d->n <= 700000 && B >= 32;
+    const int64_t most = container_bits(d->bits) == 2 ? (d->n <= 1000 ? 2300000 : 1500000)
+                         : d->n < 400 ? 1200000 : d->n <= 600 ? 1700000 : d->n > 1000 ? 700000 : d->bits == 3 ? 1250000 : d->n <= 900 ? 1000000 : 700000;
+    return B * d->n <= most;
 }
 
 // Uniform rows too wide for the column and stream engines: the persistent grid up to 16 MB a step, 4 bits n 100,000 x 64 G 23 R 42, x 300

@@ -584,12 +584,15 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
 }
 
 // Level tables: split by features, or by rows where the features make too few 16-byte units for the CTAs.  us per step by features / by
-// rows / lean: 3 bits n 64 (2 units) x 512 5.1 / 5.2 / 5.6, x 1,024 8.4 / 7.1 / 6.9, n 120 (4) x 1,024 6.5 / 7.2 / 7.2, x 2,048 11.5 / 11.3 / 10.0,
-// n 512 (16) x 512 3.6 / 6.5 / 8.3, x 2,048 8.7 / 15.3 / 14.5; 2 bits n 120 (2) x 256 4.0 / 4.8 / 5.1, x 512 6.2 / 6.3 / 5.9; n 1,019 (16) x 1,024
-// 7.5 / 14.3 / 13.4.
+// rows: 3 bits n 17 to 32 (1 unit) x 180 3.72 / 3.86, x 240 4.33 / 4.02, n 64 (2) x 420 4.49 / 4.82, x 500 4.86 / 5.02, x 600 5.89 / 5.65, n 96 (3) x
+// 800 6.11 / 6.50, n 120 (4) x 1,024 6.5 / 7.2, x 2,048 11.5 / 11.3, n 512 (16) x 2,048 8.7 / 15.3; 4 bits n 32 x 180 3.90 / 4.01, x 240 4.55 /
+// 4.18, n 64 x 420 4.85 / 4.98, x 500 5.25 / 5.18, n 96 x 800 6.59 / 6.67; 2 bits n 33 to 64 (1) x 180 4.23 / 4.29, x 240 4.98 / 4.55, n 100 (2) x 500
+// 6.04 / 6.11, x 600 7.40 / 7.00, n 190 (3) x 800 8.10 / 8.34; n 1,019 (16) x 1,024 7.5 / 14.3.  With a quantized vector the features do a little
+// longer: 3 bits n 64 x 600 8.30 / 8.43, 4 bits x 500 7.35 / 7.57.
 static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
     const int64_t B = p->batch < d->m ? p->batch : d->m, units = (d->n * container_bits(d->bits) + 127) / 128;
-    return B <= (container_bits(d->bits) == 2 ? 240 : 300) * units;
+    if (container_bits(d->bits) == 2) return B <= 240 * units - (units == 1 ? 55 : 0);
+    return B <= 300 * units - (units == 1 || (units <= 3 && p->model_bits == 0 && p->grad_bits == 0) ? 100 : 0);
 }
 
 // Uniform grids: split by features, or by rows where the features make too little work for the CTAs, or a batch is so long that it goes

@@ -960,6 +960,22 @@ def test_auto_on_rows_wider_than_a_cluster(ctx, m, n, bits, batch, optimal, engi
     assert ctx.zipml_last_engine() == engine and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
 
 
+@pytest.mark.parametrize("m,n,bits,batch,kernel", [
+    (420, 31, 3, 200, "sgd_table_kernel"), (450, 31, 3, 201, "sgd_cluster_kernel"), (400, 64, 2, 185, "sgd_table_kernel"),
+    (400, 61, 2, 186, "sgd_cluster_kernel"), (2500, 590, 3, 2400, "sgd_lean_kernel"), (3000, 590, 3, 2950, "sgd_kernel"),
+], ids=str)
+def test_auto_on_level_tables(ctx, m, n, bits, batch, kernel):
+    """Either side of the lines of AUTO's rule for level tables, with the kernel it takes and the oracle's result."""
+    _, A, b, _ = workload("c4", m, n, seed=4)
+    ods = oracle.quantize(A, bits, seed=3, mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 64)[0])
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-3)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-3)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+
+
 REGS = [(binding.REG_L2, 0.5), (binding.REG_L1, 0.02), (binding.REG_NONNEG, 0.0), (binding.REG_LSSVM, 0.5)]
 
 
