@@ -278,6 +278,7 @@ def test_sgd_epoch_parity(ctx, case, engine):
     (100, 1, 2, 7, False), (300, 5, 8, 64, False), (90, 16, 4, 1, False), (1200, 23, 8, 512, False), (260, 61, 4, 33, False),
     (700, 250, 2, 64, False), (70, 2048, 8, 16, False), (60, 1999, 4, 16, False), (300, 1000, 1, 16, False), (500, 37, 3, 100, True),
     (130, 250, 2, 16, True), (40, 2000, 4, 3, True), (2500, 30, 6, 1024, False),
+    (5800, 16, 2, 2880, False),          # a batch that leaves room for one slot of codes
 ])
 def test_solo_engine(ctx, m, n, bits, batch, table):
     """The one-block engine at the edges of its lane splits (rows, words and features left over), with a batch order, a
