@@ -35,7 +35,7 @@ NOMINAL_HBM_GBS = 8000.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one epoch launch, quoted from the ncu captures summarised under
 # profiles/ (a run cannot measure them itself): (workload, engine) -> (bytes, where they come from)
 NCU_TRAFFIC = {
-    ("c2", 5): (203.04e6 + 3.76e6, "profiles/sgd_cluster_kernel_c2_full.md"),
+    ("c2", 5): (202.11e6 + 3.52e6, "profiles/sgd_feature_kernel_256x1000.md"),
     ("c5", 6): (4 * (591.80e6 + 6.29e6), "profiles/sgd_stream_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
     ("c5", 7): (4 * (538.45e6 + 4.86e6), "profiles/sgd_column_kernel_c5_full.md, 16,384-row capture scaled x4 by the rows"),
 }
@@ -93,9 +93,13 @@ def latency_model(ctx, engine_ran, n, step_bytes, peak_gbs):
     """What the minibatch chain allows: a step moves step_bytes and cannot start before the previous step's model
     exists, so it costs at least step_bytes / BW plus its exchanges between SMs (measured here with the library's
     communication skeleton: publish through L2, bounded-spin barrier, read the others' data).  ceiling_frac =
-    S / (S / BW + k t_exchange) / BW with t_compute taken as zero: an upper bound on roofline.frac."""
+    S / (S / BW + k t_exchange) / BW with t_compute taken as zero: an upper bound on roofline.frac.  None for the engines
+    whose CTAs do not meet through L2 in a step: the one-block engine exchanges nothing, the cluster engine's CTAs store
+    into each other's shared memory, which takes less than the skeleton's round."""
+    if engine_ran in (5, 8):
+        return None
     k = 1 if engine_ran in (6, 7) else 2           # stream, column: the dots; the others: gradient parts out, model back
-    ctas = {5: 16}.get(engine_ran, 128)            # the cluster engine is one cluster of at most 16 CTAs
+    ctas = 128
     floats = max(4, (n // ctas + 3) // 4 * 4)
     try:
         t_ns = ctx.zipml_barrier_latency(ctas, floats, 2000)
