@@ -278,8 +278,9 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
     if (cb == 8 ? 4 * B > 3 * d->row_bytes : 3 * B > 4 * d->row_bytes) return ZIPML_ENGINE_RING;
     const int64_t blocks = (d->row_bytes + 127) / 128;                 // CTAs of the column engine
     if (2 * blocks >= ctx->sm_count) {
-        // At least half the device.  (At 32 to 255 rows of 4-bit codes the stream engine keeps what it had, C 9.2 S 11.1 at 10 KB x
-        // 128: callers rely on that choice.)
+        // At least half the device.  At 32 to 255 rows of 4-bit codes the choice of the stream engine for short steps is a pinned one,
+        // not the faster: 10 KB x 32 C 8.2 S 10.4, x 128 8.9 / 10.8, x 224 9.3 / 11.7; 16 KB x 128 9.7 / 11.3.  (Rows that the column
+        // engine declines, 32 KB x 128 S 14.3, go to the stream engine anyway.)
         if (B >= 256 || cb == 8 || B < 32) return ZIPML_ENGINE_COLUMN;
         return ZIPML_ENGINE_STREAM;
     }

@@ -1,7 +1,7 @@
 // Variance-optimal level placement (paper Section 3): a one-pass per-feature histogram over equal
 // bins of the normalised range ("Discretization"), then the dynamic programme
 //   T(k, m) = min_j T(k-1, j) + V(j, m)
-// over the bin edges ("Dynamic Programming with Candidate Points") in exact 64-bit integers.
+// over the bin edges ("Dynamic Programming with Candidate Points"), exact: integers below 2^53, held in doubles.
 #include "common.cuh"
 #include "internal.h"
 

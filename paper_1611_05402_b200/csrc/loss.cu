@@ -379,9 +379,11 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
         unsigned* ticket = reinterpret_cast<unsigned*>(wdig + (8 / cb) * 4 * vec_bytes);
         // 16 warps per SM, 16 rows per warp and turn (four spans in flight take 128 registers a thread); with fewer rows smaller
         // blocks, so that every SM has some, and where there are not rows for two warps of all schedulers several to 16 rows.
-        // Measured, us: 2 bits 1,000,000 x 2,048 253 with shifted codes and two spans -> 225 (4.7 TB/s, bound by the masks and
-        // products), 4 bits 1,000,000 x 1,000 270 -> 185 (5.5 TB/s), 8 bits 300,000 x 2,000 264 -> 257; few rows: 4 bits 3,997 x 6,576
-        // 99 -> 29, 245 x 2,710 42 -> 26, 2 bits 8,000 x 32,000 176 -> 63.
+        // Measured, us: 2 bits 1,000,000 x 2,048 253 with shifted codes and two spans -> 225 (4.7 TB/s), 4 bits
+        // 1,000,000 x 1,000 270 -> 185 (5.5 TB/s), 8 bits 300,000 x 2,000 264 -> 257; few rows: 4 bits 3,997 x 6,576 99 -> 29, 245 x
+        // 2,710 42 -> 26, 2 bits 8,000 x 32,000 176 -> 63.  Bound by the bytes in flight: of the cycles between
+        // two instructions of a warp its loads take 6.1 of 11.6 at 2 bits (the masks keep the ALU pipe 48 % busy), 11.6 of 17.1 at 4
+        // and 23.8 of 28.4 at 8; the digits, which every warp reads again, are half of the sectors that L2 serves.
         const int64_t turns = (d->m + 15) / 16, spans = vec_bytes / 64;
         int warps = (int)(turns / ctx->sm_count), kp = 1, kp_shift = 0;
         warps = warps > 16 ? 16 : warps < 1 ? 1 : warps;

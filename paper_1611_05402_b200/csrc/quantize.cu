@@ -202,7 +202,7 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 // multiplication with the staged reciprocal of the cell's width, corrected (quotient below).  Such a call
 // needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
 // non-finite values, are gathered on the way.
-// What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 63 %; 24 warps per SM: fewer
+// What bounds it: dense rows, the integer products (that pipe 71 % busy, issue slots 63 %; 24 warps per SM: fewer
 // registers per thread spill, more leave too few warps); sparse rows, issue slots and DRAM together.
 // Measured, whole call with the range pass, before -> now: 100,003 x 1,001 at 8 bits 395 -> 278 us, 65,536 x 32,768 of
 // 5 % non-zeros at 4 bits 6,127 -> 3,639 us; 500,000 x 512 on 3-bit tables 1,520 -> 890 us (no range pass any more).

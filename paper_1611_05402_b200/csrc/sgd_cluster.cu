@@ -601,7 +601,9 @@ static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
 // 7.06 / 5.99; 2 bits n 256 x 128 3.04 / 2.83, n 1,000 x 64 2.82 / 3.33, x 512 4.05 / 4.58, x 4,096 8.04 / 7.66.
 static bool features_pay(const zipml_dataset* d, const zipml_sgd_params* p) {
     const int64_t B = p->batch < d->m ? p->batch : d->m;
-    // (from 2^24 entries a step a quantized vector goes to the ring engine, a choice that callers rely on)
+    // From 2^24 entries a step a quantized vector leaves this form: wide rows then go to the ring engine, a pinned choice, and rows that
+    // the form by rows holds go there.  Not the faster side at 2 bits 4,096 x 4,096 (features 13.8, rows 22.9, ring 43.5); longer batches
+    // this form does not hold anyway (4 bits 2,048 x 8,192 rows 20.1, ring 45.9).
     if ((p->model_bits > 0 || p->grad_bits > 0) && B * d->n >= 1 << 24) return false;
     return d->n >= (container_bits(d->bits) == 2 ? 900 : 480) && B <= 5 * d->n;
 }

@@ -3,10 +3,11 @@
 // footnote form; "End-to-end Quantization").
 //
 // A small step is a chain of hand-overs; its arithmetic is little.  Split by features the model and the gradient stay in the CTA that owns
-// them; what travels is a row's two dots to the row's owner, in double, and its two residuals back:
+// them; what travels is a row's two dots to the row's owner, as integers, and its two residuals back:
 //   * dots: a warp takes 16 rows of the own columns (mma.sync m16n8k32 u8 x s8 against the digits of w = step * x~: exact integer sums)
 //     and stores the two of a row into its owner's shared memory (st.async, 16 bytes);
-//   * the owner of a row adds the nb parts, 16 lanes a row, subtracts the label; each lane stores the residuals of two rows into one CTA;
+//   * the owner of a row adds the nb parts, 16 lanes a row, in the largest of the CTAs' units, and what the copying warp has made of
+//     lo^T x~ and the row's label meanwhile, an integer in the same unit; each lane stores the residuals of two rows into one CTA;
 //   * every CTA takes the largest residual of all rows for the scale and writes their digits: 16 rows of plane 1 with r2 and 16 rows of
 //     plane 2 with r1 are the 32 entries of one contraction;                                                  barrier
 //   * gradient: a warp takes a column and a part of the row blocks (transposing ldmatrix) and leaves a low and a high integer per feature;
@@ -14,7 +15,7 @@
 //   * sums over the parts, exact integers until they meet lo and step in double (codes less a constant centre in fp32 lost 10 to 37 times
 //     the precision on rows that are mostly zeros: 1.2e-6 of the gradient at 256 x 1,000, 4e-8 now); Q4, update, Q3, w;   barrier
 //     and the digits of w, four balanced base-256 digits per entry, with the power of two of the CTA's largest.            barrier
-// Bound by the chain of dependent instructions: some 660 a warp and step at 48 % of the issue slots (8 bits 256 x 1,000: dots 1.1 k cycles,
+// Bound by the chain of dependent instructions: some 680 a warp and step at 50 % of the issue slots (8 bits 256 x 1,000: dots 1.1 k cycles,
 // hand-overs 0.8 k and 0.2 k, digits of the residuals 0.7 k, gradient 0.7 k, update 0.6 k, digits of w 0.6 k); a quantized gradient and
 // model add a norm over the CTAs each, 2.1 k.  Measured against the form split by rows, us per step: 8 bits 256 x 1,000 3.3 -> 2.9, 2 bits
 // 1,024 x 2,048 with both quantized 9.0 -> 7.6, 8 bits 512 x 2,000 5.9 -> 4.6, 4 bits 128 x 4,000 5.9 -> 3.5; against the column engine 8 bits
