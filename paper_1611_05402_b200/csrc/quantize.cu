@@ -183,29 +183,34 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 // Quantize + pack.  A thread owns four consecutive features (8, 16 or 32 bits of a plane's row) and kQuantRows
 // consecutive rows per pass: the features' lo and inv are loaded once, the rows' loads and Philox chains are
 // independent and overlap, and the next pass's samples are on their way while this pass draws.
-//   Cell and threshold.  With t = (v - lo) * inv rounded as the grid prescribes, tc = clamp(t, 0, s) and
-//     r = 2^23 + tc rounded down, the cell is the low byte of r, and 2^24 * p = 2^24 * (tc - floor tc) comes out of
-//     two exact FMAs; up <=> (word >> 8) < ceil(2^24 p) <=> word < ceil(2^24 p) << 8, so the draws are compared as
-//     they are (u24 * 2^-24 < p is exact in fp32, u24 an integer; p <= 0 or NaN: never up).  t >= s lands in code s
-//     with p = 0: no special case for the upper end.
+//   Cell and threshold.  With t = (v - lo) * inv rounded as the grid prescribes and tc = clamp(t, 0, s), p = tc - floor tc:
+//     up <=> (word >> 8) < ceil(2^24 p) (u24 * 2^-24 < p is exact in fp32, u24 an integer; p <= 0 or NaN: never up).
+//     Cell and threshold together, floor(tc) << 24 plus ceil(2^24 p), are ceil(2^24 tc): one conversion.  A draw is an
+//     addition whose carry reaches the cell in the upper byte, from where byte permutes collect the codes.  t >= s lands in
+//     code s with p = 0: no special case for the upper end.
 //   Draws.  One Philox block serves a feature pair: counter (row, row's upper half, pair, draw), words {first feature copy
 //     1, copy 2, second feature copy 1, copy 2}, the top 24 bits of a word the uniform integer.  The round keys depend on
 //     the seed alone and arrive as kernel parameters (an operand of the xor).  The 32 x 32 -> 64-bit products are what
 //     the rounds cost (half of the FMA pipe takes them): of the first two rounds' four, two depend only on the pair
 //     (kept for the thread's life) and two only on the row (shared by the thread's pairs): 17 a block, not 20.
-//   Sparse rows.  A pair whose two values are their features' lowest level has code 0 in both planes for certain.
-//     Where at most a quarter of a warp's pairs are anything else (5 % non-zeros: a tenth), the lanes put those in a
-//     queue in shared memory and share them out evenly -- cell, threshold, draw and all, one round per 512 elements
-//     instead of 16 per lane -- each answer or-ed into its owner's words.
-// Level tables: the block's tables are staged in shared memory as [level][feature of the thread][thread column], so
-// that a warp's look-ups are free of bank conflicts whatever its codes are; the cell is found by bisection and p by a
-// multiplication with the staged reciprocal of the cell's width, corrected (quotient below).  Such a call
-// needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
+//   Sparse rows.  A pair whose two values lie on grid points (5 % non-zeros: nine pairs in ten) has no draw to make.
+//     Where at most a quarter of a warp's pairs are anything else, the lanes put those thresholds in a queue in shared
+//     memory and share them out evenly, one Philox block per 32 pairs instead of eight per lane; the four answers of a pair go to its
+//     owner's word, whose bits a shift and a mask add to the codes.  (Queueing the samples, with cells and thresholds
+//     done by whoever draws, saves conversions and loses more to shared memory, which was 87 % busy: 148 us per
+//     4,096 x 32,768, now 134.)
+// Level tables: the block's tables are staged in shared memory as [feature of the thread][level][thread column], so
+// that a warp's look-ups are free of bank conflicts whatever its codes are; the cell is found by bisection, whose offset is the cell's
+// number times 256, and p by a multiplication with the staged reciprocal of the cell's width, corrected (quotient below).
+// Blocks with a cell too narrow or too wide for that divide instead; a quotient too small for it is between 0 and
+// 2^-24 anyway and its threshold 1, or 0 where the division would round to 0 (the staged least numerator).  No calls, and no branch a
+// sample: 85 -> 71 instructions a sample, 890 -> 655 us on 500,000 x 512 at 3 bits.  Such a
+// call needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
 // non-finite values, are gathered on the way.
-// What bounds it: dense rows, the integer products (that pipe 71 % busy, issue slots 63 %; 24 warps per SM: fewer
-// registers per thread spill, more leave too few warps); sparse rows, issue slots and DRAM together.
-// Measured, whole call with the range pass, before -> now: 100,003 x 1,001 at 8 bits 395 -> 278 us, 65,536 x 32,768 of
-// 5 % non-zeros at 4 bits 6,127 -> 3,639 us; 500,000 x 512 on 3-bit tables 1,520 -> 890 us (no range pass any more).
+// What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 62 %; 24 warps per SM: fewer
+// registers per thread spill, more leave too few warps); sparse rows, issue slots (75 %) and DRAM (60 %) together.
+// Measured, whole call with the range pass, samples queued and conversions of their own for cell and threshold ->
+// now: 100,003 x 1,001 at 8 bits 279 -> 262 us, 65,536 x 4,096 of 5 % non-zeros at 4 bits 484 -> 450.
 // ---------------------------------------------------------------------------------------------
 constexpr int kQuantRows = 4;                  // rows per thread and pass
 constexpr int kQuantTableCols = 64;            // thread columns per block with level tables
@@ -239,38 +244,25 @@ __device__ __forceinline__ Philox4 philox_rounds(uint32_t c0, uint32_t c1, uint3
     return out;
 }
 
-// Integer steps of the kernel below, worded so that they run on the ALU pipe: the Philox products fill the half of the
-// FMA pipe that integer multiplies share, and left to itself the compiler puts shifts and additions there too.
-template <int S>
-__device__ __forceinline__ uint32_t shift_left(uint32_t v) {
-    uint32_t d;
-    if constexpr (S == 8) asm("prmt.b32 %0, %1, 0, 0x2104;" : "=r"(d) : "r"(v));
-    else asm("shf.l.wrap.b32 %0, 0, %1, %2;" : "=r"(d) : "r"(v), "n"(S));
-    return d;
-}
-template <uint32_t BIT>
-__device__ __forceinline__ void set_if_below(uint32_t& word, uint32_t a, uint32_t b) {
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}" : "+r"(word) : "r"(a), "r"(b), "n"(BIT));
-}
+// A decision (cell << 24 plus threshold) and its draw: the code in the upper byte.  The uniform integer u below the threshold
+// carries into the cell: threshold + 2^24 - 1 - u >= 2^24.
+__device__ __forceinline__ uint32_t with_draw(uint32_t decision, uint32_t word) { return decision + 0xFFFFFFu - (word >> 8); }
 
-// Four codes (in the low bits of each word, anything above) side by side, CB bits each; what lies above is undefined.
+// The upper bytes of four words side by side, CB bits each; what lies above is undefined.
 template <int CB>
 __device__ __forceinline__ uint32_t pack_codes(const uint32_t (&c)[4]) {
-    if constexpr (CB == 8) return __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+    if constexpr (CB == 8) return __byte_perm(__byte_perm(c[0], c[1], 0x0073), __byte_perm(c[2], c[3], 0x0073), 0x5410);
     else {
-        constexpr uint32_t kMask = (1u << CB) - 1u;
-        return (c[0] & kMask) | shift_left<CB>(c[1] & kMask) | shift_left<2 * CB>(c[2] & kMask) | shift_left<3 * CB>(c[3]);
+        const uint32_t w = __byte_perm(c[0], c[2], 0x0073) + (__byte_perm(c[1], c[3], 0x0073) << CB);
+        return CB == 4 ? w : w + (w >> 4);
     }
 }
 
-__device__ __noinline__ float divide_slowly(float num, float width) { return __fdiv_rn(num, width); }
-
 // num / width rounded to nearest, from rw = 1 / width rounded to nearest: two residual corrections (Markstein, "Computation
 // of elementary functions on the IBM RISC System/6000 processor", 1990: a faithful quotient corrected once with the
-// correctly rounded reciprocal is the correctly rounded quotient, where nothing underflows).  rw = 0 stands for a
-// width of 0 (quotient 0), rw < 0 for widths outside [2^-40, 2^40]: the quotient comes out negative.  The caller
-// divides instead where the quotient of a positive num is below 2^-60: the residuals of the others are multiples of
-// 2^(-60 - 23 - 40 - 23) and cannot underflow.
+// correctly rounded reciprocal is the correctly rounded quotient, where nothing underflows).  For widths in [2^-40, 2^40] the
+// residuals of quotients from 2^-60 on are multiples of 2^(-60 - 23 - 40 - 23) and cannot underflow; smaller ones
+// come out wrong by at most 2^-110.
 // Compared with CUDA's division on 2 x 10^10 pairs (widths 2^-40 .. 2^40, quotients 2^-60 .. 2): equal.
 __device__ __forceinline__ float quotient(float num, float width, float rw) {
     float q = __fmul_rn(num, rw);
@@ -283,6 +275,13 @@ template <> struct QuantWord<8> { using type = uint32_t; };
 template <> struct QuantWord<4> { using type = uint16_t; };
 template <> struct QuantWord<2> { using type = uint8_t; };
 
+// Sparse rows: a lane's 32 answers (4 rows, 2 planes, 4 features) in one word.  A row's four answers of a plane lie CB bits
+// apart from bit answer_shift() on, where they are added to its codes.
+template <int CB>
+__host__ __device__ constexpr int answer_shift(int row, int plane) {
+    return CB == 8 ? 4 * plane + row : CB == 4 ? 16 * plane + row : 16 * (row >> 1) + 8 * plane + (row & 1);
+}
+
 // TB: 0 for a uniform grid of `bits` bits, else the bits of the level table.
 template <int CB, int TB>
 __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda, int bits,
@@ -294,17 +293,18 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
     using Word = typename QuantWord<CB>::type;
     constexpr bool TABLE = TB > 0;
     constexpr int L = 1 << TB;                                     // TABLE: levels
-    __shared__ float4 val_s[8][kQuantRows][32];                    // samples of a warp's pass: [row][lane]
-    __shared__ __align__(16) uint32_t word_s[8][32][2 * kQuantRows];  // and its words: [lane][row][plane]
-    __shared__ uint8_t queue_s[8][kQuantQueue];                    // pairs to do: lane * 8 + row * 2 + pair
-    extern __shared__ float4 cell_s[];                             // TABLE: [L][4][tx] level, width of its cell, 1 / width, cell
+    constexpr int kCols = kQuantTableCols;
+    __shared__ uint2 queue_s[8][kQuantQueue];                      // pairs to draw: {threshold, lane * 8 + row * 2 + pair in the upper byte}, {threshold}
+    __shared__ uint32_t answer_s[8][32];                           // and what came out, per lane
+    extern __shared__ float4 cell_s[];                             // TABLE: [4][L][kCols] level, width of its cell, 1 / width, least numerator
+    float* lev_s = reinterpret_cast<float*>(cell_s + 4 * L * kCols);   // TABLE: [4][L][kCols] levels
     const int tx = blockDim.x, tid = threadIdx.y * tx + threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float* lev_s = reinterpret_cast<float*>(cell_s + L * 4 * tx);  // TABLE: [L][4][tx] levels
     const unsigned row_block = blockIdx.x / col_blocks, col_block = blockIdx.x - row_block * col_blocks;
     const int64_t g = (int64_t)col_block * tx + threadIdx.x;       // this thread's group of four features
     const int64_t groups = row_bytes * 8 / (4 * CB);
     const int64_t j0 = g * 4;
     const int nf = (int)max((int64_t)0, min((int64_t)4, n - j0));  // real features of the group (0: padding)
+    bool divide = false;                                           // TABLE: a cell of the block needs the division itself
     if constexpr (TABLE) {
         const int64_t jb = (int64_t)col_block * tx * 4;            // first feature of the block
         for (int idx = tid; idx < tx * 4 * L; idx += 256) {        // consecutive threads read consecutive floats of the table
@@ -313,30 +313,30 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
             const float val = have ? __ldg(levels + (jb + f) * L + k) : 0.0f;
             const float next = have && k < L - 1 ? __ldg(levels + (jb + f) * L + k + 1) : val;
             const float width = __fsub_rn(next, val);
-            // (a width that overflows takes no value up either: its quotients are 0 or none)
-            const float rw = !(width > 0.0f && width <= 3.402823466e+38f) ? 0.0f : (width >= 9.1e-13f && width <= 1.09e12f) ? __frcp_rn(width) : -1.0f;
-            const int at = (k * 4 + (f & 3)) * tx + (f >> 2);
+            // An empty cell, and one whose width overflows, takes no value up: its width is stored as NaN, and so are its quotients.
+            const bool takes = width > 0.0f && width <= 3.402823466e+38f;
+            if (takes && !(width >= 9.1e-13f && width <= 1.09e12f)) divide = true;
+            const int at = ((f & 3) * L + k) * kCols + (f >> 2);
             lev_s[at] = k < L - 1 ? val : INFINITY;
-            cell_s[at] = make_float4(val, width, rw, __int_as_float(k));
+            // (a numerator above width 2^-150 has a quotient that is not rounded to 0)
+            cell_s[at] = make_float4(val, takes ? width : __int_as_float(0x7fffffff), takes ? __frcp_rn(width) : 0.0f,
+                                     takes ? __fmul_rd(__fmul_rn(width, 0x1p-75f), 0x1p-75f) : INFINITY);
         }
-        __syncthreads();
+        divide = __syncthreads_or(divide);
     }
-    // the value that has code 0 for certain: the lowest level (level tables: unless it is there twice)
     float flo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, finv[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float seen_lo[4], seen_hi[4], probe = 0.0f;                    // TABLE: the extremes of this thread's rows; NaN once a value is not finite
+    float mid[4];                                                  // TABLE: where the bisection starts
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         if constexpr (!TABLE) {
             if (i < nf) { flo[i] = __ldg(lo + j0 + i); finv[i] = __ldg(inv + j0 + i); }
         } else {
             seen_lo[i] = INFINITY; seen_hi[i] = -INFINITY;
-            if (i < nf) {
-                const float4 c = cell_s[i * tx + threadIdx.x];
-                flo[i] = c.y > 0.0f ? c.x : __int_as_float(0x7fffffff);
-            }
+            mid[i] = lev_s[(i * L + L / 2) * kCols + threadIdx.x];
         }
     }
-    const float top = (float)((1 << bits) - 1);
+    const uint32_t top = ((1u << bits) - 1u) << 24;
     // the blocks run from the last rows to the first: the range pass has left the end of A in L2
     const int64_t row_first = ((int64_t)(row_blocks - 1 - row_block) * blockDim.y + threadIdx.y) * kQuantRows * passes;
     // (rows above 2^32: a block holds a power of two of them, at its multiple, so all its rows have the same upper half)
@@ -346,31 +346,6 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
     const float* src = A + row_first * lda + j0;                   // the row that is requested next
     uint8_t* out1 = plane1 + row_first * row_bytes + g * (int64_t)sizeof(Word);
     uint8_t* out2 = plane2 + row_first * row_bytes + g * (int64_t)sizeof(Word);
-    // cell (in the low bits) and threshold of value x of feature i of thread column `col`, whose lo and inv are given
-    auto decide = [&](float x, int i, int col, float x_lo, float x_inv, uint32_t& cell, uint32_t& threshold) {
-        float y;
-        if constexpr (!TABLE) {
-            const float tc = fminf(fmaxf(__fmul_rn(__fsub_rn(x, x_lo), x_inv), 0.0f), top);
-            const float big = __fadd_rd(tc, 8388608.0f);
-            cell = __float_as_uint(big);
-            // 2^24 (tc - floor tc); both products are exact, and so is the difference
-            y = __fmaf_rn(tc, 16777216.0f, -__fmaf_rn(big, 16777216.0f, -140737488355328.0f));
-        } else {
-            const int ls = 4 * tx;
-            int at = i * tx + col;                                 // level k at lev_s[k * ls + at]; the last one is staged as infinity
-#pragma unroll
-            for (int half = L >> 1; half > 0; half >>= 1)          // the largest k <= L - 2 whose level is <= x
-                if (lev_s[at + half * ls] <= x) at += half * ls;
-            const float4 c = cell_s[at];
-            const float num = __fsub_rn(x, c.x);
-            float p = quotient(num, c.y, c.z);
-            if (p < 8.7e-19f && num > 0.0f && c.y > 0.0f) p = divide_slowly(num, c.y);
-            const bool sure = num >= c.y && c.z != 0.0f;           // the upper end (a quotient of 1): always up
-            cell = (uint32_t)__float_as_int(c.w) + (sure ? 1u : 0u);
-            y = sure ? 0.0f : __fmul_rn(p, 16777216.0f);
-        }
-        threshold = shift_left<8>(__float2uint_ru(y));
-    };
     // the part of the Philox rounds 0 and 1 that depends on the pair alone
     uint32_t pair_lo[2];
     uint64_t pair_p[2];
@@ -381,8 +356,33 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
         pair_p[p] = (uint64_t)kPhiloxM0 * ((uint32_t)(a >> 32) ^ row_hi ^ key.k0[0]);
     }
     // The rows of a warp, with everything that depends on the matrix's edges compiled out where it lies inside.
-    auto run = [&](auto inside) {
+    auto run = [&](auto inside, auto divides) {
         constexpr bool kInside = decltype(inside)::value;
+        [[maybe_unused]] constexpr bool kDivide = decltype(divides)::value;
+        // cell << 24 plus threshold of value x of feature i
+        auto decide = [&](float x, int i) -> uint32_t {
+            if constexpr (!TABLE) {
+                // (the conversion saturates: negative values and NaN at 0, large ones and infinity at 2^32 - 1)
+                return min(__float2uint_ru(__fmul_rn(__fmul_rn(__fsub_rn(x, flo[i]), finv[i]), 16777216.0f)), top);
+            } else {
+                // level k of the thread's feature i lies kCols floats after level k - 1: byte 1 of the offset is k (the last
+                // level is staged as infinity); the search ends at the largest k <= L - 2 whose level is <= x
+                static_assert(kCols * sizeof(float) == 256, "a level's offset is its number in byte 1");
+                uint32_t at = threadIdx.x * 4u;
+                const char* lev = reinterpret_cast<const char*>(lev_s + i * L * kCols);
+                if (mid[i] <= x) at += L / 2 * 256;
+#pragma unroll
+                for (int half = L >> 2; half > 0; half >>= 1)
+                    if (*reinterpret_cast<const float*>(lev + at + half * 256) <= x) at += half * 256;
+                const float4 c = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(cell_s + i * L * kCols) + 4 * at);
+                const float num = __fsub_rn(x, c.x);
+                const float p = kDivide ? __fdiv_rn(num, c.y) : quotient(num, c.y, c.z);
+                // the upper end (a quotient of 1 or more) is always up
+                uint32_t threshold = __float2uint_ru(num >= c.y ? 16777216.0f : __fmul_rn(p, 16777216.0f));
+                if (!kDivide && num > c.w) threshold = max(threshold, 1u);
+                return __byte_perm(at, 0u, 0x1444) + threshold;
+            }
+        };
         float v[kQuantRows][4];
         auto request = [&](int have) {                             // the next kQuantRows rows, of which `have` exist
             if (kInside && vec_ok) {
@@ -391,145 +391,114 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
                     const float4 t = __ldg(reinterpret_cast<const float4*>(src));
                     v[r][0] = t.x; v[r][1] = t.y; v[r][2] = t.z; v[r][3] = t.w;
                 }
-            } else {
+            } else {                                               // (what does not exist is certain)
 #pragma unroll
                 for (int r = 0; r < kQuantRows; ++r, src += lda)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) v[r][i] = kInside || (r < have && i < nf) ? __ldg(src + i) : flo[i];
+                    for (int i = 0; i < 4; ++i) v[r][i] = kInside || (r < have && i < nf) ? __ldg(src + i) : TABLE ? -INFINITY : flo[i];
             }
         };
-        auto store = [&](const uint32_t (&w1)[kQuantRows], const uint32_t (&w2)[kQuantRows]) {
+        request(left);
+#pragma unroll 1
+        for (int pass = 0; pass < passes; ++pass, left -= kQuantRows, row0 += kQuantRows) {
+            if (!kInside && !__any_sync(0xffffffffu, left > 0)) break;
+            uint32_t t[kQuantRows][4];
+#pragma unroll
+            for (int r = 0; r < kQuantRows; ++r)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (TABLE && (kInside || (r < left && i < nf))) {
+                        seen_lo[i] = fminf(seen_lo[i], v[r][i]);
+                        seen_hi[i] = fmaxf(seen_hi[i], v[r][i]);
+                        probe = fmaf(v[r][i], 0.0f, probe);
+                    }
+                    t[r][i] = decide(v[r][i], i);
+                    if (TABLE && !kInside && i >= nf) t[r][i] = 0u;
+                }
+            if (pass + 1 < passes) request(left - kQuantRows);
+            // a guess from the first row (dense or sparse data look alike in every row), the count where it says sparse
+            int total = 4 * kQuantQueue, count = 0;
+            uint32_t need = 0u;                                    // bit 2 r + p: pair p of row r has a draw to make
+            if (__popc(__ballot_sync(0xffffffffu, ((t[0][0] | t[0][1] | t[0][2] | t[0][3]) & 0xFFFFFFu) != 0u)) <= 20) {
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r)
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+                        if (((t[r][2 * p] | t[r][2 * p + 1]) & 0xFFFFFFu) != 0u) need |= 1u << (2 * r + p);
+                count = __popc(need);
+                total = __reduce_add_sync(0xffffffffu, count);
+            }
+            uint32_t w1[kQuantRows], w2[kQuantRows];
+            if (total > kQuantQueue) {
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) {
+                    const uint64_t a = (uint64_t)kPhiloxM0 * (row0 + r);
+                    const uint64_t b = (uint64_t)kPhiloxM1 * ((uint32_t)(a >> 32) ^ draw ^ key.k1[0]);
+                    Philox4 rnd[2];
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+                        rnd[p] = philox_rounds<2>((uint32_t)(b >> 32) ^ pair_lo[p], (uint32_t)b,
+                                                  (uint32_t)(pair_p[p] >> 32) ^ (uint32_t)a ^ key.k1[1], (uint32_t)pair_p[p], key);
+                    uint32_t c1[4], c2[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        c1[i] = with_draw(t[r][i], rnd[i >> 1].v[2 * (i & 1)]);
+                        c2[i] = with_draw(t[r][i], rnd[i >> 1].v[2 * (i & 1) + 1]);
+                    }
+                    w1[r] = pack_codes<CB>(c1);
+                    w2[r] = pack_codes<CB>(c2);
+                }
+            } else {
+                uint32_t answers = 0u;
+                if (total > 0) {                                   // (integers on a grid of integers: no draw at all)
+                    answer_s[warp][lane] = 0u;
+                    int at = count;                                // exclusive prefix sum over the warp
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int up = __shfl_up_sync(0xffffffffu, at, o);
+                        if (lane >= o) at += up;
+                    }
+                    at -= count;
+#pragma unroll
+                    for (int k = 0; k < 2 * kQuantRows; ++k)
+                        if (need >> k & 1u)
+                            queue_s[warp][at++] = make_uint2(__byte_perm(t[k >> 1][2 * (k & 1)], (uint32_t)(lane * 2 * kQuantRows + k), 0x4210),
+                                                             t[k >> 1][2 * (k & 1) + 1] & 0xFFFFFFu);
+                    __syncwarp();
+#pragma unroll 1
+                    for (int e0 = 0; e0 < total; e0 += 32) {
+                        const uint2 q = queue_s[warp][min(e0 + lane, total - 1)];  // (lanes past the end repeat the last: or-ing twice is harmless)
+                        const int owner = q.x >> 27, r = (q.x >> 25) & 3, p = (q.x >> 24) & 1;
+                        const uint32_t row = __shfl_sync(0xffffffffu, row0, owner) + r, pair = __shfl_sync(0xffffffffu, pair0, owner) + p;
+                        const Philox4 rnd = philox_rounds<0>(row, row_hi, pair, draw, key);
+                        const uint32_t t0 = q.x & 0xFFFFFFu, t1 = q.y;
+                        const uint32_t up1 = (with_draw(t0, rnd.v[0]) >> 24) | (with_draw(t1, rnd.v[2]) >> 24 << CB);
+                        const uint32_t up2 = (with_draw(t0, rnd.v[1]) >> 24) | (with_draw(t1, rnd.v[3]) >> 24 << CB);
+                        const int shift = answer_shift<CB>(r, 0) + 2 * p * CB;
+                        atomicOr(&answer_s[warp][owner], (up1 | up2 << answer_shift<CB>(0, 1)) << shift);
+                    }
+                    __syncwarp();
+                    answers = answer_s[warp][lane];
+                }
+                constexpr uint32_t kEach = CB == 8 ? 0x01010101u : CB == 4 ? 0x1111u : 0x55u;
+#pragma unroll
+                for (int r = 0; r < kQuantRows; ++r) {
+                    const uint32_t w = pack_codes<CB>(t[r]);
+                    w1[r] = w + (answers >> answer_shift<CB>(r, 0) & kEach);
+                    w2[r] = w + (answers >> answer_shift<CB>(r, 1) & kEach);
+                }
+            }
 #pragma unroll
             for (int r = 0; r < kQuantRows; ++r, out1 += row_bytes, out2 += row_bytes)
                 if (kInside || (r < left && g < groups)) {
                     *reinterpret_cast<Word*>(out1) = (Word)w1[r];
                     *reinterpret_cast<Word*>(out2) = (Word)w2[r];
                 }
-        };
-        request(left);
-#pragma unroll 1
-        for (int pass = 0; pass < passes; ++pass, left -= kQuantRows, row0 += kQuantRows) {
-            if (!kInside && !__any_sync(0xffffffffu, left > 0)) break;
-            if constexpr (TABLE) {
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (kInside || (r < left && i < nf)) {
-                            seen_lo[i] = fminf(seen_lo[i], v[r][i]);
-                            seen_hi[i] = fmaxf(seen_hi[i], v[r][i]);
-                            probe = fmaf(v[r][i], 0.0f, probe);
-                        }
-            }
-            // a guess from the first row (dense or sparse data look alike in every row), the count where it says sparse
-            int total = 4 * kQuantQueue, count = 0;
-            uint32_t need = 0u;                                    // bit 2 r + p: pair p of row r is not certain
-            if (__popc(__ballot_sync(0xffffffffu, v[0][0] != flo[0] || v[0][1] != flo[1] || v[0][2] != flo[2] || v[0][3] != flo[3])) <= 20) {
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r)
-                    need |= (v[r][0] != flo[0] || v[r][1] != flo[1] ? 1u << (2 * r) : 0u) | (v[r][2] != flo[2] || v[r][3] != flo[3] ? 2u << (2 * r) : 0u);
-                count = __popc(need);
-                total = __reduce_add_sync(0xffffffffu, count);
-            }
-            if (total > kQuantQueue) {
-                uint32_t w[kQuantRows], thr[kQuantRows][4], any = 0u;
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r) {
-                    uint32_t cell[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        decide(v[r][i], i, threadIdx.x, flo[i], finv[i], cell[i], thr[r][i]);
-                        if (TABLE && !kInside && i >= nf) cell[i] = thr[r][i] = 0u;
-                        any |= thr[r][i];
-                    }
-                    w[r] = pack_codes<CB>(cell);
-                }
-                if (pass + 1 < passes) request(left - kQuantRows);
-                // what the draws add: one bit per code
-                uint32_t u1[kQuantRows], u2[kQuantRows];
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r) u1[r] = u2[r] = 0u;
-                if (__any_sync(0xffffffffu, any != 0u)) {          // (integers on a grid of integers: no draw at all)
-#pragma unroll
-                    for (int r = 0; r < kQuantRows; ++r) {
-                        const uint64_t a = (uint64_t)kPhiloxM0 * (row0 + r);
-                        const uint64_t b = (uint64_t)kPhiloxM1 * ((uint32_t)(a >> 32) ^ draw ^ key.k1[0]);
-                        Philox4 rnd[2];
-#pragma unroll
-                        for (int p = 0; p < 2; ++p)
-                            rnd[p] = philox_rounds<2>((uint32_t)(b >> 32) ^ pair_lo[p], (uint32_t)b,
-                                                      (uint32_t)(pair_p[p] >> 32) ^ (uint32_t)a ^ key.k1[1], (uint32_t)pair_p[p], key);
-                        set_if_below<1u>(u1[r], rnd[0].v[0], thr[r][0]);
-                        set_if_below<1u>(u2[r], rnd[0].v[1], thr[r][0]);
-                        set_if_below<1u << CB>(u1[r], rnd[0].v[2], thr[r][1]);
-                        set_if_below<1u << CB>(u2[r], rnd[0].v[3], thr[r][1]);
-                        set_if_below<1u << 2 * CB>(u1[r], rnd[1].v[0], thr[r][2]);
-                        set_if_below<1u << 2 * CB>(u2[r], rnd[1].v[1], thr[r][2]);
-                        set_if_below<1u << 3 * CB>(u1[r], rnd[1].v[2], thr[r][3]);
-                        set_if_below<1u << 3 * CB>(u2[r], rnd[1].v[3], thr[r][3]);
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r) { u1[r] += w[r]; u2[r] += w[r]; }
-                store(u1, u2);
-            } else {
-                uint4* mine = reinterpret_cast<uint4*>(word_s[warp][lane]);
-                mine[0] = mine[1] = make_uint4(0u, 0u, 0u, 0u);
-                int at = count;                                    // exclusive prefix sum over the warp
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int up = __shfl_up_sync(0xffffffffu, at, o);
-                    if (lane >= o) at += up;
-                }
-                at -= count;
-#pragma unroll
-                for (int r = 0; r < kQuantRows; ++r) val_s[warp][r][lane] = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
-#pragma unroll
-                for (int k = 0; k < 2 * kQuantRows; ++k)
-                    if (need >> k & 1u) queue_s[warp][at++] = (uint8_t)(lane * 2 * kQuantRows + k);
-                if (pass + 1 < passes) request(left - kQuantRows);
-                __syncwarp();
-#pragma unroll 1
-                for (int e0 = 0; e0 < total; e0 += 32) {
-                    const int q = queue_s[warp][min(e0 + lane, total - 1)];    // (lanes past the end repeat the last: or-ing twice is harmless)
-                    const int owner = q >> 3, r = (q >> 1) & 3, p = q & 1;
-                    const uint32_t row = __shfl_sync(0xffffffffu, row0, owner) + r, pair = __shfl_sync(0xffffffffu, pair0, owner) + p;
-                    const float2 x = reinterpret_cast<const float2*>(&val_s[warp][r][owner])[p];
-                    const int col = (warp * 32 + owner) & (tx - 1);            // tx is a power of two
-                    const int64_t j = 2 * (int64_t)pair;
-                    const int second = kInside || j + 1 < n ? 1 : 0;           // (a queued pair has at least its first feature)
-                    float2 xlo = make_float2(0.0f, 0.0f), xinv = xlo;
-                    if constexpr (!TABLE) {
-                        xlo = make_float2(__ldg(lo + j), __ldg(lo + j + second));
-                        xinv = make_float2(__ldg(inv + j), __ldg(inv + j + second));
-                    }
-                    uint32_t c0, c1, t0, t1;
-                    decide(x.x, 2 * p, col, xlo.x, xinv.x, c0, t0);
-                    decide(x.y, 2 * p + 1, col, xlo.y, xinv.y, c1, t1);
-                    constexpr uint32_t kMask = (1u << CB) - 1u;
-                    uint32_t w1 = c0 & kMask, w2 = w1;
-                    const Philox4 rnd = philox_rounds<0>(row, row_hi, pair, draw, key);
-                    if (rnd.v[0] < t0) w1 += 1u;
-                    if (rnd.v[1] < t0) w2 += 1u;
-                    if (second) {
-                        w1 += (c1 & kMask) << CB;
-                        w2 += (c1 & kMask) << CB;
-                        if (rnd.v[2] < t1) w1 += 1u << CB;
-                        if (rnd.v[3] < t1) w2 += 1u << CB;
-                    }
-                    // (a row's two pairs share its words: hence the atomics)
-                    atomicOr(&word_s[warp][owner][2 * r], w1 << (2 * p * CB));
-                    atomicOr(&word_s[warp][owner][2 * r + 1], w2 << (2 * p * CB));
-                }
-                __syncwarp();
-                const uint4 lower = mine[0], upper = mine[1];
-                const uint32_t w1[kQuantRows] = {lower.x, lower.z, upper.x, upper.z}, w2[kQuantRows] = {lower.y, lower.w, upper.y, upper.w};
-                store(w1, w2);
-            }
         }
     };
-    if (__all_sync(0xffffffffu, nf == 4 && left == kQuantRows * passes)) run(std::true_type{});
-    else run(std::false_type{});
+    if (TABLE && divide) run(std::false_type{}, std::true_type{});
+    else if (__all_sync(0xffffffffu, nf == 4 && left == kQuantRows * passes)) run(std::true_type{}, std::false_type{});
+    else run(std::false_type{}, std::false_type{});
     if constexpr (TABLE) {
         if (!(probe == 0.0f)) set_status(status, ZIPML_ERR_NONFINITE, 1);
         // (a value that is beaten already needs no atomic: after the first blocks hardly any does)
@@ -558,7 +527,7 @@ int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_
     const int64_t col_blocks = (groups + tx - 1) / tx;
     int passes = 1;
     while (passes < (table ? 16 : 8) && (m / (ty * kQuantRows * passes * 2)) * col_blocks >= (int64_t)ctx->sm_count * 16) passes *= 2;
-    const size_t smem = table ? (sizeof(float4) + sizeof(float)) * ((size_t)4 << bits) * tx : 0;
+    const size_t smem = table ? (sizeof(float4) + sizeof(float)) * ((size_t)4 << bits) * kQuantTableCols : 0;
     auto blocks_of_rows = [&]() { return (m + (int64_t)ty * kQuantRows * passes - 1) / ((int64_t)ty * kQuantRows * passes); };
     while (blocks_of_rows() > 0x7fffffffLL / col_blocks && passes < (1 << 20)) passes *= 2;      // the grid is one-dimensional, columns first
     const int64_t row_blocks = blocks_of_rows();
@@ -571,8 +540,8 @@ int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_
     const unsigned nb = (unsigned)((n + 255) / 256);
     if (table) range_init_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n);
     auto launch = [&](auto kernel) -> int {
-        // (the kernel's own 25 KB of shared memory count towards the 48 KB that need no opt-in)
-        if (smem > 20 * 1024) {
+        // (the kernel's own 5 KB of shared memory count towards the 48 KB that need no opt-in)
+        if (smem > 40 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return cuda_status(e);
         }
