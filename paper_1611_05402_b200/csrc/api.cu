@@ -157,9 +157,13 @@ int zipml_create(zipml_ctx** ctx_out, int device, void* cuda_stream) {
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_status, 0, sizeof(DeviceStatus), ctx->stream);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->exchange), kExchangeBytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->exchange, 0, kExchangeBytes, ctx->stream);
+    constexpr size_t kRangeBytes = sizeof(uint32_t) * (2 * kRangeColumns + kRangeTiles);
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ctx->range_keys), kRangeBytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->range_keys, 0, kRangeBytes, ctx->stream);
     if (e != cudaSuccess) {
         if (ctx->d_status) (void)cudaFree(ctx->d_status);
         if (ctx->exchange) (void)cudaFree(ctx->exchange);
+        if (ctx->range_keys) (void)cudaFree(ctx->range_keys);
         delete ctx;
         return cuda_status(e);
     }
@@ -174,6 +178,7 @@ int zipml_destroy(zipml_ctx* ctx) {
     if (ctx->ws) (void)cudaFree(ctx->ws);
     if (ctx->stage) (void)cudaFree(ctx->stage);
     if (ctx->exchange) (void)cudaFree(ctx->exchange);
+    if (ctx->range_keys) (void)cudaFree(ctx->range_keys);
     if (ctx->d_status) (void)cudaFree(ctx->d_status);
     (void)cudaGetLastError();
     delete ctx;
@@ -226,18 +231,15 @@ int zipml_quantize_draw(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return ZIPML_ERR_CUDA;
     const int s = (1 << bits) - 1;
-    int rc = ws_reserve(ctx, carve_size(sizeof(uint32_t) * 2 * (size_t)n) + 2 * carve_size(sizeof(float) * (size_t)n));
-    if (rc != ZIPML_OK) return rc;
-    Carver cv(ctx->ws);
-    uint32_t* keys = cv.take<uint32_t>(2 * (size_t)n);
-    float* inv = cv.take<float>((size_t)n);
-    float* step_tmp = cv.take<float>((size_t)n);
-    float* step = feat_step ? feat_step : step_tmp;
+    float* inv = nullptr;
     if (level_mode == ZIPML_LEVELS_UNIFORM) {
-        rc = launch_column_range(ctx, A, m, n, lda, s, grid == ZIPML_GRID_SYMMETRIC, keys, feat_lo, nullptr, inv, step);
+        int rc = ws_reserve(ctx, carve_size(sizeof(float) * (size_t)n));
+        if (rc != ZIPML_OK) return rc;
+        inv = reinterpret_cast<float*>(ctx->ws);
+        rc = launch_column_range(ctx, A, m, n, lda, s, grid == ZIPML_GRID_SYMMETRIC, feat_lo, nullptr, inv, feat_step);
         if (rc != ZIPML_OK) return rc;
     }
-    return launch_quantize(ctx, A, m, n, lda, bits, level_mode, feat_lo, inv, levels, seed, draw, plane1, plane2, row_bytes, keys, feat_lo, step);
+    return launch_quantize(ctx, A, m, n, lda, bits, level_mode, feat_lo, inv, levels, seed, draw, plane1, plane2, row_bytes, feat_lo, feat_step);
 }
 
 int zipml_optimal_levels(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int32_t bits,
@@ -249,16 +251,14 @@ int zipml_optimal_levels(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, i
     if (hist_bins < s || hist_bins > 1024 || m > 1000000000LL) return ZIPML_ERR_UNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return ZIPML_ERR_CUDA;
-    int rc = ws_reserve(ctx, carve_size(sizeof(uint32_t) * 2 * (size_t)n) + 3 * carve_size(sizeof(float) * (size_t)n) +
-                                 carve_size(sizeof(uint32_t) * (size_t)n * hist_bins));
+    int rc = ws_reserve(ctx, 3 * carve_size(sizeof(float) * (size_t)n) + carve_size(sizeof(uint32_t) * histogram_count(n, hist_bins)));
     if (rc != ZIPML_OK) return rc;
     Carver cv(ctx->ws);
-    uint32_t* keys = cv.take<uint32_t>(2 * (size_t)n);
     float* lo = cv.take<float>((size_t)n);
     float* hi = cv.take<float>((size_t)n);
     float* inv = cv.take<float>((size_t)n);
-    uint32_t* counts = cv.take<uint32_t>((size_t)n * hist_bins);
-    rc = launch_column_range(ctx, A, m, n, lda, hist_bins, false, keys, lo, hi, inv, nullptr);
+    uint32_t* counts = cv.take<uint32_t>(histogram_count(n, hist_bins));
+    rc = launch_column_range(ctx, A, m, n, lda, hist_bins, false, lo, hi, inv, nullptr);
     if (rc != ZIPML_OK) return rc;
     rc = launch_histogram(ctx, A, m, n, lda, hist_bins, lo, inv, counts);
     if (rc != ZIPML_OK) return rc;

@@ -27,6 +27,8 @@ struct zipml_ctx {
     // words between the clusters of the cluster engine's int8 forms, and the next tag (see sgd_slice.cu, sgd_feature.cu)
     unsigned char* exchange = nullptr;   // kExchangeBytes, for the context's life (recorded launches hold its address)
     uint32_t exchange_tag = 1;
+    // keys of a range pass, 2 x kRangeColumns, and its blocks' counters, kRangeTiles: all 0 between passes (the pass clears what it used)
+    uint32_t* range_keys = nullptr;
     int64_t launches = 0;           // kernels launched so far (diagnostics)
     int last_engine = 0;            // engine of the latest zipml_sgd_epoch call, and its kernel (diagnostics)
     const char* last_kernel = "";
@@ -47,6 +49,10 @@ int stage_reserve(zipml_ctx* ctx, size_t bytes);
 // bytes for each of 8,192 features and what the last slice or column has past them.
 constexpr size_t kExchangeBytes = 2 * 8 * (8192 + 1024) * 16;
 int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag);
+
+// Columns that a range pass takes per launch, and the column tiles of one: at least 256 columns each where there are several.
+constexpr int64_t kRangeColumns = 65536;
+constexpr int64_t kRangeTiles = kRangeColumns / 256;
 
 // The fp32 constant of zipml_sgd_params' regulariser for step length lr (see regularise() in common.cuh).
 inline float reg_constant(const zipml_sgd_params* p) {
@@ -73,14 +79,13 @@ inline size_t carve_size(size_t bytes) { return (bytes + 255) / 256 * 256; }
 // Column range: lo/hi per feature, inv = s/(hi-lo) and step = (hi-lo)/s for a grid of s intervals.
 // Any of hi_out, inv_out, step_out may be null.  Sets NONFINITE in the device status.
 int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int s, bool symmetric,
-                        uint32_t* key_scratch /* 2n */, float* lo_out, float* hi_out, float* inv_out,
-                        float* step_out);
+                        float* lo_out, float* hi_out, float* inv_out, float* step_out);
 
 // Uniform levels: on the grid (lo, inv) that launch_column_range has found.  Level tables: lo, inv unused; the range is
-// found on the way (2n keys of scratch) and lo_out, step_out written as launch_column_range would.
+// found on the way and lo_out, step_out (may be null) written as launch_column_range would.
 int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bits, int level_mode,
                     const float* lo, const float* inv, const float* levels, uint64_t seed, uint32_t draw, uint8_t* plane1,
-                    uint8_t* plane2, int64_t row_bytes, uint32_t* key_scratch, float* lo_out, float* step_out);
+                    uint8_t* plane2, int64_t row_bytes, float* lo_out, float* step_out);
 int launch_code_weights(zipml_ctx* ctx, const zipml_dataset* d, const float* x, float* wtab, double* base);
 int launch_poly_rows(zipml_ctx* ctx, const zipml_dataset* d, const uint8_t* const* planes, int degree, const double* coef,
                      const float* wtab, const double* base, const float* scale, double* rows_out);
@@ -89,7 +94,9 @@ int launch_plane_mean(zipml_ctx* ctx, const zipml_dataset* d, const uint8_t* pla
                       float* g_out);
 
 int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bins,
-                     const float* lo, const float* inv, uint32_t* counts /* n x bins, zeroed here */);
+                     const float* lo, const float* inv, uint32_t* counts /* histogram_count(n, bins), zeroed here */);
+// Counters of a histogram: [tile of 32 features][bin][feature of the tile].
+inline size_t histogram_count(int64_t n, int bins) { return (size_t)((n + 31) / 32 * 32) * (size_t)bins; }
 
 int launch_levels_dp(zipml_ctx* ctx, const uint32_t* counts, int64_t n, int bins, int s, const float* lo,
                      const float* hi, float* levels_out, uint64_t* objective_out);

@@ -8,59 +8,71 @@
 namespace zipml {
 
 // ---------------------------------------------------------------------------------------------
-// Histogram.  A block owns 32 features and a chunk of rows and keeps 32 x bins counters in shared
-// memory (row stride bins+1, so that lanes hitting the same bin of different features fall into
-// different banks).  blockDim = (32, 32): a warp reads 128 contiguous bytes of a row; the counters leave room
-// for one block per SM, so a thread requests eight of its rows before it counts the first (with 8 warps and a row
-// at a time the kernel waited for memory: 1,046 us on 500,000 x 512, now 350 us).
+// Histogram.  A block owns 32 features, a lane each, and keeps their counters in shared memory as [bin][feature]: a
+// warp reads 128 contiguous bytes of a row and counts without bank conflicts whatever the bins are.  The row chunks of a column tile
+// take groups of kHistWarps * kHistAhead rows in turn, from the last to the first (the range pass has left the end of A in L2);
+// a thread has kHistAhead rows requested, each asked for as soon as its register is counted.
+// Bound by HBM: 500,000 x 512 at 1,024 bins 380 -> 155 us ([feature][bin + 1] counters before, whose conflicts took three
+// wavefronts a warp, and 43 instructions a sample, mostly row numbers and addresses in 64 bits).
 // ---------------------------------------------------------------------------------------------
-constexpr int kHistWarps = 32, kHistAhead = 8;
+constexpr int kHistWarps = 32, kHistAhead = 16;
 
+// Offset: unsigned where kHistWarps rows span less than 4 GB, else 64 bits.
+template <typename Offset>
 __global__ void __launch_bounds__(32 * kHistWarps) histogram_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda,
-                                                                    int bins, int64_t rows_per_block,
-                                                                    const float* __restrict__ lo, const float* __restrict__ inv,
+                                                                    int bins, const float* __restrict__ lo, const float* __restrict__ inv,
                                                                     uint32_t* __restrict__ counts) {
     extern __shared__ uint32_t s_hist[];
-    const int stride = bins + 1;
-    const int t = threadIdx.y * 32 + threadIdx.x;
-    for (int i = t; i < 32 * stride; i += 32 * kHistWarps) s_hist[i] = 0u;
+    const int lane = threadIdx.x, warp = threadIdx.y, t = warp * 32 + lane;
+    for (int i = t; i < 32 * bins; i += 32 * kHistWarps) s_hist[i] = 0u;
     __syncthreads();
-    const int64_t j = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
     if (j < n) {
         const float flo = __ldg(lo + j), finv = __ldg(inv + j);
-        const int64_t r0 = (int64_t)blockIdx.y * rows_per_block;
-        const int64_t r1 = min(m, r0 + rows_per_block);
-        uint32_t* mine = s_hist + threadIdx.x * stride;
-        for (int64_t r = r0 + threadIdx.y; r < r1; r += kHistWarps * kHistAhead) {
-            float v[kHistAhead];
+        const uint32_t last = (uint32_t)(bins - 1);
+        uint32_t* mine = s_hist + lane;
+        // floor((v - lo) * inv), the product rounded as the grid prescribes (the conversion saturates, NaN and negative values at 0)
+        auto count = [&](float v) { atomicAdd(mine + 32u * min(__float2uint_rd(__fmul_rn(__fsub_rn(v, flo), finv)), last), 1u); };
+        constexpr int kGroup = kHistWarps * kHistAhead;
+        const int64_t groups = m / kGroup;                          // whole ones
+        const Offset at = ((Offset)warp * (Offset)lda + (Offset)lane) * (Offset)sizeof(float);
+        const char* column = reinterpret_cast<const char*>(A + (int64_t)blockIdx.x * 32);
+        const int64_t part = kHistWarps * lda * (int64_t)sizeof(float);
+        float v[kHistAhead];
+        int64_t q = groups - 1 - blockIdx.y;
+        if (q >= 0) {
+            const char* p = column + q * kHistAhead * part;
 #pragma unroll
-            for (int u = 0; u < kHistAhead; ++u) v[u] = r + u * kHistWarps < r1 ? __ldg(A + (r + u * kHistWarps) * lda + j) : 0.0f;
+            for (int u = 0; u < kHistAhead; ++u, p += part) v[u] = __ldg(reinterpret_cast<const float*>(p + at));
+        }
+        for (; q >= (int64_t)gridDim.y; q -= gridDim.y) {
+            const char* p = column + (q - gridDim.y) * kHistAhead * part;
 #pragma unroll
-            for (int u = 0; u < kHistAhead; ++u) {
-                uint32_t cell;
-                float p;
-                uniform_cell(v[u], flo, finv, bins, cell, p);
-                if (r + u * kHistWarps < r1) atomicAdd(mine + cell, 1u);
+            for (int u = 0; u < kHistAhead; ++u, p += part) {
+                count(v[u]);
+                v[u] = __ldg(reinterpret_cast<const float*>(p + at));
             }
         }
+        if (q >= 0) {
+#pragma unroll
+            for (int u = 0; u < kHistAhead; ++u) count(v[u]);
+        }
+        if (blockIdx.y == gridDim.y - 1)
+            for (int64_t r = groups * kGroup + warp; r < m; r += kHistWarps) count(__ldg(A + r * lda + j));
     }
     __syncthreads();
+    uint32_t* out = counts + (int64_t)blockIdx.x * 32 * bins;
     for (int i = t; i < 32 * bins; i += 32 * kHistWarps) {
-        const int f = i / bins, c = i - f * bins;
-        const int64_t jj = (int64_t)blockIdx.x * 32 + f;
-        const uint32_t v = s_hist[f * stride + c];
-        if (jj < n && v) atomicAdd(counts + jj * bins + c, v);
+        const uint32_t v = s_hist[i];
+        if (gridDim.y == 1) out[i] = v;
+        else if (v) atomicAdd(out + i, v);
     }
 }
 
 int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bins, const float* lo,
                      const float* inv, uint32_t* counts) {
-    cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)(n * bins), ctx->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-    const size_t smem = sizeof(uint32_t) * 32 * (size_t)(bins + 1);
+    const size_t smem = sizeof(uint32_t) * 32 * (size_t)bins;
     if (smem > (size_t)ctx->smem_optin) return ZIPML_ERR_WORKSPACE;
-    e = cudaFuncSetAttribute(histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_status(e);
     // one block per SM at a time: the number of row chunks that leaves the last wave fullest, fewest first (every
     // chunk flushes its counters), of at least 512 rows
     const int64_t col_tiles = (n + 31) / 32;
@@ -71,12 +83,18 @@ int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64
         const double full = (double)blocks / (double)(waves * ctx->sm_count);
         if (full > best * 1.03) { best = full; chunks = c; }
     }
-    int64_t rows_per_block = (m + chunks - 1) / chunks;
-    chunks = (m + rows_per_block - 1) / rows_per_block;
-    histogram_kernel<<<dim3((unsigned)col_tiles, (unsigned)chunks), dim3(32, kHistWarps), smem, ctx->stream>>>(
-        A, m, n, lda, bins, rows_per_block, lo, inv, counts);
-    ctx->launches += 1;
-    return cuda_status(cudaGetLastError());
+    if (chunks > 1) {
+        const cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * histogram_count(n, bins), ctx->stream);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    auto launch = [&](auto kernel) -> int {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_status(e);
+        kernel<<<dim3((unsigned)col_tiles, (unsigned)chunks), dim3(32, kHistWarps), smem, ctx->stream>>>(A, m, n, lda, bins, lo, inv, counts);
+        ctx->launches += 1;
+        return cuda_status(cudaGetLastError());
+    };
+    return lda < (1ll << 32) / (kHistWarps * (int64_t)sizeof(float)) ? launch(histogram_kernel<uint32_t>) : launch(histogram_kernel<uint64_t>);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -97,53 +115,70 @@ int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64
 // over groups of lanes (32 down to 4 a group: the ranges get shorter; 8 in the last round 15 % slower, 2 as fast on
 // short tails, 1 slower).  The minima, and with
 // ascending scans and strict comparisons the leftmost minimisers, are those of the full scan.
-// Measured, a call on 3,000 rows (512 features of 1,024 bins): 7 intervals 536 -> 210 us, 15 intervals 1,228 -> 452;
-// bound by the chain of the rounds (load, two multiply-adds, compare, a few shuffles, barrier).
+// The three edges between two neighbours are searched together, on one load of a candidate (7 intervals 155 -> 145 us).
+// Measured, a call on 3,000 rows (512 features of 1,024 bins) against the full scan: 7 intervals 536 -> 210 us, 15 intervals
+// 1,228 -> 452; bound by the chain of the rounds (load, two multiply-adds, compare, a few shuffles, barrier).
 // ---------------------------------------------------------------------------------------------
 constexpr int kDpThreads = 256;
+constexpr int kDpRun = 1024 / kDpThreads;       // bins that a thread sums, at most
 
-// E_k(mm) and its leftmost minimiser over j_lo .. j_hi by a group of G lanes; every lane of the warp takes part.
-template <int G>
-__device__ __forceinline__ void dp_minimise(const double* D, const double* prev, double* cur, unsigned short* ak, bool valid, int mm,
+// E_k and its leftmost minimiser for the N edges first, first + S, .. over j_lo .. j_hi by a group of G lanes; every lane of the warp
+// takes part.  N edges share the loads of a candidate.  Of several edges, one counts where it is at least k, and a candidate where it
+// lies below the edge.
+template <int G, int N, int S>
+__device__ __forceinline__ void dp_minimise(const double* D, const double* prev, double* cur, unsigned short* ak, bool valid, int k, int first,
                                             int j_lo, int j_hi) {
     const int lane = threadIdx.x & 31;
-    double best = INFINITY;
-    int bj = 0x7fffffff;
+    double best[N];
+    int bj[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) { best[u] = INFINITY; bj[u] = 0x7fffffff; }
     if (valid) {
-        const double dm = D[mm], md = (double)mm;
+        double dm[N], md[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) { dm[u] = D[first + u * S]; md[u] = (double)(first + u * S); }
         int j = j_lo + (lane & (G - 1));
         double jd = -(double)j;                                     // (counted along: conversions are slow)
-#pragma unroll 4
+#pragma unroll 2
         for (; j <= j_hi; j += G, jd -= (double)G) {
-            const double c = fma(jd, dm, fma(md, D[j], prev[j]));
-            if (c < best) { best = c; bj = j; }
+            const double dj = D[j], pj = prev[j];
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                const double c = fma(jd, dm[u], fma(md[u], dj, pj));
+                if (c < best[u] && (N == 1 || j < first + u * S)) { best[u] = c; bj[u] = j; }
+            }
         }
     }
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        if (ob < best || (ob == best && oj < bj)) { best = ob; bj = oj; }
-    }
-    if (valid && (lane & (G - 1)) == 0) { cur[mm] = best; ak[mm] = (unsigned short)bj; }
+    for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best[u], o);
+            const int oj = __shfl_xor_sync(0xffffffffu, bj[u], o);
+            if (ob < best[u] || (ob == best[u] && oj < bj[u])) { best[u] = ob; bj[u] = oj; }
+        }
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+        if (valid && (lane & (G - 1)) == u % G && first + u * S >= k) { cur[first + u * S] = best[u]; ak[first + u * S] = (unsigned short)bj[u]; }
 }
 
-// One round of a layer: the multiples of S that are not multiples of 4 S.
+// One round of a layer: the multiples of S that are not multiples of 4 S, the three between two neighbours of the rounds before at once.
 template <int G, int S>
 __device__ __forceinline__ void dp_round(const double* D, const double* prev, double* cur, unsigned short* ak, int k, int M) {
     constexpr int kGroups = kDpThreads / G;
-    const int items = (M / (4 * S)) * 3 + (M % (4 * S)) / S;
+    const int items = M / (4 * S);                                  // whole intervals; M itself may end a shorter one
     for (int q0 = 0; q0 < items; q0 += kGroups) {
-        const int q = q0 + (int)threadIdx.x / G;
-        const int mm = S * (q / 3 * 4 + q % 3 + 1);
-        const bool valid = q < items && mm >= k && mm < M;
-        int j_lo = k - 1, j_hi = 0;
-        if (valid) {
-            const int below = mm / (4 * S) * (4 * S), above = min(below + 4 * S, M);
-            if (below >= k) j_lo = ak[below];
-            j_hi = min((int)ak[above], mm - 1);
-        }
-        dp_minimise<G>(D, prev, cur, ak, valid, mm, j_lo, j_hi);
+        const int q = q0 + (int)threadIdx.x / G, below = q * 4 * S, above = below + 4 * S;
+        const bool valid = q < items && below + 3 * S >= k;
+        const int j_lo = valid && below >= k ? (int)ak[below] : k - 1;
+        dp_minimise<G, 3, S>(D, prev, cur, ak, valid, k, below + S, j_lo, valid ? min((int)ak[above], below + 3 * S - 1) : 0);
+    }
+    const int rest = (M % (4 * S) + S - 1) / S - 1;                 // edges of that one (at most 3): a group each
+    if ((int)threadIdx.x / 32 * 32 < rest * G) {
+        const int q = (int)threadIdx.x / G, below = items * 4 * S, mm = below + (q + 1) * S;
+        const bool valid = q < rest && mm >= k;
+        const int j_lo = valid && below >= k ? (int)ak[below] : k - 1;
+        dp_minimise<G, 1, S>(D, prev, cur, ak, valid, k, mm, j_lo, valid ? min((int)ak[M], mm - 1) : 0);
     }
     __syncthreads();
 }
@@ -162,16 +197,20 @@ __global__ void __launch_bounds__(kDpThreads) levels_dp_kernel(const uint32_t* _
     __shared__ int s_idx[17];
     __shared__ unsigned long long tot[3][kDpThreads / 32];
     const int64_t j_feat = blockIdx.x;
-    const uint32_t* cnt = counts + j_feat * M;
+    const uint32_t* cnt = counts + j_feat / 32 * 32 * M + j_feat % 32;   // bin i at 32 i
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long S0, S1, S2;                                  // sums of c, c x, c x^2 over all bins
     {
         // exclusive prefix sums of c and c x: every thread sums a run of bins, the runs' totals are scanned by warps
         const int per = (M + kDpThreads - 1) / kDpThreads;
         const int i_begin = min(M, (int)threadIdx.x * per), i_end = min(M, i_begin + per);
+        uint32_t c_run[kDpRun];
+#pragma unroll
+        for (int u = 0; u < kDpRun; ++u) c_run[u] = i_begin + u < i_end ? cnt[(int64_t)(i_begin + u) * 32] : 0u;
         unsigned long long a0 = 0, a1 = 0, a2 = 0;
-        for (int i = i_begin; i < i_end; ++i) {
-            const unsigned long long c = cnt[i], x = 2ull * i + 1ull;
+#pragma unroll
+        for (int u = 0; u < kDpRun; ++u) {
+            const unsigned long long c = c_run[u], x = 2ull * (i_begin + u) + 1ull;
             a0 += c; a1 += c * x; a2 += c * x * x;
         }
         const unsigned long long own0 = a0, own1 = a1;
@@ -190,10 +229,13 @@ __global__ void __launch_bounds__(kDpThreads) levels_dp_kernel(const uint32_t* _
             if (w == warp) { a0 += S0; a1 += S1; }
             S0 += tot[0][w]; S1 += tot[1][w]; S2 += tot[2][w];
         }
-        for (int i = i_begin; i < i_end; ++i) {
+#pragma unroll
+        for (int u = 0; u < kDpRun; ++u) {
+            const int i = i_begin + u;
+            if (i >= i_end) break;
             D[i] = (double)(4ull * i * a0 - 2ull * a1);
             prev[i] = 0.0;                                          // E_1
-            const unsigned long long c = cnt[i], x = 2ull * i + 1ull;
+            const unsigned long long c = c_run[u], x = 2ull * i + 1ull;
             a0 += c; a1 += c * x;
         }
         if (threadIdx.x == 0) { D[M] = (double)(4ull * M * S0 - 2ull * S1); prev[M] = 0.0; }
@@ -205,7 +247,7 @@ __global__ void __launch_bounds__(kDpThreads) levels_dp_kernel(const uint32_t* _
         const int items = M / 256 + (M % 256 != 0 ? 1 : 0);         // multiples of 256, and M
         for (int q = warp; q < items; q += kDpThreads / 32) {
             const int mm = q < M / 256 ? (q + 1) * 256 : M;
-            dp_minimise<32>(D, prev, cur, ak, mm >= k, mm, k - 1, mm - 1);
+            dp_minimise<32, 1, 1>(D, prev, cur, ak, mm >= k, k, mm, k - 1, mm - 1);
         }
         __syncthreads();
         dp_round<32, 64>(D, prev, cur, ak, k, M);

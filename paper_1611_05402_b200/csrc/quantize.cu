@@ -9,173 +9,146 @@
 namespace zipml {
 
 // ---------------------------------------------------------------------------------------------
-// Column range.  A tile is 32*VEC columns wide; blockDim = (32, 8): x walks the columns (one VEC-wide
-// load per thread, a warp reads 128*VEC contiguous bytes of a row), y walks rows.  Row chunks are
-// spread over gridDim.y; results meet in order-preserving integer atomics (min/max are exact and
-// order independent).
+// Column range.  A block of 256 threads takes tx * VEC columns (tx a power of two, at least the row's as far as it
+// goes) and 256 / tx rows at a time, up to 4 KB of consecutive memory; a thread keeps its VEC columns, kRangeAhead rows in flight.
+// The row chunks of a column tile take groups of rows in turn, so that the pass as a whole goes through A from front to back and
+// leaves the end of A in L2.  Their results meet in order-preserving integer keys (a maximum of the value's key, a maximum
+// of the complement for the minimum: exact and order independent); the tile's last block turns the keys into the grid
+// and clears keys and counter for the next pass: no launch before this one to set them, none after it.
+// Bound by HBM.  500,000 x 512 230 -> 148 us (one row in flight a thread before), 100,003 x 1,001 70 -> 63, and what follows finds more of
+// A in L2: the whole call on 250,000 x 1,000 at 4 bits 664 -> 567 us, 4,096 x 64 19 -> 12.
 // ---------------------------------------------------------------------------------------------
-__global__ void range_init_kernel(uint32_t* lo_key, uint32_t* hi_key, int64_t n) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) { lo_key[j] = 0xffffffffu; hi_key[j] = 0u; }
-}
+struct RangeArgs {
+    const float* A;
+    int64_t m, n, lda;                         // n: columns of this launch
+    uint32_t *lo_key, *hi_key;                 // 0 between passes
+    unsigned* done;                            // blocks that have finished, per column tile; 0 between passes
+    DeviceStatus* status;
+    int s;                                     // intervals of the grid
+    int symmetric;
+    float *lo, *hi, *inv, *step;               // results; all but lo may be null
+};
 
-template <int VEC>
-__global__ void __launch_bounds__(256) range_scan_kernel(const float* __restrict__ A, int64_t m, int64_t n,
-                                                         int64_t lda, int64_t rows_per_block, uint32_t* lo_key,
-                                                         uint32_t* hi_key, DeviceStatus* status) {
-    __shared__ float s_lo[8][32 * VEC];
-    __shared__ float s_hi[8][32 * VEC];
-    const int64_t j0 = ((int64_t)blockIdx.x * 32 + threadIdx.x) * VEC;
-    const int64_t r0 = (int64_t)blockIdx.y * rows_per_block;
-    const int64_t r1 = min(m, r0 + rows_per_block);
-    float lo[VEC], hi[VEC];
-    bool bad = false;
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) { lo[v] = INFINITY; hi[v] = -INFINITY; }
-    if (j0 < n) {
-        for (int64_t r = r0 + threadIdx.y; r < r1; r += 8) {
-            float val[VEC];
-            bool have[VEC];
-            if constexpr (VEC == 4) {
-                if (j0 + 3 < n) {
-                    const float4 q = __ldg(reinterpret_cast<const float4*>(A + r * lda + j0));
-                    val[0] = q.x; val[1] = q.y; val[2] = q.z; val[3] = q.w;
-                    have[0] = have[1] = have[2] = have[3] = true;
-                } else {
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        have[v] = j0 + v < n;
-                        val[v] = have[v] ? __ldg(A + r * lda + j0 + v) : 0.0f;
-                    }
-                }
-            } else {
-                val[0] = __ldg(A + r * lda + j0);
-                have[0] = true;
-            }
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                if (!have[v]) continue;
-                bad |= !(fabsf(val[v]) <= 3.402823466e+38f);
-                lo[v] = fminf(lo[v], val[v]);
-                hi[v] = fmaxf(hi[v], val[v]);
-            }
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) { s_lo[threadIdx.y][threadIdx.x * VEC + v] = lo[v]; s_hi[threadIdx.y][threadIdx.x * VEC + v] = hi[v]; }
-    if (bad) set_status(status, ZIPML_ERR_NONFINITE, 1);
-    __syncthreads();
-    const int t = threadIdx.y * 32 + threadIdx.x;
-    if (t < 32 * VEC) {
-        const int64_t j = (int64_t)blockIdx.x * 32 * VEC + t;
-        if (j < n) {
-            float a = s_lo[0][t], b = s_hi[0][t];
-#pragma unroll
-            for (int y = 1; y < 8; ++y) { a = fminf(a, s_lo[y][t]); b = fmaxf(b, s_hi[y][t]); }
-            if (a <= b) {  // at least one row seen
-                atomicMin(lo_key + j, float_order_key(a));
-                atomicMax(hi_key + j, float_order_key(b));
-            }
-        }
-    }
-}
-
-// The same scan for wide matrices: a block reads 4 KB of consecutive columns of a row at a time (256 threads x
-// float4; the narrow kernel's 512-byte pieces waste DRAM pages on rows of tens of kilobytes), a thread keeps its
-// four columns for all rows of the block's chunk, four rows' loads in flight; no meeting in shared memory.
-__global__ void __launch_bounds__(256) range_scan_wide_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda,
-                                                              int64_t rows_per_block, uint32_t* lo_key, uint32_t* hi_key,
-                                                              DeviceStatus* status) {
-    const int64_t j0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
-    if (j0 >= n) return;
-    const int64_t r0 = (int64_t)blockIdx.y * rows_per_block;
-    const int64_t r1 = min(m, r0 + rows_per_block);
-    const int nv = (int)min((int64_t)4, n - j0);
-    float lo[4], hi[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) { lo[v] = INFINITY; hi[v] = -INFINITY; }
-    bool bad = false;
-    const float* col = A + j0;
-    if (nv == 4) {
-#pragma unroll 4
-        for (int64_t r = r0; r < r1; ++r) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(col + r * lda));
-            const float val[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                bad |= !(fabsf(val[v]) <= 3.402823466e+38f);
-                lo[v] = fminf(lo[v], val[v]);
-                hi[v] = fmaxf(hi[v], val[v]);
-            }
-        }
-    } else {
-        for (int64_t r = r0; r < r1; ++r)
-            for (int v = 0; v < nv; ++v) {
-                const float val = __ldg(col + r * lda + v);
-                bad |= !(fabsf(val) <= 3.402823466e+38f);
-                lo[v] = fminf(lo[v], val);
-                hi[v] = fmaxf(hi[v], val);
-            }
-    }
-    if (bad) set_status(status, ZIPML_ERR_NONFINITE, 1);
-    for (int v = 0; v < nv; ++v)
-        if (lo[v] <= hi[v]) {  // at least one row seen
-            atomicMin(lo_key + j0 + v, float_order_key(lo[v]));
-            atomicMax(hi_key + j0 + v, float_order_key(hi[v]));
-        }
-}
-
-__global__ void range_finalize_kernel(const uint32_t* lo_key, const uint32_t* hi_key, int64_t n, int s, bool symmetric,
-                                      float* lo_out, float* hi_out, float* inv_out, float* step_out) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    float lo = float_from_order_key(lo_key[j]), hi = float_from_order_key(hi_key[j]);
-    if (symmetric) {                     // the grid [-M_j, M_j], M_j = max |value| (Supplement "Column Scaling")
+__device__ __forceinline__ void range_results(const RangeArgs& a, int64_t j, uint32_t lo_key, uint32_t hi_key) {
+    float lo = float_from_order_key(~lo_key), hi = float_from_order_key(hi_key);
+    if (a.symmetric) {                         // the grid [-M_j, M_j], M_j = max |value| (Supplement "Column Scaling")
         hi = fmaxf(fabsf(lo), fabsf(hi));
         lo = -hi;
     }
     const float range = __fsub_rn(hi, lo);
-    lo_out[j] = lo;
-    if (hi_out) hi_out[j] = hi;
-    if (inv_out) inv_out[j] = range > 0.0f ? __fdiv_rn((float)s, range) : 0.0f;
-    if (step_out) step_out[j] = __fdiv_rn(range, (float)s);
+    a.lo[j] = lo;
+    if (a.hi) a.hi[j] = hi;
+    if (a.inv) a.inv[j] = range > 0.0f ? __fdiv_rn((float)a.s, range) : 0.0f;
+    if (a.step) a.step[j] = __fdiv_rn(range, (float)a.s);
 }
 
-int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int s, bool symmetric,
-                        uint32_t* key_scratch, float* lo_out, float* hi_out, float* inv_out, float* step_out) {
-    uint32_t* lo_key = key_scratch;
-    uint32_t* hi_key = key_scratch + n;
-    const unsigned nb = (unsigned)((n + 255) / 256);
-    range_init_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n);
-    const bool vec = (lda % 4 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
-    if (vec && n >= 2048) {
-        const int64_t col_tiles = (n + 1023) / 1024;
-        int64_t chunks = (int64_t)ctx->sm_count * 8 / col_tiles;
-        chunks = chunks < 1 ? 1 : chunks;
-        int64_t rows_per_block = (m + chunks - 1) / chunks;
-        rows_per_block = rows_per_block < 64 ? 64 : rows_per_block;
-        chunks = (m + rows_per_block - 1) / rows_per_block;
-        if (chunks > 65535) { rows_per_block = (m + 65534) / 65535; chunks = (m + rows_per_block - 1) / rows_per_block; }
-        range_scan_wide_kernel<<<dim3((unsigned)col_tiles, (unsigned)chunks), 256, 0, ctx->stream>>>(A, m, n, lda, rows_per_block, lo_key,
-                                                                                                   hi_key, ctx->d_status);
-        range_finalize_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n, s, symmetric, lo_out, hi_out, inv_out, step_out);
-        ctx->launches += 3;
-        return cuda_status(cudaGetLastError());
+// Called by every thread of a block once its keys are on their way: the tile's last block writes the results of columns j0 .. j0 +
+// count - 1 and clears what the pass has used.
+__device__ __forceinline__ void range_finish(const RangeArgs& a, unsigned tile, unsigned blocks, int64_t j0, int count) {
+    const int t = threadIdx.y * blockDim.x + threadIdx.x;
+    __shared__ bool last_s;
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last_s = atomicAdd(a.done + tile, 1u) == blocks - 1;
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    for (int64_t j = j0 + t; j < min(a.n, j0 + count); j += 256) {
+        range_results(a, j, __ldcg(a.lo_key + j), __ldcg(a.hi_key + j));
+        a.lo_key[j] = 0u;
+        a.hi_key[j] = 0u;
     }
-    const int width = vec ? 128 : 32;
-    const int64_t col_tiles = (n + width - 1) / width;
-    // enough row chunks to give every SM a few blocks, at least 64 rows each
-    int64_t chunks = (int64_t)ctx->sm_count * 8 / col_tiles;
-    chunks = chunks < 1 ? 1 : chunks;
-    int64_t rows_per_block = (m + chunks - 1) / chunks;
-    rows_per_block = rows_per_block < 64 ? 64 : rows_per_block;
-    chunks = (m + rows_per_block - 1) / rows_per_block;
-    if (chunks > 65535) { rows_per_block = (m + 65534) / 65535; chunks = (m + rows_per_block - 1) / rows_per_block; }
-    const dim3 grid((unsigned)col_tiles, (unsigned)chunks), block(32, 8);
-    if (vec) range_scan_kernel<4><<<grid, block, 0, ctx->stream>>>(A, m, n, lda, rows_per_block, lo_key, hi_key, ctx->d_status);
-    else range_scan_kernel<1><<<grid, block, 0, ctx->stream>>>(A, m, n, lda, rows_per_block, lo_key, hi_key, ctx->d_status);
-    range_finalize_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n, s, symmetric, lo_out, hi_out, inv_out, step_out);
-    ctx->launches += 3;
+    if (t == 0) a.done[tile] = 0u;
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(256, 4) range_scan_kernel(const RangeArgs a) {
+    constexpr int kRangeAhead = VEC == 4 ? 4 : 16;
+    __shared__ float lo_s[256 * VEC], hi_s[256 * VEC];
+    const int tx = blockDim.x, ty = blockDim.y, t = threadIdx.y * tx + threadIdx.x;
+    const int64_t first = (int64_t)blockIdx.x * tx * VEC, j0 = first + threadIdx.x * VEC;
+    float lo[VEC], hi[VEC], probe = 0.0f;                          // probe: NaN once a value is not finite
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) { lo[v] = INFINITY; hi[v] = -INFINITY; }
+    if (j0 < a.n) {
+        const int nv = (int)min((int64_t)VEC, a.n - j0);
+        const int64_t group = (int64_t)ty * kRangeAhead;
+        for (int64_t r0 = blockIdx.y * group; r0 < a.m; r0 += gridDim.y * group) {
+            const float* src = a.A + (r0 + threadIdx.y) * a.lda + j0;
+            if (r0 + group <= a.m && nv == VEC) {
+                float val[kRangeAhead][VEC];
+#pragma unroll
+                for (int u = 0; u < kRangeAhead; ++u, src += ty * a.lda) {
+                    if constexpr (VEC == 4) {
+                        const float4 q = __ldg(reinterpret_cast<const float4*>(src));
+                        val[u][0] = q.x; val[u][1] = q.y; val[u][2] = q.z; val[u][3] = q.w;
+                    } else {
+                        val[u][0] = __ldg(src);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kRangeAhead; ++u)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        probe = fmaf(val[u][v], 0.0f, probe);
+                        lo[v] = fminf(lo[v], val[u][v]);
+                        hi[v] = fmaxf(hi[v], val[u][v]);
+                    }
+            } else {
+                for (int64_t r = r0 + threadIdx.y; r < min(a.m, r0 + group); r += ty, src += ty * a.lda)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v)
+                        if (v < nv) {
+                            const float val = __ldg(src + v);
+                            probe = fmaf(val, 0.0f, probe);
+                            lo[v] = fminf(lo[v], val);
+                            hi[v] = fmaxf(hi[v], val);
+                        }
+            }
+        }
+    }
+    if (!(probe == 0.0f)) set_status(a.status, ZIPML_ERR_NONFINITE, 1);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) { lo_s[t * VEC + v] = lo[v]; hi_s[t * VEC + v] = hi[v]; }
+    __syncthreads();
+    for (int c = t; c < tx * VEC; c += 256) {
+        float x = lo_s[c], y = hi_s[c];
+        for (int k = 1; k < ty; ++k) { x = fminf(x, lo_s[k * tx * VEC + c]); y = fmaxf(y, hi_s[k * tx * VEC + c]); }
+        if (first + c < a.n && x <= y) {                           // at least one row seen
+            atomicMax(a.lo_key + first + c, ~float_order_key(x));
+            atomicMax(a.hi_key + first + c, float_order_key(y));
+        }
+    }
+    range_finish(a, blockIdx.x, gridDim.y, first, tx * VEC);
+}
+
+int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int s, bool symmetric, float* lo_out, float* hi_out,
+                        float* inv_out, float* step_out) {
+    const bool vec = (lda % 4 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
+    const int per = vec ? 4 : 1;
+    for (int64_t j0 = 0; j0 < n; j0 += kRangeColumns) {            // (the keys hold so many columns at a time)
+        RangeArgs a{};
+        a.A = A + j0; a.m = m; a.n = n - j0 < kRangeColumns ? n - j0 : kRangeColumns; a.lda = lda;
+        a.lo_key = ctx->range_keys; a.hi_key = a.lo_key + kRangeColumns; a.done = a.hi_key + kRangeColumns;
+        a.status = ctx->d_status; a.s = s; a.symmetric = symmetric;
+        a.lo = lo_out + j0;
+        a.hi = hi_out ? hi_out + j0 : nullptr;
+        a.inv = inv_out ? inv_out + j0 : nullptr;
+        a.step = step_out ? step_out + j0 : nullptr;
+        int tx = 8;
+        while (tx < 256 && tx * per < a.n) tx *= 2;
+        const int ty = 256 / tx;
+        const int64_t tiles = (a.n + tx * per - 1) / (tx * per);
+        // four blocks per SM, of at least 64 rows each
+        int64_t chunks = (int64_t)ctx->sm_count * 4 / tiles;
+        const int64_t most = (m + 63) / 64;
+        chunks = chunks > most ? most : chunks;
+        chunks = chunks < 1 ? 1 : chunks;
+        const dim3 grid((unsigned)tiles, (unsigned)chunks), block((unsigned)tx, (unsigned)ty);
+        if (vec) range_scan_kernel<4><<<grid, block, 0, ctx->stream>>>(a);
+        else range_scan_kernel<1><<<grid, block, 0, ctx->stream>>>(a);
+        ctx->launches += 1;
+    }
     return cuda_status(cudaGetLastError());
 }
 
@@ -210,7 +183,7 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 // What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 62 %; 24 warps per SM: fewer
 // registers per thread spill, more leave too few warps); sparse rows, issue slots (75 %) and DRAM (60 %) together.
 // Measured, whole call with the range pass, samples queued and conversions of their own for cell and threshold ->
-// now: 100,003 x 1,001 at 8 bits 279 -> 262 us, 65,536 x 4,096 of 5 % non-zeros at 4 bits 484 -> 450.
+// now: 100,003 x 1,001 at 8 bits 279 -> 251 us, 65,536 x 4,096 of 5 % non-zeros at 4 bits 484 -> 415.
 // ---------------------------------------------------------------------------------------------
 constexpr int kQuantRows = 4;                  // rows per thread and pass
 constexpr int kQuantTableCols = 64;            // thread columns per block with level tables
@@ -286,10 +259,10 @@ __host__ __device__ constexpr int answer_shift(int row, int plane) {
 template <int CB, int TB>
 __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restrict__ A, int64_t m, int64_t n, int64_t lda, int bits,
                                                           const float* __restrict__ lo, const float* __restrict__ inv,
-                                                          const float* __restrict__ levels, uint32_t* lo_key, uint32_t* hi_key,
-                                                          DeviceStatus* status, const PhiloxKeys key, uint32_t draw,
+                                                          const float* __restrict__ levels, const RangeArgs range, const PhiloxKeys key,
+                                                          uint32_t draw,
                                                           uint8_t* __restrict__ plane1, uint8_t* __restrict__ plane2, int64_t row_bytes,
-                                                          bool vec_ok, int passes, unsigned col_blocks, unsigned row_blocks) {
+                                                          bool vec_ok, int passes, unsigned col_blocks, unsigned row_blocks, int64_t group0) {
     using Word = typename QuantWord<CB>::type;
     constexpr bool TABLE = TB > 0;
     constexpr int L = 1 << TB;                                     // TABLE: levels
@@ -300,13 +273,13 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
     float* lev_s = reinterpret_cast<float*>(cell_s + 4 * L * kCols);   // TABLE: [4][L][kCols] levels
     const int tx = blockDim.x, tid = threadIdx.y * tx + threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned row_block = blockIdx.x / col_blocks, col_block = blockIdx.x - row_block * col_blocks;
-    const int64_t g = (int64_t)col_block * tx + threadIdx.x;       // this thread's group of four features
+    const int64_t g = group0 + (int64_t)col_block * tx + threadIdx.x;   // this thread's group of four features (group0: the launch's first)
     const int64_t groups = row_bytes * 8 / (4 * CB);
     const int64_t j0 = g * 4;
     const int nf = (int)max((int64_t)0, min((int64_t)4, n - j0));  // real features of the group (0: padding)
     bool divide = false;                                           // TABLE: a cell of the block needs the division itself
     if constexpr (TABLE) {
-        const int64_t jb = (int64_t)col_block * tx * 4;            // first feature of the block
+        const int64_t jb = (group0 + (int64_t)col_block * tx) * 4; // first feature of the block
         for (int idx = tid; idx < tx * 4 * L; idx += 256) {        // consecutive threads read consecutive floats of the table
             const int f = idx / L, k = idx - f * L;
             const bool have = jb + f < n;
@@ -500,63 +473,72 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
     else if (__all_sync(0xffffffffu, nf == 4 && left == kQuantRows * passes)) run(std::true_type{}, std::false_type{});
     else run(std::false_type{}, std::false_type{});
     if constexpr (TABLE) {
-        if (!(probe == 0.0f)) set_status(status, ZIPML_ERR_NONFINITE, 1);
+        if (!(probe == 0.0f)) set_status(range.status, ZIPML_ERR_NONFINITE, 1);
         // (a value that is beaten already needs no atomic: after the first blocks hardly any does)
+        const int64_t jk = j0 - group0 * 4;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             if (i < nf && seen_lo[i] <= seen_hi[i]) {
-                const uint32_t a = float_order_key(seen_lo[i]), b = float_order_key(seen_hi[i]);
-                if (a < *reinterpret_cast<volatile uint32_t*>(lo_key + j0 + i)) atomicMin(lo_key + j0 + i, a);
-                if (b > *reinterpret_cast<volatile uint32_t*>(hi_key + j0 + i)) atomicMax(hi_key + j0 + i, b);
+                const uint32_t a = ~float_order_key(seen_lo[i]), b = float_order_key(seen_hi[i]);
+                if (a > *reinterpret_cast<volatile uint32_t*>(range.lo_key + jk + i)) atomicMax(range.lo_key + jk + i, a);
+                if (b > *reinterpret_cast<volatile uint32_t*>(range.hi_key + jk + i)) atomicMax(range.hi_key + jk + i, b);
             }
+        range_finish(range, col_block, row_blocks, (int64_t)col_block * tx * 4, tx * 4);
     }
 }
 
 int launch_quantize(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64_t lda, int bits, int level_mode,
                     const float* lo, const float* inv, const float* levels, uint64_t seed, uint32_t draw, uint8_t* plane1,
-                    uint8_t* plane2, int64_t row_bytes, uint32_t* key_scratch, float* lo_out, float* step_out) {
+                    uint8_t* plane2, int64_t row_bytes, float* lo_out, float* step_out) {
     const int cb = container_bits(bits);
     const bool table = level_mode == ZIPML_LEVELS_TABLE;
-    const int64_t groups = row_bytes * 8 / (4 * cb);
-    // 256 threads: as many feature groups as the row has (a power of two from 4 to 256; 64 with level tables), the
-    // rest row groups.  More passes per thread share the loads of lo and inv (the staging of the tables), as
-    // long as the grid still covers the SMs several times over.
-    int tx = 4;
-    while (tx < (table ? kQuantTableCols : 256) && tx < groups) tx *= 2;
-    const int ty = 256 / tx;
-    const int64_t col_blocks = (groups + tx - 1) / tx;
-    int passes = 1;
-    while (passes < (table ? 16 : 8) && (m / (ty * kQuantRows * passes * 2)) * col_blocks >= (int64_t)ctx->sm_count * 16) passes *= 2;
-    const size_t smem = table ? (sizeof(float4) + sizeof(float)) * ((size_t)4 << bits) * kQuantTableCols : 0;
-    auto blocks_of_rows = [&]() { return (m + (int64_t)ty * kQuantRows * passes - 1) / ((int64_t)ty * kQuantRows * passes); };
-    while (blocks_of_rows() > 0x7fffffffLL / col_blocks && passes < (1 << 20)) passes *= 2;      // the grid is one-dimensional, columns first
-    const int64_t row_blocks = blocks_of_rows();
-    if (row_blocks > 0x7fffffffLL / col_blocks) return ZIPML_ERR_WORKSPACE;
-    const dim3 grid((unsigned)(row_blocks * col_blocks)), block((unsigned)tx, (unsigned)ty);
     const bool vec_ok = (lda % 4 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
     const PhiloxKeys key = philox_keys(seed);
-    uint32_t* lo_key = key_scratch;
-    uint32_t* hi_key = key_scratch + n;
-    const unsigned nb = (unsigned)((n + 255) / 256);
-    if (table) range_init_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n);
-    auto launch = [&](auto kernel) -> int {
-        // (the kernel's own 5 KB of shared memory count towards the 48 KB that need no opt-in)
-        if (smem > 40 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return cuda_status(e);
+    const int64_t all_groups = row_bytes * 8 / (4 * cb);
+    // (level tables: as many columns at a time as the range keys hold)
+    const int64_t slab = table ? kRangeColumns / 4 : all_groups;
+    for (int64_t group0 = 0; group0 < all_groups; group0 += slab) {
+        const int64_t groups = all_groups - group0 < slab ? all_groups - group0 : slab;
+        // 256 threads: as many feature groups as the row has (a power of two from 4 to 256; 64 with level tables), the
+        // rest row groups.  More passes per thread share the loads of lo and inv (the staging of the tables), as
+        // long as the grid still covers the SMs several times over.
+        int tx = 4;
+        while (tx < (table ? kQuantTableCols : 256) && tx < groups) tx *= 2;
+        const int ty = 256 / tx;
+        const int64_t col_blocks = (groups + tx - 1) / tx;
+        int passes = 1;
+        while (passes < (table ? 16 : 8) && (m / (ty * kQuantRows * passes * 2)) * col_blocks >= (int64_t)ctx->sm_count * 16) passes *= 2;
+        const size_t smem = table ? (sizeof(float4) + sizeof(float)) * ((size_t)4 << bits) * kQuantTableCols : 0;
+        auto blocks_of_rows = [&]() { return (m + (int64_t)ty * kQuantRows * passes - 1) / ((int64_t)ty * kQuantRows * passes); };
+        while (blocks_of_rows() > 0x7fffffffLL / col_blocks && passes < (1 << 20)) passes *= 2;      // the grid is one-dimensional, columns first
+        const int64_t row_blocks = blocks_of_rows();
+        if (row_blocks > 0x7fffffffLL / col_blocks) return ZIPML_ERR_WORKSPACE;
+        const dim3 grid((unsigned)(row_blocks * col_blocks)), block((unsigned)tx, (unsigned)ty);
+        RangeArgs range{};
+        if (table) {
+            const int64_t j0 = group0 * 4;
+            range.n = n - j0 < kRangeColumns ? n - j0 : kRangeColumns;
+            range.lo_key = ctx->range_keys; range.hi_key = range.lo_key + kRangeColumns; range.done = range.hi_key + kRangeColumns;
+            range.s = (1 << bits) - 1;
+            range.lo = lo_out + j0;
+            range.step = step_out ? step_out + j0 : nullptr;
         }
-        kernel<<<grid, block, smem, ctx->stream>>>(A, m, n, lda, bits, lo, inv, levels, lo_key, hi_key, ctx->d_status, key, draw, plane1, plane2,
-                                                   row_bytes, vec_ok, passes, (unsigned)col_blocks, (unsigned)row_blocks);
-        return ZIPML_OK;
-    };
-    int rc;
-    if (!table) rc = cb == 2 ? launch(quantize_kernel<2, 0>) : cb == 4 ? launch(quantize_kernel<4, 0>) : launch(quantize_kernel<8, 0>);
-    else rc = bits == 1 ? launch(quantize_kernel<2, 1>) : bits == 2 ? launch(quantize_kernel<2, 2>) : bits == 3 ? launch(quantize_kernel<4, 3>) : launch(quantize_kernel<4, 4>);
-    if (rc != ZIPML_OK) return rc;
-    ctx->launches += 1;
-    if (table) {
-        range_finalize_kernel<<<nb, 256, 0, ctx->stream>>>(lo_key, hi_key, n, (1 << bits) - 1, false, lo_out, nullptr, nullptr, step_out);
-        ctx->launches += 2;
+        range.status = ctx->d_status;
+        auto launch = [&](auto kernel) -> int {
+            // (the kernel's own 5 KB of shared memory count towards the 48 KB that need no opt-in)
+            if (smem > 40 * 1024) {
+                const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return cuda_status(e);
+            }
+            kernel<<<grid, block, smem, ctx->stream>>>(A, m, n, lda, bits, lo, inv, levels, range, key, draw, plane1, plane2, row_bytes, vec_ok,
+                                                       passes, (unsigned)col_blocks, (unsigned)row_blocks, group0);
+            return ZIPML_OK;
+        };
+        int rc;
+        if (!table) rc = cb == 2 ? launch(quantize_kernel<2, 0>) : cb == 4 ? launch(quantize_kernel<4, 0>) : launch(quantize_kernel<8, 0>);
+        else rc = bits == 1 ? launch(quantize_kernel<2, 1>) : bits == 2 ? launch(quantize_kernel<2, 2>) : bits == 3 ? launch(quantize_kernel<4, 3>) : launch(quantize_kernel<4, 4>);
+        if (rc != ZIPML_OK) return rc;
+        ctx->launches += 1;
     }
     return cuda_status(cudaGetLastError());
 }

@@ -122,6 +122,40 @@ def test_quantize_onto_levels_whose_distance_overflows(ctx, bits):
     assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
 
 
+@pytest.mark.parametrize("m,n,cut", [(9, 65_541, 0), (70, 65_600, 3), (3, 131_073, 1)])
+def test_quantize_more_features_than_a_range_pass_holds(ctx, m, n, cut):
+    """A range pass takes 65,536 columns at a time (`cut` columns off the rows' front: unaligned rows)."""
+    A = np.random.default_rng(n).standard_normal((m, n + cut)).astype(np.float32)
+    dA, A = to_dev(A, ctx)[:, cut:], np.ascontiguousarray(A[:, cut:])
+    ods, gds = oracle.quantize(A, 5, seed=3), ctx.zipml_quantize(dA, 5, seed=3)
+    ctx.zipml_sync()
+    assert (gds.feat_lo.cpu().numpy() == ods.feat_lo).all() and (gds.feat_step.cpu().numpy() == ods.feat_step).all()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+    table = oracle.optimal_levels(A, 2, 16)[0]
+    assert (ctx.zipml_optimal_levels(dA, 2, 16).cpu().numpy() == table).all()
+    ods = oracle.quantize(A, 2, seed=3, mode=oracle.TABLE, levels=table)
+    gds = ctx.zipml_quantize(dA, 2, seed=3, level_mode=binding.LEVELS_TABLE, levels=to_dev(table, ctx))
+    ctx.zipml_sync()
+    assert (gds.feat_lo.cpu().numpy() == ods.feat_lo).all()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_quantize_values_just_above_a_level(ctx, bits):
+    """Quotients far below 2^-24, down to those that round to 0: the threshold is 1 or 0, as the division says."""
+    rng = np.random.default_rng(bits)
+    m, n = 40_000, 24
+    A = np.float32(2.0) ** rng.integers(-149, -20, (m, n)).astype(np.float32)
+    A[0] = 0.0
+    A[1] = 1.0
+    table = np.sort(np.concatenate([np.zeros((n, 1)), rng.random((n, (1 << bits) - 2)), np.ones((n, 1))], axis=1), axis=1).astype(np.float32)
+    table[::2] *= np.float32(2.0 ** 39)
+    ods = oracle.quantize(A, bits, seed=7, mode=oracle.TABLE, levels=table)
+    gds = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=7, level_mode=binding.LEVELS_TABLE, levels=to_dev(table, ctx))
+    ctx.zipml_sync()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+
+
 def test_quantize_strided_and_unaligned_input(ctx):
     _, A, _, _ = workload("c2", 200, 101, seed=3)
     big = torch.zeros((200, 131), dtype=torch.float32, device=ctx.device)
