@@ -978,6 +978,8 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     int R = p->column_chunk_rows > 0 ? p->column_chunk_rows : 128;
     if (R > kColMaxChunkRows) R = kColMaxChunkRows;
     if (R > (B + 31) / 32 * 32) R = (int)((B + 31) / 32 * 32);
+    R = (R + 31) / 32 * 32;
+    if (R == 96 && B > R) R = 64;             // (several chunks a step: of a length whose tasks the A warps share evenly)
     const int nch_max = (int)((B + R - 1) / R);
     const int bpad = nch_max * R;
     // One dot word per row and plane for all CTAs (tuning: grid_feature_parts = words, each shared by a group of
@@ -1000,8 +1002,16 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     if (slots_b < 2) slots_b = 2;
     if (slots_b > slots - 2) slots_b = slots - 2;
     if (slots_b > kColMaxSlots) slots_b = kColMaxSlots;
+    const int stride = kColAWarps * 32 / R;
+    if (nch_max > 1 && slots_b > slots - stride) slots_b = slots - stride;
     int slots_a = slots - slots_b;
     if (slots_a > kColMaxSlots) slots_a = kColMaxSlots;
+    // An A warp sees every `stride`-th chunk.  The ring holds a multiple of that, so that the warp has itself waited for the copy that
+    // was in a slot before the one it waits for: a barrier tells two neighbouring phases apart, not the third (with three slots
+    // and chunks that land out of turn, warps read and freed slots before their copies were there).  Where a step has a single chunk, its
+    // dots follow from all before.
+    if (nch_max > 1) slots_a = slots_a / stride * stride;
+    if (slots_a < 1 || slots_b < 1) return ZIPML_ERR_WORKSPACE;
     const size_t smem = fixed + (size_t)slots * slot_bytes;
     const void* kernel = column_kernel_ptr(cb);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -748,6 +748,21 @@ def test_column_engine(ctx, case):
     assert e.value.code == binding.ERR_UNSUPPORTED
 
 
+@pytest.mark.parametrize("chunk,ring_b", [(128, 3), (96, 0), (64, 11), (64, 2), (32, 24)])
+def test_column_engine_rings_of_any_size(ctx, chunk, ring_b):
+    """Chunk lengths and ring sizes whose slots the warps see in every pattern; several chunks a step."""
+    m, n, batch = 2100, 9001, 700
+    _, A, b, _ = workload("c2", m, n, seed=5)
+    ods = oracle.quantize(A, 8, seed=3)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    x_ref, g_ref = oracle.sgd_epoch(ods, b, x0, batch, 1e-5, want_grad=True)
+    x, g = to_dev(x0, ctx), torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, 1e-5, engine=binding.ENGINE_COLUMN, column_chunk_rows=chunk, grid_row_parts=ring_b, grad_out=g)
+    ctx.zipml_sync()
+    assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL and rel(g.cpu().numpy()[0], g_ref[0]) <= GRAD_TOL
+
+
 def test_column_engine_limits(ctx):
     """Rows narrower than one column block, rows wider than one block per SM and batches above 8,192 are declined."""
     _, A, b, _ = workload("c1", 200, 64, seed=1)
