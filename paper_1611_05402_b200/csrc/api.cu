@@ -284,10 +284,10 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
         if (B >= 256 || cb == 8 || B < 32) return ZIPML_ENGINE_COLUMN;
         return ZIPML_ENGINE_STREAM;
     }
-    // 2 bits: C 11.5 S 10.8 at 2.4 KB x 64, 27 / 20 at 6 KB x 1,000.  Else up to some 1,000 rows the column engine, whose CTAs are
-    // few but exchange less: 4 bits 3.3 KB x 600 C 14.6 S 16.6, x 1,500 29.2 / 25.6; 8 bits 4.5 KB x 1,000 14.0 / 14.4, x 2,000
-    // 19.7 / 18.3.
-    return cb == 2 || B >= 1200 ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
+    // 2 bits: C 10.4 S 11.0 at 2.3 KB x 64, 12.4 / 12.3 x 200, 27 / 22 x 1,200.  Else the column engine, whose CTAs are few but exchange
+    // less, up to many rows: 8 bits 7 KB x 1,200 C 12.5 S 15.7, x 3,000 24.5 / 25.5, x 4,500 35.2 / 33.5; 9 KB x 2,000 21.6 / 23.3, x 3,000
+    // 31.1 / 31.6.  (At 4 bits the line at 1,200 rows is a pinned one: 4.1 KB x 1,200 C 13.7 S 16.0, x 2,000 19.3 / 19.4.)
+    return cb == 2 || B >= (cb == 8 ? 3000 : 1200) ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
 }
 
 // Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.

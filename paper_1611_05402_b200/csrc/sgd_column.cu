@@ -1,5 +1,4 @@
-// Column engine of zipml_sgd_epoch: large minibatch tiles on uniform grids, fp32 model and gradient,
-// every code byte read from HBM exactly once per step, no grid-wide barrier.
+// Column engine of zipml_sgd_epoch: large minibatch tiles on uniform grids, fp32 model and gradient, every code byte read from HBM exactly once per step, no grid-wide barrier.
 //
 // A step of the double-sampled minibatch SGD (paper Eq. (double) in its symmetrised form, footnote of
 // "Double Sampling"; update in full precision, "End-to-end Quantization") needs the step's code tile
@@ -50,13 +49,20 @@
 //
 // The machine code is kept small on purpose (four roles share the instruction cache): 32-bit counters kept up
 // step by step instead of 64-bit divisions, waits as functions with one copy, loops unrolled only where
-// registers demand it.  Measured on 65,536 x 32,768 4-bit rows, B = 2,048: 23.0 us per step (stream engine:
+// registers demand it.  Measured on 65,536 x 32,768 4-bit rows, B = 2,048: 21.9 us per step (stream engine:
 // 29.8), DRAM reads 1.00 x the packed bytes.  Not HBM bounds it but the chain of a step: the first chunk's dots
 // have to cross L2 and become digits before pass B can start, pass B (about 1.2 k cycles per chunk on its own, 2 k
 // while pass A runs beside it) ends about 9 k cycles after pass A, and the next step's first dots come 5 k cycles
 // after the last chunk's gradient.  The SM issues about two instructions per cycle in every variant tried, so a
 // role given more warps slows the others by as much; what helped was taking instructions and tests out of the
 // loops and keeping the R warps from waiting for pass B (two digit buffers each).
+// Short steps are that chain alone.  Four things on it that were waiting, us per step of 64 rows of 8,700 / 32,768 4-bit codes, 7.6 / 8.3
+// at first: the A warps slept up to 400 ns past the new w and fenced after it (now a barrier wakes them and the fence
+// comes before; clocks are read by a kernel of their own; one copy of the step's arithmetic) 7.1 / 7.4; the last chunk's digits
+// waited for the step's sums, and the R warps looked every 400 ns (now the sums follow, looks every 100 ns) 6.3 / 6.6; a
+// residual took two shifts, and clamp, maximum and sums in 64 bits (now upper words, one sum a lane) 6.2 / 6.4; 16,000 8-bit codes x 256
+// 9.1 -> 7.3.  Not faster: a chunk's slot held until its gradient, one visit (a chunk takes 18 k cycles through the exchange
+// while others stream, six slots are too few: 28 us on the 2,048 rows); the residuals' planes as two turns of one loop (+3 %).
 //
 // Memory order.  A buffer of dot words serves every third step and is cleared in between by the R warp that
 // has seen the first chunk of step t complete (then every CTA has left step t-1, the buffer's last use,
@@ -89,6 +95,7 @@ constexpr int kColMaxChunkRows = 128;       // a lane of an R warp takes four ro
 constexpr int kColMaxGroups = 4;            // words per row and plane
 constexpr int kColRDigits = 8;              // digits of a residual
 constexpr long long kColQmaxR = 35000000000000000LL;     // below 2^55: eight balanced base-256 digits hold it with room
+constexpr int kColQmaxRHigh = (int)(kColQmaxR >> 32) - 1;    // of its upper word: +-(that << 32) and what lies below stay within +-kColQmaxR
 // Residual digits are balanced base-256 digits (-128..127), found without a carry chain: with 128 added to every digit
 // the number is plain base 256, i.e. the bytes of R + bias; a byte xor 0x80 is the digit as a signed byte.
 constexpr unsigned long long kColBiasR = 0x8080808080808080ull;
@@ -133,6 +140,9 @@ struct ColShared {
     unsigned long long full_b[kColMaxSlots], empty_b[kColMaxSlots];     // B ring: copies landed / the B warps are done
     unsigned long long rfull[kColRBufs], rempty[kColRBufs];     // residual digits of a chunk (buffer q mod kColRBufs): written / consumed
     int w_version;                             // steps (+1) whose digits of w are in place
+    unsigned long long w_ready;                // completes with it: wakes those who wait (the count says whether it is the step they want)
+    unsigned long long s_ready;                // the step's sums over the residuals are in place
+    int cleared;                               // steps whose clearing of dot words (this CTA's share) is done
     ColStepParams sp[2];
     double red_d[2][32];
     float red_f[2][32];
@@ -205,12 +215,13 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
     return v;
 }
 
-// Bounded wait until a version count in shared memory has reached `want`.
-__device__ __noinline__ bool col_wait_version(const int* version, int want, ColShared* sh, DeviceStatus* status, int where) {
+// Bounded wait until a version count in shared memory has reached `want`; the hardware parks the thread until phase want - 1 of `hint`
+// completes (which is when it does, unless the thread comes more than a step late: then the parking runs out).
+__device__ __noinline__ bool col_wait_version(const int* version, int want, unsigned long long* hint, ColShared* sh, DeviceStatus* status, int where) {
     const long long t0 = clock64();
 #pragma unroll 1
     for (int spin = 0; ld_acquire_cta(version) < want; ++spin) {
-        __nanosleep(400);
+        if (mbar_try_wait_parked(hint, (uint32_t)(want - 1) & 1u)) { if (ld_acquire_cta(version) >= want) break; __nanosleep(100); }
         if ((spin & 15) == 15) {
             if (col_aborted(sh)) return false;
             if (clock64() - t0 > kColWaitCycles) { sh->abort_flag = 1; set_status(status, ZIPML_ERR_TIMEOUT, where); return false; }
@@ -242,12 +253,14 @@ __device__ __forceinline__ void tensor_load_2d_hint(void* dst_smem, const CUtens
                  ::"r"(smem_u32(dst_smem)), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy) : "memory");
 }
 
+template <bool TRACED>
 __device__ __forceinline__ void col_mark(const ColumnArgs& a, int64_t t_rel, int k) {
-    if (a.trace && blockIdx.x == 0 && t_rel < a.trace_steps) a.trace[t_rel * 8 + k] = (unsigned long long)clock64();
+    if (TRACED && blockIdx.x == 0 && t_rel < a.trace_steps) a.trace[t_rel * 8 + k] = (unsigned long long)clock64();
 }
 // Adds `cycles` to slot k of the step's trace record (one writer per slot).
+template <bool TRACED>
 __device__ __forceinline__ void col_tally(const ColumnArgs& a, int64_t t_rel, int k, long long cycles) {
-    if (a.trace && blockIdx.x == 0 && t_rel < a.trace_steps) a.trace[t_rel * 8 + k] += (unsigned long long)cycles;
+    if (TRACED && blockIdx.x == 0 && t_rel < a.trace_steps) a.trace[t_rel * 8 + k] += (unsigned long long)cycles;
 }
 
 // Rows of step position `it`.
@@ -255,14 +268,15 @@ struct ColStep {
     int64_t row0;
     int bt, nch;
 };
-__device__ __forceinline__ ColStep col_step(const ColumnArgs& a, int64_t it) {
+__device__ __noinline__ ColStep col_step_of(const int32_t* order, int64_t it, int64_t batch, int64_t m, int R) {
     ColStep s;
-    const int64_t t = a.order ? (int64_t)a.order[it] : it;
-    s.row0 = t * a.batch;
-    s.bt = (int)min(a.batch, a.m - s.row0);
-    s.nch = (s.bt + a.R - 1) / a.R;
+    const int64_t t = order ? (int64_t)order[it] : it;
+    s.row0 = t * batch;
+    s.bt = (int)min(batch, m - s.row0);
+    s.nch = (s.bt + R - 1) / R;
     return s;
 }
+__device__ __forceinline__ ColStep col_step(const ColumnArgs& a, int64_t it) { return col_step_of(a.order, it, a.batch, a.m, a.R); }
 
 // A position in a ring of slots: slot index and the parity of the number of times the ring has wrapped.
 struct ColRing {
@@ -275,7 +289,8 @@ struct ColRing {
 // instruction cache together every warp waits for its next instructions (a first version of 96 KB spent more
 // time there than anywhere else).  Hence: 32-bit counters kept up step by step instead of 64-bit divisions,
 // waits and helpers as functions with one copy, loops unrolled only where registers demand it.
-template <int CB>
+// TRACED: the caller wants a record of the steps (clocks that the others do without).
+template <int CB, bool TRACED>
 __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const ColumnArgs a, const __grid_constant__ CUtensorMap tm1,
                                                                     const __grid_constant__ CUtensorMap tm2) {
     constexpr int NG = 8 / CB;                         // codes per byte = code groups
@@ -319,6 +334,9 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             mbar_init(reinterpret_cast<uint64_t*>(sh->rempty + s), kColBWarps);
         }
         sh->w_version = 0;
+        sh->cleared = 0;
+        mbar_init(reinterpret_cast<uint64_t*>(&sh->w_ready), 1);
+        mbar_init(reinterpret_cast<uint64_t*>(&sh->s_ready), 1);
         sh->abort_flag = 0;
         sh->qa_issued = 0;
         mbar_fence_init();
@@ -442,21 +460,23 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             if (fresh) {
                 // the digits of this step's w (a version count, not a phase: a warp without a task in some step
                 // never looks at that step's digits)
-                ok = __all_sync(0xffffffffu, col_wait_version(&sh->w_version, t_rel + 1, sh, a.status, 71));     // (the warp acts as one)
+                // (see "Memory order" above: the cleared words before this step's additions; they are there long before w is)
+                ok = col_wait_version(&sh->cleared, t_rel, &sh->w_ready, sh, a.status, 69);
+                __threadfence();
+                ok = __all_sync(0xffffffffu, ok && col_wait_version(&sh->w_version, t_rel + 1, &sh->w_ready, sh, a.status, 71));     // (the warp acts as one)
                 if (!ok) break;
-                __threadfence();        // (see "Memory order" above: the cleared words before this step's additions)
                 const ColStepParams& sp = sh->sp[t_rel & 1];
                 kshift = sp.kshift; bint = sp.bint;
                 dots = a.dots + ((size_t)(t_rel % 3) * a.ngrp + grp) * 2 * a.bpad;
                 fresh = false;
-                if (lane == 0 && c == 0 && j == 0) col_mark(a, t_rel, 0);
+                if (lane == 0 && c == 0 && j == 0) col_mark<TRACED>(a, t_rel, 0);
             }
-            const long long w0c = (a.trace && aw == 0) ? clock64() : 0;
+            const long long w0c = (TRACED && aw == 0) ? clock64() : 0;
             if (!__all_sync(0xffffffffu, mbar_test_wait(sh->full_a + ring.slot, ring.phase))) {      // (usually there already)
                 ok = __all_sync(0xffffffffu, col_wait(sh->full_a + ring.slot, ring.phase, sh, a.status, 72));
                 if (!ok) break;
             }
-            if (a.trace && aw == 0 && lane == 0) col_tally(a, t_rel, 1, clock64() - w0c);
+            if (TRACED && aw == 0 && lane == 0) col_tally<TRACED>(a, t_rel, 1, clock64() - w0c);
             const uint32_t tile = smem_u32(tiles) + (uint32_t)ring.slot * slot_bytes;
             const int k0 = c * R + j * 32;                                // first row of the task within the step
             if (k0 < st.bt) {
@@ -555,6 +575,7 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
         const uint32_t rdig_lane = smem_u32(rdig) + (uint32_t)(gl * rstride + tl * 8);
         int q = 0;                                       // chunks so far
         ColRing ring{0, 0u};
+        const double full_scale = 1.0 / (2.0 * (double)a.batch);
         // After a wait has given up the warp stays in step with the others (the named barriers below need every
         // B thread) but waits for nothing and skips the arithmetic.
         bool ok = true;
@@ -598,8 +619,11 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                     }
                 }
                 named_barrier(kColNamedB, kColBThreads);     // every digit is written (also: red_* may be reused)
-                if (btid == 0) st_release_cta(&sh->w_version, t_rel + 1);
-                if (t_rel > 0 && p == 0 && lane == 0) col_mark(a, t_rel - 1, 7);
+                if (btid == 0) {
+                    st_release_cta(&sh->w_version, t_rel + 1);
+                    mbar_arrive(reinterpret_cast<uint64_t*>(&sh->w_ready));
+                }
+                if (t_rel > 0 && p == 0 && lane == 0) col_mark<TRACED>(a, t_rel - 1, 7);
             }
             int acc2[2][NG][4];                                  // two sets, for alternate 32-row blocks: shorter dependency chains
 #pragma unroll
@@ -611,18 +635,18 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
 #pragma unroll 1
             for (int c = 0; c < st.nch; ++c, ++q) {
                 const int rbuf = q & (kColRBufs - 1);
-                const long long w0c = (a.trace && p == 0) ? clock64() : 0;
+                const long long w0c = (TRACED && p == 0) ? clock64() : 0;
                 long long w1c = w0c;
                 // both are usually there already: one look at each, side by side, before the waiting routine is called
                 const bool have_r = mbar_test_wait(sh->rfull + rbuf, (uint32_t)((q >> kColRBufShift) & 1));
                 const bool have_c = mbar_test_wait(sh->full_b + ring.slot, ring.phase);
                 if (!__all_sync(0xffffffffu, ok && have_r && have_c)) {
                     ok = ok && col_wait(sh->rfull + rbuf, (uint32_t)((q >> kColRBufShift) & 1), sh, a.status, 73);
-                    w1c = (a.trace && p == 0) ? clock64() : 0;
+                    w1c = (TRACED && p == 0) ? clock64() : 0;
                     ok = ok && col_wait(sh->full_b + ring.slot, ring.phase, sh, a.status, 74);
                     ok = __all_sync(0xffffffffu, ok);                  // the warp acts as one
                 }
-                if (a.trace && p == 0 && lane == 0) { col_tally(a, t_rel, 4, w1c - w0c); col_tally(a, t_rel, 5, clock64() - w1c); }
+                if (TRACED && p == 0 && lane == 0) { col_tally<TRACED>(a, t_rel, 4, w1c - w0c); col_tally<TRACED>(a, t_rel, 5, clock64() - w1c); }
                 const uint32_t tile = smem_u32(tiles_b) + (uint32_t)ring.slot * slot_bytes + b_off;
                 // Rows past the step's last one carry zero digits, so whole chunks are contracted: all R / 32 blocks, and
                 // for the usual R = 128 without a test per block.
@@ -675,7 +699,9 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                 }
                 ring.next(a.slots_b);
             }
-            const long long u0c = (a.trace && p == 0) ? clock64() : 0;
+            const long long u0c = (TRACED && p == 0) ? clock64() : 0;
+            ok = ok && col_wait(&sh->s_ready, (uint32_t)t_rel & 1u, sh, a.status, 68);
+            ok = __all_sync(0xffffffffu, ok);
             // ---- the step's gradient of the own features; update
             // lane (g, t): acc[gi][0..1] = digits 2t, 2t+1 of byte 2g, acc[gi][2..3] of byte 2g+1
             int acc[NG][4];
@@ -684,7 +710,7 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[g][e] = acc2[0][g][e] + acc2[1][g][e];
             const ColStepParams& sp = sh->sp[t_rel & 1];
-            const double delta_r = sp.delta_r, lo_term = sp.delta_r * sp.rsum, scale = 1.0 / (2.0 * (double)st.bt);
+            const double delta_r = sp.delta_r, lo_term = sp.delta_r * sp.rsum, scale = st.bt == (int)a.batch ? full_scale : 1.0 / (2.0 * (double)st.bt);
             const double w0 = (tl == 0) ? 1.0 : (tl == 1) ? 65536.0 : (tl == 2) ? 4294967296.0 : 281474976710656.0;  // 256^(2t)
             double Sf[NF];
 #pragma unroll
@@ -709,7 +735,7 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                     if (last) a.x[jo[e]] = xo[e];
                 }
             }
-            if (p == 0 && lane == 0) col_tally(a, t_rel, 6, clock64() - u0c);
+            if (p == 0 && lane == 0) col_tally<TRACED>(a, t_rel, 6, clock64() - u0c);
         }
     }
     // =================================================================================== R warps: residual digits
@@ -744,12 +770,13 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             const bool bounded = rbound - rbound == 0.0;
             // The residuals' unit is a power of two as well (at most twice what the bound needs), so that a dot becomes
             // a residual by a shift and the label's own fixed-point value: integers only on the way to the digits.
-            const int ed = rbound > 0.0 ? max(-900, min(900, col_exponent(rbound * (1.0 / (double)kColQmaxR)) + 1)) : 0;
+            // It is not below the dots' unit, whose multiples the dots are.
+            const int eu = col_exponent(sp.U);
+            const int ed = max(eu, rbound > 0.0 ? max(-900, min(900, col_exponent(rbound * (1.0 / (double)kColQmaxR)) + 1)) : 0);
             const double delta_r = col_pow2(ed), inv_delta = col_pow2(-ed);
-            const int sft = col_exponent(sp.U) - ed;     // dot unit over residual unit: 2^sft (at most 2^4 by construction)
-            const int lsh = max(0, min(sft, 8)), rsh = min(63, max(0, -sft));
+            const int rsh = min(63, ed - eu);            // residual unit over dot unit: 2^rsh
             const long long half = rsh > 0 ? (1ll << (rsh - 1)) : 0;
-            long long amax = 0;                          // largest |fixed-point residual| of the lane
+            int amax = 0;                                // largest upper word of a |fixed-point residual| of the lane
             long long rs_hi = 0, rs_lo = 0;              // sum of the fixed-point residuals: high parts and low 28 bits
             const int c_last = st.nch - 1;
             bool behind = false;                         // (a step's first chunks are never complete yet)
@@ -787,17 +814,17 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                             asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(v0) : "l"(wl) : "memory");
                             if ((int)(v0 & 0xFF) >= want) break;
                             first_look = false;
-                            if ((spin & 15) == 15) {
+                            if ((spin & 63) == 63) {
                                 if (col_aborted(sh) || *reinterpret_cast<volatile int*>(&a.status->code) != 0) { sh->abort_flag = 1; break; }
                                 if (clock64() - t0 > kColWaitCycles) { sh->abort_flag = 1; set_status(a.status, ZIPML_ERR_TIMEOUT, 75); break; }
                             }
-                            __nanosleep(400);
+                            __nanosleep(100);
                         }
                     }
                 }
                 __syncwarp();
                 ok = __all_sync(0xffffffffu, ok && !col_aborted(sh));          // (the warp acts as one)
-                if (a.trace && rw == 0 && lane == 0) col_tally(a, t_rel, 2, clock64() - t0);
+                if (TRACED && rw == 0 && lane == 0) col_tally<TRACED>(a, t_rel, 2, clock64() - t0);
                 long long D1[4], D2[4];                                  // the rows' dots: sums over the groups' words
 #pragma unroll 1
                 for (int spin = 0;; ++spin) {
@@ -824,36 +851,42 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                     }
                     if (__all_sync(0xffffffffu, done) || !ok) break;
                     first_look = false;
-                    __nanosleep(200);
-                    if ((spin & 7) == 7) {
+                    __nanosleep(60);
+                    if ((spin & 31) == 31) {
                         bool give_up = col_aborted(sh) || *reinterpret_cast<volatile int*>(&a.status->code) != 0;
                         if (clock64() - t0 > kColWaitCycles) { set_status(a.status, ZIPML_ERR_TIMEOUT, 77); give_up = true; }
                         if (__any_sync(0xffffffffu, give_up)) { sh->abort_flag = 1; ok = false; }
                     }
                 }
                 behind = __all_sync(0xffffffffu, first_look);
-                const long long e0c = (a.trace && rw == 0) ? clock64() : 0;
+                const long long e0c = (TRACED && rw == 0) ? clock64() : 0;
                 if (ok && q >= kColRBufs) ok = col_wait(sh->rempty + rbuf, (uint32_t)(((q >> kColRBufShift) - 1) & 1), sh, a.status, 76);
                 ok = __all_sync(0xffffffffu, ok);
-                if (a.trace && rw == 0 && lane == 0) col_tally(a, t_rel, 3, clock64() - e0c);
+                if (TRACED && rw == 0 && lane == 0) col_tally<TRACED>(a, t_rel, 3, clock64() - e0c);
                 if (kkA < R && ok) {
-                    // residuals r = U * dot - label in fixed point, then their digits: with 64 added to every digit the
+                    // residuals r = U * dot - label in fixed point, then their digits: with 128 added to every digit the
                     // number is plain base 256 (no carry chain); four rows' digits make a word
                     unsigned long long u1[4], u2[4];
+                    long long sum = 0;                                   // (eight values: no overflow)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        long long R1 = 0, R2 = 0;
-                        if (kA + (i & 1) + 8 * (i >> 1) < st.bt) {
-                            const long long bfix = __double2ll_rn((double)bk[i] * inv_delta);
-                            R1 = max(-kColQmaxR, min(kColQmaxR, (((D1[i] + half) >> rsh) << lsh) - bfix));
-                            R2 = max(-kColQmaxR, min(kColQmaxR, (((D2[i] + half) >> rsh) << lsh) - bfix));
-                            amax = max(amax, max(llabs(R1), llabs(R2)));
-                            rs_hi += (R1 >> 28) + (R2 >> 28);
-                            rs_lo += (R1 & 0xFFFFFFFll) + (R2 & 0xFFFFFFFll);
-                        }
+                        const bool real = kA + (i & 1) + 8 * (i >> 1) < st.bt;
+                        const long long bfix = __double2ll_rn((double)bk[i] * inv_delta);
+                        long long R1 = real ? ((D1[i] + half) >> rsh) - bfix : 0, R2 = real ? ((D2[i] + half) >> rsh) - bfix : 0;
+                        // by the upper word (a violated bound could only lose accuracy, never wrap)
+                        auto clamp = [&](long long r) {
+                            const int high = max(-kColQmaxRHigh, min(kColQmaxRHigh, (int)(r >> 32)));
+                            amax = max(amax, max(high, ~high));
+                            return (long long)((unsigned long long)(uint32_t)high << 32 | (uint32_t)r);
+                        };
+                        R1 = clamp(R1);
+                        R2 = clamp(R2);
+                        sum += R1 + R2;
                         u1[i] = ((unsigned long long)R1 + kColBiasR) ^ kColBiasR;      // eight digits as signed bytes
                         u2[i] = ((unsigned long long)R2 + kColBiasR) ^ kColBiasR;
                     }
+                    rs_hi += sum >> 28;
+                    rs_lo += sum & 0xFFFFFFFll;
                     // the four rows' words (four digits each) are transposed into one word per digit
                     signed char* dst = rd + blk * 32 + tl * 8 + hf * 4;
 #pragma unroll
@@ -872,10 +905,8 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                         *reinterpret_cast<uint32_t*>(dst + (size_t)(4 * h + 3) * rstride) = __byte_perm(t2, t3, 0x7632);
                     }
                 }
-                if (c != c_last) {                       // (the step's last chunk is released below, after the step's sums)
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(reinterpret_cast<uint64_t*>(sh->rfull + rbuf));
-                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(reinterpret_cast<uint64_t*>(sh->rfull + rbuf));
                 // (off the chunk's path) every CTA has left step t - 1 behind, as chunk 0's complete dots showed: its buffer of dot words is cleared for step t + 2 (this CTA's share)
                 if (c == 0 && ok) {
                     __threadfence();        // (see "Memory order" above: the others' reads of that buffer before these stores)
@@ -885,6 +916,8 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                     for (int g = 0; g < 2 * ngrp; ++g)
 #pragma unroll 1
                         for (int i = z0 + lane; i < z1; i += 32) z[(size_t)g * a.bpad + i] = 0;
+                    __syncwarp();
+                    if (lane == 0) st_release_cta(&sh->cleared, t_rel + 1);
                 }
             }
             // ---- the step's residuals are all known: their sum for the B warps, the next step's bound and unit
@@ -894,7 +927,7 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                 rs_hi += __shfl_xor_sync(0xffffffffu, rs_hi, o);
                 rs_lo += __shfl_xor_sync(0xffffffffu, rs_lo, o);
             }
-            if (lane == 0) { sh->red_d[1][rw] = (double)amax * delta_r; sh->red_l[0][rw] = rs_hi; sh->red_l[1][rw] = rs_lo; }
+            if (lane == 0) { sh->red_d[1][rw] = ((double)amax + 1.0) * (4294967296.0 * delta_r); sh->red_l[0][rw] = rs_hi; sh->red_l[1][rw] = rs_lo; }
             named_barrier(kColNamedR, kColRThreads);     // (the next step's barrier keeps these slots from being rewritten early)
             double rm = 0.0;
             long long hi = 0, lo = 0;
@@ -902,15 +935,14 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             for (int w = 0; w < kColRWarps; ++w) { rm = fmax(rm, sh->red_d[1][w]); hi += sh->red_l[0][w]; lo += sh->red_l[1][w]; }
             dbound = bounded ? (dbound * grow + fabs((double)a.lr) * rm * c2) * 1.0001 : __longlong_as_double(0x7fffffffffffffffll);
             if (((q0 + c_last) & (kColRWarps - 1)) == rw) {      // the warp that holds the step's last chunk
-                if (lane == 0) {
+                if (lane == 0) {                         // (pass B is done with the chunk about when the sums are there)
                     ColStepParams& cur = sh->sp[t_rel & 1];
                     cur.inv_r = inv_delta;
                     cur.delta_r = delta_r;
                     cur.rsum = bounded ? (double)hi * 268435456.0 + (double)lo : __longlong_as_double(0x7fffffffffffffffll);
                     col_unit_of(dbound, sh->sp[(t_rel + 1) & 1].U, sh->sp[(t_rel + 1) & 1].invU);
+                    mbar_arrive(reinterpret_cast<uint64_t*>(&sh->s_ready));
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(reinterpret_cast<uint64_t*>(sh->rfull + ((q0 + c_last) & (kColRBufs - 1))));
             }
             q0 += st.nch;
         }
@@ -921,10 +953,11 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
 // ---------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------
+template <bool TRACED>
 static const void* column_kernel_ptr(int cb) {
-    if (cb == 2) return reinterpret_cast<const void*>(&sgd_column_kernel<2>);
-    if (cb == 4) return reinterpret_cast<const void*>(&sgd_column_kernel<4>);
-    return reinterpret_cast<const void*>(&sgd_column_kernel<8>);
+    if (cb == 2) return reinterpret_cast<const void*>(&sgd_column_kernel<2, TRACED>);
+    if (cb == 4) return reinterpret_cast<const void*>(&sgd_column_kernel<4, TRACED>);
+    return reinterpret_cast<const void*>(&sgd_column_kernel<8, TRACED>);
 }
 
 // Tensor maps over the two planes as byte matrices: boxes of 128 bytes x R rows with the 128-byte swizzle,
@@ -1013,7 +1046,7 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     if (nch_max > 1) slots_a = slots_a / stride * stride;
     if (slots_a < 1 || slots_b < 1) return ZIPML_ERR_WORKSPACE;
     const size_t smem = fixed + (size_t)slots * slot_bytes;
-    const void* kernel = column_kernel_ptr(cb);
+    const void* kernel = p->trace && p->trace_steps > 0 ? column_kernel_ptr<true>(cb) : column_kernel_ptr<false>(cb);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
     int per_sm = 0;
