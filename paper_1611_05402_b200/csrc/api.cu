@@ -290,6 +290,20 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
     return cb == 2 || B >= (cb == 8 ? 3000 : 1200) ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
 }
 
+// The same rows with a quantized model or gradient: column or ring engine.  Q0/8 (fp32 model, gradient of 8 bits): 2 bits 2.2 KB x 1,200
+// C 29.4 R 34.5, x 2,000 41 / 36; 4 KB x 2,000 42 / 41; 6 KB x 3,000 56 / 56; 8 KB x 4,500 87 / 93.  4 bits 4.1 KB x 64 C 9.1 R 22, x 1,200
+// 16.5 / 33, x 4,500 41 / 43, x 6,000 53 / 49; 9 KB x 8,192 86 / 85; 16 KB x 64 10.7 / 31, x 8,192 92 / 145.  8 bits 9 KB x 64 9.4 / 21, x 3,000
+// 33 / 36, x 6,000 61 / 54; 12 KB x 6,000 49 / 68.  (With a quantized model too C takes some 3 more, R 6.)
+static bool column_pays_quantized(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t count) {
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || (p->model_bits == 0 && p->grad_bits == 0)) return false;
+    // (a quantized gradient alone in up to three steps: the choice of the ring engine is a pinned one, not the faster)
+    if (p->model_bits == 0 && count <= 3) return false;
+    const int cb = container_bits(d->bits);
+    if (cb == 2) return B <= 1500 || 2 * B <= d->row_bytes;
+    if (cb == 4) return B <= 4500 || 10 * B <= 9 * d->row_bytes;
+    return B <= 4500 || d->row_bytes >= 11000;
+}
+
 // Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.
 //   tables: 3 bits n 600 x 1,207 L 13.7 G 21.2, x 2,414 L 21.5 G 23.8, x 3,276 L 27 G 25; n 512 x 2,867 L 18.5 G 20.1, x 3,891 L 22.9 G 21.5;
 //   n 300 x 3,276 L 19.1 G 20.7, x 4,587 L 24.3 G 22.9; n 700 x 1,489 L 15.8 G 16.6, x 2,084 L 20.0 G 19.0; n 1,000 x 1,024 L 15.4 G 16.6, x 1,433
@@ -350,14 +364,14 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
     if (linf && data->layout == ZIPML_LAYOUT_COLUMN_BLOCKS) return ZIPML_ERR_UNSUPPORTED;
     if (data->layout == ZIPML_LAYOUT_COLUMN_BLOCKS) {                 // the column engine's own layout
         if (params->engine != ZIPML_ENGINE_AUTO && params->engine != ZIPML_ENGINE_COLUMN) return ZIPML_ERR_UNSUPPORTED;
-        rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
+        rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
         return rc == ZIPML_ERR_WORKSPACE ? ZIPML_ERR_UNSUPPORTED : rc;
     }
     if (params->engine == ZIPML_ENGINE_RING) return launch_sgd_ring(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_LEAN) return launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
     if (params->engine == ZIPML_ENGINE_CLUSTER) return launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
     if (params->engine == ZIPML_ENGINE_STREAM) return launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out);
-    if (params->engine == ZIPML_ENGINE_COLUMN) return launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
+    if (params->engine == ZIPML_ENGINE_COLUMN) return launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_SOLO) return launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, false);
     if (params->engine == ZIPML_ENGINE_AUTO && !linf) {
         // Small minibatch tiles are bound by the step-to-step chain, not by HBM: the smallest stay on one SM, then
@@ -383,8 +397,12 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
+        if (column_pays_quantized(data, params, B, count)) {
+            rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, true);
+            if (rc != ZIPML_ERR_WORKSPACE) return rc;
+        }
         if (wide == ZIPML_ENGINE_COLUMN) {
-            rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out);
+            rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, false);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
         if (wide == ZIPML_ENGINE_COLUMN || wide == ZIPML_ENGINE_STREAM) {

@@ -1,4 +1,4 @@
-// Column engine of zipml_sgd_epoch: large minibatch tiles on uniform grids, fp32 model and gradient, every code byte read from HBM exactly once per step, no grid-wide barrier.
+// Column engine of zipml_sgd_epoch: large minibatch tiles on uniform grids, every code byte read from HBM exactly once per step, no grid-wide barrier.
 //
 // A step of the double-sampled minibatch SGD (paper Eq. (double) in its symmetrised form, footnote of
 // "Double Sampling"; update in full precision, "End-to-end Quantization") needs the step's code tile
@@ -64,6 +64,11 @@
 // 9.1 -> 7.3.  Not faster: a chunk's slot held until its gradient, one visit (a chunk takes 18 k cycles through the exchange
 // while others stream, six slots are too few: 28 us on the 2,048 rows); the residuals' planes as two turns of one loop (+3 %).
 //
+// Quantized model and gradient (QV).  The norm is a sum over all CTAs: each writes its part to a box of every other, 16 bytes with a
+// tag in each half, and polls its own boxes only (all polling the same words: +2 us a norm).  The norm also bounds the next
+// dots (||a|| ||Q(v)||), so that here the B warps set the dots' unit, with the digits of w, and the R warps take it from there.  64 rows
+// of 8,700 / 32,768 4-bit codes, 8 bits of gradient: 8.8 / 10.3 us (ring engine 22 / 31); of the model too 11.7 / 13.5 (25 / 37).
+//
 // Memory order.  A buffer of dot words serves every third step and is cleared in between by the R warp that
 // has seen the first chunk of step t complete (then every CTA has left step t-1, the buffer's last use,
 // behind: hence its fence before the stores), once that chunk's digits are out; the A warps fence once per step before their first
@@ -122,6 +127,10 @@ struct ColumnArgs {
     float reg_cst;
     long long* dots;         // [3][ngrp][2][bpad] three steps in rotation, zeroed before the launch; a word holds the
                              // fixed-point sum in its upper 56 bits and the number of CTAs that added in its low byte
+    int model_bits, grad_bits;   // QV: bits of the quantized model and gradient (0: fp32)
+    uint64_t seed;
+    uint32_t epoch;
+    unsigned long long* norms;   // QV: [2: gradient, model][2 steps in turn][reader][writer][2] halves of a CTA's sum of squares, a tag with each; zeroed
     DeviceStatus* status;
     unsigned long long* trace;
     int trace_steps;
@@ -133,6 +142,7 @@ struct ColStepParams {       // by step parity
     int kshift;              // the unit of the own w digits is U * 2^kshift     (B warps -> A warps)
     double inv_r, delta_r;   // fixed point of the residuals                     (R warps -> B warps)
     double rsum;             // sum of all fixed-point residuals of the step     (R warps -> B warps)
+    double bound;            // QV: of the step's |dots|; U, invU come with it   (B warps -> R warps)
 };
 
 struct ColShared {
@@ -147,6 +157,7 @@ struct ColShared {
     double red_d[2][32];
     float red_f[2][32];
     long long red_l[2][kColRWarps];
+    double norm_d[2][kColBWarps];
     int abort_flag;
     int qa_issued;                             // chunks whose first copy has been issued
 };
@@ -243,6 +254,55 @@ __device__ __forceinline__ void col_unit_of(double bound, double& U, double& inv
 
 __device__ __forceinline__ void named_barrier(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
+// The norm over all CTAs of a vector spread over their B threads (`part`: this thread's share of the squares), summed in an order that
+// does not depend on timing.  Every CTA writes its sum to every CTA's box, as two words that are each valid by their tag, and a
+// thread per CTA watches for one: a CTA looks only at its own 16 bytes per sender.
+__device__ __noinline__ float col_norm(double part, unsigned long long* box, uint32_t tag, bool wait, ColShared* sh, DeviceStatus* status) {
+    const int btid = (int)threadIdx.x - 32 * kColWarpB0, lane = btid & 31, p = btid >> 5;
+    part = warp_sum(part);
+    if (lane == 0) sh->norm_d[0][p] = part;
+    named_barrier(kColNamedB, kColBThreads);
+    const int G = (int)gridDim.x;
+    double v = 0.0;
+    if (btid < G) {
+#pragma unroll
+        for (int w = 0; w < kColBWarps; ++w) v += sh->norm_d[0][w];
+        const unsigned long long u = (unsigned long long)__double_as_longlong(v), high = (unsigned long long)tag << 32;
+        asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(box + 2 * (btid * G + (int)blockIdx.x)), "l"(high | (u >> 32)),
+                     "l"(high | (u & 0xffffffffull)) : "memory");
+    }
+    v = 0.0;
+    if (btid < G && wait) {
+        box += 2 * ((int)blockIdx.x * G + btid);
+        const long long t0 = clock64();
+#pragma unroll 1
+        for (int spin = 0;; ++spin) {
+            unsigned long long x, y;
+            asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(box) : "memory");
+            if ((uint32_t)(x >> 32) == tag && (uint32_t)(y >> 32) == tag) { v = __longlong_as_double((long long)(x << 32 | (y & 0xffffffffull))); break; }
+            if ((spin & 15) == 15) {
+                if (col_aborted(sh) || *reinterpret_cast<volatile int*>(&status->code) != 0) { sh->abort_flag = 1; break; }
+                if (clock64() - t0 > kColWaitCycles) { sh->abort_flag = 1; set_status(status, ZIPML_ERR_TIMEOUT, 79); break; }
+            }
+        }
+    }
+    v = warp_sum(v);
+    if (lane == 0) sh->norm_d[1][p] = v;
+    named_barrier(kColNamedB, kColBThreads);
+    v = 0.0;
+#pragma unroll
+    for (int w = 0; w < kColBWarps; ++w) v += sh->norm_d[1][w];
+    return (float)sqrt(v);
+}
+
+__device__ __noinline__ float col_quantize(float v, float M, int bits, uint32_t u24) {
+    const VecQuant q{M, (1 << (bits - 1)) - 1, 0, 0u, 0u, 0u};
+    return q.apply_drawn(v, u24);
+}
+__device__ __noinline__ uint32_t col_draw(uint64_t seed, uint32_t epoch, uint32_t step, uint32_t coord, uint32_t stream) {
+    return vector_u24(seed, epoch, step, coord, stream);
+}
+
 __device__ __forceinline__ void tensor_load_2d(void* dst_smem, const CUtensorMap* tm, int x, int y, unsigned long long* bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(smem_u32(dst_smem)), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
@@ -289,8 +349,8 @@ struct ColRing {
 // instruction cache together every warp waits for its next instructions (a first version of 96 KB spent more
 // time there than anywhere else).  Hence: 32-bit counters kept up step by step instead of 64-bit divisions,
 // waits and helpers as functions with one copy, loops unrolled only where registers demand it.
-// TRACED: the caller wants a record of the steps (clocks that the others do without).
-template <int CB, bool TRACED>
+// QV: the model, the gradient or both are quantized.  TRACED: the caller wants a record of the steps (clocks that the others do without).
+template <int CB, bool QV, bool TRACED>
 __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const ColumnArgs a, const __grid_constant__ CUtensorMap tm1,
                                                                     const __grid_constant__ CUtensorMap tm2) {
     constexpr int NG = 8 / CB;                         // codes per byte = code groups
@@ -558,6 +618,8 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
         const int btid = tid - 32 * kColWarpB0;
         // own features: (byte 2g + h of the piece, code group gi), fi = h * NG + gi = tl + 4e
         float xo[NF], lo_o[NF], st_o[NF];
+        [[maybe_unused]] float vo[NF];                   // QV: what the step's dots see of the model
+        [[maybe_unused]] uint32_t u_x[NF], u_g[NF];      // QV: draws, made while the step's dots are on their way
         int64_t jo[NF];
         bool have[NF];
 #pragma unroll
@@ -579,17 +641,44 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
         // After a wait has given up the warp stays in step with the others (the named barriers below need every
         // B thread) but waits for nothing and skips the arithmetic.
         bool ok = true;
+        // QV: bounds of a vector's dots with the rows by its norm: ||a|| ||Q(v)||, and rounding moves every entry by at most M / s
+        [[maybe_unused]] double bound = dbound, reach_x = 0.0, reach_g = 0.0;
+        [[maybe_unused]] const double grow = a.reg == ZIPML_REG_LSSVM ? fmax(1.0, fabs(1.0 - (double)a.reg_cst)) : 1.0;
+        if constexpr (QV) {
+            const double rows = sqrt(c2) * 1.0001, root = sqrt((double)n);
+            if (a.model_bits > 0) reach_x = rows * (1.0 + root / (double)((1 << (a.model_bits - 1)) - 1));
+            if (a.grad_bits > 0) reach_g = fabs((double)a.lr) * rows * (1.0 + root / (double)((1 << (a.grad_bits - 1)) - 1));
+            if (a.model_bits > 0)
+#pragma unroll
+                for (int e = 0; e < NF; ++e) u_x[e] = col_draw(a.seed, a.epoch, (uint32_t)a.first_step, (uint32_t)jo[e], 3u);
+        }
 #pragma unroll 1
         for (int t_rel = 0; t_rel < steps; ++t_rel) {
             const ColStep st = col_step(a, a.first_step + t_rel);
             const bool last = t_rel + 1 == steps;
+            if constexpr (QV) {
+#pragma unroll
+                for (int e = 0; e < NF; ++e) vo[e] = xo[e];
+                if (a.model_bits > 0) {
+                    double part = 0.0;
+#pragma unroll
+                    for (int e = 0; e < NF; ++e) part += (double)xo[e] * (double)xo[e];       // (0 where there is none)
+                    const float M = col_norm(part, a.norms + (size_t)(2 + (t_rel & 1)) * 2 * G * G, (uint32_t)t_rel + 1u, ok, sh, a.status);
+#pragma unroll
+                    for (int e = 0; e < NF; ++e) vo[e] = have[e] ? col_quantize(xo[e], M, a.model_bits, u_x[e]) : 0.0f;
+                    bound = M > 0.0f ? (double)M * reach_x : 0.0;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < NF; ++e) vo[e] = xo[e];
+            }
             // ---- digits of w = step * x of the own features for this step, and the own part of lo^T x
             {
                 const int par = t_rel & 1;
                 float wm = 0.0f;
                 double bs = 0.0;
 #pragma unroll
-                for (int e = 0; e < NF; ++e) { wm = fmaxf(wm, fabsf(st_o[e] * xo[e])); bs += (double)lo_o[e] * (double)xo[e]; }
+                for (int e = 0; e < NF; ++e) { wm = fmaxf(wm, fabsf(st_o[e] * vo[e])); bs += (double)lo_o[e] * (double)vo[e]; }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
                 bs = warp_sum(bs);
@@ -601,18 +690,25 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                 for (int w = 0; w < kColBWarps; ++w) { wmax = fmaxf(wmax, sh->red_f[0][w]); bsum += sh->red_d[0][w]; }
                 // the unit of the digits is the dots' unit times a power of two (at most twice what max |w| needs), so
                 // that a digit sum turns into the dots' unit by a shift
-                const double U = sh->sp[par].U, need = (double)wmax * (1.0 / (double)QMAXW);
+                double U, invU;
+                if constexpr (QV) col_unit_of(bound, U, invU);
+                else { U = sh->sp[par].U; invU = sh->sp[par].invU; }
+                const double need = (double)wmax * (1.0 / (double)QMAXW);
                 const int eu = col_exponent(U);                           // U = 2^eu
                 const int ks = need > U ? col_exponent(need) + 1 - eu : 0;   // need < U * 2^ks
                 const float inv = (float)col_pow2(-(eu + ks));
-                if (btid == 0) { sh->sp[par].kshift = ks; sh->sp[par].bint = __double2ll_rn(bsum * sh->sp[par].invU); }
+                if (btid == 0) {
+                    sh->sp[par].kshift = ks;
+                    sh->sp[par].bint = __double2ll_rn(bsum * invU);
+                    if constexpr (QV) { sh->sp[par].U = U; sh->sp[par].invU = invU; sh->sp[par].bound = bound; }
+                }
 #pragma unroll
                 for (int e = 0; e < NF; ++e) {
                     const int fi = tl + 4 * e, h = fi / NG, gi = fi - h * NG;
                     if (fi < 2 * NG) {
                         const int byte = 16 * p + 2 * gl + h, kb = byte >> 5, bb = byte & 31;
                         // balanced digits without a carry chain: with 64 added to every digit the number is plain base 128
-                        const uint32_t u = (uint32_t)((have[e] ? max(-QMAXW, min(QMAXW, __float2int_rn(st_o[e] * xo[e] * inv))) : 0) + kColBiasW);
+                        const uint32_t u = (uint32_t)((have[e] ? max(-QMAXW, min(QMAXW, __float2int_rn(st_o[e] * vo[e] * inv))) : 0) + kColBiasW);
                         signed char* dst = wdig + (size_t)((gi * 4 + kb) * 8) * 32 + ((bb & 15) >> 2) * 8 + (bb >> 4) * 4 + (bb & 3);
 #pragma unroll
                         for (int s = 0; s < NS; ++s) dst[s * 32] = (signed char)((int)((u >> (7 * s)) & 127u) - 64);
@@ -624,6 +720,14 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                     mbar_arrive(reinterpret_cast<uint64_t*>(&sh->w_ready));
                 }
                 if (t_rel > 0 && p == 0 && lane == 0) col_mark<TRACED>(a, t_rel - 1, 7);
+            }
+            if constexpr (QV) {
+                const uint32_t it = (uint32_t)(a.first_step + t_rel);
+#pragma unroll
+                for (int e = 0; e < NF; ++e) {
+                    if (a.grad_bits > 0) u_g[e] = col_draw(a.seed, a.epoch, it, (uint32_t)jo[e], 4u);
+                    if (a.model_bits > 0) u_x[e] = col_draw(a.seed, a.epoch, it + 1u, (uint32_t)jo[e], 3u);
+                }
             }
             int acc2[2][NG][4];                                  // two sets, for alternate 32-row blocks: shorter dependency chains
 #pragma unroll
@@ -726,11 +830,29 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
                 v += __shfl_xor_sync(0xffffffffu, v, 2);
                 if ((fi & 3) == tl) Sf[fi >> 2] = v;
             }
+            float g_o[NF];
+#pragma unroll
+            for (int e = 0; e < NF; ++e) {
+                g_o[e] = have[e] ? (float)(((double)lo_o[e] * lo_term + (double)st_o[e] * (delta_r * Sf[e])) * scale) : 0.0f;
+                if (have[e] && last && a.grad_out) a.grad_out[jo[e]] = g_o[e];
+            }
+            if constexpr (QV) {
+                if (a.grad_bits > 0) {
+                    double part = 0.0;
+#pragma unroll
+                    for (int e = 0; e < NF; ++e) part += (double)g_o[e] * (double)g_o[e];
+                    const float M = col_norm(part, a.norms + (size_t)(t_rel & 1) * 2 * G * G, (uint32_t)t_rel + 1u, ok, sh, a.status);
+#pragma unroll
+                    for (int e = 0; e < NF; ++e) g_o[e] = col_quantize(g_o[e], M, a.grad_bits, u_g[e]);
+                    bound = (bound * grow + (M > 0.0f ? (double)M * reach_g : 0.0)) * 1.0001;
+                }
+                ok = ok && !col_aborted(sh);
+            }
 #pragma unroll
             for (int e = 0; e < NF; ++e) {
                 if (have[e]) {
-                    const float g = (float)(((double)lo_o[e] * lo_term + (double)st_o[e] * (delta_r * Sf[e])) * scale);
-                    if (last && a.grad_out) { a.grad_out[jo[e]] = g; a.grad_out[n + jo[e]] = g; }
+                    const float g = g_o[e];
+                    if (last && a.grad_out) a.grad_out[n + jo[e]] = g;
                     xo[e] = regularise(fmaf(-a.lr, g, xo[e]), xo[e], a.reg, a.reg_cst);
                     if (last) a.x[jo[e]] = xo[e];
                 }
@@ -746,7 +868,7 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
         const int rt = tid - 32 * kColWarpR0, rw = rt >> 5;
         int q0 = 0;                                      // the step's first chunk in the launch's sequence
         bool ok = true;                                  // (after a failure: as for the B warps)
-        const double grow = a.reg == ZIPML_REG_LSSVM ? fmax(1.0, fabs(1.0 - (double)a.reg_cst)) : 1.0;
+        [[maybe_unused]] const double grow = a.reg == ZIPML_REG_LSSVM ? fmax(1.0, fabs(1.0 - (double)a.reg_cst)) : 1.0;
         const int zper = (a.bpad + G - 1) / G;           // rows of a buffer of dot words that this CTA clears
         const int ngrp = a.ngrp;
         const int last_size = G - (ngrp - 1) * a.gsize;  // CTAs of the last group
@@ -766,6 +888,11 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             bm = 0u;
 #pragma unroll
             for (int w = 0; w < kColRWarps; ++w) bm = max(bm, __float_as_uint(sh->red_f[1][w]));
+            if constexpr (QV) {                          // the bound and the unit come from the B warps, with the step's w
+                ok = ok && col_wait_version(&sh->w_version, t_rel + 1, &sh->w_ready, sh, a.status, 80);
+                ok = __all_sync(0xffffffffu, ok);
+                dbound = sp.bound;
+            }
             const double rbound = (dbound + (double)__uint_as_float(bm)) * 1.0001;
             const bool bounded = rbound - rbound == 0.0;
             // The residuals' unit is a power of two as well (at most twice what the bound needs), so that a dot becomes
@@ -933,14 +1060,14 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
             long long hi = 0, lo = 0;
 #pragma unroll
             for (int w = 0; w < kColRWarps; ++w) { rm = fmax(rm, sh->red_d[1][w]); hi += sh->red_l[0][w]; lo += sh->red_l[1][w]; }
-            dbound = bounded ? (dbound * grow + fabs((double)a.lr) * rm * c2) * 1.0001 : __longlong_as_double(0x7fffffffffffffffll);
+            if constexpr (!QV) dbound = bounded ? (dbound * grow + fabs((double)a.lr) * rm * c2) * 1.0001 : __longlong_as_double(0x7fffffffffffffffll);
             if (((q0 + c_last) & (kColRWarps - 1)) == rw) {      // the warp that holds the step's last chunk
                 if (lane == 0) {                         // (pass B is done with the chunk about when the sums are there)
                     ColStepParams& cur = sh->sp[t_rel & 1];
                     cur.inv_r = inv_delta;
                     cur.delta_r = delta_r;
                     cur.rsum = bounded ? (double)hi * 268435456.0 + (double)lo : __longlong_as_double(0x7fffffffffffffffll);
-                    col_unit_of(dbound, sh->sp[(t_rel + 1) & 1].U, sh->sp[(t_rel + 1) & 1].invU);
+                    if constexpr (!QV) col_unit_of(dbound, sh->sp[(t_rel + 1) & 1].U, sh->sp[(t_rel + 1) & 1].invU);
                     mbar_arrive(reinterpret_cast<uint64_t*>(&sh->s_ready));
                 }
             }
@@ -953,11 +1080,11 @@ __global__ void __launch_bounds__(kColThreads, 1) sgd_column_kernel(const Column
 // ---------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------
-template <bool TRACED>
+template <bool QV, bool TRACED>
 static const void* column_kernel_ptr(int cb) {
-    if (cb == 2) return reinterpret_cast<const void*>(&sgd_column_kernel<2, TRACED>);
-    if (cb == 4) return reinterpret_cast<const void*>(&sgd_column_kernel<4, TRACED>);
-    return reinterpret_cast<const void*>(&sgd_column_kernel<8, TRACED>);
+    if (cb == 2) return reinterpret_cast<const void*>(&sgd_column_kernel<2, QV, TRACED>);
+    if (cb == 4) return reinterpret_cast<const void*>(&sgd_column_kernel<4, QV, TRACED>);
+    return reinterpret_cast<const void*>(&sgd_column_kernel<8, QV, TRACED>);
 }
 
 // Tensor maps over the two planes as byte matrices: boxes of 128 bytes x R rows with the 128-byte swizzle,
@@ -996,9 +1123,10 @@ static int encode_column_maps(zipml_ctx* ctx, const zipml_dataset* d, int R, CUt
 }
 
 int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,
-                      int64_t first_step, int64_t num_steps, float* grad_out) {
+                      int64_t first_step, int64_t num_steps, float* grad_out, bool quantized_vectors) {
     if (!ctx->cooperative) return ZIPML_ERR_WORKSPACE;
-    if (d->level_mode != ZIPML_LEVELS_UNIFORM || p->model_bits != 0 || p->grad_bits != 0 || p->model_out) return ZIPML_ERR_WORKSPACE;
+    const bool qv = p->model_bits != 0 || p->grad_bits != 0;
+    if (d->level_mode != ZIPML_LEVELS_UNIFORM || (qv && !quantized_vectors) || p->model_out) return ZIPML_ERR_WORKSPACE;
     if (d->m > 0x7fffffffLL || d->row_bytes < kColBlockBytes) return ZIPML_ERR_WORKSPACE;
     if ((d->row_bytes + kColBlockBytes - 1) / kColBlockBytes * d->m > 0x7fffffffLL) return ZIPML_ERR_WORKSPACE;     // (32-bit copy coordinates)
     const int cb = container_bits(d->bits);
@@ -1046,7 +1174,9 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     if (nch_max > 1) slots_a = slots_a / stride * stride;
     if (slots_a < 1 || slots_b < 1) return ZIPML_ERR_WORKSPACE;
     const size_t smem = fixed + (size_t)slots * slot_bytes;
-    const void* kernel = p->trace && p->trace_steps > 0 ? column_kernel_ptr<true>(cb) : column_kernel_ptr<false>(cb);
+    const bool traced = p->trace && p->trace_steps > 0;
+    const void* kernel = qv ? (traced ? column_kernel_ptr<true, true>(cb) : column_kernel_ptr<true, false>(cb))
+                            : (traced ? column_kernel_ptr<false, true>(cb) : column_kernel_ptr<false, false>(cb));
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_status(e);
     int per_sm = 0;
@@ -1061,6 +1191,7 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     size_t off = 0;
     auto piece = [&](size_t bytes) { const size_t o = off; off += carve_size(bytes); return o; };
     const size_t o_dots = piece(sizeof(long long) * 3 * 2 * (size_t)bpad * ngrp);
+    const size_t o_norms = piece(qv ? sizeof(unsigned long long) * 2 * 2 * (size_t)G * (size_t)G * 2 : 0);
     const size_t zero_bytes = off;
     const size_t o_ord = piece(sizeof(int32_t) * (size_t)(p->batch_order ? T : 0));
     rc = ws_reserve(ctx, off);
@@ -1073,6 +1204,8 @@ int launch_sgd_column(zipml_ctx* ctx, const zipml_dataset* d, const float* b, fl
     a.ngrp = ngrp; a.gsize = gsize; a.blocked = d->layout == ZIPML_LAYOUT_COLUMN_BLOCKS;
     a.lr = p->lr; a.reg = p->reg; a.reg_cst = reg_constant(p);
     a.dots = reinterpret_cast<long long*>(ctx->ws + o_dots);
+    a.model_bits = p->model_bits; a.grad_bits = p->grad_bits; a.seed = p->seed; a.epoch = (uint32_t)p->epoch;
+    a.norms = reinterpret_cast<unsigned long long*>(ctx->ws + o_norms);
     a.status = ctx->d_status;
     a.trace = reinterpret_cast<unsigned long long*>(p->trace);
     a.trace_steps = p->trace ? p->trace_steps : 0;

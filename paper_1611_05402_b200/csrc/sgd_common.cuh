@@ -129,12 +129,14 @@ struct VecQuant {
     uint64_t seed;
     uint32_t epoch, step, stream;
     __device__ __forceinline__ float apply(float v, uint32_t coord) const {
+        return apply_drawn(v, vector_u24(seed, epoch, step, coord, stream));
+    }
+    __device__ __forceinline__ float apply_drawn(float v, uint32_t u) const {
         if (!(M > 0.0f)) return 0.0f;
         const float t = __fmul_rn(__fdiv_rn(fabsf(v), M), (float)sm);
         float fl = floorf(t);
         fl = fl > (float)(sm - 1) ? (float)(sm - 1) : fl;
         const float p = __fsub_rn(t, fl);
-        const uint32_t u = vector_u24(seed, epoch, step, coord, stream);
         const uint32_t mag = (uint32_t)fl + ((__fmul_rn((float)u, 5.9604644775390625e-08f) < p) ? 1u : 0u);
         const float q = __fmul_rn(M, __fdiv_rn((float)mag, (float)sm));
         return v < 0.0f ? -q : q;

@@ -763,6 +763,36 @@ def test_column_engine_rings_of_any_size(ctx, chunk, ring_b):
     assert rel(x.cpu().numpy(), x_ref) <= MODEL_TOL and rel(g.cpu().numpy()[0], g_ref[0]) <= GRAD_TOL
 
 
+@pytest.mark.parametrize("m,n,bits,batch,model_bits,grad_bits,reg", [
+    (700, 9001, 4, 150, 8, 8, 0), (130, 16_383, 4, 16, 0, 8, 1), (600, 9403, 2, 130, 4, 6, 3), (500, 8500, 8, 97, 8, 0, 4), (300, 18_944, 5, 100, 2, 2, 2),
+], ids=str)
+def test_column_engine_with_quantized_model_and_gradient(ctx, m, n, bits, batch, model_bits, grad_bits, reg):
+    """Q3 and Q4 on rows wider than a cluster: the norms of both vectors are sums over the CTAs."""
+    _, A, b, _ = workload("c2", m, n, seed=bits)
+    ods = oracle.quantize(A, bits, seed=4)
+    gds, db = dev_dataset(ods, ctx), to_dev(b, ctx)
+    x0 = (np.random.default_rng(5).standard_normal(n) * 0.02).astype(np.float32)
+    kw = dict(model_bits=model_bits, grad_bits=grad_bits, seed=21, epoch=1, reg=reg, reg_param=1e-3 if reg else 0.0)
+    lr = 0.1 / n
+    x, g = to_dev(x0, ctx), torch.zeros((2, n), dtype=torch.float32, device=ctx.device)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, grad_out=g, **kw)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_kernel() == "sgd_column_kernel"
+    x_ref, g_ref = oracle.sgd_epoch(ods, b, x0, batch, lr, want_grad=True, **kw)
+    # (a last-bit difference in a norm may flip a draw that sits on its threshold, by one unit of one coordinate)
+    assert rel(x.cpu().numpy(), x_ref) <= 20 * MODEL_TOL
+    # without Q3, whose flips would move the later steps: the last gradient before Q4, and its quantization but for such flips
+    x, one = to_dev(x0, ctx), dict(kw, model_bits=0) if grad_bits else kw
+    ctx.zipml_sgd_epoch(gds, db, x, batch, lr, grad_out=g, **one)
+    ctx.zipml_sync()
+    x_ref, g_ref = oracle.sgd_epoch(ods, b, x0, batch, lr, want_grad=True, **one)
+    gg = g.cpu().numpy()
+    assert rel(gg[0], g_ref[0]) <= 20 * GRAD_TOL
+    if grad_bits:
+        unit = np.linalg.norm(g_ref[0]) / ((1 << (grad_bits - 1)) - 1)
+        assert (np.abs(gg[1] - g_ref[1]) > 0.5 * unit).sum() <= 3
+
+
 def test_column_engine_limits(ctx):
     """Rows narrower than one column block, rows wider than one block per SM and batches above 8,192 are declined."""
     _, A, b, _ = workload("c1", 200, 64, seed=1)
