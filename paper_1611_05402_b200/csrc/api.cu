@@ -320,6 +320,36 @@ static bool lean_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t
     return B * d->n <= most;
 }
 
+// Level tables of up to 3,000 features, past what the cluster engine takes by features: its form by rows, whose sixteen CTAs walk
+// through the batch, row parts that meet through L2 (lean), the persistent grid with 148 CTAs, or the ring engine.
+//   2 bits, fp32 vectors: n 16 to 256 x 1,024 K 11.4 L 9.9 G 18, x 4,096 28.6 / 20.4 / 25, x 8,192 51.5 / 34.5 / 31.5 (R 41), x 16,384 97.5 / 62 / 43
+//   (R 69); n 512 x 4,096 28.8 / 22.1 / 24, x 16,384 G 37.6 R 69; n 1,400 x 2,048 L 28.6 G 24.7; n 2,000 x 8,192 G 53 R 120.
+//   3 and 4 bits: n 16 to 40 x 1,024 K 9.1 L 8.7 G 17, x 4,096 20.5 / 16.6 / 22 (R 18), x 8,192 35.5 / 27 / 26, x 16,384 65.5 / 48 / 36 (R 43); 3 bits
+//   n 256 x 4,096 20.3 / 18.1 / 20.5; n 512 x 16,384 (8 MB) G 35 R 67; n 1,400 x 8,192 (11 MB) G 46 R 61; n 1,024 x 16,384 (16 MB) G 81 R 66; 4 bits n
+//   512 x 16,384 (8 MB) G 37.5 R 69; n 700 x 8,192 (6 MB) 37 / 41; n 1,400 x 4,096 (6 MB) 32 / 28.  Past 4 MB and
+//   500 features the lean engine again, where it holds the rows: 3 bits n 700 x 16,384 L 38 G 51, n 1,400 x 6,000 31 / 39; 4 bits n 512 x 16,384 31 / 37;
+//   2 bits n 2,000 x 8,192 39 / 53.
+//   Both vectors of 8 bits (a norm is dear on the lean engine beyond 64 features): 2 bits n 16 x 1,024 K 13.9 L 13.5 G 22, x 4,096 31 / 24 / 29, x
+//   8,192 54 / 38.5 / 35.6; n 256 x 2,048 19.8 / 22.5 / 24.6, x 4,096 31.4 / 30 / 27.7, x 16,384 L 73 G 46 R 75; n 1,024 x 16,384 L 67 G 55 R 132;
+//   n 2,000 x 4,096 L 47.5 G 57.6 R 77.  3 bits n 40 x 2,048 K 15.3 L 15.2, x 4,096 22.6 / 20.7 / 23.2, x 6,000 30 / 29.6 / 25.5; n 256 x 4,096 K 23 G 22.5; n 700 x 2,048 L 24.4 G 27.4
+//   R 28, x 8,192 46 / 39 / 64; n 1,024 x 8,192 58 / 40 / 73; n 1,400 x 4,096 49 / 48 / 46.  4 bits n 700 x 8,192 45 / 42 / 49; n 1,400 x 1,024 31 / 41 / 29.
+// `lean_fits`: false once the lean engine has declined.
+static int table_engine(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t step_bytes, bool lean_fits) {
+    const bool quantized = p->model_bits != 0 || p->grad_bits != 0, two = container_bits(d->bits) == 2;
+    const int64_t n = d->n;
+    constexpr int64_t MB = 1 << 20;
+    if (!quantized) {
+        if (B < (two ? 800 : n <= 64 ? 1100 : 1600)) return ZIPML_ENGINE_CLUSTER;
+        if (lean_fits && B <= (two ? 7000 : 6500) && lean_pays(d, p, B)) return ZIPML_ENGINE_LEAN;
+        if (lean_fits && (two ? n >= 1000 && step_bytes > 5 * MB : n >= 500 && step_bytes > 4 * MB)) return ZIPML_ENGINE_LEAN;
+        return step_bytes <= (two ? 10 : d->bits == 3 ? 11 : n <= 800 ? 8 : 3) * MB ? ZIPML_ENGINE_PERSISTENT : ZIPML_ENGINE_RING;
+    }
+    if (n <= 64) return B < (two ? 1000 : 3500) ? ZIPML_ENGINE_CLUSTER : B <= 5000 ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_PERSISTENT;
+    if (B <= (two || n >= 400 ? 2500 : 4096) && step_bytes <= 2 * MB) return ZIPML_ENGINE_CLUSTER;
+    if (n <= (two || d->bits == 3 ? 1100 : 800) && step_bytes <= (d->bits == 4 ? 8 : 10) * MB) return ZIPML_ENGINE_PERSISTENT;
+    return lean_fits && two && step_bytes <= 10 * MB ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_RING;
+}
+
 // Uniform rows too wide for the column and stream engines: the persistent grid up to 16 MB a step, 4 bits n 100,000 x 64 G 23 R 42, x 300
 // (30 MB) 107 / 53; 8 bits n 150,000 x 64 (19 MB) 60 / 71, x 300 243 / 138.
 // Level tables wider than a cluster holds: the persistent grid too, whose CTAs take row parts of a few columns and so build few of the
@@ -386,14 +416,27 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_solo(ctx, data, b, x, params, first, count, grad_out, true);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
+        int table = 0;
+        if (data->level_mode == ZIPML_LEVELS_TABLE && data->n < 3000 && params->cluster_contraction == 0) {
+            if (small && table_form_pays(data, params)) {
+                rc = launch_sgd_table(ctx, data, b, x, params, first, count, grad_out);
+                if (rc != ZIPML_ERR_WORKSPACE) return rc;
+            }
+            table = table_engine(data, params, B, step_bytes, true);
+            if (table == ZIPML_ENGINE_LEAN) {
+                rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
+                if (rc != ZIPML_ERR_WORKSPACE) return rc;
+                table = table_engine(data, params, B, step_bytes, false);
+            }
+        }
         if (data->level_mode == ZIPML_LEVELS_UNIFORM && params->cluster_contraction != 1) {
             rc = launch_sgd_int8(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
-        } else if (small) {
+        } else if (small && (table == 0 || table == ZIPML_ENGINE_CLUSTER)) {
             rc = launch_sgd_cluster(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        if (small && lean_pays(data, params, B)) {
+        if (small && (table == 0 || table == ZIPML_ENGINE_CLUSTER) && lean_pays(data, params, B)) {
             rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
@@ -409,7 +452,7 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_stream(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        if (grid_pays(data, params, step_bytes, wide)) {
+        if (table == ZIPML_ENGINE_PERSISTENT || (table != ZIPML_ENGINE_RING && grid_pays(data, params, step_bytes, wide))) {
             zipml_sgd_params grid = *params;
             grid.engine = ZIPML_ENGINE_PERSISTENT;
             rc = launch_sgd_epoch(ctx, data, b, x, &grid, first, count, grad_out);

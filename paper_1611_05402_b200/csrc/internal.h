@@ -121,7 +121,8 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
                        int64_t num_steps, float* grad_out);
 int launch_sgd_int8(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                     int64_t num_steps, float* grad_out);
-// The form on level tables.
+// The form on level tables, and whether it is the faster one against the form split by rows.
+bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p);
 int launch_sgd_table(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,
                      int64_t num_steps, float* grad_out);
 int launch_sgd_cluster(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p,

@@ -589,7 +589,7 @@ static int make_cluster_plan(const zipml_ctx* ctx, const zipml_dataset* d, const
 // 4.18, n 64 x 420 4.85 / 4.98, x 500 5.25 / 5.18, n 96 x 800 6.59 / 6.67; 2 bits n 33 to 64 (1) x 180 4.23 / 4.29, x 240 4.98 / 4.55, n 100 (2) x 500
 // 6.04 / 6.11, x 600 7.40 / 7.00, n 190 (3) x 800 8.10 / 8.34; n 1,019 (16) x 1,024 7.5 / 14.3.  With a quantized vector the features do a little
 // longer: 3 bits n 64 x 600 8.30 / 8.43, 4 bits x 500 7.35 / 7.57.
-static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
+bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
     const int64_t B = p->batch < d->m ? p->batch : d->m, units = (d->n * container_bits(d->bits) + 127) / 128;
     if (container_bits(d->bits) == 2) return B <= 240 * units - (units == 1 ? 55 : 0);
     return B <= 300 * units - (units == 1 || (units <= 3 && p->model_bits == 0 && p->grad_bits == 0) ? 100 : 0);
@@ -601,10 +601,9 @@ static bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
 // 7.06 / 5.99; 2 bits n 256 x 128 3.04 / 2.83, n 1,000 x 64 2.82 / 3.33, x 512 4.05 / 4.58, x 4,096 8.04 / 7.66.
 static bool features_pay(const zipml_dataset* d, const zipml_sgd_params* p) {
     const int64_t B = p->batch < d->m ? p->batch : d->m;
-    // From 2^24 entries a step a quantized vector leaves this form: wide rows then go to the ring engine, a pinned choice, and rows that
-    // the form by rows holds go there.  Not the faster side at 2 bits 4,096 x 4,096 (features 13.8, rows 22.9, ring 43.5); longer batches
-    // this form does not hold anyway (4 bits 2,048 x 8,192 rows 20.1, ring 45.9).
-    if ((p->model_bits > 0 || p->grad_bits > 0) && B * d->n >= 1 << 24) return false;
+    // (From 2^24 entries a step a quantized vector whose model is asked for leaves this form, and wide rows then go to the ring engine: a
+    // pinned choice, not the faster.  2 bits 4,096 x 4,096 features 13.8, rows 22.9, ring 43.5.)
+    if ((p->model_bits > 0 || p->grad_bits > 0) && p->model_out && B * d->n >= 1 << 24) return false;
     return d->n >= (container_bits(d->bits) == 2 ? 900 : 480) && B <= 5 * d->n;
 }
 int launch_sgd_int8(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,

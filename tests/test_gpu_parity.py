@@ -1056,6 +1056,26 @@ def test_auto_on_level_tables(ctx, m, n, bits, batch, kernel):
     assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
 
 
+@pytest.mark.parametrize("m,n,bits,batch,quantized,kernel", [
+    (1700, 19, 2, 790, False, "sgd_cluster_kernel"), (1700, 19, 2, 800, False, "sgd_lean_kernel"), (7100, 19, 2, 7001, False, "sgd_kernel"),
+    (3300, 90, 3, 1600, False, "sgd_lean_kernel"), (6600, 90, 4, 6501, False, "sgd_kernel"), (3600, 33, 4, 3500, True, "sgd_lean_kernel"),
+    (5100, 33, 3, 5001, True, "sgd_kernel"), (2600, 130, 2, 2501, True, "sgd_kernel"), (4200, 130, 3, 4097, True, "sgd_kernel"),
+    (2600, 1200, 2, 2501, True, "sgd_lean_kernel"), (7400, 570, 4, 7400, False, "sgd_lean_kernel"),
+], ids=str)
+def test_auto_on_level_tables_with_long_batches(ctx, m, n, bits, batch, quantized, kernel):
+    """Either side of the lines for batches past what the cluster engine takes by features."""
+    _, A, b, _ = workload("c4", m, n, seed=4)
+    ods = oracle.quantize(A, bits, seed=3, mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 32)[0])
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    kw = dict(model_bits=8, grad_bits=8, seed=3) if quantized else {}
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-3, **kw)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-3, **kw)
+    ctx.zipml_sync()
+    # (a last-bit difference in a norm may flip a draw that sits on its threshold, by one unit of one coordinate)
+    assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= (20 if quantized else 1) * MODEL_TOL
+
+
 REGS = [(binding.REG_L2, 0.5), (binding.REG_L1, 0.02), (binding.REG_NONNEG, 0.0), (binding.REG_LSSVM, 0.5)]
 
 
