@@ -257,16 +257,28 @@ __global__ void __launch_bounds__(1024) loss_digits_kernel(const float* __restri
 }
 
 constexpr int64_t kLossFlushSpans = 512;
+constexpr int kLossStages = 4;
 
-template <int CB>
+// 16 bytes from global to shared memory, zeros where `bytes` is 0.
+__device__ __forceinline__ void loss_copy16(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
+// SHARED: a warp's spans, 16 rows after 16 rows, as one sequence that runs kLossStages - 1 spans ahead of the arithmetic: every lane copies the 64 bytes
+// it will use into its own places of a stage (nobody else reads them: no barrier) and asks for the next as soon as it has
+// taken one.  The digits lie in shared memory: [group][digit], `digit_pitch` bytes apart, 64 past a multiple of 128, so that two digits'
+// lanes meet different banks.  Not SHARED: for digits that find no room or blocks that use them too little: from global memory to registers, four spans at a
+// time, and the digits with them (through stages without them in shared memory 20 to 40 % slower on few rows of 30,000 codes).
+template <int CB, bool SHARED>
 __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned char* __restrict__ p1, const unsigned char* __restrict__ p2,
                                                               int64_t row_bytes, int64_t m, int64_t vec_bytes, int kp_shift,
                                                               const signed char* __restrict__ wdig, const double* __restrict__ base_in,
                                                               const float* __restrict__ b, double* __restrict__ partials, unsigned* __restrict__ ticket,
                                                               double scale, double* __restrict__ out) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
+    extern __shared__ uint4 loss_smem[];                          // SHARED: [warps][kLossStages][4][32], then the digits
     __shared__ double red[40];
-    __shared__ double parts[16][32];
+    __shared__ double parts[2][16][32];                           // two turns' in turn
     __shared__ bool last;
     const int lane = threadIdx.x & 31, gl = lane >> 2, tl = lane & 3, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int kp = 1 << kp_shift, part = warp & (kp - 1);
@@ -275,24 +287,71 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
     const int64_t nblocks = (m + 15) / 16;
     const int64_t nspans = (row_bytes + 63) / 64;
     const int64_t span0 = (nspans * part) >> kp_shift, span1 = (nspans * (part + 1)) >> kp_shift;
+    uint4* stages = loss_smem + warp * kLossStages * 128 + lane;
+    const int digit_pitch = SHARED ? (int)((vec_bytes + 127) / 128 * 128 + 64) : 0;
+    unsigned char* digits = reinterpret_cast<unsigned char*>(loss_smem + warps * kLossStages * 128);
+    if constexpr (SHARED) {
+        const int pieces = (int)(vec_bytes / 16);
+        for (int i = threadIdx.x; i < NG * NS * pieces; i += blockDim.x) {
+            const int v = i / pieces, k = i - v * pieces;
+            *reinterpret_cast<uint4*>(digits + v * digit_pitch + 16 * k) = __ldg(reinterpret_cast<const uint4*>(wdig + v * vec_bytes) + k);
+        }
+        __syncthreads();
+    }
+    // the span that is asked for next
+    int64_t ask_blk = first, ask_sp = span0;
+    const unsigned char *a1, *h1, *a2, *h2;
+    auto rows_of = [&]() {
+        const int64_t ra = min(ask_blk * 16 + gl, m - 1), rh = min(ask_blk * 16 + gl + 8, m - 1);
+        a1 = p1 + ra * row_bytes + 16 * tl; h1 = p1 + rh * row_bytes + 16 * tl;
+        a2 = p2 + ra * row_bytes + 16 * tl; h2 = p2 + rh * row_bytes + 16 * tl;
+    };
+    rows_of();
+    const int64_t jump = more * 16 * row_bytes;
+    auto ask = [&](int stage) {
+        if (ask_blk < nblocks && ask_sp < span1) {
+            const int64_t off = ask_sp * 64;
+            const bool have = off + 16 * tl < row_bytes;          // rows are whole multiples of 16 bytes
+            const uint32_t bytes = have ? 16u : 0u;
+            uint4* dst = stages + stage * 128;
+            loss_copy16(dst, have ? a1 + off : p1, bytes);
+            loss_copy16(dst + 32, have ? h1 + off : p1, bytes);
+            loss_copy16(dst + 64, have ? a2 + off : p2, bytes);
+            loss_copy16(dst + 96, have ? h2 + off : p2, bytes);
+            if (++ask_sp == span1) {
+                ask_sp = span0;
+                ask_blk += more;
+                if (ask_blk * 16 + 16 <= m) { a1 += jump; h1 += jump; a2 += jump; h2 += jump; }
+                else rows_of();
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int stage = 0;
+    if constexpr (SHARED)
+#pragma unroll
+        for (int k = 0; k < kLossStages - 1; ++k) ask(k);
     double total = 0.0;
-    for (int64_t blk = first; blk < nblocks || kp > 1; blk += more) {      // (shared rows: one turn, for all warps)
-        const int64_t ra = min(blk * 16 + gl, m - 1), rh = min(blk * 16 + gl + 8, m - 1);
-        const unsigned char* a1 = p1 + ra * row_bytes + 16 * tl;
-        const unsigned char* h1 = p1 + rh * row_bytes + 16 * tl;
-        const unsigned char* a2 = p2 + ra * row_bytes + 16 * tl;
-        const unsigned char* h2 = p2 + rh * row_bytes + 16 * tl;
+    int turn = 0;
+    // (kp > 1: a block is one group of warps, which take every turn together)
+    for (int64_t blk = first; blk < nblocks; blk += more, turn ^= 1) {
         // A span adds at most 64 * 128 * 255 to a 32-bit digit sum: they are moved into 64-bit sums every
         // kLossFlushSpans spans (2^21 * 512 < 2^31), so rows of any admitted length stay exact.
         long long s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0};
         for (int64_t sp0 = span0; sp0 < span1; sp0 += kLossFlushSpans) {
         int c1[4] = {0, 0, 0, 0}, c2[4] = {0, 0, 0, 0};
         const int64_t sp1 = min(span1, sp0 + kLossFlushSpans);
-#pragma unroll 4
+#pragma unroll (SHARED ? 2 : 4)
         for (int64_t sp = sp0; sp < sp1; ++sp) {
             const int64_t off = sp * 64;
             uint4 ua = make_uint4(0u, 0u, 0u, 0u), uh = ua, va = ua, vh = ua;
-            if (off + 16 * tl < row_bytes) {                      // rows are whole multiples of 16 bytes
+            if constexpr (SHARED) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kLossStages - 2) : "memory");
+                const uint4* src = stages + stage * 128;
+                ua = src[0]; uh = src[32]; va = src[64]; vh = src[96];
+                ask((stage + kLossStages - 1) % kLossStages);
+                stage = (stage + 1) % kLossStages;
+            } else if (off + 16 * tl < row_bytes) {
                 ua = __ldcs(reinterpret_cast<const uint4*>(a1 + off));
                 uh = __ldcs(reinterpret_cast<const uint4*>(h1 + off));
                 va = __ldcs(reinterpret_cast<const uint4*>(a2 + off));
@@ -301,7 +360,9 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
                 uint4 bd = make_uint4(0u, 0u, 0u, 0u);            // digit gl of this lane's 16 bytes
-                if (gl < NS) bd = __ldg(reinterpret_cast<const uint4*>(wdig + ((int64_t)g * NS + gl) * vec_bytes + off + 16 * tl));
+                if (gl < NS)
+                    bd = SHARED ? *reinterpret_cast<const uint4*>(digits + (g * NS + gl) * digit_pitch + (int)off + 16 * tl)
+                                : __ldg(reinterpret_cast<const uint4*>(wdig + ((int64_t)g * NS + gl) * vec_bytes + off + 16 * tl));
                 mma_u8s8(c1, slice_dot_codes<CB>(ua.x, g), slice_dot_codes<CB>(uh.x, g), slice_dot_codes<CB>(ua.y, g), slice_dot_codes<CB>(uh.y, g), bd.x, bd.y);
                 mma_u8s8(c1, slice_dot_codes<CB>(ua.z, g), slice_dot_codes<CB>(uh.z, g), slice_dot_codes<CB>(ua.w, g), slice_dot_codes<CB>(uh.w, g), bd.z, bd.w);
                 mma_u8s8(c2, slice_dot_codes<CB>(va.x, g), slice_dot_codes<CB>(vh.x, g), slice_dot_codes<CB>(va.y, g), slice_dot_codes<CB>(vh.y, g), bd.x, bd.y);
@@ -311,6 +372,7 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
 #pragma unroll
         for (int e = 0; e < 4; ++e) { s1[e] += c1[e]; s2[e] += c2[e]; }
         }
+        if constexpr (!SHARED) { ask_blk += more; rows_of(); }
         // lane t < 2 holds digits 2t, 2t+1 of rows g (s[0], s[1]) and g+8 (s[2], s[3])
         double v[4];
 #pragma unroll
@@ -323,11 +385,12 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
         if (kp > 1) {
             if (tl == 0)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) parts[warp][gl * 4 + e] = v[e];
+                for (int e = 0; e < 4; ++e) parts[turn][warp][gl * 4 + e] = v[e];
             __syncthreads();
-            for (int w = 1; w < kp; ++w)
+            if (part == 0 && tl == 0)
+                for (int w = 1; w < kp; ++w)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] += part == 0 && tl == 0 ? parts[warp + w][gl * 4 + e] : 0.0;
+                    for (int e = 0; e < 4; ++e) v[e] += parts[turn][w][gl * 4 + e];
         }
         if (tl == 0 && part == 0) {
 #pragma unroll
@@ -339,7 +402,6 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
                 }
             }
         }
-        if (kp > 1) break;
     }
     total = block_sum(total, red);
     if (threadIdx.x == 0) {
@@ -377,29 +439,52 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
         const int64_t vec_bytes = (d->row_bytes + 63) / 64 * 64;
         signed char* wdig = reinterpret_cast<signed char*>(wtab);
         unsigned* ticket = reinterpret_cast<unsigned*>(wdig + (8 / cb) * 4 * vec_bytes);
-        // 16 warps per SM, 16 rows per warp and turn (four spans in flight take 128 registers a thread); with fewer rows smaller
-        // blocks, so that every SM has some, and where there are not rows for two warps of all schedulers several to 16 rows.
-        // Measured, us: 2 bits 1,000,000 x 2,048 253 with shifted codes and two spans -> 225 (4.7 TB/s), 4 bits
-        // 1,000,000 x 1,000 270 -> 185 (5.5 TB/s), 8 bits 300,000 x 2,000 264 -> 257; few rows: 4 bits 3,997 x 6,576 99 -> 29, 245 x
-        // 2,710 42 -> 26, 2 bits 8,000 x 32,000 176 -> 63.  Bound by the bytes in flight: of the cycles between
-        // two instructions of a warp its loads take 6.1 of 11.6 at 2 bits (the masks keep the ALU pipe 48 % busy), 11.6 of 17.1 at 4
-        // and 23.8 of 28.4 at 8; the digits, which every warp reads again, are half of the sectors that L2 serves.
+        // 16 warps per SM, 16 rows per warp and turn, or kp warps to 16 rows, each a part of the spans: as many as make the turns, each its spans
+        // and about two more for what it ends with, take least -- few rows would leave warps without any, long rows the last turn
+        // nearly empty.  Blocks are 16 warps (kp = 1) or one such group.
+        // Measured with L2 flushed, us, as many warps to 16 rows as fill half the chip -> this: 8 bits 20,000 x 20,000 468 -> 185,
+        // 40,000 x 20,000 558 -> 322, 30,000 x 9,000 241 -> 146, 4 bits 60,000 x 12,000 204 -> 191; in L2: 8 bits 2,797 x 1,500 18 -> 14.
         const int64_t turns = (d->m + 15) / 16, spans = vec_bytes / 64;
-        int warps = (int)(turns / ctx->sm_count), kp = 1, kp_shift = 0;
-        warps = warps > 16 ? 16 : warps < 1 ? 1 : warps;
-        while (kp < 16 && turns * kp < 8ll * ctx->sm_count && 2 * kp <= spans) { kp *= 2; ++kp_shift; }
-        if (kp > 1) warps = kp;
+        int kp_shift = 0;
+        int64_t least = INT64_MAX;
+        for (int k = 0; k <= 4 && (k == 0 || (2ll << k) <= spans); ++k) {
+            const int64_t groups = (int64_t)ctx->sm_count * 16 >> k, time = ((turns + groups - 1) / groups) * (((spans + (1 << k) - 1) >> k) + (k ? 2 : 1));
+            if (time < least) { least = time; kp_shift = k; }
+        }
+        const int kp = 1 << kp_shift;
+        int warps = kp;
+        if (kp == 1) {                                            // (fewer rows than warps: smaller blocks, on every SM)
+            const int64_t per_sm = turns / ctx->sm_count;
+            warps = per_sm > 16 ? 16 : per_sm < 1 ? 1 : (int)per_sm;
+        }
         int64_t blocks = kp > 1 ? turns : (turns + warps - 1) / warps;
-        if (kp == 1 && blocks > ctx->sm_count) blocks = ctx->sm_count;
+        const int64_t most = kp > 1 ? (int64_t)ctx->sm_count * 16 / kp : ctx->sm_count;
+        if (blocks > most) blocks = most;
         if (blocks > max_partials) return ZIPML_ERR_WORKSPACE;
         const int64_t chunks = (vec_bytes * (8 / cb) + 1023) / 1024;
         const int digit_blocks = (int)(chunks > 16 ? 16 : chunks);
         const double scale = 1.0 / (2.0 * (double)d->m);
-#define ZIPML_LAUNCH_LI(CB_) \
-    loss_digits_kernel<CB_><<<digit_blocks, 1024, 0, ctx->stream>>>(d->feat_lo, d->feat_step, x, d->n, vec_bytes, wdig, base, ticket); \
-    loss_codes_imma_kernel<CB_><<<(int)blocks, 32 * warps, 0, ctx->stream>>>(d->plane1, d->plane2, d->row_bytes, d->m, vec_bytes, kp_shift, wdig, base, b, partials, ticket, scale, loss_out)
-        if (cb == 2) { ZIPML_LAUNCH_LI(2); } else if (cb == 4) { ZIPML_LAUNCH_LI(4); } else { ZIPML_LAUNCH_LI(8); }
-#undef ZIPML_LAUNCH_LI
+        // Stages (see the kernel) where 16 warps share the digits and these fit.  Measured with L2 flushed, us, straight to registers -> stages: 2 bits
+        // 1,000,000 x 2,048 236 -> 198 (5.2 TB/s), 4 bits 1,000,000 x 1,000 206 -> 197, 8 bits 300,000 x 2,000 279 -> 259; rows of one span (20 codes of 4 bits,
+        // 13,421,773 rows) 495 -> 414.  Rows of two to five spans keep to registers, where one row's spans are all in flight at once (8 bits 1,342,178
+        // x 200 120 us against 134, 335,545 x 200 40 against 48), and so do warps of about a hundred spans in all, whose start counts: 8 bits 100,000 x 2,100
+        // (102 as counted above) 109 against 113, 4 bits 60,000 x 1,500 (26) 42 against 44; 5 bits 400,000 x 999 (121) 191 against 179.
+        const size_t ring = (size_t)warps * kLossStages * 2048, digit_bytes = (size_t)(8 / cb) * 4 * ((size_t)(vec_bytes + 127) / 128 * 128 + 64);
+        const bool shared = warps == 16 && (spans == 1 || (spans > 5 && least >= 112)) && ring + digit_bytes + 16384 <= (size_t)ctx->smem_optin;
+        const size_t smem = shared ? ring + digit_bytes : 0;
+        auto launch = [&](auto digits_kernel, auto kernel) -> int {
+            const cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+            if (e != cudaSuccess) return cuda_status(e);
+            digits_kernel<<<digit_blocks, 1024, 0, ctx->stream>>>(d->feat_lo, d->feat_step, x, d->n, vec_bytes, wdig, base, ticket);
+            kernel<<<(int)blocks, 32 * warps, smem, ctx->stream>>>(d->plane1, d->plane2, d->row_bytes, d->m, vec_bytes, kp_shift, wdig, base, b, partials,
+                                                                   ticket, scale, loss_out);
+            return ZIPML_OK;
+        };
+        const int rc = cb == 2   ? shared ? launch(loss_digits_kernel<2>, loss_codes_imma_kernel<2, true>) : launch(loss_digits_kernel<2>, loss_codes_imma_kernel<2, false>)
+                       : cb == 4 ? shared ? launch(loss_digits_kernel<4>, loss_codes_imma_kernel<4, true>) : launch(loss_digits_kernel<4>, loss_codes_imma_kernel<4, false>)
+                       : shared  ? launch(loss_digits_kernel<8>, loss_codes_imma_kernel<8, true>)
+                                 : launch(loss_digits_kernel<8>, loss_codes_imma_kernel<8, false>);
+        if (rc != ZIPML_OK) return rc;
         ctx->launches += 2;
         return cuda_status(cudaGetLastError());
     }

@@ -1168,6 +1168,23 @@ def test_loss_codes_with_few_and_many_rows(ctx, m, n, bits):
     assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
 
 
+@pytest.mark.parametrize("m,n,bits", [(40_005, 20, 4), (40_003, 200, 8), (38_001, 390, 8), (39_990, 900, 8), (266_000, 390, 8), (2_300, 2_100, 8), (4_790, 4_000, 8), (1_500, 3_500, 2)],
+                         ids=str)
+def test_loss_codes_through_stages_and_without(ctx, m, n, bits):
+    """Rows of one span, of four (no stages) and of seven, few turns of a warp (none) and many; two, eight and sixteen warps to 16 rows, one turn and three; a part
+    of the spans that has none in some warps; last rows and last spans that are cut off."""
+    _, A, b, xs = workload("c2", m, n, seed=2)
+    x = (xs * 0.9).astype(np.float32)
+    ods = oracle.quantize(A, bits, seed=3)
+    want = oracle.loss_codes(ods, b, x)
+    gds, db, dx = dev_dataset(ods, ctx), to_dev(b, ctx), to_dev(x, ctx)
+    got = ctx.zipml_loss(binding.LOSS_CODES, db, dx, data=gds)
+    again = ctx.zipml_loss(binding.LOSS_CODES, db, dx, data=gds)
+    ctx.zipml_sync()
+    assert got.item() == again.item()
+    assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
+
+
 def test_loss_codes_with_level_table_and_strided_dense(ctx):
     _, A, b, xs = workload("c4", 2000, 60, seed=1)
     lev, _ = oracle.optimal_levels(A, 3, 128)
