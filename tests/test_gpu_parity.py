@@ -1442,6 +1442,30 @@ def test_apply_gradient_is_the_end_of_a_step(ctx, grad_bits, reg, reg_param):
         ctx.zipml_sgd_apply_gradient(x, g, 0, lr, reg=1, reg_param=-1.0)
 
 
+@pytest.mark.parametrize("n,skip,bits,norm", [(1, 0, 8, 0), (3, 1, 4, 1), (127, 0, 2, 0), (2_048, 0, 8, 0), (2_049, 0, 8, 1), (4_099, 3, 6, 0), (16_384, 0, 0, 0),
+                                              (32_768, 0, 8, 0), (32_773, 0, 5, 1), (70_001, 2, 8, 0)], ids=str)
+def test_apply_gradient_of_any_size(ctx, n, skip, bits, norm):
+    """One CTA, a cluster of them, more coordinates than the cluster's threads hold; last quadruples that are cut off and vectors that do not start on 16 bytes."""
+    rng = np.random.default_rng(n)
+    x0, g0 = rng.standard_normal(n).astype(np.float32), rng.standard_normal(n).astype(np.float32)
+    room = torch.zeros((3, n + skip + 8), dtype=torch.float32, device=ctx.device)
+    x, g, applied = (room[k].reshape(-1)[skip:skip + n] for k in range(3))
+    x.copy_(to_dev(x0, ctx)); g.copy_(to_dev(g0, ctx))
+    ctx.zipml_sgd_apply_gradient(x, g, 7, 0.1, applied_out=applied, grad_bits=bits, seed=11, epoch=2, vector_norm=norm)
+    ctx.zipml_sync()
+    app = applied.cpu().numpy()
+    want = oracle.quantize_vector(g0, bits, 11, 2, 7, 4, norm=norm)[0] if bits else g0
+    if bits:                                                       # (a last-bit difference in the norm may flip a rounding, as above)
+        unit = (np.abs(g0).max() if norm else np.linalg.norm(g0.astype(np.float64))) / ((1 << (bits - 1)) - 1)
+        flips = np.abs(app - want) > 0.5 * unit
+        assert flips.sum() <= 2 and np.abs(app - want)[~flips].max() <= 1e-5 * unit
+    else:
+        assert (app == want).all()
+    exact = x0.astype(np.float64) - np.float64(np.float32(0.1)) * app          # one rounding: half a unit of the last place, and the double's
+    assert (np.abs(x.cpu().numpy() - exact) <= 0.51 * np.spacing(np.abs(exact).astype(np.float32))).all()
+    assert (room[:, n + skip:] == 0).all() and (room[:, :skip] == 0).all()     # nothing beside the vectors
+
+
 @pytest.mark.parametrize("world", [1, 2, 4])
 @pytest.mark.parametrize("case", ["plain_ragged", "q3_q4_shuffled", "wide_l2"])
 def test_row_sharded_epoch_matches_the_whole_epoch(ctx, world, case):
