@@ -28,6 +28,18 @@ static int grow(unsigned char** buf, size_t* have, size_t want, cudaStream_t str
 int ws_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->ws, &ctx->ws_bytes, bytes, ctx->stream); }
 int stage_reserve(zipml_ctx* ctx, size_t bytes) { return grow(&ctx->stage, &ctx->stage_bytes, bytes, ctx->stream); }
 
+bool early_start(zipml_ctx* ctx, int64_t steps, cudaLaunchAttribute* attr) {
+    if (steps > kEarlySteps) return false;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    return capture == cudaStreamCaptureStatusNone;
+}
+
 int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag) {
     if (bytes > kExchangeBytes) return ZIPML_ERR_WORKSPACE;
     // Tags go up from launch to launch, so the buffer is cleared only before they would wrap.  A launch that is recorded into a

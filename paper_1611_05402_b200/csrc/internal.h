@@ -50,6 +50,12 @@ int stage_reserve(zipml_ctx* ctx, size_t bytes);
 constexpr size_t kExchangeBytes = 2 * 8 * (8192 + 1024) * 16;
 int exchange_tags(zipml_ctx* ctx, size_t bytes, int64_t steps, unsigned long long** buffer, uint32_t* tag);
 
+// Fills the attribute that lets a kernel of so few steps start while the one before it on the stream ends (it waits for that one's end: see
+// after_previous_kernel).  False for longer ones, which would keep multiprocessors from other streams while they wait, and while the
+// stream is being captured, where a launch stays an ordinary one.
+constexpr int64_t kEarlySteps = 4;
+bool early_start(zipml_ctx* ctx, int64_t steps, cudaLaunchAttribute* attr);
+
 // Columns that a range pass takes per launch, and the column tiles of one: at least 256 columns each where there are several.
 constexpr int64_t kRangeColumns = 65536;
 constexpr int64_t kRangeTiles = kRangeColumns / 256;

@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(kApplyThreads) sgd_apply_kernel(const ApplyArg
     auto draws = [&](int64_t j) { return philox4x32_10((uint32_t)j >> 2, a.step, a.epoch, 4u, (uint32_t)a.seed, (uint32_t)(a.seed >> 32)); };
     Philox4 u = {};
     if (a.grad_bits > 0) u = draws(j0);
+    after_previous_kernel(1);
     const float4 g0 = apply_read(a.g, j0, a), x0 = apply_read(a.x, j0, a);
     if (a.ctas > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // (every CTA has started)
     if (a.grad_bits > 0) {
@@ -121,12 +122,13 @@ int launch_sgd_apply(zipml_ctx* ctx, float* x, const float* g, int64_t n, const 
     cfg.gridDim = dim3((unsigned)a.ctas);
     cfg.blockDim = dim3(32u * (unsigned)a.warps);
     cfg.stream = ctx->stream;
-    cudaLaunchAttribute cluster;
-    cluster.id = cudaLaunchAttributeClusterDimension;
-    cluster.val.clusterDim.x = (unsigned)a.ctas;
-    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
-    cfg.attrs = &cluster;
-    cfg.numAttrs = a.ctas > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (early_start(ctx, 1, attr + 1)) cfg.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, sgd_apply_kernel, a);
     if (e != cudaSuccess) return cuda_status(e);
     ++ctx->launches;

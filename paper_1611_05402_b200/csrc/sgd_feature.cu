@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
     mbar_fence_init();
     __syncthreads();
     slice_cluster_sync();                                // every CTA's barriers exist before anyone writes into it
+    after_previous_kernel(a.num_steps);
 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
@@ -575,7 +576,7 @@ int launch_sgd_feature(zipml_ctx* ctx, const zipml_dataset* d, const float* b, f
         if (fit >= a.clusters) break;
         most = fit;
     }
-    if (a.clusters > 1) cfg.numAttrs = 2;
+    if (a.clusters > 1 || early_start(ctx, num_steps, attr + 1)) cfg.numAttrs = 2;      // (a cooperative launch, or one that starts early)
     CUtensorMap tmaps[2];
     memset(tmaps, 0, sizeof(tmaps));
     int rc = encode_plane_maps(ctx, d, a.pitch / 4, a.box_rows, true, tmaps);

@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     mbar_fence_init();
     __syncthreads();
     slice_cluster_sync();                                // every CTA's barriers exist before anyone writes into it
+    after_previous_kernel(a.num_steps);
 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
@@ -657,7 +658,7 @@ int launch_sgd_slice(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
         if (fit >= plan.clusters) break;
         most = fit;
     }
-    if (plan.clusters > 1) cfg.numAttrs = 2;
+    if (plan.clusters > 1 || early_start(ctx, num_steps, attr + 1)) cfg.numAttrs = 2;      // (a cooperative launch, or one that starts early)
     const int64_t T = (d->m + p->batch - 1) / p->batch;
     SliceArgs a;
     memset(&a, 0, sizeof(a));

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_table_kernel(const 
     } else if (tid >= 64 && tid < 80) {
         sh->nrm_g[tid - 64] = sh->nrm_x[tid - 64] = 0.0;
     }
+    after_previous_kernel(a.num_steps);
 #pragma unroll 1
     for (int i = tid; i < F * L; i += kSliceThreads + 32) {
         const int c = i / WL % L, f = feature(i / (L * WL) * WL + i % WL);
@@ -499,7 +500,7 @@ int launch_sgd_table(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     cfg.blockDim = dim3(kSliceThreads + 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)a.nb;
     attr[0].val.clusterDim.y = 1;
@@ -510,6 +511,7 @@ int launch_sgd_table(zipml_ctx* ctx, const zipml_dataset* d, const float* b, flo
     e = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg);
     if (e != cudaSuccess) { (void)cudaGetLastError(); return ZIPML_ERR_WORKSPACE; }
     if (fit < 1) return ZIPML_ERR_WORKSPACE;
+    if (early_start(ctx, num_steps, attr + 1)) cfg.numAttrs = 2;
     if (p->batch_order) {
         rc = ws_reserve(ctx, carve_size(sizeof(int32_t) * (size_t)T));
         if (rc != ZIPML_OK) return rc;

@@ -1442,6 +1442,54 @@ def test_apply_gradient_is_the_end_of_a_step(ctx, grad_bits, reg, reg_param):
         ctx.zipml_sgd_apply_gradient(x, g, 0, lr, reg=1, reg_param=-1.0)
 
 
+@pytest.mark.parametrize("m,n,bits,batch,table,kernel", [(512, 60, 4, 16, False, "sgd_solo_kernel"), (4_096, 1_000, 8, 256, False, "sgd_feature_kernel"),
+                                                         (8_192, 1_000, 8, 1_024, False, "sgd_feature_kernel"), (2_048, 90, 2, 700, False, "sgd_slice_kernel"),
+                                                         (4_096, 400, 3, 256, True, "sgd_table_kernel"), (4_096, 20_000, 4, 128, False, None)], ids=str)
+@pytest.mark.parametrize("kw", [dict(), dict(model_bits=8, grad_bits=8)], ids=["", "quantized"])
+def test_steps_one_after_another(ctx, m, n, bits, batch, table, kernel, kw):
+    """Kernels of a step that start while the one before ends (a step's gradient, its application, the next step's, a change of x in between) leave what the
+    same calls leave with the device idle between them, recorded into a graph too."""
+    _, A, b, _ = workload("c2", m, n, seed=3)
+    levels = oracle.optimal_levels(A, bits, 64)[0] if table else None
+    gds = dev_dataset(oracle.quantize(A, bits, seed=1, **(dict(mode=oracle.TABLE, levels=levels) if table else {})), ctx)
+    db, x0 = to_dev(b, ctx), torch.linspace(-0.1, 0.1, n, device=ctx.device)
+    x, g2 = x0.clone(), torch.zeros(2 * n, device=ctx.device)
+
+    def steps(idle, count=12):
+        x.copy_(x0)
+        for k in range(count):
+            ctx.zipml_sgd_epoch(gds, db, x, batch, 0.0, first_step=k % (m // batch), num_steps=1, grad_out=g2, seed=5, **kw)
+            idle()
+            ctx.zipml_sgd_apply_gradient(x, g2[:n], k, 0.01, grad_bits=kw.get("grad_bits", 0), seed=5)
+            idle()
+            if k % 5 == 4:
+                x.mul_(0.5)
+                idle()
+        return x.clone()
+
+    want = steps(ctx.zipml_sync)
+    if kernel:
+        assert ctx.zipml_last_kernel() == kernel
+    for _ in range(8):
+        assert torch.equal(steps(lambda: None), want)
+    stream = torch.cuda.Stream(ctx.device)
+    with torch.cuda.stream(stream), binding.Context(ctx.device) as own:
+        ctx = own
+        assert torch.equal(steps(lambda: None), want)              # (grows what it needs before the recording)
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            steps(lambda: None, 4)
+        for _ in range(3):
+            graph.replay()
+        torch.cuda.synchronize()
+        recorded = x.clone()
+        steps(own.zipml_sync, 4)
+        torch.cuda.synchronize()
+        assert torch.equal(recorded, x)
+        del graph
+
+
 @pytest.mark.parametrize("n,skip,bits,norm", [(1, 0, 8, 0), (3, 1, 4, 1), (127, 0, 2, 0), (2_048, 0, 8, 0), (2_049, 0, 8, 1), (4_099, 3, 6, 0), (16_384, 0, 0, 0),
                                               (32_768, 0, 8, 0), (32_773, 0, 5, 1), (70_001, 2, 8, 0)], ids=str)
 def test_apply_gradient_of_any_size(ctx, n, skip, bits, norm):
