@@ -118,18 +118,18 @@ class ShardedEpoch:
         # positions whose batch this rank does not hold are never executed; their entries only have to be valid
         self.order_local = None if self.order is None or not T_local else [min(o, T_local - 1) for o in self.order][:T_local]
 
-    _calls = None                                                  # the two below, kept until an attribute changes
+    _calls = None                                                  # the two below and where the gradient lies, kept until an attribute changes
     _alone = False                                                 # run() is at work and nobody else sees a share
 
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
-        if name != "_calls":
+        if name not in ("_calls", "_alone"):
             object.__setattr__(self, "_calls", None)
 
     # The step's two library calls, with everything marshalled that stays the same from step to step.
     def _prepared(self):
         if self._calls is None:
-            self._calls = (self._share_call(), self._apply_call())
+            self._calls = (self._share_call(), self._apply_call(), self.g2[:self.n])
         return self._calls
 
     def _share_call(self):
@@ -144,10 +144,11 @@ class ShardedEpoch:
     def share(self, pos, t, weight):
         """weight * the mean over the rank's rows of batch t of the symmetrised gradient, at the model (or its Q3
         image for position pos) as it stands; zeros if the rank holds none of the batch.  A tensor of its own."""
-        if self.plan.count(t) == 0:
+        alone = self._alone and weight == 1.0                      # (then the batch's rows are all here)
+        if not alone and self.plan.count(t) == 0:
             import torch
             return torch.zeros(self.n, dtype=torch.float32, device=self.x.device)
-        call = self._prepared()[0]
+        call, _, g = self._prepared()
         if self.order_local is not None:
             # the library keys Q3 by the position: the step runs at position pos of a local order that names t there
             if pos >= len(self.order_local):
@@ -155,8 +156,7 @@ class ShardedEpoch:
                                  "take a position beyond its own count")
             call.batch_order[pos] = t
         call(pos)
-        g = self.g2[:self.n]
-        return g if self._alone and weight == 1.0 else g * weight
+        return g if alone else g * weight
 
     def apply(self, v, pos):
         """Q4 and the update on this rank's replica."""
