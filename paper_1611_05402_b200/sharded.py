@@ -118,12 +118,12 @@ class ShardedEpoch:
         # positions whose batch this rank does not hold are never executed; their entries only have to be valid
         self.order_local = None if self.order is None or not T_local else [min(o, T_local - 1) for o in self.order][:T_local]
 
-    _calls = None                                                  # the two below and where the gradient lies, kept until an attribute changes
+    _calls = None                                                  # the two below and where the gradient lies, kept until an attribute changes or a run begins
     _alone = False                                                 # run() is at work and nobody else sees a share
 
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
-        if name not in ("_calls", "_alone"):
+        if name != "_calls":
             object.__setattr__(self, "_calls", None)
 
     # The step's two library calls, with everything marshalled that stays the same from step to step.
