@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(1024) loss_digits_kernel(const float* __restri
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS, FPW = 32 / CB;
     __shared__ double red[40];
     __shared__ float smax[32];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // (the next kernel asks for codes meanwhile)
     double base = 0.0;
     float wm = 0.0f;
 #pragma unroll 4
@@ -283,30 +284,21 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
     const int lane = threadIdx.x & 31, gl = lane >> 2, tl = lane & 3, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int kp = 1 << kp_shift, part = warp & (kp - 1);
     const int64_t first = (int64_t)blockIdx.x * (warps >> kp_shift) + (warp >> kp_shift), more = (int64_t)gridDim.x * (warps >> kp_shift);
-    const double base = base_in[0], delta = base_in[1];
     const int64_t nblocks = (m + 15) / 16;
     const int64_t nspans = (row_bytes + 63) / 64;
     const int64_t span0 = (nspans * part) >> kp_shift, span1 = (nspans * (part + 1)) >> kp_shift;
     uint4* stages = loss_smem + warp * kLossStages * 128 + lane;
     const int digit_pitch = SHARED ? (int)((vec_bytes + 127) / 128 * 128 + 64) : 0;
     unsigned char* digits = reinterpret_cast<unsigned char*>(loss_smem + warps * kLossStages * 128);
-    if constexpr (SHARED) {
-        const int pieces = (int)(vec_bytes / 16);
-        for (int i = threadIdx.x; i < NG * NS * pieces; i += blockDim.x) {
-            const int v = i / pieces, k = i - v * pieces;
-            *reinterpret_cast<uint4*>(digits + v * digit_pitch + 16 * k) = __ldg(reinterpret_cast<const uint4*>(wdig + v * vec_bytes) + k);
-        }
-        __syncthreads();
-    }
     // the span that is asked for next
     int64_t ask_blk = first, ask_sp = span0;
-    const unsigned char *a1, *h1, *a2, *h2;
+    const unsigned char *a1 = p1, *h1 = p1, *a2 = p2, *h2 = p2;
     auto rows_of = [&]() {
         const int64_t ra = min(ask_blk * 16 + gl, m - 1), rh = min(ask_blk * 16 + gl + 8, m - 1);
         a1 = p1 + ra * row_bytes + 16 * tl; h1 = p1 + rh * row_bytes + 16 * tl;
         a2 = p2 + ra * row_bytes + 16 * tl; h2 = p2 + rh * row_bytes + 16 * tl;
     };
-    rows_of();
+    if constexpr (SHARED) rows_of();
     const int64_t jump = more * 16 * row_bytes;
     auto ask = [&](int stage) {
         if (ask_blk < nblocks && ask_sp < span1) {
@@ -331,10 +323,25 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
     if constexpr (SHARED)
 #pragma unroll
         for (int k = 0; k < kLossStages - 1; ++k) ask(k);
+    // the digits' kernel, which may still be at work, has ended; what lay before it had before it began
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const double base = *(volatile const double*)base_in, delta = *(volatile const double*)(base_in + 1);
+    if constexpr (SHARED) {
+        const int pieces = (int)(vec_bytes / 16);
+        for (int i = threadIdx.x; i < NG * NS * pieces; i += blockDim.x) {
+            const int v = i / pieces, k = i - v * pieces;
+            *reinterpret_cast<uint4*>(digits + v * digit_pitch + 16 * k) = __ldg(reinterpret_cast<const uint4*>(wdig + v * vec_bytes) + k);
+        }
+        __syncthreads();
+    }
     double total = 0.0;
     int turn = 0;
     // (kp > 1: a block is one group of warps, which take every turn together)
     for (int64_t blk = first; blk < nblocks; blk += more, turn ^= 1) {
+        if constexpr (!SHARED) {
+            ask_blk = blk;
+            rows_of();
+        }
         // A span adds at most 64 * 128 * 255 to a 32-bit digit sum: they are moved into 64-bit sums every
         // kLossFlushSpans spans (2^21 * 512 < 2^31), so rows of any admitted length stay exact.
         long long s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0};
@@ -372,7 +379,6 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
 #pragma unroll
         for (int e = 0; e < 4; ++e) { s1[e] += c1[e]; s2[e] += c2[e]; }
         }
-        if constexpr (!SHARED) { ask_blk += more; rows_of(); }
         // lane t < 2 holds digits 2t, 2t+1 of rows g (s[0], s[1]) and g+8 (s[2], s[3])
         double v[4];
 #pragma unroll
@@ -441,7 +447,7 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
         unsigned* ticket = reinterpret_cast<unsigned*>(wdig + (8 / cb) * 4 * vec_bytes);
         // 16 warps per SM, 16 rows per warp and turn, or kp warps to 16 rows, each a part of the spans: as many as make the turns, each its spans
         // and about two more for what it ends with, take least -- few rows would leave warps without any, long rows the last turn
-        // nearly empty.  Blocks are 16 warps (kp = 1) or one such group.
+        // nearly empty.  (Asking for an eighth less loses most of this: 8 bits 30,000 x 9,000, 142 against 140 so counted, 236 us against 146.)  Blocks are 16 warps (kp = 1) or one such group.
         // Measured with L2 flushed, us, as many warps to 16 rows as fill half the chip -> this: 8 bits 20,000 x 20,000 468 -> 185,
         // 40,000 x 20,000 558 -> 322, 30,000 x 9,000 241 -> 146, 4 bits 60,000 x 12,000 204 -> 191; in L2: 8 bits 2,797 x 1,500 18 -> 14.
         const int64_t turns = (d->m + 15) / 16, spans = vec_bytes / 64;
@@ -464,6 +470,7 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
         const int64_t chunks = (vec_bytes * (8 / cb) + 1023) / 1024;
         const int digit_blocks = (int)(chunks > 16 ? 16 : chunks);
         const double scale = 1.0 / (2.0 * (double)d->m);
+        // The second kernel starts while the first is at work and asks for its codes: 4 bits 20,972 x 200 13.1 -> 11.9 us, 8 bits 83,887 x 200 18.9 -> 16.4.
         // Stages (see the kernel) where 16 warps share the digits and these fit.  Measured with L2 flushed, us, straight to registers -> stages: 2 bits
         // 1,000,000 x 2,048 236 -> 198 (5.2 TB/s), 4 bits 1,000,000 x 1,000 206 -> 197, 8 bits 300,000 x 2,000 279 -> 259; rows of one span (20 codes of 4 bits,
         // 13,421,773 rows) 495 -> 414.  Rows of two to five spans keep to registers, where one row's spans are all in flight at once (8 bits 1,342,178
@@ -476,9 +483,17 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
             const cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
             if (e != cudaSuccess) return cuda_status(e);
             digits_kernel<<<digit_blocks, 1024, 0, ctx->stream>>>(d->feat_lo, d->feat_step, x, d->n, vec_bytes, wdig, base, ticket);
-            kernel<<<(int)blocks, 32 * warps, smem, ctx->stream>>>(d->plane1, d->plane2, d->row_bytes, d->m, vec_bytes, kp_shift, wdig, base, b, partials,
-                                                                   ticket, scale, loss_out);
-            return ZIPML_OK;
+            cudaLaunchConfig_t cfg;
+            memset(&cfg, 0, sizeof(cfg));
+            cfg.gridDim = dim3((unsigned)blocks);
+            cfg.blockDim = dim3(32u * (unsigned)warps);
+            cfg.dynamicSmemBytes = smem;
+            cfg.stream = ctx->stream;
+            cudaLaunchAttribute early;
+            cfg.attrs = &early;
+            cfg.numAttrs = early_start(ctx, 1, &early) ? 1 : 0;
+            return cuda_status(cudaLaunchKernelEx(&cfg, kernel, (const unsigned char*)d->plane1, (const unsigned char*)d->plane2, d->row_bytes, d->m, vec_bytes,
+                                                  kp_shift, (const signed char*)wdig, (const double*)base, b, partials, ticket, scale, loss_out));
         };
         const int rc = cb == 2   ? shared ? launch(loss_digits_kernel<2>, loss_codes_imma_kernel<2, true>) : launch(loss_digits_kernel<2>, loss_codes_imma_kernel<2, false>)
                        : cb == 4 ? shared ? launch(loss_digits_kernel<4>, loss_codes_imma_kernel<4, true>) : launch(loss_digits_kernel<4>, loss_codes_imma_kernel<4, false>)
