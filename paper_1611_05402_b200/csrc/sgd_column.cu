@@ -49,7 +49,7 @@
 //
 // The machine code is kept small on purpose (four roles share the instruction cache): 32-bit counters kept up
 // step by step instead of 64-bit divisions, waits as functions with one copy, loops unrolled only where
-// registers demand it.  Measured on 65,536 x 32,768 4-bit rows, B = 2,048: 21.9 us per step (stream engine:
+// registers demand it.  Measured on 65,536 x 32,768 4-bit rows, B = 2,048: 21.1 us per step (stream engine:
 // 29.8), DRAM reads 1.00 x the packed bytes.  Not HBM bounds it but the chain of a step: the first chunk's dots
 // have to cross L2 and become digits before pass B can start, pass B (about 1.2 k cycles per chunk on its own, 2 k
 // while pass A runs beside it) ends about 9 k cycles after pass A, and the next step's first dots come 5 k cycles
