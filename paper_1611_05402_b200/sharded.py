@@ -118,7 +118,7 @@ class ShardedEpoch:
         # positions whose batch this rank does not hold are never executed; their entries only have to be valid
         self.order_local = None if self.order is None or not T_local else [min(o, T_local - 1) for o in self.order][:T_local]
 
-    _calls = None                                                  # the two below and where the gradient lies, kept until an attribute changes or a run begins
+    _calls = None                                                  # the two below and a view of the gradient, kept until an attribute changes or a run begins
     _alone = False                                                 # run() is at work and nobody else sees a share
 
     def __setattr__(self, name, value):
@@ -156,6 +156,9 @@ class ShardedEpoch:
                                  "take a position beyond its own count")
             call.batch_order[pos] = t
         call(pos)
+        if g.data_ptr() != self.g2.data_ptr():                     # (its buffer got another storage, which the call followed)
+            g = self.g2[:self.n]
+            self._calls = (*self._calls[:2], g)
         return g if alone else g * weight
 
     def apply(self, v, pos):

@@ -147,6 +147,29 @@ def test_a_share_is_the_callers_own():
     assert torch.allclose(rank.x, torch.full((5,), x)) and torch.allclose(rank.g2[:5], torch.full((5,), g))
 
 
+def test_a_share_is_read_from_where_the_gradient_lies():
+    """Between two shares and within a run the gradient's buffer may get another storage: what is returned and applied lies there."""
+    rank = _fake_rank()
+    assert rank.share(0, 0, 1.0)[0].item() == 1.0
+    rank.g2.data = torch.zeros(10)
+    assert rank.share(1, 1, 1.0)[0].item() == 2.0
+    rank.g2.set_(torch.zeros(10))
+    assert rank.share(2, 2, 1.0)[0].item() == 3.0
+
+    alone, x = _fake_rank(), torch.zeros(5)
+    step = alone.apply
+
+    def apply(v, pos):
+        step(v, pos)
+        alone.g2.data = torch.zeros(10)
+
+    object.__setattr__(alone, "apply", apply)                                 # (what a rank that runs alone is handed after every step)
+    alone.run()
+    for pos in range(3):
+        x -= 0.5 * (x + pos + 1)
+    assert torch.allclose(alone.x, x)
+
+
 def test_a_rank_follows_its_attributes_from_step_to_step():
     """What the meeting of the ranks changes (a step length by schedule, another replica) holds from there on, as it does
     between runs."""
