@@ -176,7 +176,8 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 // that a warp's look-ups are free of bank conflicts whatever its codes are; the cell is found by bisection, whose offset is the cell's
 // number times 256, and p by a multiplication with the staged reciprocal of the cell's width, corrected (quotient below).
 // Blocks with a cell too narrow or too wide for that divide instead; a quotient too small for it is between 0 and
-// 2^-24 anyway and its threshold 1, or 0 where the division would round to 0 (the staged least numerator).  No calls, and no branch a
+// 2^-24 anyway, and its threshold is 1 if the numerator lies above the staged one from which on the division does not round to 0 and 0 if not
+// (a numerator of exactly width 2^-150, half of the smallest number, comes out of the correction as 0 or not).  No calls, and no branch a
 // sample: 85 -> 71 instructions a sample, 890 -> 655 us on 500,000 x 512 at 3 bits.  Such a
 // call needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
 // non-finite values, are gathered on the way.
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
             if (takes && !(width >= 9.1e-13f && width <= 1.09e12f)) divide = true;
             const int at = ((f & 3) * L + k) * kCols + (f >> 2);
             lev_s[at] = k < L - 1 ? val : INFINITY;
-            // (a numerator above width 2^-150 has a quotient that is not rounded to 0)
+            // (a numerator above width 2^-150 has a quotient that is not rounded to 0; at and below it it is)
             cell_s[at] = make_float4(val, takes ? width : __int_as_float(0x7fffffff), takes ? __frcp_rn(width) : 0.0f,
                                      takes ? __fmul_rd(__fmul_rn(width, 0x1p-75f), 0x1p-75f) : INFINITY);
         }
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
                 const float p = kDivide ? __fdiv_rn(num, c.y) : quotient(num, c.y, c.z);
                 // the upper end (a quotient of 1 or more) is always up
                 uint32_t threshold = __float2uint_ru(num >= c.y ? 16777216.0f : __fmul_rn(p, 16777216.0f));
-                if (!kDivide && num > c.w) threshold = max(threshold, 1u);
+                if (!kDivide) threshold = num > c.w ? max(threshold, 1u) : 0u;
                 return __byte_perm(at, 0u, 0x1444) + threshold;
             }
         };

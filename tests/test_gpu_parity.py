@@ -156,6 +156,24 @@ def test_quantize_values_just_above_a_level(ctx, bits):
     assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3, 4])
+@pytest.mark.parametrize("width", [0x1d9c282, 0x17b7084 * 2.0 ** 6, 0x1f3d096 * 2.0 ** 12, 0x1eead6c * 2.0 ** 15], ids=["2^24", "2^30", "2^36", "2^39"])
+def test_quantize_where_the_division_just_rounds_to_zero(ctx, width, bits):
+    """(x - level) / width is exactly 2^-150, which rounds to 0: no draw takes it up; the next larger x goes up on a draw of 0,
+    which each of these seeds makes for one of the samples."""
+    m, n = 300, 64
+    table = np.tile(np.float32(width) * np.arange(1 << bits, dtype=np.float32), (n, 1)).astype(np.float32)
+    tie = np.float32(np.ldexp(width, -150))
+    for seed in (45, 62, 301):
+        for v, goes_up in ((tie, 0), (np.nextafter(tie, np.float32(1)), 1)):
+            A = np.full((m, n), v, np.float32)
+            ods = oracle.quantize(A, bits, seed=seed, mode=oracle.TABLE, levels=table)
+            assert (ods.plane1 != 0).sum() + (ods.plane2 != 0).sum() == goes_up
+            gds = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=seed, level_mode=binding.LEVELS_TABLE, levels=to_dev(table, ctx))
+            ctx.zipml_sync()
+            assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+
+
 def test_quantize_strided_and_unaligned_input(ctx):
     _, A, _, _ = workload("c2", 200, 101, seed=3)
     big = torch.zeros((200, 131), dtype=torch.float32, device=ctx.device)
