@@ -265,6 +265,14 @@ __device__ __forceinline__ void loss_copy16(void* dst, const void* src, uint32_t
     asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
 }
 
+// 16 bytes of the digits, which the kernel before may still be writing when this one starts: an ordinary load (the read-only path wants
+// what does not change while the kernel lives), and one that stays behind the wait for that kernel.
+__device__ __forceinline__ uint4 loss_digits_at(const signed char* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // SHARED: a warp's spans, 16 rows after 16 rows, as one sequence that runs kLossStages - 1 spans ahead of the arithmetic: every lane copies the 64 bytes
 // it will use into its own places of a stage (nobody else reads them: no barrier) and asks for the next as soon as it has
 // taken one.  The digits lie in shared memory: [group][digit], `digit_pitch` bytes apart, 64 past a multiple of 128, so that two digits'
@@ -273,7 +281,7 @@ __device__ __forceinline__ void loss_copy16(void* dst, const void* src, uint32_t
 template <int CB, bool SHARED>
 __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned char* __restrict__ p1, const unsigned char* __restrict__ p2,
                                                               int64_t row_bytes, int64_t m, int64_t vec_bytes, int kp_shift,
-                                                              const signed char* __restrict__ wdig, const double* __restrict__ base_in,
+                                                              const signed char* wdig, const double* base_in,
                                                               const float* __restrict__ b, double* __restrict__ partials, unsigned* __restrict__ ticket,
                                                               double scale, double* __restrict__ out) {
     constexpr int NG = IntPath<CB>::NG, NS = IntPath<CB>::NS;
@@ -330,7 +338,7 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
         const int pieces = (int)(vec_bytes / 16);
         for (int i = threadIdx.x; i < NG * NS * pieces; i += blockDim.x) {
             const int v = i / pieces, k = i - v * pieces;
-            *reinterpret_cast<uint4*>(digits + v * digit_pitch + 16 * k) = __ldg(reinterpret_cast<const uint4*>(wdig + v * vec_bytes) + k);
+            *reinterpret_cast<uint4*>(digits + v * digit_pitch + 16 * k) = loss_digits_at(wdig + v * vec_bytes + 16 * k);
         }
         __syncthreads();
     }
@@ -369,7 +377,7 @@ __global__ void __launch_bounds__(512) loss_codes_imma_kernel(const unsigned cha
                 uint4 bd = make_uint4(0u, 0u, 0u, 0u);            // digit gl of this lane's 16 bytes
                 if (gl < NS)
                     bd = SHARED ? *reinterpret_cast<const uint4*>(digits + (g * NS + gl) * digit_pitch + (int)off + 16 * tl)
-                                : __ldg(reinterpret_cast<const uint4*>(wdig + ((int64_t)g * NS + gl) * vec_bytes + off + 16 * tl));
+                                : loss_digits_at(wdig + ((int64_t)g * NS + gl) * vec_bytes + off + 16 * tl);
                 mma_u8s8(c1, slice_dot_codes<CB>(ua.x, g), slice_dot_codes<CB>(uh.x, g), slice_dot_codes<CB>(ua.y, g), slice_dot_codes<CB>(uh.y, g), bd.x, bd.y);
                 mma_u8s8(c1, slice_dot_codes<CB>(ua.z, g), slice_dot_codes<CB>(uh.z, g), slice_dot_codes<CB>(ua.w, g), slice_dot_codes<CB>(uh.w, g), bd.z, bd.w);
                 mma_u8s8(c2, slice_dot_codes<CB>(va.x, g), slice_dot_codes<CB>(vh.x, g), slice_dot_codes<CB>(va.y, g), slice_dot_codes<CB>(vh.y, g), bd.x, bd.y);

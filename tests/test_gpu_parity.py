@@ -1203,6 +1203,24 @@ def test_loss_codes_through_stages_and_without(ctx, m, n, bits):
     assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
 
 
+def test_losses_one_after_another_see_their_own_digits(ctx):
+    """Losses of several models and shapes (with and without stages; their digits lie elsewhere in the same scratch) with no wait between
+    them: each is what it is on an idle device."""
+    calls = []
+    for m, n, bits in ((40_003, 200, 8), (39_990, 900, 8), (266_000, 390, 8), (2_300, 2_100, 8), (40_005, 20, 4)):
+        _, A, b, xs = workload("c2", m, n, seed=2)
+        gds, db = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=3), to_dev(b, ctx)
+        for scale in (0.9, -30.0, 1e-3):
+            dx = to_dev((xs * scale).astype(np.float32), ctx)
+            out = ctx.zipml_loss(binding.LOSS_CODES, db, dx, data=gds)
+            ctx.zipml_sync()
+            calls.append((gds, db, dx, out.item()))
+    order = np.random.default_rng(4).integers(0, len(calls), 200)
+    outs = [ctx.zipml_loss(binding.LOSS_CODES, calls[k][1], calls[k][2], data=calls[k][0]) for k in order]
+    ctx.zipml_sync()
+    assert [o.item() for o in outs] == [calls[k][3] for k in order]
+
+
 def test_loss_codes_with_level_table_and_strided_dense(ctx):
     _, A, b, xs = workload("c4", 2000, 60, seed=1)
     lev, _ = oracle.optimal_levels(A, 3, 128)
