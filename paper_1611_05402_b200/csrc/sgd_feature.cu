@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
-    auto batch_at = [&](int k) { return k < steps ? (a.order ? __ldg(a.order + a.first_step + k) : (int)a.first_step + k) : 0; };
+    auto batch_at = [&](int k) { return k < steps ? (a.order ? a.order[a.first_step + k] : (int)a.first_step + k) : 0; };
     auto own_of = [&](int batch) { return max(0, min(own, (batch < whole ? (int)a.batch : a.rows_last) - row_base - bi * a.rpo)); };
     if (warp == kSliceWarps) {
         // -------------------------------------------------------------------- the copying warp, which also sees to lo^T x~
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_feature_kernel(cons
     const int gl = lane >> 2, tl = lane & 3, lm = lane >> 3, l8 = lane & 7;
     const int P = 1 << a.p_shift, pp = tid & (P - 1), k_own = tid >> a.p_shift, f_own = bi * F + k_own;
     const bool mine = k_own < F && f_own < n, writes = mine && pp == 0;
-    const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
+    const float st = mine ? a.step[f_own] : 0.0f, lof = mine ? a.lo[f_own] : 0.0f;
     const double lo_double = lof, st_low = (double)st / (double)(1 << (CB * (k_own % NG)));     // (codes were multiplied where they lie in their byte)
     float x = mine ? a.x[f_own] : 0.0f;
     auto draw = [&](int k, uint32_t stream) { return slice_draw(a.seed, a.epoch, (uint32_t)a.first_step + (uint32_t)k, (uint32_t)f_own, stream); };

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
-    auto batch_at = [&](int k) { return k < steps ? (a.order ? __ldg(a.order + a.first_step + k) : (int)a.first_step + k) : 0; };
+    auto batch_at = [&](int k) { return k < steps ? (a.order ? a.order[a.first_step + k] : (int)a.first_step + k) : 0; };
     const int row_base = (cl * a.nb + bi) * a.rc, chunks = MANY ? a.chunks : 1;
     const int rows_full = min(a.rc, (int)a.batch - row_base), rows_last = min(a.rc, a.rows_last - row_base);
     auto rows_of = [&](int batch, int chunk) { return max(0, min(a.cr, (batch < whole ? rows_full : rows_last) - chunk * a.cr)); };
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     // labels: a lane of the first rb warps forms one residual, of this row of the CTA
     const int res_row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
     auto label_of = [&](int batch, int chunk) {
-        return warp < rb && res_row < rows_of(batch, chunk) ? __ldg(a.b + batch * a.batch + row_base + chunk * a.cr + res_row) : 0.0f;
+        return warp < rb && res_row < rows_of(batch, chunk) ? a.b[batch * a.batch + row_base + chunk * a.cr + res_row] : 0.0f;
     };
     float label = label_of(batch, 0);
 
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     const int f_own = bi * SF + k_own;
     const bool mine = owner && k_own < SF && f_own < n;
     const int c0 = 1 << (a.bits - 1);
-    const float st = mine ? __ldg(a.step + f_own) : 0.0f, lof = mine ? __ldg(a.lo + f_own) : 0.0f;
+    const float st = mine ? a.step[f_own] : 0.0f, lof = mine ? a.lo[f_own] : 0.0f;
     const double mid = fma((double)c0, (double)st, (double)lof);
     const double st_low = (double)st / (double)(1 << (CB * (k_own % NG)));    // (codes were multiplied where they lie in their byte)
     float x = mine ? a.x[f_own] : 0.0f;

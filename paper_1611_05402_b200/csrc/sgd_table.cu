@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_table_kernel(const 
 #pragma unroll 1
     for (int i = tid; i < F * L; i += kSliceThreads + 32) {
         const int c = i / WL % L, f = feature(i / (L * WL) * WL + i % WL);
-        lev[i] = f < n && c < a.real_levels ? __ldg(a.levels + (size_t)f * a.real_levels + c) : 0.0f;
+        lev[i] = f < n && c < a.real_levels ? a.levels[(size_t)f * a.real_levels + c] : 0.0f;
     }
 #pragma unroll 1
     for (int g = tid; g < F; g += kSliceThreads + 32) xown[g] = feature(g) < n ? a.x[feature(g)] : 0.0f;
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_table_kernel(const 
 
     // steps are counted from the call's first one; a batch is named by its index
     const int steps = (int)a.num_steps, whole = a.whole;
-    auto batch_at = [&](int k) { return k < steps ? (a.order ? __ldg(a.order + a.first_step + k) : (int)a.first_step + k) : 0; };
+    auto batch_at = [&](int k) { return k < steps ? (a.order ? a.order[a.first_step + k] : (int)a.first_step + k) : 0; };
     auto own_of = [&](int batch) { return max(0, min(own, (batch < whole ? (int)a.batch : a.rows_last) - bi * a.rpo)); };
     if (warp == kSliceWarps) {
         // -------------------------------------------------------------------- the copying warp
