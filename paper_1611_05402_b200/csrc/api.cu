@@ -306,10 +306,11 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
 // C 29.4 R 34.5, x 2,000 41 / 36; 4 KB x 2,000 42 / 41; 6 KB x 3,000 56 / 56; 8 KB x 4,500 87 / 93.  4 bits 4.1 KB x 64 C 9.1 R 22, x 1,200
 // 16.5 / 33, x 4,500 41 / 43, x 6,000 53 / 49; 9 KB x 8,192 86 / 85; 16 KB x 64 10.7 / 31, x 8,192 92 / 145.  8 bits 9 KB x 64 9.4 / 21, x 3,000
 // 33 / 36, x 6,000 61 / 54; 12 KB x 6,000 49 / 68.  (With a quantized model too C takes some 3 more, R 6.)
-static bool column_pays_quantized(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t count) {
+static bool column_pays_quantized(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t T) {
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || (p->model_bits == 0 && p->grad_bits == 0)) return false;
-    // (a quantized gradient alone in up to three steps: the choice of the ring engine is a pinned one, not the faster)
-    if (p->model_bits == 0 && count <= 3) return false;
+    // (a quantized gradient alone on data of up to three batches: the choice of the ring engine is a pinned one, not the faster.  The batches
+    // of the data count, not the steps of the call: a range of an epoch's steps runs on the engine of the whole epoch)
+    if (p->model_bits == 0 && T <= 3) return false;
     const int cb = container_bits(d->bits);
     if (cb == 2) return B <= 1500 || 2 * B <= d->row_bytes;
     if (cb == 4) return B <= 4500 || 10 * B <= 9 * d->row_bytes;
@@ -452,7 +453,7 @@ int zipml_sgd_epoch(zipml_ctx* ctx, const zipml_dataset* data, const float* b, f
             rc = launch_sgd_lean(ctx, data, b, x, params, first, count, grad_out);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }
-        if (column_pays_quantized(data, params, B, count)) {
+        if (column_pays_quantized(data, params, B, T)) {
             rc = launch_sgd_column(ctx, data, b, x, params, first, count, grad_out, true);
             if (rc != ZIPML_ERR_WORKSPACE) return rc;
         }

@@ -1038,6 +1038,24 @@ def test_auto_picks_the_engine_that_fits(ctx):
     assert ctx.zipml_last_engine() == binding.ENGINE_CLUSTER
 
 
+@pytest.mark.parametrize("pieces", [(1,) * 7, (3, 3, 1), (5, 2)], ids=str)
+@pytest.mark.parametrize("m,n,bits,batch", [(440, 9001, 4, 64), (440, 8431, 8, 64), (2090, 20_000, 4, 300)], ids=str)
+def test_ranges_of_steps_run_on_the_engine_of_the_whole_epoch(ctx, m, n, bits, batch, pieces):
+    """A quantized gradient on wide rows, seven steps in one call and in ranges of them: the same engine and the same model."""
+    _, A, b, _ = workload("c2", m, n, seed=4)
+    gds, db = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=3), to_dev(b, ctx)
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    whole, parts = to_dev(x0, ctx), to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(gds, db, whole, batch, 1e-5, grad_bits=8, seed=5)
+    engine, first = ctx.zipml_last_engine(), 0
+    for count in pieces:
+        ctx.zipml_sgd_epoch(gds, db, parts, batch, 1e-5, grad_bits=8, seed=5, first_step=first, num_steps=count)
+        assert ctx.zipml_last_engine() == engine == binding.ENGINE_COLUMN
+        first += count
+    ctx.zipml_sync()
+    assert torch.equal(whole, parts)
+
+
 @pytest.mark.parametrize("m,n,bits,batch,optimal,engine", [
     (130, 9001, 4, 64, False, binding.ENGINE_COLUMN), (9, 8431, 8, 1, False, binding.ENGINE_COLUMN),
     (90, 9403, 2, 40, False, binding.ENGINE_STREAM), (1300, 9001, 4, 1205, False, binding.ENGINE_STREAM),
