@@ -600,10 +600,11 @@ bool table_form_pays(const zipml_dataset* d, const zipml_sgd_params* p) {
 // 3.10, x 1,024 4.12 / 4.41, n 1,000 x 256 3.15 / 3.56, n 2,000 x 2,048 6.6 / 9.5; 4 bits n 250 x 256 3.19 / 2.92, n 512 x 2,048 5.15 / 5.27, x 4,096
 // 7.06 / 5.99; 2 bits n 256 x 128 3.04 / 2.83, n 1,000 x 64 2.82 / 3.33, x 512 4.05 / 4.58, x 4,096 8.04 / 7.66.
 static bool features_pay(const zipml_dataset* d, const zipml_sgd_params* p) {
-    const int64_t B = p->batch < d->m ? p->batch : d->m;
-    // (From 2^24 entries a step a quantized vector whose model is asked for leaves this form, and wide rows then go to the ring engine: a
-    // pinned choice, not the faster.  2 bits 4,096 x 4,096 features 13.8, rows 22.9, ring 43.5.)
-    if ((p->model_bits > 0 || p->grad_bits > 0) && p->model_out && B * d->n >= 1 << 24) return false;
+    const int64_t B = p->batch < d->m ? p->batch : d->m, T = (d->m + p->batch - 1) / p->batch;
+    // (From 2^24 entries a step a quantized vector on data of up to three batches leaves this form, and wide rows then go to the ring
+    // engine: a pinned choice, not the faster.  2 bits 4,096 x 4,096 features 13.8, rows 22.9, ring 43.5.  Whether the model is asked
+    // for makes no difference.)
+    if ((p->model_bits > 0 || p->grad_bits > 0) && T <= 3 && B * d->n >= 1 << 24) return false;
     return d->n >= (container_bits(d->bits) == 2 ? 900 : 480) && B <= 5 * d->n;
 }
 int launch_sgd_int8(zipml_ctx* ctx, const zipml_dataset* d, const float* b, float* x, const zipml_sgd_params* p, int64_t first_step,

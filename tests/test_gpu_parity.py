@@ -1056,6 +1056,21 @@ def test_ranges_of_steps_run_on_the_engine_of_the_whole_epoch(ctx, m, n, bits, b
     assert torch.equal(whole, parts)
 
 
+@pytest.mark.parametrize("m,n,bits,batch", [(9000, 8192, 2, 2048), (17_000, 4096, 2, 4096)], ids=str)
+def test_asking_for_the_model_changes_nothing(ctx, m, n, bits, batch):
+    """2^24 entries a step and both vectors quantized, with model_out and without: the same kernel and the same bits."""
+    _, A, b, _ = workload("c3", m, n, seed=7)
+    gds, db = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=4), to_dev(b, ctx)
+    x0 = (np.random.default_rng(5).standard_normal(n) * 0.02).astype(np.float32)
+    x, y, seen = to_dev(x0, ctx), to_dev(x0, ctx), torch.zeros(n, device=ctx.device)
+    kw = dict(model_bits=8, grad_bits=8, seed=21)
+    ctx.zipml_sgd_epoch(gds, db, x, batch, 5e-4, **kw)
+    kernel = ctx.zipml_last_kernel()
+    ctx.zipml_sgd_epoch(gds, db, y, batch, 5e-4, model_out=seen, **kw)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_kernel() == kernel == "sgd_feature_kernel" and torch.equal(x, y) and seen.abs().sum().item() > 0
+
+
 @pytest.mark.parametrize("m,n,bits,batch,optimal,engine", [
     (130, 9001, 4, 64, False, binding.ENGINE_COLUMN), (9, 8431, 8, 1, False, binding.ENGINE_COLUMN),
     (90, 9403, 2, 40, False, binding.ENGINE_STREAM), (1300, 9001, 4, 1205, False, binding.ENGINE_STREAM),
