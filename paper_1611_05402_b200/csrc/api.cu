@@ -357,7 +357,15 @@ static int table_engine(const zipml_dataset* d, const zipml_sgd_params* p, int64
         if (lean_fits && (two ? n >= 1000 && step_bytes > 5 * MB : n >= 500 && step_bytes > 4 * MB)) return ZIPML_ENGINE_LEAN;
         return step_bytes <= (two ? 10 : d->bits == 3 ? 11 : n <= 800 ? 8 : 3) * MB ? ZIPML_ENGINE_PERSISTENT : ZIPML_ENGINE_RING;
     }
-    if (n <= 64) return B < (two ? 1000 : 3500) ? ZIPML_ENGINE_CLUSTER : B <= 5000 ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_PERSISTENT;
+    if (n <= 64) {
+        if (B < (two ? 1000 : 3500)) return ZIPML_ENGINE_CLUSTER;
+        if (B > 5000) return ZIPML_ENGINE_PERSISTENT;
+        if (lean_fits) return ZIPML_ENGINE_LEAN;
+        // (rows that lie far apart: the stride sizes what the lean engine stages.  2 bits n 16 x 1,200 G 24.7 R 24.5, n 40 x 3,000 25.5 / 30.0, n 64 x 4,900
+        // 28.0 / 37.3; 3 bits n 40 x 3,600 22.6 / 22.0; 4 bits n 16 x 3,600 24.4 / 23.3, n 64 x 4,900 24.1 / 25.9)
+        if (step_bytes <= 2 * MB) return ZIPML_ENGINE_CLUSTER;
+        return two || B > 4000 ? ZIPML_ENGINE_PERSISTENT : ZIPML_ENGINE_RING;
+    }
     if (B <= (two || n >= 400 ? 2500 : 4096) && step_bytes <= 2 * MB) return ZIPML_ENGINE_CLUSTER;
     if (n <= (two || d->bits == 3 ? 1100 : 800) && step_bytes <= (d->bits == 4 ? 8 : 10) * MB) return ZIPML_ENGINE_PERSISTENT;
     return lean_fits && two && step_bytes <= 10 * MB ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_RING;

@@ -1107,6 +1107,28 @@ def test_auto_on_level_tables(ctx, m, n, bits, batch, kernel):
     assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
 
 
+@pytest.mark.parametrize("m,n,bits,batch,kernel", [(3100, 40, 2, 3000, "sgd_kernel"), (5000, 61, 4, 4900, "sgd_kernel"), (3700, 33, 3, 3600, "sgd_ring_kernel"),
+                                                    (1100, 40, 2, 1000, "sgd_kernel")], ids=str)
+def test_auto_on_level_tables_whose_rows_lie_far_apart(ctx, m, n, bits, batch, kernel):
+    """Quantized vectors on few features whose row stride is more than the lean engine holds: what AUTO takes in its place."""
+    _, A, b, _ = workload("c4", m, n, seed=4)
+    ods = oracle.quantize(A, bits, seed=3, mode=oracle.TABLE, levels=oracle.optimal_levels(A, bits, 32)[0])
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    kw = dict(model_bits=8, grad_bits=8, seed=3)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-3, **kw)
+    far = dev_dataset(ods, ctx)
+    planes = []
+    for plane in (far.plane1, far.plane2):
+        planes.append(torch.zeros((m, 2048), dtype=torch.uint8, device=ctx.device))
+        planes[-1][:, :far.row_bytes] = plane
+    gds = binding.Dataset(planes[0], planes[1], m, n, bits, ods.mode, far.feat_lo, None, far.levels)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(gds, to_dev(b, ctx), x, batch, 1e-3, **kw)
+    ctx.zipml_sync()
+    # (a last-bit difference in a norm may flip a draw that sits on its threshold, by one unit of one coordinate)
+    assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= 20 * MODEL_TOL
+
+
 @pytest.mark.parametrize("m,n,bits,batch,quantized,kernel", [
     (1700, 19, 2, 790, False, "sgd_cluster_kernel"), (1700, 19, 2, 800, False, "sgd_lean_kernel"), (7100, 19, 2, 7001, False, "sgd_kernel"),
     (3300, 90, 3, 1600, False, "sgd_lean_kernel"), (6600, 90, 4, 6501, False, "sgd_kernel"), (3600, 33, 4, 3500, True, "sgd_lean_kernel"),
