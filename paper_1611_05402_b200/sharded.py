@@ -129,7 +129,7 @@ class ShardedEpoch:
     # The step's two library calls, with everything marshalled that stays the same from step to step.
     def _prepared(self):
         if self._calls is None:
-            self._calls = (self._share_call(), self._apply_call(), self.g2[:self.n])
+            self._calls = (self._share_call(), self._apply_call(), self.g2[:self.n], self.g2.data_ptr())
         return self._calls
 
     def _share_call(self):
@@ -148,7 +148,7 @@ class ShardedEpoch:
         if not alone and self.plan.count(t) == 0:
             import torch
             return torch.zeros(self.n, dtype=torch.float32, device=self.x.device)
-        call, _, g = self._prepared()
+        call, _, g, at = self._prepared()
         if self.order_local is not None:
             # the library keys Q3 by the position: the step runs at position pos of a local order that names t there
             if pos >= len(self.order_local):
@@ -156,9 +156,9 @@ class ShardedEpoch:
                                  "take a position beyond its own count")
             call.batch_order[pos] = t
         call(pos)
-        if g.data_ptr() != self.g2.data_ptr():                     # (its buffer got another storage, which the call followed)
+        if self.g2.data_ptr() != at:                               # (its buffer got another storage, which the call followed)
             g = self.g2[:self.n]
-            self._calls = (*self._calls[:2], g)
+            self._calls = (*self._calls[:2], g, self.g2.data_ptr())
         return g if alone else g * weight
 
     def apply(self, v, pos):
