@@ -1056,6 +1056,28 @@ def test_ranges_of_steps_run_on_the_engine_of_the_whole_epoch(ctx, m, n, bits, b
     assert torch.equal(whole, parts)
 
 
+@pytest.mark.parametrize("n,bits,batch,engine", [
+    (4110, 8, 2500, binding.ENGINE_COLUMN), (4110, 8, 2501, binding.ENGINE_RING), (4128, 8, 3200, binding.ENGINE_COLUMN), (4128, 8, 3201, binding.ENGINE_RING),
+    (6528, 8, 4500, binding.ENGINE_COLUMN), (8200, 4, 4000, binding.ENGINE_COLUMN), (8200, 4, 4001, binding.ENGINE_RING),
+], ids=str)
+def test_auto_on_wide_rows_with_a_quantized_gradient(ctx, n, bits, batch, engine):
+    """Either side of the lines between column and ring engine, and the ring engine's result."""
+    m = 3 * batch + 5
+    g = torch.Generator(device=ctx.device)
+    g.manual_seed(n + batch)
+    A = torch.rand((m, n), generator=g, device=ctx.device)
+    b, x0 = A[:, :100].sum(dim=1) * 0.1, torch.randn(n, generator=g, device=ctx.device) * 0.01
+    gds = ctx.zipml_quantize(A, bits, seed=3)
+    x, x_ref = x0.clone(), x0.clone()
+    kw = dict(grad_bits=8, seed=5)
+    ctx.zipml_sgd_epoch(gds, b, x, batch, 1e-5, **kw)
+    took = ctx.zipml_last_engine()
+    ctx.zipml_sgd_epoch(gds, b, x_ref, batch, 1e-5, engine=binding.ENGINE_RING, **kw)
+    ctx.zipml_sync()
+    # (a last-bit difference in a norm may flip a draw that sits on its threshold, by one unit of one coordinate)
+    assert took == engine and rel(x.cpu().numpy(), x_ref.cpu().numpy()) <= 20 * MODEL_TOL
+
+
 @pytest.mark.parametrize("m,n,bits,batch", [(9000, 8192, 2, 2048), (17_000, 4096, 2, 4096)], ids=str)
 def test_asking_for_the_model_changes_nothing(ctx, m, n, bits, batch):
     """2^24 entries a step and both vectors quantized, with model_out and without: the same kernel and the same bits."""
