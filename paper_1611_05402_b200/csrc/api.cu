@@ -298,8 +298,9 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
     }
     // 2 bits: C 10.4 S 11.0 at 2.3 KB x 64, 12.4 / 12.3 x 200, 27 / 22 x 1,200.  Else the column engine, whose CTAs are few but exchange
     // less, up to many rows: 8 bits 7 KB x 1,200 C 12.5 S 15.7, x 3,000 24.5 / 25.5, x 4,500 35.2 / 33.5; 9 KB x 2,000 21.6 / 23.3, x 3,000
-    // 31.1 / 31.6.  (At 4 bits the line at 1,200 rows is a pinned one: 4.1 KB x 1,200 C 13.7 S 16.0, x 2,000 19.3 / 19.4.)
-    return cb == 2 || B >= (cb == 8 ? 3000 : 1200) ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
+    // 31.1 / 31.6; but rows of an odd multiple of 16 bytes, whose pieces begin in the middle of a sector, 6,512 bytes x 1,300 0.90 times S, x 2,200
+    // 24.4 / 23.4, x 2,900 30.5 / 27.8, 8,016 x 1,300 0.98, x 1,700 22.4 / 20.6, x 2,900 34.8 / 29.3.  (At 4 bits the line at 1,200 rows is a pinned one: 4.1 KB x 1,200 C 13.7 S 16.0, x 2,000 19.3 / 19.4.)
+    return cb == 2 || B >= (cb == 8 ? (d->row_bytes % 32 == 0 ? 3000 : 1500) : 1200) ? ZIPML_ENGINE_STREAM : ZIPML_ENGINE_COLUMN;
 }
 
 // The same rows with a quantized model or gradient: column or ring engine.  Q0/8 (fp32 model, gradient of 8 bits): 2 bits 2.2 KB x 1,200

@@ -1113,6 +1113,22 @@ def test_auto_on_rows_wider_than_a_cluster(ctx, m, n, bits, batch, optimal, engi
     assert ctx.zipml_last_engine() == engine and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
 
 
+@pytest.mark.parametrize("n,batch,engine", [
+    (6512, 1499, binding.ENGINE_COLUMN), (6512, 1500, binding.ENGINE_STREAM), (6528, 2999, binding.ENGINE_COLUMN), (6528, 3000, binding.ENGINE_STREAM),
+], ids=str)
+def test_auto_on_rows_that_begin_in_the_middle_of_a_sector(ctx, n, batch, engine):
+    """8-bit rows of an odd multiple of 16 bytes and of an even one, either side of the lines between column and stream engine."""
+    m = batch + 70
+    _, A, b, _ = workload("c2", m, n, seed=4)
+    ods = oracle.quantize(A, 8, seed=3)
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-5)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-5)
+    ctx.zipml_sync()
+    assert ctx.zipml_last_engine() == engine and rel(x.cpu().numpy(), x_ref) <= MODEL_TOL
+
+
 @pytest.mark.parametrize("m,n,bits,batch,kernel", [
     (420, 31, 3, 200, "sgd_table_kernel"), (450, 31, 3, 201, "sgd_cluster_kernel"), (400, 64, 2, 185, "sgd_table_kernel"),
     (400, 61, 2, 186, "sgd_cluster_kernel"), (2500, 590, 3, 2400, "sgd_lean_kernel"), (3000, 590, 3, 2950, "sgd_kernel"),
