@@ -347,7 +347,8 @@ static bool lean_pays(const zipml_dataset* d, const zipml_sgd_params* p, int64_t
 //   2 bits n 2,000 x 8,192 39 / 53.
 //   Both vectors of 8 bits (a norm is dear on the lean engine beyond 64 features): 2 bits n 16 x 1,024 K 13.9 L 13.5 G 22, x 4,096 31 / 24 / 29, x
 //   8,192 54 / 38.5 / 35.6; n 256 x 2,048 19.8 / 22.5 / 24.6, x 4,096 31.4 / 30 / 27.7, x 16,384 L 73 G 46 R 75; n 1,024 x 16,384 L 67 G 55 R 132;
-//   n 2,000 x 4,096 L 47.5 G 57.6 R 77.  3 bits n 40 x 2,048 K 15.3 L 15.2, x 4,096 22.6 / 20.7 / 23.2, x 6,000 30 / 29.6 / 25.5; n 256 x 4,096 K 23 G 22.5; n 700 x 2,048 L 24.4 G 27.4
+//   n 2,000 x 4,096 L 47.5 G 57.6 R 77; just above 2 MB a step up to n 2,560 x 2,048 the ring engine still: n 2,200 L 48.9 R 46.5, x 2,200 52.8 / 53.2, n
+//   2,550 x 1,900 52.5 / 47.2, x 2,400 48.3 / 53.5, n 2,600 x 2,048 46.9 / 51.4.  3 bits n 40 x 2,048 K 15.3 L 15.2, x 4,096 22.6 / 20.7 / 23.2, x 6,000 30 / 29.6 / 25.5; n 256 x 4,096 K 23 G 22.5; n 700 x 2,048 L 24.4 G 27.4
 //   R 28, x 8,192 46 / 39 / 64; n 1,024 x 8,192 58 / 40 / 73; n 1,400 x 4,096 49 / 48 / 46.  4 bits n 700 x 8,192 45 / 42 / 49; n 1,400 x 1,024 31 / 41 / 29.
 // `lean_fits`: false once the lean engine has declined.
 static int table_engine(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t step_bytes, bool lean_fits) {
@@ -371,7 +372,7 @@ static int table_engine(const zipml_dataset* d, const zipml_sgd_params* p, int64
     }
     if (B <= (two || n >= 400 ? 2500 : 4096) && step_bytes <= 2 * MB) return ZIPML_ENGINE_CLUSTER;
     if (n <= (two || d->bits == 3 ? 1100 : 800) && step_bytes <= (d->bits == 4 ? 8 : 10) * MB) return ZIPML_ENGINE_PERSISTENT;
-    return lean_fits && two && step_bytes <= 10 * MB ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_RING;
+    return lean_fits && two && step_bytes <= 10 * MB && (B > 2100 || n > 2560) ? ZIPML_ENGINE_LEAN : ZIPML_ENGINE_RING;
 }
 
 // Uniform rows too wide for the column and stream engines: the persistent grid up to 16 MB a step, 4 bits n 100,000 x 64 G 23 R 42, x 300

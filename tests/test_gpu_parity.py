@@ -1187,6 +1187,22 @@ def test_auto_on_level_tables_with_long_batches(ctx, m, n, bits, batch, quantize
     assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= (20 if quantized else 1) * MODEL_TOL
 
 
+@pytest.mark.parametrize("m,n,batch,kernel", [(2300, 2300, 2100, "sgd_ring_kernel"), (2300, 2300, 2101, "sgd_lean_kernel"), (2300, 2561, 2100, "sgd_lean_kernel")],
+                         ids=str)
+def test_auto_on_2_bit_tables_with_both_vectors_quantized(ctx, m, n, batch, kernel):
+    """Either side of the line between ring and lean engine just above 2 MB a step."""
+    _, A, b, _ = workload("c4", m, n, seed=4)
+    ods = oracle.quantize(A, 2, seed=3, mode=oracle.TABLE, levels=oracle.optimal_levels(A, 2, 32)[0])
+    x0 = (np.random.default_rng(2).standard_normal(n) * 0.1).astype(np.float32)
+    kw = dict(model_bits=8, grad_bits=8, seed=3)
+    x_ref, _ = oracle.sgd_epoch(ods, b, x0, batch, 1e-4, **kw)
+    x = to_dev(x0, ctx)
+    ctx.zipml_sgd_epoch(dev_dataset(ods, ctx), to_dev(b, ctx), x, batch, 1e-4, **kw)
+    ctx.zipml_sync()
+    # (a last-bit difference in a norm may flip a draw that sits on its threshold, by one unit of one coordinate)
+    assert ctx.zipml_last_kernel() == kernel and rel(x.cpu().numpy(), x_ref) <= 20 * MODEL_TOL
+
+
 REGS = [(binding.REG_L2, 0.5), (binding.REG_L1, 0.02), (binding.REG_NONNEG, 0.0), (binding.REG_LSSVM, 0.5)]
 
 
