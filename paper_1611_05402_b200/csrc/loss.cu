@@ -483,9 +483,12 @@ int launch_loss_codes(zipml_ctx* ctx, const zipml_dataset* d, const float* b, co
         // 1,000,000 x 2,048 236 -> 198 (5.2 TB/s), 4 bits 1,000,000 x 1,000 206 -> 197, 8 bits 300,000 x 2,000 279 -> 259; rows of one span (20 codes of 4 bits,
         // 13,421,773 rows) 495 -> 414.  Rows of two to five spans keep to registers, where one row's spans are all in flight at once (8 bits 1,342,178
         // x 200 120 us against 134, 335,545 x 200 40 against 48), and so do warps of about a hundred spans in all, whose start counts: 8 bits 100,000 x 2,100
-        // (102 as counted above) 109 against 113, 4 bits 60,000 x 1,500 (26) 42 against 44; 5 bits 400,000 x 999 (121) 191 against 179.
+        // (102 as counted above) 109 against 113, 4 bits 60,000 x 1,500 (26) 42 against 44; 5 bits 400,000 x 999 (121) 191 against 179.  So do rows of 8-bit
+        // codes that are whole 128-byte lines, of which a warp's requests split none: 524,288 x 1,024 212 against 224 with L2 flushed, 183 against
+        // 200 call after call, 262,144 x 2,048 194 against 211 (at 4 bits stages win the first and lose the second by 4 to 6 %: kept).
         const size_t ring = (size_t)warps * kLossStages * 2048, digit_bytes = (size_t)(8 / cb) * 4 * ((size_t)(vec_bytes + 127) / 128 * 128 + 64);
-        const bool shared = warps == 16 && (spans == 1 || (spans > 5 && least >= 112)) && ring + digit_bytes + 16384 <= (size_t)ctx->smem_optin;
+        const bool lines = cb == 8 && d->row_bytes % 128 == 0;
+        const bool shared = warps == 16 && (spans == 1 || (spans > 5 && least >= 112)) && !lines && ring + digit_bytes + 16384 <= (size_t)ctx->smem_optin;
         const size_t smem = shared ? ring + digit_bytes : 0;
         auto launch = [&](auto digits_kernel, auto kernel) -> int {
             const cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;

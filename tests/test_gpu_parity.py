@@ -1312,6 +1312,19 @@ def test_loss_codes_through_stages_and_without(ctx, m, n, bits):
     assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
 
 
+@pytest.mark.parametrize("n", [1024, 1023, 1008, 384])
+def test_loss_codes_on_rows_of_whole_lines(ctx, n):
+    """8-bit rows that are whole 128-byte lines (no stages), with and without padding in the last one, and rows that are not (stages)."""
+    m = 45_003
+    _, A, b, xs = workload("c2", m, n, seed=2)
+    x = (xs * 0.9).astype(np.float32)
+    ods = oracle.quantize(A, 8, seed=3)
+    want = oracle.loss_codes(ods, b, x)
+    got = ctx.zipml_loss(binding.LOSS_CODES, to_dev(b, ctx), to_dev(x, ctx), data=dev_dataset(ods, ctx))
+    ctx.zipml_sync()
+    assert abs(got.item() - want) <= LOSS_TOL * max(abs(want), oracle.loss_dense(A, b, x))
+
+
 def test_losses_one_after_another_see_their_own_digits(ctx):
     """Losses of several models and shapes (with and without stages; their digits lie elsewhere in the same scratch) with no wait between
     them: each is what it is on an idle device."""
