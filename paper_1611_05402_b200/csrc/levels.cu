@@ -115,7 +115,9 @@ int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64
 // over groups of lanes (32 down to 4 a group: the ranges get shorter; 8 in the last round 15 % slower, 2 as fast on
 // short tails, 1 slower).  The minima, and with
 // ascending scans and strict comparisons the leftmost minimisers, are those of the full scan.
-// The three edges between two neighbours are searched together, on one load of a candidate (7 intervals 155 -> 145 us).
+// The three edges between two neighbours are searched together, on one load of a candidate (7 intervals 155 -> 145 us), but for few bins of
+// many features, whose edges have a group each and whose idle warps rest (20,000 features, 15 intervals: 17 bins 1,067 -> 820 us, 256 bins 2,665 -> 2,470;
+// in one kernel with the other form both took 1.2 to 1.9 times as long).
 // Measured, a call on 3,000 rows (512 features of 1,024 bins) against the full scan: 7 intervals 536 -> 210 us, 15 intervals
 // 1,228 -> 452; bound by the chain of the rounds (load, two multiply-adds, compare, a few shuffles, barrier).
 // ---------------------------------------------------------------------------------------------
@@ -163,9 +165,23 @@ __device__ __forceinline__ void dp_minimise(const double* D, const double* prev,
 }
 
 // One round of a layer: the multiples of S that are not multiples of 4 S, the three between two neighbours of the rounds before at once.
-template <int G, int S>
+// FEW (bins): a group for every edge, and the warps that are left over rest.
+template <int G, int S, bool FEW>
 __device__ __forceinline__ void dp_round(const double* D, const double* prev, double* cur, unsigned short* ak, int k, int M) {
     constexpr int kGroups = kDpThreads / G;
+    if constexpr (FEW) {
+        const int edges = M / (4 * S) * 3 + M % (4 * S) / S;        // (the last may be M itself)
+        for (int q0 = 0; q0 < edges; q0 += kGroups) {
+            const int q = q0 + (int)threadIdx.x / G, below = q / 3 * (4 * S), mm = below + (q % 3 + 1) * S;
+            const bool valid = q < edges && mm >= k && mm < M;
+            if (__any_sync(0xffffffffu, valid)) {
+                const int j_lo = valid && below >= k ? (int)ak[below] : k - 1;
+                dp_minimise<G, 1, S>(D, prev, cur, ak, valid, k, mm, j_lo, valid ? min((int)ak[min(below + 4 * S, M)], mm - 1) : 0);
+            }
+        }
+        __syncthreads();
+        return;
+    }
     const int items = M / (4 * S);                                  // whole intervals; M itself may end a shorter one
     for (int q0 = 0; q0 < items; q0 += kGroups) {
         const int q = q0 + (int)threadIdx.x / G, below = q * 4 * S, above = below + 4 * S;
@@ -183,6 +199,7 @@ __device__ __forceinline__ void dp_round(const double* D, const double* prev, do
     __syncthreads();
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(kDpThreads) levels_dp_kernel(const uint32_t* __restrict__ counts, int bins, int s,
                                                                const float* __restrict__ lo,
                                                                const float* __restrict__ hi,
@@ -250,10 +267,10 @@ __global__ void __launch_bounds__(kDpThreads) levels_dp_kernel(const uint32_t* _
             dp_minimise<32, 1, 1>(D, prev, cur, ak, mm >= k, k, mm, k - 1, mm - 1);
         }
         __syncthreads();
-        dp_round<32, 64>(D, prev, cur, ak, k, M);
-        dp_round<16, 16>(D, prev, cur, ak, k, M);
-        dp_round<8, 4>(D, prev, cur, ak, k, M);
-        dp_round<4, 1>(D, prev, cur, ak, k, M);
+        dp_round<32, 64, FEW>(D, prev, cur, ak, k, M);
+        dp_round<16, 16, FEW>(D, prev, cur, ak, k, M);
+        dp_round<8, 4, FEW>(D, prev, cur, ak, k, M);
+        dp_round<4, 1, FEW>(D, prev, cur, ak, k, M);
         double* t = prev; prev = cur; cur = t;
     }
     if (threadIdx.x == 0) {
@@ -279,10 +296,11 @@ int launch_levels_dp(zipml_ctx* ctx, const uint32_t* counts, int64_t n, int bins
                      const float* hi, float* levels_out, uint64_t* objective_out) {
     const size_t smem = sizeof(double) * 3 * (size_t)(bins + 1) + sizeof(unsigned short) * (size_t)(s + 1) * (bins + 1);
     if (smem > (size_t)ctx->smem_optin) return ZIPML_ERR_WORKSPACE;
-    cudaError_t e = cudaFuncSetAttribute(levels_dp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_status(e);
     if (n > 0x7fffffffLL) return ZIPML_ERR_WORKSPACE;
-    levels_dp_kernel<<<(unsigned)n, kDpThreads, smem, ctx->stream>>>(
+    auto kernel = bins <= 256 && n >= 8ll * ctx->sm_count ? levels_dp_kernel<true> : levels_dp_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_status(e);
+    kernel<<<(unsigned)n, kDpThreads, smem, ctx->stream>>>(
         counts, bins, s, lo, hi, levels_out, reinterpret_cast<unsigned long long*>(objective_out));
     ctx->launches += 1;
     return cuda_status(cudaGetLastError());
