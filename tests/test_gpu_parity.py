@@ -157,6 +157,27 @@ def test_quantize_values_just_above_a_level(ctx, bits):
 
 
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
+@pytest.mark.parametrize("m,n,nonzero", [(1, 1, 1.0), (131, 3, 1.0), (67, 9, 0.05), (40_003, 5, 0.3), (4_099, 33, 0.02), (530, 257, 0.04), (1025, 130, 0.2)], ids=str)
+def test_quantize_onto_levels_where_most_samples_are_certain(ctx, m, n, nonzero, bits):
+    """Rows of few features (their padding is most of what a warp holds), sparse rows, and rows that turn dense after a sparse start or
+    the other way round; features whose lowest level is there twice or whose values are constant."""
+    rng = np.random.default_rng(m + n + bits)
+    A = np.where(rng.random((m, n)) < nonzero, rng.random((m, n)), 0.0).astype(np.float32)
+    A[m // 4: m // 2] = rng.random((m // 2 - m // 4, n), dtype=np.float32)
+    A[-1], A[0] = 1.0, 0.0
+    table = np.sort(rng.random((n, 1 << bits), dtype=np.float32), axis=1)
+    table[:, 0], table[:, -1] = 0.0, 1.0
+    if bits > 1:
+        table[1::3, 1] = 0.0
+    A[:, 2::5] = 0.0
+    ods = oracle.quantize(A, bits, seed=17, mode=oracle.TABLE, levels=table)
+    gds = ctx.zipml_quantize(to_dev(A, ctx), bits, seed=17, level_mode=binding.LEVELS_TABLE, levels=to_dev(table, ctx))
+    ctx.zipml_sync()
+    assert (gds.plane1.cpu().numpy() == ods.plane1).all() and (gds.plane2.cpu().numpy() == ods.plane2).all()
+    assert (gds.feat_lo.cpu().numpy() == ods.feat_lo).all()
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3, 4])
 @pytest.mark.parametrize("width", [0x1d9c282, 0x17b7084 * 2.0 ** 6, 0x1f3d096 * 2.0 ** 12, 0x1eead6c * 2.0 ** 15], ids=["2^24", "2^30", "2^36", "2^39"])
 def test_quantize_where_the_division_just_rounds_to_zero(ctx, width, bits):
     """(x - level) / width is exactly 2^-150, which rounds to 0: no draw takes it up; the next larger x goes up on a draw of 0,
