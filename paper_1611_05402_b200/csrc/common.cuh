@@ -58,19 +58,6 @@ __device__ __forceinline__ uint32_t vector_u24(uint64_t seed, uint32_t epoch, ui
     return b.v[coord & 3u] >> 8;
 }
 
-// Cell and up-probability on a uniform grid of s intervals (s < 2^22): t = (v - lo) * inv with every
-// operation rounded on its own (no contraction into an FMA), cell = clamp(floor t, 0, s-1), p = t - cell.
-// The floor needs no conversion instruction: 2^23 + t' rounded down keeps floor(t') in its mantissa.
-// A NaN lands in cell 0 with p = NaN (never up); -inf in cell 0, +inf in the last cell, always up.
-__device__ __forceinline__ void uniform_cell(float v, float lo, float inv, int s, uint32_t& cell, float& p) {
-    const float t = __fmul_rn(__fsub_rn(v, lo), inv);
-    const float tc = fmaxf(t, 0.0f);                                        // NaN -> 0
-    float fl = __fsub_rn(__fadd_rd(tc, 8388608.0f), 8388608.0f);            // floor(tc), exact for tc < 2^23
-    fl = fminf(fl, (float)(s - 1));
-    cell = __float_as_uint(__fadd_rn(fl, 8388608.0f)) & 0x7FFFFFu;
-    p = __fsub_rn(t, fl);
-}
-
 // Regulariser applied to y = x - lr g, coordinate by coordinate (paper Eq. (proxupdate); reg 4: the
 // least-squares SVM term of the Supplement).  cst is the per-call constant in fp32: 1/(1 + lr c),
 // lr lambda or lr c.  Every operation is one IEEE fp32 rounding.
