@@ -64,10 +64,15 @@ enum {
 };
 /* How zipml_sgd_epoch runs its minibatch chain.  Results do not depend on the choice. */
 enum {
-    ZIPML_ENGINE_AUTO = 0,      /* solo for the smallest steps; cluster where its forms hold the rows;
-                                   else column, else stream, by code width, row length and batch
-                                   (uniform grid, fp32 model and gradient), else ring; lean and
-                                   persistent on level tables no cluster holds                        */
+    ZIPML_ENGINE_AUTO = 0,      /* solo for the smallest steps; cluster where its forms hold the rows.
+                                   Else, uniform grids: column, stream or ring by code width, row length
+                                   and batch (with a quantized model or gradient column or ring), rows
+                                   too wide for these also persistent.  Level tables: lean, persistent or
+                                   ring by width and batch, also for batches that a cluster would hold
+                                   but takes longer for.  The choice follows the data's shape, its codes
+                                   and the batch, not the range of steps a call takes (an epoch in
+                                   several calls stays on one engine); a call with model_out does without
+                                   the stream and column engines                                      */
     ZIPML_ENGINE_STEPWISE = 1,  /* a few kernel launches per minibatch                               */
     ZIPML_ENGINE_PERSISTENT = 2, /* one cooperative launch per call, grid barriers between the phases */
     ZIPML_ENGINE_RING = 3,       /* one cooperative launch; producer warp streams code chunks through a
@@ -88,16 +93,18 @@ enum {
                                     model or gradient, batches above 8192 rows.
                                     zipml_sgd_params.stream_prefetch overrides how many eighths of the
                                     next step's tile are requested into L2 ahead of time               */
-    ZIPML_ENGINE_COLUMN = 7,     /* one cooperative launch for large tiles on uniform grids with an fp32
-                                    model and gradient, rows of 128 bytes .. 128 bytes x the number of
-                                    SMs: a CTA owns a 128-byte column block of the packed rows for the
+    ZIPML_ENGINE_COLUMN = 7,     /* one cooperative launch for large tiles on uniform grids, rows of
+                                    128 bytes .. 128 bytes x the number of SMs: a CTA owns a 128-byte column block of the packed rows for the
                                     whole launch; chunks of rows visit shared memory once for the dots
                                     and once more, out of L2, for the gradient, so the codes are read
                                     from HBM once per step; CTAs exchange only the rows' dots (integer
                                     atomics that count their own completion), there is no grid-wide
                                     barrier.  The only engine that takes ZIPML_LAYOUT_COLUMN_BLOCKS
                                     (where its copies are contiguous; AUTO picks it for such data).
-                                    ZIPML_ERR_WORKSPACE for what it does not cover (as for STREAM)     */
+                                    A quantized model or gradient it takes on row-major planes from AUTO;
+                                    asked for by name it answers ZIPML_ERR_WORKSPACE to them, on column
+                                    blocks ZIPML_ERR_UNSUPPORTED.  ZIPML_ERR_WORKSPACE for what else it
+                                    does not cover (as for STREAM)                                     */
     ZIPML_ENGINE_SOLO = 8        /* one thread block for the whole chain: steps so small that handing
                                    values between SMs costs more than their arithmetic.
                                    ZIPML_ERR_WORKSPACE for more than 2,048 features or tiles above 48 KiB
@@ -174,7 +181,9 @@ typedef struct zipml_sgd_params {
                                    mark 4.  Stream engine: 0 step start, 1 own dots added, 2 barrier
                                    passed, 3 residual digits ready, 4 own gradient blocks summed,
                                    5 model updated and digits published, 6 dots and labels read,
-                                   7 residual scale known.  Column engine (the buffer must be zeroed):
+                                   7 residual scale known.  Column engine (the buffer must be zeroed;
+                                   AUTO may take this engine, for quantized vectors too: see
+                                   zipml_last_engine):
                                    0 clock at the step's first dots, 7 clock when the next w is out;
                                    cycles that warp 0 of a role spent waiting in the step: 1 A warp
                                    for first-visit copies, 2 R warp for complete dots (of its chunks),
@@ -195,7 +204,7 @@ typedef struct zipml_sgd_params {
                                    eighths of the next step's tile into L2 ahead of time             */
     int32_t column_chunk_rows;  /* tuning, column engine: 0 = automatic, else rows of a minibatch that
                                    travel through shared memory together (a multiple of 32; values
-                                   above 128 count as 128)                                            */
+                                   above 128 count as 128, 96 as 64 where a step has several chunks)  */
     int32_t vector_norm;        /* scale M(v) of Q3 and Q4 (Supplement Eq. (quant2) leaves it general):
                                    ZIPML_NORM_L2 = ||v||_2, the paper's choice and the default;
                                    ZIPML_NORM_LINF = max |v_i| (lower variance; the largest entry is exact).
