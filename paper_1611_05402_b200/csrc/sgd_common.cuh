@@ -79,6 +79,18 @@ __device__ __forceinline__ void after_previous_kernel(int64_t steps) {
     if (steps <= kEarlySteps) asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The same pointer, known to the compiler only from here on; and an ordinary load through one, which is scheduled as freely as a read-only
+// one: nothing that the kernel writes lies there.
+__device__ __forceinline__ const float* from_here_on(const float* p) {
+    asm volatile("" : "+l"(p));
+    return p;
+}
+__device__ __forceinline__ float load_freely(const float* p) {
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
