@@ -307,8 +307,9 @@ static int wide_rows_engine(const zipml_ctx* ctx, const zipml_dataset* d, const 
 // C 29.4 R 34.5, x 2,000 41 / 36; 4 KB x 2,000 42 / 41; 6 KB x 3,000 56 / 56; 8 KB x 4,500 87 / 93.  4 bits 4.1 KB x 64 C 9.1 R 22, x 1,200
 // 16.5 / 33, x 3,600 39 / 40, x 4,500 46 / 44, 5 KB x 4,500 47 / 48; 9 KB x 8,192 86 / 85; 16 KB x 64 10.7 / 31, x 8,192 92 / 145.  8 bits 9 KB x 64
 // 9.4 / 21; rows of an odd multiple of 16 bytes, whose pieces begin in the middle of a sector: 4,112 bytes x 2,400 26 / 28, x 3,000 32 / 30, 6,512 x 3,000 35 / 34,
-// 8,016 x 2,700 1.07 times R, 9,008 x 3,000 37 / 36; others: 4,160 bytes x 3,000 0.95 times R, x 3,500 1.05, 6,528 x 4,500 1.04, 8,000 x 4,500
-// 41 / 41, 9,024 x 4,500 0.88; 12 KB x 6,000 49 / 68.  (With a quantized model too C takes some 3 more, R 6.)
+// 8,016 x 2,700 1.07 times R, 9,008 x 3,000 37 / 36; others: 4,160 bytes x 3,000 0.95 times R, x 3,500 1.05, 6,528 x 4,000 0.99, x 4,500 1.04, 8,000 x 4,000
+// 37 / 38, 9,024 x 4,500 0.88; 12 KB x 6,000 49 / 68.  (With a quantized model too C takes some 3 more, R 6; single steps cost C some 7 more, R 5: at
+// the lines 0.07 to 0.15 of a step.)
 static bool column_pays_quantized(const zipml_dataset* d, const zipml_sgd_params* p, int64_t B, int64_t T) {
     if (d->level_mode != ZIPML_LEVELS_UNIFORM || (p->model_bits == 0 && p->grad_bits == 0)) return false;
     // (a quantized gradient alone on data of up to three batches: the choice of the ring engine is a pinned one, not the faster.  The batches
@@ -316,8 +317,10 @@ static bool column_pays_quantized(const zipml_dataset* d, const zipml_sgd_params
     if (p->model_bits == 0 && T <= 3) return false;
     const int cb = container_bits(d->bits);
     if (cb == 2) return B <= 1500 || 2 * B <= d->row_bytes;
-    if (cb == 4) return B <= 4000 || 10 * B <= 9 * d->row_bytes;
-    return d->row_bytes >= 11000 || B <= (d->row_bytes % 32 != 0 ? 2500 : d->row_bytes < 6000 ? 3200 : 4500);
+    if (cb == 4) return B <= 4000 || 10 * B <= (d->row_bytes >= 8000 ? 9 : 7) * d->row_bytes;
+    if (d->row_bytes >= 11000) return true;
+    if (d->row_bytes % 32 != 0) return B <= (d->row_bytes < 9000 ? 2500 : 3200);
+    return B <= (d->row_bytes < 6000 ? 3200 : d->row_bytes < 9000 ? 4000 : 4500);
 }
 
 // Small steps that the cluster engine declined: row parts that meet through L2 (lean), or the ring's or grid's 148 CTAs.
