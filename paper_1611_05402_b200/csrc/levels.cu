@@ -116,7 +116,7 @@ int launch_histogram(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, int64
 // short tails, 1 slower).  The minima, and with
 // ascending scans and strict comparisons the leftmost minimisers, are those of the full scan.
 // The three edges between two neighbours are searched together, on one load of a candidate (7 intervals 155 -> 145 us), but for few bins of
-// many features, whose edges have a group each and whose idle warps rest (20,000 features, 15 intervals: 17 bins 1,067 -> 820 us, 256 bins 2,665 -> 2,470;
+// many features, whose edges have a group each and whose idle warps rest (20,000 features, 15 intervals: 17 bins 1,067 -> 683 us, 256 bins 2,665 -> 2,265;
 // in one kernel with the other form both took 1.2 to 1.9 times as long).
 // Measured, a call on 3,000 rows (512 features of 1,024 bins) against the full scan: 7 intervals 536 -> 210 us, 15 intervals
 // 1,228 -> 452; bound by the chain of the rounds (load, two multiply-adds, compare, a few shuffles, barrier).

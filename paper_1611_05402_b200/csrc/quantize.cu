@@ -173,12 +173,12 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 //     done by whoever draws, saves conversions and loses more to shared memory, which was 87 % busy: 148 us per
 //     4,096 x 32,768, now 134.)
 // Level tables: the block's tables are staged in shared memory as [feature of the thread][level][thread column], so
-// that a warp's look-ups are free of bank conflicts whatever its codes are; the cell is found by bisection, whose offset is the cell's
+// that a warp's look-ups are free of bank conflicts whatever its codes are (from 32 thread columns on; of fewer, two rows' lanes share a column's bank); the cell is found by bisection, whose offset is the cell's
 // number times 256, and p by a multiplication with the staged reciprocal of the cell's width, corrected (quotient below).
 // Blocks with a cell too narrow or too wide for that divide instead; a quotient too small for it is between 0 and
 // 2^-24 anyway, and its threshold is 1 if the numerator lies above the staged one from which on the division does not round to 0 and 0 if not
 // (a numerator of exactly width 2^-150, half of the smallest number, comes out of the correction as 0 or not).  No calls, and no branch a
-// sample: 85 -> 71 instructions a sample, 890 -> 655 us on 500,000 x 512 at 3 bits.  Such a
+// sample: 85 -> 71 instructions a sample, 890 -> 655 us (665 with the thresholds of the smallest quotients exact) on 500,000 x 512 at 3 bits.  Such a
 // call needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
 // non-finite values, are gathered on the way.
 // What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 62 %; 24 warps per SM: fewer

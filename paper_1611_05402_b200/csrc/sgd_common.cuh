@@ -73,7 +73,7 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 // In a kernel that early_start may launch, and by all of its threads: what comes before this may run while the kernel before it on the stream
 // still does, and so touches no global memory.  After it that kernel has ended and its writes are seen -- by ordinary loads: the read-only path
 // (__ldg) wants what does not change while the kernel lives -- and the next one may start in turn (two at most
-// are on the device).  Sixteen single steps of 256 x 1,000, gradient and application each a launch: 242 us -> 222, of which the host's launches
+// are on the device).  Sixteen single steps of 256 x 1,000, gradient and application each a launch: 242 us (240 to 249 from device to device) -> 222, of which the host's launches
 // are the most; 512 x 8,000 a step 18.8 -> 16.6, 128 x 32,768 29.0 -> 26.8.  (Not in the solo kernel, whose epochs lost 0.4 to 2 % to it.)
 __device__ __forceinline__ void after_previous_kernel(int64_t steps) {
     if (steps <= kEarlySteps) asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
