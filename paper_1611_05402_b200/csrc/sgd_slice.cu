@@ -196,9 +196,12 @@ __global__ void __launch_bounds__(kSliceThreads + 32, 1) sgd_slice_kernel(const 
     int batch = batch_at(0), batch_next = batch_at(1);
     // labels: a lane of the first rb warps forms one residual, of this row of the CTA
     const int res_row = warp * 16 + 2 * ((lane >> 2) & 3) + (lane & 1) + 8 * ((lane >> 1) & 1);
-    const float* labels = from_here_on(a.b);
+    // (MANY: where the load stands suits it, moved it costs 1 % a step: 8,192 x 1,999 at 6 bits 643 -> 648 us an epoch; else it has to move: 2 bits
+    // 500 x 256 3.53 -> 3.34 us)
+    const float* labels = MANY ? a.b : from_here_on(a.b);
     auto label_of = [&](int batch, int chunk) {
-        return warp < rb && res_row < rows_of(batch, chunk) ? load_freely(labels + batch * a.batch + row_base + chunk * a.cr + res_row) : 0.0f;
+        if constexpr (MANY) return warp < rb && res_row < rows_of(batch, chunk) ? a.b[batch * a.batch + row_base + chunk * a.cr + res_row] : 0.0f;
+        else return warp < rb && res_row < rows_of(batch, chunk) ? load_freely(labels + batch * a.batch + row_base + chunk * a.cr + res_row) : 0.0f;
     };
     float label = label_of(batch, 0);
 
