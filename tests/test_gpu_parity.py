@@ -178,7 +178,7 @@ def test_quantize_onto_levels_where_most_samples_are_certain(ctx, m, n, nonzero,
 
 
 @pytest.mark.parametrize("bits", [1, 2, 3, 4])
-@pytest.mark.parametrize("width", [0x1d9c282, 0x17b7084 * 2.0 ** 6, 0x1f3d096 * 2.0 ** 12, 0x1eead6c * 2.0 ** 15], ids=["2^24", "2^30", "2^36", "2^39"])
+@pytest.mark.parametrize("width", [6.0, 46.0, 0x1d9c282, 0x17b7084 * 2.0 ** 6, 0x1f3d096 * 2.0 ** 12, 0x1eead6c * 2.0 ** 15], ids=["6", "46", "2^24", "2^30", "2^36", "2^39"])
 def test_quantize_where_the_division_just_rounds_to_zero(ctx, width, bits):
     """(x - level) / width is exactly 2^-150, which rounds to 0: no draw takes it up; the next larger x goes up on a draw of 0,
     which each of these seeds makes for one of the samples."""
