@@ -178,7 +178,7 @@ int launch_column_range(zipml_ctx* ctx, const float* A, int64_t m, int64_t n, in
 // Blocks with a cell too narrow or too wide for that divide instead; a quotient too small for it is between 0 and
 // 2^-24 anyway, and its threshold is 1 if the numerator lies above the staged one from which on the division does not round to 0 and 0 if not
 // (a numerator of exactly width 2^-150, half of the smallest number, comes out of the correction as 0 or not).  No calls, and no branch a
-// sample: 85 -> 71 instructions a sample, 890 -> 655 us (665 with the thresholds of the smallest quotients exact) on 500,000 x 512 at 3 bits.  Such a
+// sample: 85 -> 71 instructions a sample, 890 -> 655 us on 500,000 x 512 at 3 bits.  Such a
 // call needs no range pass before this kernel: the feature's extremes, which it returns and which carry the check for
 // non-finite values, are gathered on the way.
 // What bounds it: dense rows, the integer products (that pipe 73 % busy, issue slots 62 %; 24 warps per SM: fewer
@@ -291,13 +291,13 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
             const float val = have ? __ldg(levels + (jb + f) * L + k) : 0.0f;
             const float next = have && k < L - 1 ? __ldg(levels + (jb + f) * L + k + 1) : val;
             const float width = __fsub_rn(next, val);
-            // An empty cell, and one whose width overflows, takes no value up: its width is stored as NaN, and so are its quotients.
+            // An empty cell, and one whose width overflows, takes no value up: its reciprocal is stored as 0, and so are its quotients.
             const bool takes = width > 0.0f && width <= 3.402823466e+38f;
             if (takes && !(width >= 9.1e-13f && width <= 1.09e12f)) divide = true;
             const int at = (fc & 3) * kFeature + k * kCols + (fc >> 2);
             lev_s[at] = k < L - 1 ? val : INFINITY;
             // (a numerator above width 2^-150 has a quotient that is not rounded to 0; at and below it it is)
-            cell_s[at] = make_float4(val, takes ? width : __int_as_float(0x7fffffff), takes ? __frcp_rn(width) : 0.0f,
+            cell_s[at] = make_float4(val, takes ? width : 1.0f, takes ? __frcp_rn(width) : 0.0f,
                                      takes ? __fmul_rd(__fmul_rn(width, 0x1p-75f), 0x1p-75f) : INFINITY);
         }
         divide = __syncthreads_or(divide);
@@ -354,9 +354,9 @@ __global__ void __launch_bounds__(256, 3) quantize_kernel(const float* __restric
                     if (*reinterpret_cast<const float*>(lev + at + half * 256) <= x) at += half * 256;
                 const float4 c = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(cell_s + i * kFeature) + 4 * at);
                 const float num = __fsub_rn(x, c.x);
-                const float p = kDivide ? __fdiv_rn(num, c.y) : quotient(num, c.y, c.z);
+                const float p = kDivide ? (c.z != 0.0f ? __fdiv_rn(num, c.y) : 0.0f) : quotient(num, c.y, c.z);
                 // the upper end (a quotient of 1 or more) is always up
-                uint32_t threshold = __float2uint_ru(num >= c.y ? 16777216.0f : __fmul_rn(p, 16777216.0f));
+                uint32_t threshold = __float2uint_ru(fminf(__fmul_rn(p, 16777216.0f), 16777216.0f));
                 if (!kDivide) threshold = num > c.w ? max(threshold, 1u) : 0u;
                 return __byte_perm(at, 0u, 0x1444) + threshold;
             }
